@@ -281,38 +281,36 @@ template <typename R, typename OT> __device__ __forceinline__ OT to_out(R v) {
 // ------------------------------------------------- per-frequency tables
 // Tridiagonal solve of one frequency block T_k = tridiag(e, d, e), n x n,
 // stored by its row excess sigma = d + 2e and off-diagonal e (Section 3: one
-// tridiagonal system per frequency).  The row is cut into chunks of CH-1
-// unknowns separated by single "separator" unknowns; chunks are solved
-// locally (Thomas with the shared pivots of the constant-coefficient chunk),
-// the separators form a smaller tridiagonal system (Schur complement) solved
-// by cyclic reduction, and each chunk is corrected with its Green's
-// functions.  Everything here is per frequency k and RHS-independent, so the
-// host computes it once in FP64.
-template <typename R, int CH>
-struct TriTab {
-  cx<R> invp[CH];   // 1/p_i, pivots of the chunk LU (prefix-shared by all sizes)
-  cx<R> bp[CH];     // e/p_i
-  cx<R> fc[CH];     // -e * (T_c^{-1} e_1)_i, regular chunk size c = CH-1
-  cx<R> fl[CH];     // -e * (T_cl^{-1} e_1)_i, last chunk size cl
-  cx<R> e;          // off-diagonal
-  cx<R> sig_reg, off_reg;    // separator rows with regular chunks on both sides
-  cx<R> sig_last, off_last;  // last separator row (regular | last chunk)
-};
-
-// Recursive form for rows whose separator systems are again regular
-// (n + 1 a power of CH times a chunk count at every level, e.g. n = 2^p - 1):
-// level l is the constant-coefficient system (sigma_l, e_l) of the level-(l-1)
-// separators, cut again into chunks of CH-1 unknowns plus a separator, down
-// to a last level of at most CH-1 unknowns solved by one Thomas sweep.  Per
-// level: chunk pivots, Green's function and off-diagonal.
+// tridiagonal system per frequency), by recursive substructuring: the row is
+// cut into chunks of CH-1 unknowns, each followed by a single "separator"
+// unknown, and a last chunk of 1 .. CH unknowns; chunks are solved locally
+// (Thomas with the shared pivots of the constant-coefficient chunk), the
+// separators form a smaller tridiagonal system (Schur complement) of the same
+// kind, solved the same way one level up, and each chunk is corrected with
+// its Green's functions.  Down to a last level of at most CH unknowns, which
+// is a single last chunk.
+//
+// The class that is closed under this step is the constant-coefficient
+// system (sigma, e) whose last row alone has another diagonal, written
+// sigma_L - e - o_L (excess sigma_L, virtual right coupling o_L; level 0 has
+// sigma_L = sigma, o_L = e): so any n >= 1 is served, and n + 1 a multiple of
+// CH at every level is the case in which the last chunk is like the others.
+// Everything here is per frequency k and RHS-independent, so the host
+// computes it once in FP64.  Zeros in the tables keep the device code free of
+// lengths: invp[CH-1] = 0 clears a chunk's separator slot, invt and fl are
+// zero past the last chunk's end.
 constexpr int kRecLevels = 6;
 template <typename R, int CH>
-struct RecTab {
-  cx<R> invp[kRecLevels][CH];
-  cx<R> bp[kRecLevels][CH];
-  cx<R> fc[kRecLevels][CH];
-  cx<R> e[kRecLevels];
+struct RecLev {
+  cx<R> invp[CH];   // 1/p_i, pivots of the chunk LU, i < CH-1
+  cx<R> invt[CH];   // the same for the last chunk (its last pivot differs)
+  cx<R> bp[CH];     // e/p_i, shared by both
+  cx<R> fc[CH];     // -e (T_c^{-1} e_1)_i, regular chunk of c = CH-1 unknowns
+  cx<R> fl[CH];     // the same for the last chunk
+  cx<R> e;          // off-diagonal
+  cx<R> pad;
 };
+// The table of frequency k is tab[k levels .. k levels + levels).
 
 // Factor L1 of the four-step FP32 time transform, ell = L1 L2 (ell = 256 ...
 // 4096, L1 >= L2, both in {16, 32, 64}).
@@ -320,13 +318,16 @@ __host__ __device__ constexpr int four_l1(int64_t ell) {
   return ell >= 2048 ? 64 : (ell >= 512 ? 32 : 16);
 }
 
-// Level-0 coefficients of the recursive form (RecTab level 0, FP32) for the
+// Level-0 coefficients of the recursive form (RecLev level 0, FP32) for the
 // fused four-step apply, as float4 pairs in structure-of-arrays order: pair j
 // of frequency k at fuse32[j * ell + (k mod L1) L2 + k / L1], so that the
 // frequencies k = k1 + L1 k2 (k1 fixed) that one CTA of the transform holds
 // are adjacent.  Pairs 0-7: (invp_0, invp_1) ... (invp_14, e); pairs 8-14:
-// (bp_0, bp_1) ... (bp_12, bp_13); pairs 15-22: (fc_0, fc_1) ... (fc_14, 0).
-constexpr int kFusePairs = 23;
+// (bp_0, bp_1) ... (bp_12, bp_13); pairs 15-22: (fc_0, fc_1) ... (fc_14, bp_14);
+// pairs 23-30: (invt_0, invt_1) ... (invt_14, invt_15); pairs 31-38: the same
+// of fl (the last chunk of a row whose n + 1 is no multiple of 16).
+constexpr int kFusePairs = 23, kFusePairsRagged = 39;
+constexpr int kFuseTailInv = 23, kFuseTailGreen = 31;
 
 // Stencil of the block circulant P (Section 3) for the compensated
 // residual: block A_j (time lag j, j < taps) is c0_j on the diagonal and c1_j
@@ -360,12 +361,10 @@ struct Ctx {
   int P32 = 1, P64 = 1;      // chunks per row
 
   // device-side constants (owned)
-  void *tab32 = nullptr;   // TriTab<float, ch32>[nk]; the transposed symbols are their conjugates
-  void *tab64 = nullptr;   // TriTab<double, ch64>[nk]
-  void *rec32 = nullptr;   // RecTab<float, ch32>[nk] when the recursive form applies
-  void *rec64 = nullptr;   // RecTab<double, ch64>[nk]
-  void *fuse32 = nullptr;  // float4[kFusePairs][ell]: level-0 tables of the fused apply
-  int lev32 = 0, lev64 = 0;             // levels of the recursive form (0: not applicable)
+  void *rec32 = nullptr;   // RecLev<float, ch32>[nk][lev32]; the transposed symbols are their conjugates
+  void *rec64 = nullptr;   // RecLev<double, ch64>[nk][lev64]
+  void *fuse32 = nullptr;  // float4[kFusePairs(Ragged)][ell]: level-0 tables of the fused apply
+  int lev32 = 1, lev64 = 1;             // levels of the recursive form
   int clu32 = 1, clu64 = 1;             // CTAs per row (cluster size) for rows beyond one CTA
   int cta32 = 0, cta64 = 0;             // threads per CTA in the cluster form
   int lsz32[kRecLevels] = {0}, lsz64[kRecLevels] = {0};   // unknowns per level
@@ -502,7 +501,7 @@ cudaError_t launch_tridiag(const Ctx &c, void *spec, int prec, int transpose,
                            cudaStream_t s);
 // The FP32 apply with the tridiagonal solves folded into the four-step
 // transform (ell = 256 ... 4096 a power of two, the recursive form of the
-// solve, n + 1 = 16 P): forward transform + level-0 chunk solves into spec
+// solve with at least two levels): forward transform + level-0 chunk solves into spec
 // and the chunks' separator data into sep, the separator system per
 // frequency (into sep as well), corrections + inverse transform.  sep
 // (fused_sep_bytes) lies fused_sep_offset(c) bytes after spec: the spectrum

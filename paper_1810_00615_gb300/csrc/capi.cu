@@ -88,150 +88,116 @@ void excess_form(const Ctx &c, const cd &cM, double cK, cd &sig, cd &e) {
 template <typename R>
 cx<R> to_cx(const cd &z) { return aao::mk((R)z.real(), (R)z.imag()); }
 
-// Thomas solve on a chunk of `len` unknowns with the shared pivots.
-void chunk_solve(const std::vector<cd> &invp, const std::vector<cd> &bp, const cd &e,
-                 const std::vector<cd> &rhs, int len, std::vector<cd> &out) {
-  out.assign(len, cd(0, 0));
-  out[0] = rhs[0] * invp[0];
-  for (int i = 1; i < len; i++) out[i] = (rhs[i] - e * out[i - 1]) * invp[i];
-  for (int i = len - 2; i >= 0; i--) out[i] = out[i] - bp[i] * out[i + 1];
+// Chunks of a system of m unknowns with chunk length CH (CH-1 unknowns + one
+// separator, the last chunk 1 .. CH unknowns): the number of separators.
+int64_t separators(int64_t m, int CH) { return m >= CH + 1 ? (m - 1 - CH) / CH + 1 : 0; }
+
+// The table construction runs 2 CH dependent complex operations per level and
+// frequency, so it uses the plain complex struct: std::complex products and
+// quotients carry NaN and overflow recoveries that cost more than the
+// arithmetic (a context at n 1568, ell 1440 took 3.4 ms to make with them,
+// 1.4 ms with these).
+using zd = cx<double>;
+inline zd zrecip(zd a) {
+  const double d = 1.0 / (a.re * a.re + a.im * a.im);
+  return aao::mk(a.re * d, -a.im * d);
+}
+template <typename R>
+cx<R> to_cx(zd z) { return aao::mk((R)z.re, (R)z.im); }
+
+// Thomas solve on a chunk of `len` unknowns: pivots 1/p_i and e/p_i; every
+// right-hand side entry is b but the first (b0) and the last (bl).
+inline void chunk_solve(const zd *invp, const zd *bp, zd e, zd b0, zd b, zd bl, int len, zd *out) {
+  out[0] = (len == 1 ? bl : b0) * invp[0];
+  for (int i = 1; i < len; i++)
+    out[i] = aao::cfnms(i + 1 < len ? b : bl, e, out[i - 1]) * invp[i];
+  for (int i = len - 2; i >= 0; i--) out[i] = aao::cfnms(out[i], bp[i], out[i + 1]);
 }
 
+// Tables of the recursive form (aao_internal.cuh, RecLev), all in FP64.
+// Level l is the system (sigma, e) with last-row excess sigma_L and virtual
+// right coupling o_L, so its last diagonal is sigma_L - e - o_L.
+//   pivots in excess form: q_0 = sigma - e, q_i = sigma - e q_{i-1}/p_{i-1},
+//     p_i = q_i - e; the last row: q = sigma_L - e q/p (sigma_L - e alone),
+//     p = q - o_L;
+//   Green's functions g = T_c^{-1} e_1 (regular chunk), gl (last chunk), and
+//     w = T_c^{-1} (sigma 1), wl = Tlast^{-1} (sigma, ..., sigma, sigma_L):
+//     1 + e (g_0 + g_{c-1}) = w_0 and 1 + e gl_0 + o_L gl_{cl-1} = wl_0, so
+//     the separators' excesses sigma - 2 e w_0 and sigma - e w_0 - e wl_0
+//     come without cancellation;
+//   level l+1: off-diagonal -e^2 g_{c-1}, virtual coupling -e o_L gl_{cl-1}.
 template <typename R, int CH>
-void build_tables(const Ctx &c, int64_t cl, std::vector<aao::TriTab<R, CH>> &tabs) {
-  tabs.assign((size_t)c.nk, aao::TriTab<R, CH>{});
-  const int cr = CH - 1;
+void build_rec_tables(const Ctx &c, int levels, const int *lsz,
+                      std::vector<aao::RecLev<R, CH>> &tabs) {
+  tabs.assign((size_t)c.nk * (size_t)levels, aao::RecLev<R, CH>{});
+  constexpr int cr = CH - 1;
+  const zd zero = aao::mk(0.0, 0.0), one = aao::mk(1.0, 0.0);
+  zd invp[CH], bp[CH], invt[CH], g[CH], w[CH], gl[CH], wl[CH];
   for (int64_t k = 0; k < c.nk; k++) {
-    cd cM, sig, e;
+    cd cM, sig0, e0;
     double cK;
     block_symbol(c, k, cM, cK);
-    excess_form(c, cM, cK, sig, e);
-    // pivots of the constant-coefficient LU in excess form:
-    // q_0 = sigma - e, q_i = sigma - e q_{i-1} / p_{i-1}, p_i = q_i - e
-    std::vector<cd> invp(CH), bp(CH);
-    cd q = sig - e, p = q - e;
-    for (int i = 0; i < CH; i++) {
-      if (i > 0) {
-        q = sig - e * q / p;
-        p = q - e;
-      }
-      invp[i] = 1.0 / p;
-      bp[i] = e / p;
-    }
-    std::vector<cd> unit_first(CH, cd(0, 0)), ones(CH, cd(1, 0));
-    unit_first[0] = 1.0;
-    std::vector<cd> gc, wc, gl, wl;
-    chunk_solve(invp, bp, e, unit_first, cr, gc);
-    chunk_solve(invp, bp, e, ones, cr, wc);
-    chunk_solve(invp, bp, e, unit_first, (int)cl, gl);
-    chunk_solve(invp, bp, e, ones, (int)cl, wl);
-    auto &T = tabs[(size_t)k];
-    for (int i = 0; i < CH; i++) {
-      T.invp[i] = to_cx<R>(invp[i]);
-      T.bp[i] = to_cx<R>(bp[i]);
-      T.fc[i] = to_cx<R>(i < cr ? -e * gc[i] : cd(0, 0));
-      T.fl[i] = to_cx<R>(i < cl ? -e * gl[i] : cd(0, 0));
-    }
-    T.e = to_cx<R>(e);
-    // separator rows: sigma' = sigma (1 - e (w_left[0] + w_right[0])),
-    // couplings -e^2 g[len-1] (identity 1 + e (g[0] + g[len-1]) = sigma w[0])
-    T.sig_reg = to_cx<R>(sig * (1.0 - 2.0 * e * wc[0]));
-    T.off_reg = to_cx<R>(-e * e * gc[cr - 1]);
-    T.sig_last = to_cx<R>(sig * (1.0 - e * (wc[0] + wl[0])));
-    T.off_last = to_cx<R>(-e * e * gl[cl - 1]);
-  }
-}
-
-// Tables of the recursive form: level l is (sigma_l, e_l); its chunks of
-// CH-1 unknowns have pivots invp/bp and Green's function g; the separators
-// form level l+1 with sigma_{l+1} = sigma_l (1 - 2 e_l w_l[0]) and
-// e_{l+1} = -e_l^2 g_l[CH-2] (w_l = T^{-1} 1), all in FP64.
-template <typename R, int CH>
-void build_rec_tables(const Ctx &c, int levels, std::vector<aao::RecTab<R, CH>> &tabs) {
-  tabs.assign((size_t)c.nk, aao::RecTab<R, CH>{});
-  const int cr = CH - 1;
-  for (int64_t k = 0; k < c.nk; k++) {
-    cd cM, sig, e;
-    double cK;
-    block_symbol(c, k, cM, cK);
-    excess_form(c, cM, cK, sig, e);
-    auto &T = tabs[(size_t)k];
+    excess_form(c, cM, cK, sig0, e0);
+    zd sig = aao::mk(sig0.real(), sig0.imag()), e = aao::mk(e0.real(), e0.imag());
+    zd sig_l = sig, off_l = e;
     for (int l = 0; l < levels; l++) {
-      std::vector<cd> invp(CH), bp(CH);
-      cd q = sig - e, pv = q - e;
+      auto &V = tabs[(size_t)k * (size_t)levels + (size_t)l];
+      const int M = l + 1 < levels ? lsz[l + 1] : 0;   // separators
+      const int cl = lsz[l] - M * CH;                  // unknowns of the last chunk
+      zd q = sig - e, qp = zero;
       for (int i = 0; i < CH; i++) {
-        if (i > 0) {
-          q = sig - e * q / pv;
-          pv = q - e;
-        }
-        invp[i] = 1.0 / pv;
-        bp[i] = e / pv;
+        if (i > 0) q = sig - e * q * invp[i - 1];
+        invp[i] = zrecip(q - e);
+        bp[i] = e * invp[i];
+        if (i == cl - 2) qp = q * invp[i];
       }
-      std::vector<cd> unit_first(CH, cd(0, 0)), ones(CH, cd(1, 0)), g, w;
-      unit_first[0] = 1.0;
-      chunk_solve(invp, bp, e, unit_first, cr, g);
-      chunk_solve(invp, bp, e, ones, cr, w);
+      for (int i = 0; i < CH; i++) invt[i] = i < cl - 1 ? invp[i] : zero;
+      invt[cl - 1] = zrecip((cl == 1 ? sig_l - e : sig_l - e * qp) - off_l);
+      chunk_solve(invt, bp, e, one, zero, cl == 1 ? one : zero, cl, gl);
+      chunk_solve(invt, bp, e, sig, sig, sig_l, cl, wl);
+      chunk_solve(invp, bp, e, one, zero, zero, cr, g);
+      chunk_solve(invp, bp, e, one, one, one, cr, w);
       for (int i = 0; i < CH; i++) {
-        T.invp[l][i] = to_cx<R>(invp[i]);
-        T.bp[l][i] = to_cx<R>(bp[i]);
-        T.fc[l][i] = to_cx<R>(i < cr ? -e * g[i] : cd(0, 0));
+        V.invp[i] = to_cx<R>(i < cr ? invp[i] : zero);
+        V.invt[i] = to_cx<R>(invt[i]);
+        V.bp[i] = to_cx<R>(bp[i]);
+        V.fc[i] = to_cx<R>(i < cr ? zero - e * g[i] : zero);
+        V.fl[i] = to_cx<R>(i < cl ? zero - e * gl[i] : zero);
       }
-      T.e[l] = to_cx<R>(e);
-      const cd sig_next = sig * (1.0 - 2.0 * e * w[0]);
-      const cd e_next = -e * e * g[cr - 1];
-      sig = sig_next;
-      e = e_next;
+      V.e = to_cx<R>(e);
+      const zd sw = e * sig * w[0];
+      sig_l = sig - sw - e * wl[0];
+      sig = sig - 2.0 * sw;
+      off_l = zero - e * off_l * gl[cl - 1];
+      e = zero - e * e * g[cr - 1];
     }
   }
 }
 
-// Level sizes of the recursive form, or 0 levels if some chunked level is
-// not an exact multiple of CH (then the cyclic-reduction kernel is used).
+// Level sizes of the recursive form.
 int rec_levels(int64_t n, int CH, int *lsz) {
   int levels = 0;
-  int64_t m = n;
-  while (true) {
-    if (levels >= aao::kRecLevels) return 0;
+  for (int64_t m = n; m > 0 && levels < aao::kRecLevels; m = separators(m, CH))
     lsz[levels++] = (int)m;
-    if (m <= CH - 1) break;
-    if ((m + 1) % CH != 0) return 0;
-    m = (m + 1) / CH - 1;
-  }
-  if (levels < 2) return 0;   // a single chunk: the plain kernel is as good
   return levels;
 }
 
-// The recursive kernel stages the whole row in shared memory.
-bool rec_fits(int64_t n, int CH, size_t elem) {
-  return (size_t)((n + 1) / CH) * CH * elem <= 160 * 1024;
-}
-
-// Form of the per-frequency solve: one CTA per row (recursive form when the
-// staged row fits in shared memory), or a cluster of S CTAs of `tpb`
-// threads when the row is longer than one CTA can hold.
+// Form of the per-frequency solve: one CTA per row, or, for a row that one
+// CTA cannot stage in shared memory and that divides into equal chunks, a
+// cluster of S CTAs of `tpb` threads.
 void choose_form(int64_t n, int CH, size_t elem, int tpb, int &lev, int *lsz, int &clu, int &cta) {
   clu = 1;
   cta = 0;
   lev = rec_levels(n, CH, lsz);
-  if (lev == 0) return;
   const int64_t P = (n + 1) / CH;
-  if (P <= 1024 && rec_fits(n, CH, elem)) return;
+  if (P <= 1024 && (size_t)P * CH * elem <= 160 * 1024) return;
+  for (int l = 0; l + 1 < lev; l++)
+    if ((lsz[l] + 1) % CH != 0) return;
+  if (lsz[lev - 1] > CH - 1) return;
   if (P % tpb == 0 && P / tpb >= 2 && P / tpb <= 8) {
     clu = (int)(P / tpb);
     cta = tpb;
-    return;
   }
-  lev = 0;
-}
-
-
-
-// Chunks of a row of n unknowns with chunk length CH (CH-1 unknowns + one
-// separator); returns the chunk count P and the last chunk's size cl.
-void chunking(int64_t n, int CH, int &P, int64_t &cl) {
-  const int64_t M = (n >= CH + 1) ? ((n - 1 - CH) / CH + 1) : 0;
-  P = (int)(M + 1);
-  cl = n - M * CH;
 }
 
 template <typename T>
@@ -361,61 +327,48 @@ cudaError_t upload_dst_tables(Ctx &c) {
 // (Re)compute everything that depends on kappa, the steps or tau.
 int refresh_constants(Ctx &c) {
   // per-frequency tridiagonal tables
-  {
-    int64_t cl;
-    chunking(c.n, c.ch32, c.P32, cl);
-    std::vector<aao::TriTab<float, 16>> t32;
-    build_tables<float, 16>(c, cl, t32);
-    AAO_CK(c, upload(&c.tab32, t32));
-    chunking(c.n, c.ch64, c.P64, cl);
-    if (c.ch64 == 8) {
-      std::vector<aao::TriTab<double, 8>> t64;
-      build_tables<double, 8>(c, cl, t64);
-      AAO_CK(c, upload(&c.tab64, t64));
-    } else {
-      std::vector<aao::TriTab<double, 16>> t64;
-      build_tables<double, 16>(c, cl, t64);
-      AAO_CK(c, upload(&c.tab64, t64));
-    }
-  }
-  // recursive tables where the row structure allows them
+  c.P32 = (int)separators(c.n, c.ch32) + 1;
+  c.P64 = (int)separators(c.n, c.ch64) + 1;
   choose_form(c.n, c.ch32, sizeof(cx<float>), 1024, c.lev32, c.lsz32, c.clu32, c.cta32);
-  if (c.lev32 > 0) {
-    std::vector<aao::RecTab<float, 16>> r32;
-    build_rec_tables<float, 16>(c, c.lev32, r32);
+  {
+    std::vector<aao::RecLev<float, 16>> r32;
+    build_rec_tables<float, 16>(c, c.lev32, c.lsz32, r32);
     AAO_CK(c, upload(&c.rec32, r32));
     // level 0 again, in the layout of the fused four-step apply
     if (c.lev32 >= 2 && c.ell >= 256 && c.ell <= 4096 && (c.ell & (c.ell - 1)) == 0) {
       const int64_t L1 = aao::four_l1(c.ell), L2 = c.ell / L1;
-      std::vector<float4> ft((size_t)aao::kFusePairs * (size_t)c.ell, make_float4(0, 0, 0, 0));
+      const bool ragged = (c.n + 1) % 16 != 0;
+      const int pairs = ragged ? aao::kFusePairsRagged : aao::kFusePairs;
+      std::vector<float4> ft((size_t)pairs * (size_t)c.ell, make_float4(0, 0, 0, 0));
       auto pack = [](const cx<float> &a, const cx<float> &b) {
         return make_float4(a.re, a.im, b.re, b.im);
       };
-      const cx<float> zero = aao::mk(0.f, 0.f);
       for (int64_t k = 0; k < c.nk; k++) {
-        const auto &T = r32[(size_t)k];
+        const auto &T = r32[(size_t)k * (size_t)c.lev32];
         const size_t pos = (size_t)((k % L1) * L2 + k / L1);
         auto at = [&](int j) -> float4 & { return ft[(size_t)j * (size_t)c.ell + pos]; };
-        for (int j = 0; j < 7; j++) at(j) = pack(T.invp[0][2 * j], T.invp[0][2 * j + 1]);
-        at(7) = pack(T.invp[0][14], T.e[0]);
-        for (int j = 0; j < 7; j++) at(8 + j) = pack(T.bp[0][2 * j], T.bp[0][2 * j + 1]);
-        for (int j = 0; j < 7; j++) at(15 + j) = pack(T.fc[0][2 * j], T.fc[0][2 * j + 1]);
-        at(22) = pack(T.fc[0][14], zero);
+        for (int j = 0; j < 7; j++) at(j) = pack(T.invp[2 * j], T.invp[2 * j + 1]);
+        at(7) = pack(T.invp[14], T.e);
+        for (int j = 0; j < 7; j++) at(8 + j) = pack(T.bp[2 * j], T.bp[2 * j + 1]);
+        for (int j = 0; j < 7; j++) at(15 + j) = pack(T.fc[2 * j], T.fc[2 * j + 1]);
+        at(22) = pack(T.fc[14], T.bp[14]);
+        for (int j = 0; ragged && j < 8; j++) {
+          at(aao::kFuseTailInv + j) = pack(T.invt[2 * j], T.invt[2 * j + 1]);
+          at(aao::kFuseTailGreen + j) = pack(T.fl[2 * j], T.fl[2 * j + 1]);
+        }
       }
       AAO_CK(c, upload(&c.fuse32, ft));
     }
   }
   choose_form(c.n, c.ch64, sizeof(cx<double>), 512, c.lev64, c.lsz64, c.clu64, c.cta64);
-  if (c.lev64 > 0) {
-    if (c.ch64 == 8) {
-      std::vector<aao::RecTab<double, 8>> r64;
-      build_rec_tables<double, 8>(c, c.lev64, r64);
-      AAO_CK(c, upload(&c.rec64, r64));
-    } else {
-      std::vector<aao::RecTab<double, 16>> r64;
-      build_rec_tables<double, 16>(c, c.lev64, r64);
-      AAO_CK(c, upload(&c.rec64, r64));
-    }
+  if (c.ch64 == 8) {
+    std::vector<aao::RecLev<double, 8>> r64;
+    build_rec_tables<double, 8>(c, c.lev64, c.lsz64, r64);
+    AAO_CK(c, upload(&c.rec64, r64));
+  } else {
+    std::vector<aao::RecLev<double, 16>> r64;
+    build_rec_tables<double, 16>(c, c.lev64, c.lsz64, r64);
+    AAO_CK(c, upload(&c.rec64, r64));
   }
   // DST-in-space form: cM_k per frequency, (m_j, cK k_j) per mode
   if (c.space == AAO_SPACE_DST) AAO_CK(c, upload_dst_tables(c));
@@ -627,11 +580,6 @@ int check_ws(const Ctx &c, int restart) {
   return AAO_OK;
 }
 
-// The FP32 apply with the tridiagonal solves folded into the four-step
-// transform: forward transform + chunk solves (class FFT_FORWARD), the
-// separator systems (TRIDIAG), corrections + inverse transform
-// (FFT_INVERSE).  Input x (FP64) or x32 (FP32); output YT, with base
-// (FP64 output) y = base - P^{-1} x.
 // Extent checks of the apply's launches (on by default; -DAAO_DEBUG_BOUNDS=0
 // drops them): the bytes each kernel's grid reads or writes in a workspace
 // region, from the launch geometry, against the region's size.  A failure
@@ -664,6 +612,11 @@ bool apply_extents_ok(const Ctx &c, const aao::WsLayout &L, bool fused) {
   return true;
 }
 
+// The FP32 apply with the tridiagonal solves folded into the four-step
+// transform: forward transform + chunk solves (class FFT_FORWARD), the
+// separator systems (TRIDIAG), corrections + inverse transform
+// (FFT_INVERSE).  Input x (FP64) or x32 (FP32); output YT, with base
+// (FP64 output) y = base - P^{-1} x.
 template <typename YT>
 cudaError_t precond_fused(Ctx &c, const double *x, const float *x32, YT *y, int tr,
                           cudaStream_t s, const float *base = nullptr) {
@@ -699,7 +652,7 @@ cudaError_t precond_fused(Ctx &c, const double *x, const float *x32, YT *y, int 
   return run(c, AAO_K_FFT_INVERSE, s, [&] { return inverse(0); });
 }
 
-// One application of P^{-1} (or P^{-T}); with yprev, of P^{-1}(x - E yprev).// One application of P^{-1} (or P^{-T}); with yprev, of P^{-1}(x - E yprev).
+// One application of P^{-1} (or P^{-T}); with yprev, of P^{-1}(x - E yprev).
 // YT = float stores an FP32 result (FP32 preconditioner only): the values
 // the FP32 inverse transform produces are then kept as they are.  With base
 // (FP32 preconditioner, FP64 result) the result is base - P^{-1} x.
@@ -1264,7 +1217,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
 void aao_destroy(aao_ctx *ctx) {
   if (!ctx) return;
   Ctx &c = ctx->c;
-  void *ptrs[] = {c.tab32, c.tab64, c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.beta, c.beta_p,
+  void *ptrs[] = {c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.beta, c.beta_p,
                   c.mv_rows, c.mv_rows_p, c.mv_d0, c.mv_o0,
                   c.sigk, c.sigk32, c.dtw32, c.dtw64, c.dst_cm32, c.dst_cm64,
                   c.dst_mk32, c.dst_mk64};

@@ -62,13 +62,14 @@ cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x3
   auto *sb = sepbuf_of(sep);
   auto *tb = static_cast<const float4 *>(c.fuse32);
   const int P = c.P32, tr = transpose ? 1 : 0;
-  const int rb = (int)sizeof(RecTab<float, fft::kFuseCH>);   // one frequency's table
+  const int ragged = (c.n + 1) % fft::kFuseCH != 0;
+  const int rb = c.lev32 * (int)sizeof(RecLev<float, fft::kFuseCH>);   // one frequency's table
 #define AAO_FS(L)                                                                                  \
   case L:                                                                                          \
     return x ? fft::four_forward_solve<L, double>(c.n, c.n_pad, P, x, sp, sb, c.tw32, s, inter,   \
-                                                  tb, tr, part, c.rec32, rb)                       \
+                                                  tb, tr, ragged, part, c.rec32, rb)                       \
              : fft::four_forward_solve<L, float>(c.n, c.n_pad, P, x32, sp, sb, c.tw32, s, inter,  \
-                                                 tb, tr, part, c.rec32, rb);
+                                                 tb, tr, ragged, part, c.rec32, rb);
   switch (c.ell) {
     AAO_FS(256) AAO_FS(512) AAO_FS(1024) AAO_FS(2048) AAO_FS(4096)
     default: return cudaErrorNotSupported;
@@ -87,12 +88,13 @@ cudaError_t fft_inverse_f32_correct(const Ctx &c, const void *spec, void *sep, d
   const cx<float> *sv = sepsol_of(c, sep);
   auto *tb = static_cast<const float4 *>(c.fuse32);
   const int P = c.P32, tr = transpose ? 1 : 0;
+  const int ragged = (c.n + 1) % fft::kFuseCH != 0;
 #define AAO_IC(L)                                                                               \
   case L:                                                                                       \
     return y ? fft::four_inverse_correct<L, double>(c.n, c.n_pad, P, sp, sv, P, y, c.tw32, s,  \
-                                                    inter, base, tb, tr, part)                  \
+                                                    inter, base, tb, tr, ragged, part)                  \
              : fft::four_inverse_correct<L, float>(c.n, c.n_pad, P, sp, sv, P, y32, c.tw32, s, \
-                                                   inter, nullptr, tb, tr, part);
+                                                   inter, nullptr, tb, tr, ragged, part);
   switch (c.ell) {
     AAO_IC(256) AAO_IC(512) AAO_IC(1024) AAO_IC(2048) AAO_IC(4096)
     default: return cudaErrorNotSupported;

@@ -5,8 +5,9 @@
 //
 // The solve is the recursive substructuring of tridiag.cu: the row of n
 // unknowns is cut into chunks of 15 unknowns, each followed by a separator
-// unknown (n + 1 = 16 P, P chunks, P - 1 separators).  Its three steps map
-// onto the transform:
+// unknown (P chunks, P - 1 separators); where n + 1 is no multiple of 16
+// ("ragged") the last chunk has 1 .. 16 unknowns and tables of its own, which
+// only the CTAs that hold it read.  Its three steps map onto the transform:
 //
 //   forward 2 + local solves: inter -> DFT over t2 -> the half spectrum
 //       X_k (k <= ell/2) of this CTA's 64 real columns, i.e. four chunks of
@@ -150,7 +151,7 @@ constexpr int kInvSeps = 5;     // separators p0-1 .. p0+3 around the CTA's four
 // Forward 2 with the level-0 solves.  grid (ncx / W, L1/2 + 1); fuse_smem
 // bytes of dynamic shared memory.  nchunks = P; spec rows have n_pad >= 16 P
 // elements; sepbuf: P float4 per frequency.
-template <int L, int W>
+template <int L, int W, bool RAGGED>
 __global__ void __launch_bounds__(kFourT, AAO_FUSE_MINB)
 k_fft4_forward2_solve(const cx<float> *__restrict__ inter, cx<float> *__restrict__ spec,
                       float4 *__restrict__ sepbuf, int ncx, int64_t n_pad, int nchunks,
@@ -227,14 +228,31 @@ k_fft4_forward2_solve(const cx<float> *__restrict__ inter, cx<float> *__restrict
     cx<float> e, ip0, ip1;
     unpair(tf[7 * L2], ip0, e);                           // (invp_14, e)
     const cx<float> sep = v[kFuseCH - 1];
-    unpair(tf[0], ip0, ip1);
-    v[0] = v[0] * ip0;
-    v[1] = cfnms(v[1], e, v[0]) * ip1;
+    if (RAGGED && p + 1 == nchunks) {
+      // the last chunk's own pivots, zero past its end, from global memory
+      // (only one column block of the grid gets here); bp_14 beside fc_14
+      const float4 *gt = ft + (size_t)kFuseTailInv * L + G.pos(f);
+      const float sg = conj_sym ? -1.f : 1.f;
 #pragma unroll
-    for (int i = 2; i < kFuseCH - 1; i += 2) {
-      unpair(tf[(i / 2) * L2], ip0, ip1);
-      v[i] = cfnms(v[i], e, v[i - 1]) * ip0;
-      if (i + 1 < kFuseCH - 1) v[i + 1] = cfnms(v[i + 1], e, v[i]) * ip1;
+      for (int i = 0; i < kFuseCH; i += 2) {
+        const float4 iv = __ldg(gt + (size_t)(i / 2) * L);
+        const cx<float> t0 = mk(iv.x, sg * iv.y), t1 = mk(iv.z, sg * iv.w);
+        v[i] = (i > 0 ? cfnms(v[i], e, v[i - 1]) : v[i]) * t0;
+        v[i + 1] = cfnms(v[i + 1], e, v[i]) * t1;
+      }
+      const float4 b14 = __ldg(ft + (size_t)22 * L + G.pos(f));
+      v[14] = cfnms(v[14], mk(b14.z, sg * b14.w), v[15]);
+    } else {
+      unpair(tf[0], ip0, ip1);
+      v[0] = v[0] * ip0;
+      v[1] = cfnms(v[1], e, v[0]) * ip1;
+#pragma unroll
+      for (int i = 2; i < kFuseCH - 1; i += 2) {
+        unpair(tf[(i / 2) * L2], ip0, ip1);
+        v[i] = cfnms(v[i], e, v[i - 1]) * ip0;
+        if (i + 1 < kFuseCH - 1) v[i + 1] = cfnms(v[i + 1], e, v[i]) * ip1;
+      }
+      v[kFuseCH - 1] = mk(0.f, 0.f);
     }
 #pragma unroll
     for (int i = kFuseCH - 4; i >= 0; i -= 2) {           // i = 12, 10, ..., 0
@@ -249,7 +267,6 @@ k_fft4_forward2_solve(const cx<float> *__restrict__ inter, cx<float> *__restrict
     // kept in L2 for the separator kernel that reads it next
     st_hint4(&sepbuf[(size_t)k * nchunks + p], make_float4(v[0].re, v[0].im, part.re, part.im),
              pol_keep);
-    v[kFuseCH - 1] = mk(0.f, 0.f);
   }
   __syncthreads();   // every read of S0/S1 is done: they become the staging rows
   if (live) {
@@ -278,7 +295,7 @@ k_fft4_forward2_solve(const cx<float> *__restrict__ inter, cx<float> *__restrict
 // Corrections + inverse A.  grid (ncx / W, L1/2 + 1).  spec: the local
 // solutions of k_fft4_forward2_solve; sep: the separator values s_p of
 // frequency k at sep[k sstride + p], p < P - 1 (k_tridiag_reduced).
-template <int L, int W>
+template <int L, int W, bool RAGGED>
 __global__ void __launch_bounds__(kFourT, AAO_FUSE_MINB)
 k_fft4_inverseA_correct(const cx<float> *__restrict__ spec, const cx<float> *__restrict__ sep,
                         cx<float> *__restrict__ inter, int ncx, int64_t n_pad, int nchunks,
@@ -370,13 +387,26 @@ k_fft4_inverseA_correct(const cx<float> *__restrict__ spec, const cx<float> *__r
     // v_i + s_{p-1} f_i + s_p f_{14-i}, v_15 = s_p (the staged values are
     // zero left of the first chunk and right of the last)
     const cx<float> sl = sS[f * kInvSeps + q], sr = sS[f * kInvSeps + q + 1];
-    cx<float> fcv[kFuseCH];
+    if (RAGGED && p + 1 == nchunks) {
+      // the last chunk's own Green's function (zero past its end; no
+      // separator follows it)
+      const float4 *gt = ft + (size_t)kFuseTailGreen * L + G.pos(f);
+      const float sg = conj_sym ? -1.f : 1.f;
 #pragma unroll
-    for (int j = 0; j < kFuseCH; j += 2) unpair(sT[(j / 2) * L2 + f], fcv[j], fcv[j + 1]);
+      for (int i = 0; i < kFuseCH; i += 2) {
+        const float4 g2 = __ldg(gt + (size_t)(i / 2) * L);
+        v[i] = cfma(v[i], sl, mk(g2.x, sg * g2.y));
+        v[i + 1] = cfma(v[i + 1], sl, mk(g2.z, sg * g2.w));
+      }
+    } else {
+      cx<float> fcv[kFuseCH];
 #pragma unroll
-    for (int i = 0; i < kFuseCH - 1; i++)
-      v[i] = cfma(cfma(v[i], sl, fcv[i]), sr, fcv[kFuseCH - 2 - i]);
-    v[kFuseCH - 1] = sr;
+      for (int j = 0; j < kFuseCH; j += 2) unpair(sT[(j / 2) * L2 + f], fcv[j], fcv[j + 1]);
+#pragma unroll
+      for (int i = 0; i < kFuseCH - 1; i++)
+        v[i] = cfma(cfma(v[i], sl, fcv[i]), sr, fcv[kFuseCH - 2 - i]);
+      v[kFuseCH - 1] = sr;
+    }
   }
   __syncthreads();   // every read of the staging rows is done: they become S0/S1
   if (active) {
@@ -441,7 +471,7 @@ k_fft4_inverseA_correct(const cx<float> *__restrict__ spec, const cx<float> *__r
 template <int L, typename XT>
 cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *x, cx<float> *spec,
                                float4 *sepbuf, const cx<float> *tw, cudaStream_t s, void *inter,
-                               const float4 *tabs, int conj, int part = 0,
+                               const float4 *tabs, int conj, int ragged, int part = 0,
                                const void *rtab = nullptr, int rtab_bytes = 0) {
   constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2, W = kFourW;
   constexpr size_t sm1 = (size_t)L1 * W * sizeof(cx<float>);
@@ -458,9 +488,10 @@ cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *
     if (e != cudaSuccess) return e;
   }
   if (part != 1) {
-    e = kernel_setup((const void *)k_fft4_forward2_solve<L, W>, kFourT, sm2, nullptr, true);
+    auto kern = ragged ? k_fft4_forward2_solve<L, W, true> : k_fft4_forward2_solve<L, W, false>;
+    e = kernel_setup((const void *)kern, kFourT, sm2, nullptr, true);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_fft4_forward2_solve<L, W>, dim3((unsigned)(ncx / W), L1 / 2 + 1),
+    e = launch_pdl(kern, dim3((unsigned)(ncx / W), L1 / 2 + 1),
                    dim3(kFourT), sm2, s, ip, spec, sepbuf, ncx, n_pad, nchunks, tw,
                    four_discard_ok(ip, spec, n_pad) ? 1 : 0, tabs, conj,
                    static_cast<const char *>(rtab), rtab_bytes);
@@ -476,7 +507,7 @@ template <int L, typename OT>
 cudaError_t four_inverse_correct(int64_t n, int64_t n_pad, int nchunks, const cx<float> *spec,
                                  const cx<float> *sep, int64_t sstride, OT *y, const cx<float> *tw,
                                  cudaStream_t s, void *inter, const float *base,
-                                 const float4 *tabs, int conj, int part = 0) {
+                                 const float4 *tabs, int conj, int ragged, int part = 0) {
   constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2, W = kFourW;
   constexpr size_t sm1 = (size_t)L1 * W * sizeof(cx<float>);
   constexpr size_t sm2 = fuse_smem<L, kInvPairs, kInvSeps>();
@@ -485,9 +516,10 @@ cudaError_t four_inverse_correct(int64_t n, int64_t n_pad, int nchunks, const cx
   const int dis = four_discard_ok(ip, spec, n_pad) ? 1 : 0;
   cudaError_t e = cudaSuccess;
   if (part != 2) {
-    e = kernel_setup((const void *)k_fft4_inverseA_correct<L, W>, kFourT, sm2, nullptr, true);
+    auto kern = ragged ? k_fft4_inverseA_correct<L, W, true> : k_fft4_inverseA_correct<L, W, false>;
+    e = kernel_setup((const void *)kern, kFourT, sm2, nullptr, true);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_fft4_inverseA_correct<L, W>, dim3((unsigned)(ncx / W), L1 / 2 + 1),
+    e = launch_pdl(kern, dim3((unsigned)(ncx / W), L1 / 2 + 1),
                    dim3(kFourT), sm2, s, spec, sep, ip, ncx, n_pad, nchunks, sstride, tw, dis,
                    tabs, conj);
     note_launch();
