@@ -344,6 +344,15 @@ struct CircDF {
   int int_weights;   // 1 where the a_j are those integers (not the literal heat form)
 };
 
+// Four-step factorisation ell = L1 L2 of the run-time time transform
+// (fft_steps.cuh) and the radices of its two short transforms; L = 0 where it
+// does not serve ell.
+struct StepPlan {
+  int L, L1, L2;
+  int np1, np2;
+  int rad1[4], rad2[4];
+};
+
 // ------------------------------------------------------------ context
 struct Ctx {
   int64_t n = 0, ell = 0, N = 0;
@@ -368,6 +377,7 @@ struct Ctx {
   int clu32 = 1, clu64 = 1;             // CTAs per row (cluster size) for rows beyond one CTA
   int cta32 = 0, cta64 = 0;             // threads per CTA in the cluster form
   int lsz32[kRecLevels] = {0}, lsz64[kRecLevels] = {0};   // unknowns per level
+  StepPlan step32{}, step64{};    // run-time four-step transforms (set by fft_plan)
   cx<float> *tw32 = nullptr;      // exp(-2 pi i m/ell), m < ell
   cx<double> *tw64 = nullptr;
   int space = AAO_SPACE_TRIDIAG;  // per-frequency solver
@@ -435,7 +445,7 @@ struct MvRow {
 
 struct WsLayout {
   size_t spec = 0, spec_bytes = 0;
-  size_t inter = 0, inter_bytes = 0;   // two-kernel forward FFT scratch (0: none)
+  size_t inter = 0, inter_bytes = 0;   // four-step FFT scratch (0: none)
   size_t red = 0, red_bytes = 0;
   size_t rf32 = 0;        // refined apply: z0 (N floats)
   size_t rf64 = 0;        // refined apply: residual, Neumann right-hand side (2 x N doubles)
@@ -473,7 +483,8 @@ cudaError_t kernel_setup(const void *kern, int threads, size_t smem, int *reside
 // Time-axis FFTs: x (and, for a Neumann term, the previous iterate y) ->
 // half spectrum; half spectrum -> y.  One instantiation per precision.
 // `inter` (may be NULL: single-kernel transform) is the scratch of the
-// two-kernel forward transform, fft_inter_bytes_* bytes.
+// four-step transforms, fft_inter_bytes_* bytes.
+void fft_plan(Ctx &c);   // sets c.step32 and c.step64 from c.ell
 cudaError_t fft_forward_f32(const Ctx &c, const double *x, const double *yprev, void *spec,
                             cudaStream_t s, void *inter = nullptr);
 cudaError_t fft_inverse_f32(const Ctx &c, const void *spec, double *y, cudaStream_t s,
@@ -491,8 +502,10 @@ cudaError_t fft_forward_f32_yf(const Ctx &c, const double *x, const float *yprev
 // Does the four-step FP32 transform serve this context's ell (a power of
 // two, 256 ... 4096, and the kernels built in)?
 bool fft_four_supported(const Ctx &c);
+// Is there a forward transform of an FP32 block vector for this ell?
+bool fft_f32_input_supported(const Ctx &c);
 // FP32 block vector -> FP32 half spectrum by the four-step kernels
-// (cudaErrorNotSupported for other lengths or without scratch).
+// (cudaErrorNotSupported where none serves the length, or without scratch).
 cudaError_t fft_forward_f32_from_f32(const Ctx &c, const float *x, void *spec, cudaStream_t s,
                                      void *inter);
 cudaError_t fft_inverse_f32_to_f32(const Ctx &c, const void *spec, float *y, cudaStream_t s,
@@ -506,14 +519,16 @@ cudaError_t launch_tridiag(const Ctx &c, void *spec, int prec, int transpose,
 // frequency (into sep as well), corrections + inverse transform.  sep
 // (fused_sep_bytes) lies fused_sep_offset(c) bytes after spec: the spectrum
 // region is sized for complex128 and FP32 uses its first half.  Exactly one
-// of x / x32 and of y / y32 is given; base (FP64 y only): y = base - result.
+// of x / x32 and, for the result, of y / y32 is given; base (FP64 y only): y =
+// base - result.  The forward half also takes a Neumann iterate y or y32 beside
+// x: it then transforms x - E y.
 bool fft_fused_supported(const Ctx &c);
 size_t fused_sep_offset(const Ctx &c);
 size_t fused_sep_bytes(const Ctx &c);
 // part: 0 both kernels of the half, 1 the first, 2 the second.
-cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x32, void *spec,
-                                  void *sep, int transpose, cudaStream_t s, void *inter,
-                                  int part = 0);
+cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x32,
+                                  const double *y, const float *y32, void *spec, void *sep,
+                                  int transpose, cudaStream_t s, void *inter, int part = 0);
 cudaError_t launch_tridiag_reduced_fused(const Ctx &c, void *sep, int transpose, cudaStream_t s);
 cudaError_t launch_tridiag_reduced(const Ctx &c, const void *sepbuf, void *sepsol, int transpose,
                                    cudaStream_t s);

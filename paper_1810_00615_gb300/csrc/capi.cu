@@ -92,26 +92,40 @@ cx<R> to_cx(const cd &z) { return aao::mk((R)z.real(), (R)z.imag()); }
 // separator, the last chunk 1 .. CH unknowns): the number of separators.
 int64_t separators(int64_t m, int CH) { return m >= CH + 1 ? (m - 1 - CH) / CH + 1 : 0; }
 
-// The table construction runs 2 CH dependent complex operations per level and
-// frequency, so it uses the plain complex struct: std::complex products and
-// quotients carry NaN and overflow recoveries that cost more than the
-// arithmetic (a context at n 1568, ell 1440 took 3.4 ms to make with them,
-// 1.4 ms with these).
-using zd = cx<double>;
-inline zd zrecip(zd a) {
-  const double d = 1.0 / (a.re * a.re + a.im * a.im);
-  return aao::mk(a.re * d, -a.im * d);
+// Four complex numbers, one per frequency.  The table construction is a chain
+// of about 2 CH dependent operations per level, so it runs four frequencies
+// side by side, in plain arithmetic: std::complex products and quotients
+// carry NaN and overflow recoveries that cost more than the arithmetic.
+struct zq {
+  double re[4], im[4];
+};
+template <class F>
+inline zq zmap(F &&f) {
+  zq z;
+  for (int u = 0; u < 4; u++) f(u, z.re[u], z.im[u]);
+  return z;
 }
-template <typename R>
-cx<R> to_cx(zd z) { return aao::mk((R)z.re, (R)z.im); }
-
-// Thomas solve on a chunk of `len` unknowns: pivots 1/p_i and e/p_i; every
-// right-hand side entry is b but the first (b0) and the last (bl).
-inline void chunk_solve(const zd *invp, const zd *bp, zd e, zd b0, zd b, zd bl, int len, zd *out) {
-  out[0] = (len == 1 ? bl : b0) * invp[0];
-  for (int i = 1; i < len; i++)
-    out[i] = aao::cfnms(i + 1 < len ? b : bl, e, out[i - 1]) * invp[i];
-  for (int i = len - 2; i >= 0; i--) out[i] = aao::cfnms(out[i], bp[i], out[i + 1]);
+inline zq operator-(const zq &a, const zq &b) {
+  return zmap([&](int u, double &r, double &i) { r = a.re[u] - b.re[u]; i = a.im[u] - b.im[u]; });
+}
+inline zq operator*(const zq &a, const zq &b) {
+  return zmap([&](int u, double &r, double &i) {
+    r = a.re[u] * b.re[u] - a.im[u] * b.im[u];
+    i = a.re[u] * b.im[u] + a.im[u] * b.re[u];
+  });
+}
+inline zq fnms(const zq &a, const zq &b, const zq &c) {   // a - b c
+  return zmap([&](int u, double &r, double &i) {
+    r = a.re[u] - b.re[u] * c.re[u] + b.im[u] * c.im[u];
+    i = a.im[u] - b.re[u] * c.im[u] - b.im[u] * c.re[u];
+  });
+}
+inline zq recip(const zq &a) {
+  return zmap([&](int u, double &r, double &i) {
+    const double d = 1.0 / (a.re[u] * a.re[u] + a.im[u] * a.im[u]);
+    r = a.re[u] * d;
+    i = -a.im[u] * d;
+  });
 }
 
 // Tables of the recursive form (aao_internal.cuh, RecLev), all in FP64.
@@ -131,45 +145,70 @@ void build_rec_tables(const Ctx &c, int levels, const int *lsz,
                       std::vector<aao::RecLev<R, CH>> &tabs) {
   tabs.assign((size_t)c.nk * (size_t)levels, aao::RecLev<R, CH>{});
   constexpr int cr = CH - 1;
-  const zd zero = aao::mk(0.0, 0.0), one = aao::mk(1.0, 0.0);
-  zd invp[CH], bp[CH], invt[CH], g[CH], w[CH], gl[CH], wl[CH];
-  for (int64_t k = 0; k < c.nk; k++) {
-    cd cM, sig0, e0;
-    double cK;
-    block_symbol(c, k, cM, cK);
-    excess_form(c, cM, cK, sig0, e0);
-    zd sig = aao::mk(sig0.real(), sig0.imag()), e = aao::mk(e0.real(), e0.imag());
-    zd sig_l = sig, off_l = e;
+  const zq zero = zmap([](int, double &r, double &i) { r = i = 0.0; });
+  const zq one = zmap([](int, double &r, double &i) { r = 1.0; i = 0.0; });
+  zq invp[CH], bp[CH], invt[CH], g[CH], w[CH], gl[CH], wl[CH], fc[CH], fl[CH];
+  for (int64_t k0 = 0; k0 < c.nk; k0 += 4) {
+    const int cnt = (int)std::min<int64_t>(4, c.nk - k0);
+    zq sig = one, e = one;
+    for (int u = 0; u < 4; u++) {
+      cd cM, s0, e0;
+      double cK;
+      block_symbol(c, k0 + (u < cnt ? u : 0), cM, cK);
+      excess_form(c, cM, cK, s0, e0);
+      sig.re[u] = s0.real(); sig.im[u] = s0.imag();
+      e.re[u] = e0.real(); e.im[u] = e0.imag();
+    }
+    zq sig_l = sig, off_l = e;
     for (int l = 0; l < levels; l++) {
-      auto &V = tabs[(size_t)k * (size_t)levels + (size_t)l];
       const int M = l + 1 < levels ? lsz[l + 1] : 0;   // separators
       const int cl = lsz[l] - M * CH;                  // unknowns of the last chunk
-      zd q = sig - e, qp = zero;
+      zq q = sig - e, qp = zero;
       for (int i = 0; i < CH; i++) {
-        if (i > 0) q = sig - e * q * invp[i - 1];
-        invp[i] = zrecip(q - e);
+        if (i > 0) q = fnms(sig, e, q * invp[i - 1]);
+        invp[i] = recip(q - e);
         bp[i] = e * invp[i];
         if (i == cl - 2) qp = q * invp[i];
       }
       for (int i = 0; i < CH; i++) invt[i] = i < cl - 1 ? invp[i] : zero;
-      invt[cl - 1] = zrecip((cl == 1 ? sig_l - e : sig_l - e * qp) - off_l);
-      chunk_solve(invt, bp, e, one, zero, cl == 1 ? one : zero, cl, gl);
-      chunk_solve(invt, bp, e, sig, sig, sig_l, cl, wl);
-      chunk_solve(invp, bp, e, one, zero, zero, cr, g);
-      chunk_solve(invp, bp, e, one, one, one, cr, w);
-      for (int i = 0; i < CH; i++) {
-        V.invp[i] = to_cx<R>(i < cr ? invp[i] : zero);
-        V.invt[i] = to_cx<R>(invt[i]);
-        V.bp[i] = to_cx<R>(bp[i]);
-        V.fc[i] = to_cx<R>(i < cr ? zero - e * g[i] : zero);
-        V.fl[i] = to_cx<R>(i < cl ? zero - e * gl[i] : zero);
+      invt[cl - 1] = recip((cl == 1 ? sig_l - e : fnms(sig_l, e, qp)) - off_l);
+      invp[cr] = zero;   // a chunk has CH-1 unknowns: its separator slot stays zero
+      g[0] = w[0] = invp[0];
+      gl[0] = invt[0];
+      wl[0] = (cl == 1 ? sig_l : sig) * invt[0];
+      for (int i = 1; i < CH; i++) {
+        g[i] = fnms(zero, e, g[i - 1]) * invp[i];
+        w[i] = fnms(one, e, w[i - 1]) * invp[i];
+        gl[i] = fnms(zero, e, gl[i - 1]) * invt[i];
+        wl[i] = fnms(i < cl - 1 ? sig : sig_l, e, wl[i - 1]) * invt[i];
       }
-      V.e = to_cx<R>(e);
-      const zd sw = e * sig * w[0];
-      sig_l = sig - sw - e * wl[0];
-      sig = sig - 2.0 * sw;
-      off_l = zero - e * off_l * gl[cl - 1];
-      e = zero - e * e * g[cr - 1];
+      for (int i = CH - 2; i >= 0; i--) {
+        g[i] = fnms(g[i], bp[i], g[i + 1]);
+        w[i] = fnms(w[i], bp[i], w[i + 1]);
+        gl[i] = fnms(gl[i], bp[i], gl[i + 1]);
+        wl[i] = fnms(wl[i], bp[i], wl[i + 1]);
+      }
+      for (int i = 0; i < CH; i++) {
+        fc[i] = fnms(zero, e, g[i]);
+        fl[i] = fnms(zero, e, gl[i]);
+      }
+      for (int u = 0; u < cnt; u++) {
+        auto &V = tabs[(size_t)(k0 + u) * (size_t)levels + (size_t)l];
+        auto at = [u](const zq &z) { return aao::mk((R)z.re[u], (R)z.im[u]); };
+        for (int i = 0; i < CH; i++) {
+          V.invp[i] = at(invp[i]);
+          V.invt[i] = at(invt[i]);
+          V.bp[i] = at(bp[i]);
+          V.fc[i] = at(fc[i]);
+          V.fl[i] = at(fl[i]);
+        }
+        V.e = at(e);
+      }
+      const zq sw = e * sig * w[0];
+      sig_l = fnms(sig - sw, e, wl[0]);
+      sig = sig - sw - sw;
+      off_l = fnms(zero, e * off_l, gl[cl - 1]);
+      e = fnms(zero, e * e, g[cr - 1]);
     }
   }
 }
@@ -615,11 +654,15 @@ bool apply_extents_ok(const Ctx &c, const aao::WsLayout &L, bool fused) {
 // The FP32 apply with the tridiagonal solves folded into the four-step
 // transform: forward transform + chunk solves (class FFT_FORWARD), the
 // separator systems (TRIDIAG), corrections + inverse transform
-// (FFT_INVERSE).  Input x (FP64) or x32 (FP32); output YT, with base
-// (FP64 output) y = base - P^{-1} x.
+// (FFT_INVERSE).  Input x (FP64) or x32 (FP32), with yprev x - E yprev; output
+// YT, with base (FP64 output) y = base - P^{-1} x.
 template <typename YT>
-cudaError_t precond_fused(Ctx &c, const double *x, const float *x32, YT *y, int tr,
-                          cudaStream_t s, const float *base = nullptr) {
+cudaError_t precond_fused(Ctx &c, const double *x, const float *x32, const YT *yprev, YT *y,
+                          int tr, cudaStream_t s, const float *base = nullptr) {
+  const double *yp64 = nullptr;
+  const float *yp32 = nullptr;
+  if constexpr (sizeof(YT) == 8) yp64 = yprev;
+  else yp32 = yprev;
   const aao::WsLayout L = aao::ws_layout(c, 0);
   if (!apply_extents_ok(c, L, true)) return cudaErrorInvalidValue;
   void *spec = c.ws + L.spec;
@@ -629,12 +672,12 @@ cudaError_t precond_fused(Ctx &c, const double *x, const float *x32, YT *y, int 
   // which serialise the chain); otherwise each half is one launcher call
   const bool each = c.prof_on;
   cudaError_t e = run(c, AAO_K_FFT_FORWARD, s, [&] {
-    return aao::fft_forward_f32_solve(c, x, x32, spec, sep, tr, s, inter, each ? 1 : 0);
+    return aao::fft_forward_f32_solve(c, x, x32, yp64, yp32, spec, sep, tr, s, inter, each ? 1 : 0);
   });
   if (e != cudaSuccess) return e;
   if (each) {
     e = run(c, AAO_K_FFT_FORWARD_SOLVE, s, [&] {
-      return aao::fft_forward_f32_solve(c, x, x32, spec, sep, tr, s, inter, 2);
+      return aao::fft_forward_f32_solve(c, x, x32, yp64, yp32, spec, sep, tr, s, inter, 2);
     });
     if (e != cudaSuccess) return e;
   }
@@ -663,8 +706,8 @@ cudaError_t precond_once(Ctx &c, const double *x, const YT *yprev, YT *y, int tr
   void *spec = c.ws + L.spec;
   void *inter = L.inter_bytes ? c.ws + L.inter : nullptr;
   const bool f32 = c.prec == AAO_PREC_FP32;
-  if (f32 && !yprev && inter && aao::fft_fused_supported(c))
-    return precond_fused<YT>(c, x, nullptr, y, tr, s, base);
+  if (f32 && inter && aao::fft_fused_supported(c))
+    return precond_fused<YT>(c, x, nullptr, yprev, y, tr, s, base);
   if (!apply_extents_ok(c, L, false)) return cudaErrorInvalidValue;
   cudaError_t e = run(c, AAO_K_FFT_FORWARD, s, [&] {
     if constexpr (sizeof(YT) == 4) return aao::fft_forward_f32_yf(c, x, yprev, spec, s, inter);
@@ -691,15 +734,16 @@ cudaError_t precond_refined(Ctx &c, const double *x, double *y, int tr, cudaStre
   double *r = reinterpret_cast<double *>(c.ws + L.rf64);
   cudaError_t e = precond_once<float>(c, x, nullptr, z0, tr, s);
   if (e != cudaSuccess) return e;
-  // where the four-step transform serves, r stays FP32 (its precision) and
+  // where a four-step transform serves, r stays FP32 (its precision) and
   // the correction's forward transform reads it directly
   void *inter = L.inter_bytes ? c.ws + L.inter : nullptr;
-  if (inter && aao::fft_four_supported(c)) {
+  if (inter && aao::fft_f32_input_supported(c)) {
     float *r32 = reinterpret_cast<float *>(r);
     void *spec = c.ws + L.spec;
     e = run(c, AAO_K_REFINE, s, [&] { return aao::launch_circ_residual_df(c, z0, x, r32, tr, s); });
     if (e != cudaSuccess) return e;
-    if (aao::fft_fused_supported(c)) return precond_fused<double>(c, nullptr, r32, y, tr, s, z0);
+    if (aao::fft_fused_supported(c))
+      return precond_fused<double>(c, nullptr, r32, nullptr, y, tr, s, z0);
     e = run(c, AAO_K_FFT_FORWARD, s, [&] { return aao::fft_forward_f32_from_f32(c, r32, spec, s, inter); });
     if (e != cudaSuccess) return e;
     e = run(c, AAO_K_TRIDIAG, s, [&] { return aao::launch_tridiag(c, spec, c.prec, tr, s); });
@@ -1181,6 +1225,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
   c.ch32 = 16;
   c.ch64 = (n <= 8191) ? 8 : 16;
   cudaGetDevice(&c.device);
+  aao::fft_plan(c);
   int st = AAO_OK;
   if (n > kMaxNAnyShape) {
     // rows longer than one CTA need the recursive cluster form in both precisions

@@ -2,34 +2,39 @@
 #include "fft_dispatch.cuh"
 
 namespace aao {
+void fft_plan(Ctx &c) {
+  fft::step_plan(c.ell, false, c.step32);
+  fft::step_plan(c.ell, true, c.step64);
+}
 cudaError_t fft_forward_f32(const Ctx &c, const double *x, const double *y, void *spec,
                             cudaStream_t s, void *inter) {
-  return fft::forward_any<float, double>(c.ell, c.n, c.n_pad, x, y, c.sigk32,
+  return fft::forward_any<float, double>(c.ell, c.step32, c.n, c.n_pad, x, y, c.sigk32,
                                          static_cast<cx<float> *>(spec), c.tw32, s, inter);
 }
 cudaError_t fft_inverse_f32(const Ctx &c, const void *spec, double *y, cudaStream_t s,
                             void *inter, const float *base) {
-  return fft::inverse_any<float, double>(c.ell, c.n, c.n_pad,
+  return fft::inverse_any<float, double>(c.ell, c.step32, c.n, c.n_pad,
                                          static_cast<const cx<float> *>(spec), y, c.tw32, s, inter,
                                          base);
 }
 cudaError_t fft_forward_f32_yf(const Ctx &c, const double *x, const float *y, void *spec,
                                cudaStream_t s, void *inter) {
-  return fft::forward_any<float, float>(c.ell, c.n, c.n_pad, x, y, c.sigk32,
+  return fft::forward_any<float, float>(c.ell, c.step32, c.n, c.n_pad, x, y, c.sigk32,
                                         static_cast<cx<float> *>(spec), c.tw32, s, inter);
 }
-size_t fft_inter_bytes_f32(const Ctx &c) { return fft::inter_bytes_any<float>(c.ell, c.n); }
-bool fft_four_supported(const Ctx &c) {
-  return AAO_FFT_FOUR && c.ell >= 256 && c.ell <= 4096 && (c.ell & (c.ell - 1)) == 0;
+size_t fft_inter_bytes_f32(const Ctx &c) { return fft::inter_bytes_any<float>(c.ell, c.step32, c.n); }
+bool fft_four_supported(const Ctx &c) { return fft::use_four<float>(c.ell); }
+bool fft_f32_input_supported(const Ctx &c) {
+  return fft::use_four<float>(c.ell) || c.step32.L;
 }
 cudaError_t fft_forward_f32_from_f32(const Ctx &c, const float *x, void *spec, cudaStream_t s,
                                      void *inter) {
-  return fft::forward_four_f32_input(c.ell, c.n, c.n_pad, x, static_cast<cx<float> *>(spec),
+  return fft::forward_four_f32_input(c.ell, c.step32, c.n, c.n_pad, x, static_cast<cx<float> *>(spec),
                                      c.tw32, s, inter);
 }
 cudaError_t fft_inverse_f32_to_f32(const Ctx &c, const void *spec, float *y, cudaStream_t s,
                                    void *inter) {
-  return fft::inverse_any<float, float>(c.ell, c.n, c.n_pad,
+  return fft::inverse_any<float, float>(c.ell, c.step32, c.n, c.n_pad,
                                         static_cast<const cx<float> *>(spec), y, c.tw32, s, inter);
 }
 
@@ -54,24 +59,29 @@ static float4 *sepbuf_of(void *sep) { return static_cast<float4 *>(sep); }
 static cx<float> *sepsol_of(const Ctx &c, void *sep) {
   return reinterpret_cast<cx<float> *>(static_cast<float4 *>(sep) + (size_t)c.nk * c.P32);
 }
-cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x32, void *spec,
-                                  void *sep, int transpose, cudaStream_t s, void *inter,
-                                  int part) {
-  if (!fft_fused_supported(c) || !inter || (!x == !x32)) return cudaErrorNotSupported;
+cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x32,
+                                  const double *y, const float *y32, void *spec, void *sep,
+                                  int transpose, cudaStream_t s, void *inter, int part) {
+  if (!fft_fused_supported(c) || !inter || (!x == !x32) || (y && y32) || (x32 && (y || y32)))
+    return cudaErrorNotSupported;
   auto *sp = static_cast<cx<float> *>(spec);
   auto *sb = sepbuf_of(sep);
   auto *tb = static_cast<const float4 *>(c.fuse32);
   const int P = c.P32, tr = transpose ? 1 : 0;
   const int ragged = (c.n + 1) % fft::kFuseCH != 0;
   const int rb = c.lev32 * (int)sizeof(RecLev<float, fft::kFuseCH>);   // one frequency's table
-#define AAO_FS(L)                                                                                  \
-  case L:                                                                                          \
-    return x ? fft::four_forward_solve<L, double>(c.n, c.n_pad, P, x, sp, sb, c.tw32, s, inter,   \
-                                                  tb, tr, ragged, part, c.rec32, rb)                       \
-             : fft::four_forward_solve<L, float>(c.n, c.n_pad, P, x32, sp, sb, c.tw32, s, inter,  \
-                                                 tb, tr, ragged, part, c.rec32, rb);
+#define AAO_FS(L)                                                                                 \
+  case L:                                                                                         \
+    if (x32)                                                                                      \
+      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x32, y32, c.sigk32, sp, sb, c.tw32, s,  \
+                                        inter, tb, tr, ragged, part, c.rec32, rb);                \
+    if (y32)                                                                                      \
+      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y32, c.sigk32, sp, sb, c.tw32, s,    \
+                                        inter, tb, tr, ragged, part, c.rec32, rb);                \
+    return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y, c.sigk32, sp, sb, c.tw32, s, inter, \
+                                      tb, tr, ragged, part, c.rec32, rb);
   switch (c.ell) {
-    AAO_FS(256) AAO_FS(512) AAO_FS(1024) AAO_FS(2048) AAO_FS(4096)
+    AAO_FOUR_CASES(AAO_FS)
     default: return cudaErrorNotSupported;
   }
 #undef AAO_FS
@@ -96,7 +106,7 @@ cudaError_t fft_inverse_f32_correct(const Ctx &c, const void *spec, void *sep, d
              : fft::four_inverse_correct<L, float>(c.n, c.n_pad, P, sp, sv, P, y32, c.tw32, s, \
                                                    inter, nullptr, tb, tr, ragged, part);
   switch (c.ell) {
-    AAO_IC(256) AAO_IC(512) AAO_IC(1024) AAO_IC(2048) AAO_IC(4096)
+    AAO_FOUR_CASES(AAO_IC)
     default: return cudaErrorNotSupported;
   }
 #undef AAO_IC

@@ -104,11 +104,19 @@ __device__ __forceinline__ void dft_columns(cx<float> *S, const cx<float> *__res
 }
 
 // Forward 1.  grid (ncx / W, L2 = t2); L1 W complex of dynamic shared memory.
-// XT: FP64 input (converted to FP32 on the way in) or FP32 input.
-template <int L, int W, typename XT = double>
+// XT: FP64 input (converted to FP32 on the way in) or FP32 input.  With YT a
+// type, the input is a Neumann term's x - E y, (E y)_t = sigk_t (2 y_i -
+// y_{i-1} - y_{i+1}): each y is loaded and converted to FP32 once, into a tile
+// of its own, where its neighbours find it (twice the dynamic shared memory,
+// plus two halo columns).  At n 4095, ell 4096 a term's first kernel took 128
+// us when every element loaded and converted all three, 105 us with the
+// neighbours from warp shuffles and the edge lanes' from memory.
+template <int L, int W, typename XT = double, typename YT = void>
 __global__ void __launch_bounds__(kFourT)
-k_fft4_forward1(const XT *__restrict__ x, cx<float> *__restrict__ inter, int n, int ncx,
+k_fft4_forward1(const XT *__restrict__ x, const YT *__restrict__ y,
+                const float *__restrict__ sigk, cx<float> *__restrict__ inter, int n, int ncx,
                 const cx<float> *__restrict__ tw) {
+  constexpr bool NEUMANN = !std::is_void<YT>::value;
   constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2;
   extern __shared__ __align__(16) unsigned char four_smem[];
   cx<float> *S = reinterpret_cast<cx<float> *>(four_smem);
@@ -126,8 +134,9 @@ k_fft4_forward1(const XT *__restrict__ x, cx<float> *__restrict__ inter, int n, 
   // column q = thread % 2W, the same for every u
   const int q = threadIdx.x % (2 * W), i = i0 + q;
   const bool in = i < n;
-  pdl_wait(x);   // x is the previous kernel's output
-  const XT *px = x + (size_t)(L2 * (threadIdx.x / (2 * W)) + t2) * n + i;
+  pdl_wait(x, y);   // x and y are earlier kernels' output
+  const int row0 = L2 * (threadIdx.x / (2 * W)) + t2;       // time step of u = 0
+  const XT *px = x + (size_t)row0 * n + i;
   const size_t ustride = (size_t)RPU * L2 * n;
 #pragma unroll
   for (int b0 = 0; b0 < NE; b0 += B) {
@@ -141,6 +150,47 @@ k_fft4_forward1(const XT *__restrict__ x, cx<float> *__restrict__ inter, int n, 
     for (int u = 0; u < B; u++) {
       if constexpr (sizeof(XT) == 8) Sf[(b0 + u) * kFourT + threadIdx.x] = to_f32(d[u]);
       else Sf[(b0 + u) * kFourT + threadIdx.x] = d[u];
+    }
+  }
+  if constexpr (NEUMANN) {
+    // the iterate's tile beside x's (each value converted once), with its two
+    // neighbour columns; then x - E y in place of x
+    float *Yf = reinterpret_cast<float *>(S + L1 * W);
+    float(*Yh)[2] = reinterpret_cast<float(*)[2]>(Yf + L1 * 2 * W);
+    const YT *py = y + (size_t)row0 * n + i;
+#pragma unroll
+    for (int b0 = 0; b0 < NE; b0 += B) {
+      YT d[B];
+#pragma unroll
+      for (int u = 0; u < B; u++) d[u] = in ? __ldg(py + (b0 + u) * ustride) : (YT)0;
+#pragma unroll
+      for (int u = 0; u < B; u++) Yf[(b0 + u) * kFourT + threadIdx.x] = from_any<float>(d[u]);
+    }
+    if (threadIdx.x < 2 * L1) {
+      const int r = threadIdx.x >> 1, ih = (threadIdx.x & 1) ? i0 + 2 * W : i0 - 1;
+      Yh[r][threadIdx.x & 1] =
+          (ih >= 0 && ih < n) ? from_any<float>(__ldg(y + (size_t)(L2 * r + t2) * n + ih)) : 0.f;
+    }
+    __syncthreads();
+    // a warp per row, two adjacent columns per lane
+    static_assert(W == 32, "a warp per row");
+    const int lane = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const float2 *Y2 = reinterpret_cast<const float2 *>(Yf);
+    float2 *X2 = reinterpret_cast<float2 *>(Sf);
+    const float *sg = sigk + L2 * r0 + t2;
+#pragma unroll
+    for (int u = 0; u < L1 * W / kFourT; u++) {
+      const int r = (kFourT / 32) * u + r0;
+      const float2 c = Y2[r * W + lane];
+      const float h = Yh[r][lane >> 4];                 // lane 0: left halo, 31: right
+      float l = __shfl_up_sync(0xffffffffu, c.y, 1), g = __shfl_down_sync(0xffffffffu, c.x, 1);
+      if (lane == 0) l = h;
+      if (lane == 31) g = h;
+      const float k = __ldg(sg + (kFourT / 32) * L2 * u);
+      float2 v = X2[r * W + lane];
+      v.x -= k * ((c.x + c.x) - l - c.y);
+      v.y -= k * ((c.y + c.y) - c.x - g);
+      X2[r * W + lane] = v;
     }
   }
   pdl_trigger();
@@ -400,19 +450,44 @@ inline bool four_discard_ok(const void *inter, const void *spec, int64_t n_pad) 
          (reinterpret_cast<uintptr_t>(spec) & 255) == 0 && (n_pad % 16) == 0;
 }
 
-template <int L, typename XT = double>
-cudaError_t four_forward(int64_t n, int64_t n_pad, const XT *x, cx<float> *spec,
-                         const cx<float> *tw, cudaStream_t s, void *inter) {
+// The first forward kernel: of x, or of x - E y with a Neumann iterate y.
+template <int L, typename XT, typename YT>
+cudaError_t four_forward1(int64_t n, const XT *x, const YT *y, const float *sigk,
+                          const cx<float> *tw, cudaStream_t s, cx<float> *ip) {
   constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2, W = kFourW;
   constexpr size_t sm1 = (size_t)L1 * W * sizeof(cx<float>);
+  const int ncx = (int)four_ncx(n);
+  const dim3 grid((unsigned)(ncx / W), L2);
+  cudaError_t e;
+  if constexpr (sizeof(XT) == 8) {
+    if (y) {
+      constexpr size_t smn = 2 * sm1 + 2 * (size_t)L1 * sizeof(float);
+      e = kernel_setup((const void *)k_fft4_forward1<L, W, XT, YT>, kFourT, smn);
+      if (e != cudaSuccess) return e;
+      e = launch_pdl(k_fft4_forward1<L, W, XT, YT>, grid, dim3(kFourT), smn, s, x, y, sigk, ip,
+                     (int)n, ncx, tw);
+      note_launch();
+      return e;
+    }
+  }
+  e = kernel_setup((const void *)k_fft4_forward1<L, W, XT, void>, kFourT, sm1);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_fft4_forward1<L, W, XT, void>, grid, dim3(kFourT), sm1, s, x,
+                 (const void *)nullptr, sigk, ip, (int)n, ncx, tw);
+  note_launch();
+  return e;
+}
+
+template <int L, typename XT, typename YT>
+cudaError_t four_forward(int64_t n, int64_t n_pad, const XT *x, const YT *y, const float *sigk,
+                         cx<float> *spec, const cx<float> *tw, cudaStream_t s, void *inter) {
+  constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2, W = kFourW;
   constexpr size_t sm2 = 2 * (size_t)L2 * W * sizeof(cx<float>);
   const int ncx = (int)four_ncx(n);
   cx<float> *ip = static_cast<cx<float> *>(inter);
-  cudaError_t e = kernel_setup((const void *)k_fft4_forward1<L, W, XT>, kFourT, sm1);
+  cudaError_t e = four_forward1<L>(n, x, y, sigk, tw, s, ip);
   if (e == cudaSuccess) e = kernel_setup((const void *)k_fft4_forward2<L, W>, kFourT, sm2);
   if (e != cudaSuccess) return e;
-  k_fft4_forward1<L, W, XT><<<dim3((unsigned)(ncx / W), L2), kFourT, sm1, s>>>(x, ip, (int)n, ncx, tw);
-  note_launch();
   k_fft4_forward2<L, W><<<dim3((unsigned)(ncx / W), L1 / 2 + 1), kFourT, sm2, s>>>(
       ip, spec, (int)n, ncx, n_pad, tw, four_discard_ok(ip, spec, n_pad) ? 1 : 0);
   note_launch();

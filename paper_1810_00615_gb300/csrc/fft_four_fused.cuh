@@ -466,25 +466,20 @@ k_fft4_inverseA_correct(const cx<float> *__restrict__ spec, const cx<float> *__r
   }
 }
 
-// x (FP64 or FP32) -> local solutions in spec and the chunks' separator data
+// x (FP64 or FP32; with y the Neumann term's x - E y) -> local solutions in spec and the chunks' separator data
 // in sepbuf: forward 1 (part 1), forward 2 + solves (part 2), or both (0).
-template <int L, typename XT>
-cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *x, cx<float> *spec,
-                               float4 *sepbuf, const cx<float> *tw, cudaStream_t s, void *inter,
+template <int L, typename XT, typename YT>
+cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *x, const YT *y,
+                               const float *sigk, cx<float> *spec, float4 *sepbuf, const cx<float> *tw, cudaStream_t s, void *inter,
                                const float4 *tabs, int conj, int ragged, int part = 0,
                                const void *rtab = nullptr, int rtab_bytes = 0) {
-  constexpr int L1 = Four<L>::L1, L2 = Four<L>::L2, W = kFourW;
-  constexpr size_t sm1 = (size_t)L1 * W * sizeof(cx<float>);
+  constexpr int L1 = Four<L>::L1, W = kFourW;
   constexpr size_t sm2 = fuse_smem<L, kFwdPairs, 0>();
   const int ncx = (int)four_ncx(n);
   cx<float> *ip = static_cast<cx<float> *>(inter);
   cudaError_t e = cudaSuccess;
   if (part != 2) {
-    e = kernel_setup((const void *)k_fft4_forward1<L, W, XT>, kFourT, sm1);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(k_fft4_forward1<L, W, XT>, dim3((unsigned)(ncx / W), L2), dim3(kFourT), sm1, s,
-                   x, ip, (int)n, ncx, tw);
-    note_launch();
+    e = four_forward1<L>(n, x, y, sigk, tw, s, ip);
     if (e != cudaSuccess) return e;
   }
   if (part != 1) {

@@ -1,0 +1,525 @@
+// Four-step time-axis FFT for any ell = L1 L2 = 2^a 3^b 5^c with run-time
+// factors, in FP32 and FP64: the lengths and precisions that the power-of-two
+// FP32 kernels of fft_four.cuh do not serve.
+//
+// The factorisation, the four kernels and the intermediate's layout
+// [k1][t2][complex column] are those of fft_four.cuh; here L1 and L2 are
+// kernel arguments.  A CTA holds the rows of 32 complex columns of G values of
+// t2 (L1 rows each) or of G k1 groups (two members of L2 rows each) in shared
+// memory; a warp takes one butterfly of all 32 columns at a time (lane =
+// column), so every index, twiddle and branch is uniform over the warp and
+// its run-time arithmetic is paid once per 32 columns.  G fills the eight
+// warps where the factors are short: with one t2 of 8 rows per CTA (ell =
+// 128) a pass had one butterfly, and the kernels took 9-10 us each at n 8191.  The passes run out of place between two buffers,
+// so that a thread holds one butterfly: in place, with all butterflies of a
+// warp in registers between two barriers, the run-time radices spilled 1 to 8
+// KB a thread and the kernels ran at half the speed.
+//
+// Why: the single mixed-radix kernel holds whole time series, 8 columns of
+// ell = 1440 in 196 KB, which left 98 CTAs of 8 warps for n = 1568 (12% of the
+// warps; 44 us forward, 35-59 us inverse), and the FP64 panel kernels had 64
+// CTAs for n = 1024, ell = 1024, their FP64 pipe 82% busy on 64 of 152 SMs
+// (75 + 52 us, with row passes of 7 and 21 us).  Here the same shapes give
+// 49 x 36 and 16 x 32 CTAs.
+// FP64 is bound by the FP64 pipe, FP32 by latency and issue.
+#pragma once
+#include "fft_time.cuh"
+#include "fft_mixed.cuh"
+
+namespace aao {
+namespace fft {
+namespace {   // included by both precision units: one private copy each
+
+constexpr int kStepT = 256, kStepW = 32, kStepWarps = kStepT / 32;
+// Shorter transforms run as one kernel.
+#ifndef AAO_STEPS_MIN
+#define AAO_STEPS_MIN 16
+#endif
+
+// Resident CTAs per SM the kernels are compiled for.
+template <typename R> struct StepOcc { static constexpr int V = sizeof(R) == 8 ? 3 : 4; };
+
+// ---- butterflies beyond fft_time.cuh's 2, 4, 8, 16 and fft_mixed.cuh's 3, 5
+// 6 = 2 x 3 and 10 = 2 x 5 by the Good-Thomas index maps (no twiddles):
+// n = n1 M + 2 n2, k = M k1 + (M + 1) k2 mod 2M for M = 3, 5 (2^-1 mod M =
+// (M + 1)/2).
+template <typename R, int DIR, int M>
+__device__ __forceinline__ void dft_2m(cx<R> *v) {
+  cx<R> a[2][M];
+#pragma unroll
+  for (int q = 0; q < M; q++) {
+    const cx<R> x0 = v[(2 * q) % (2 * M)], x1 = v[(M + 2 * q) % (2 * M)];
+    a[0][q] = x0 + x1;
+    a[1][q] = x0 - x1;
+  }
+  dft_mixed<R, DIR, M>(a[0]);
+  dft_mixed<R, DIR, M>(a[1]);
+#pragma unroll
+  for (int q = 0; q < M; q++) {
+    v[((M + 1) * q) % (2 * M)] = a[0][q];
+    v[(M + (M + 1) * q) % (2 * M)] = a[1][q];
+  }
+}
+
+// 9 = 3 x 3 (Cooley-Tukey, w = exp(DIR 2 pi i / 9)).
+template <typename R, int DIR>
+__device__ __forceinline__ void dft9(cx<R> *v) {
+  cx<R> a[3][3];
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    a[q][0] = v[q]; a[q][1] = v[q + 3]; a[q][2] = v[q + 6];
+    dft3<R, DIR>(a[q]);
+  }
+  const R c1 = (R)0.76604444311897803520, s1 = (R)0.64278760968653932632;    // 2 pi / 9
+  const R c2 = (R)0.17364817766693034885, s2 = (R)0.98480775301220805937;    // 4 pi / 9
+  const R c4 = (R)-0.93969262078590838405, s4 = (R)0.34202014332566873304;   // 8 pi / 9
+  auto rot = [](cx<R> z, R c, R s) { const R d = DIR < 0 ? -s : s; return mk(z.re * c - z.im * d, z.re * d + z.im * c); };
+  a[1][1] = rot(a[1][1], c1, s1);
+  a[1][2] = rot(a[1][2], c2, s2);
+  a[2][1] = rot(a[2][1], c2, s2);
+  a[2][2] = rot(a[2][2], c4, s4);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; k1++) {
+    cx<R> b[3] = {a[0][k1], a[1][k1], a[2][k1]};
+    dft3<R, DIR>(b);
+    v[k1] = b[0]; v[k1 + 3] = b[1]; v[k1 + 6] = b[2];
+  }
+}
+
+template <typename R, int DIR, int RAD>
+__device__ __forceinline__ void dft_step(cx<R> *v) {
+  if constexpr (RAD == 6) dft_2m<R, DIR, 3>(v);
+  else if constexpr (RAD == 10) dft_2m<R, DIR, 5>(v);
+  else if constexpr (RAD == 9) dft9<R, DIR>(v);
+  else dft_mixed<R, DIR, RAD>(v);
+}
+
+// q / d for 0 <= q < 512, 1 <= d <= 128 by a multiplication (exact: the error
+// of ceil(2^16 / d) is below 1, and 512 <= 2^16 / d).
+struct SmallDiv {
+  unsigned m;
+  __device__ __forceinline__ explicit SmallDiv(int d) : m((65536u + (unsigned)d - 1u) / (unsigned)d) {}
+  __device__ __forceinline__ int operator()(int q) const { return (int)(((unsigned)q * m) >> 16); }
+};
+
+// One Stockham pass of radix RAD over nmem buffers of N rows each (buffer m
+// at src + m N 32), out of place.  nmem N <= 256 rows in all.
+template <typename R, int DIR, int RAD>
+__device__ __forceinline__ void pass_step(const cx<R> *src, cx<R> *dst, int nmem, int N, int Ns,
+                                          int L, const cx<R> *__restrict__ tw) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nb = N / RAD, tot = nmem * nb, tstep = L / (Ns * RAD);
+  const SmallDiv by_nb(nb), by_ns(Ns);
+  for (int b = warp; b < tot; b += kStepWarps) {
+    const int m = by_nb(b), j = b - m * nb;
+    const int jd = by_ns(j), jm = j - jd * Ns;
+    const cx<R> *s = src + (m * N + j) * kStepW + lane;
+    cx<R> v[RAD];
+#pragma unroll
+    for (int r = 0; r < RAD; r++) v[r] = s[r * nb * kStepW];
+    if (jm) {
+#pragma unroll
+      for (int r = 1; r < RAD; r++) v[r] = twiddle<R, DIR>(v[r], tw[jm * tstep * r]);
+    }
+    dft_step<R, DIR, RAD>(v);
+    cx<R> *d = dst + (m * N + jd * Ns * RAD + jm) * kStepW + lane;
+#pragma unroll
+    for (int r = 0; r < RAD; r++) d[r * Ns * kStepW] = v[r];
+  }
+}
+
+// N-point DFTs down the rows of every column of nmem buffers, natural order
+// in and out, between a (the input) and b; returns the buffer that holds the
+// result.  All threads call it; a barrier before it is the caller's.
+template <typename R, int DIR>
+__device__ __forceinline__ cx<R> *dft_steps(cx<R> *a, cx<R> *b, int nmem, int N, int np,
+                                            const int *rad, int L, const cx<R> *__restrict__ tw) {
+  int Ns = 1;
+  for (int p = 0; p < np; p++) {
+    const int r = rad[p];
+#define AAO_PS(RAD) case RAD: pass_step<R, DIR, RAD>(a, b, nmem, N, Ns, L, tw); break;
+    switch (r) {
+      AAO_PS(2) AAO_PS(3) AAO_PS(4) AAO_PS(5) AAO_PS(6) AAO_PS(8) AAO_PS(9) AAO_PS(10)
+      default: break;
+    }
+#undef AAO_PS
+    __syncthreads();
+    Ns *= r;
+    cx<R> *t = a; a = b; b = t;
+  }
+  return a;
+}
+
+constexpr int kStepB = 8;   // rows a warp keeps in flight
+
+// Forward 1.  grid (ncx / 32, ceil(L2 / G) groups of t2); 2 G L1 x 32 complex
+// of dynamic shared memory.  XT: stored input type; NEUMANN: the input is
+// x - E y (load_real).
+template <typename R, typename XT, bool NEUMANN, typename YT>
+__global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
+k_steps_forward1(const XT *__restrict__ x, const YT *__restrict__ y, const R *__restrict__ sigk,
+                 cx<R> *__restrict__ inter, int n, int ncx, const cx<R> *__restrict__ tw,
+                 StepPlan pl, int G) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
+  R *Sf = reinterpret_cast<R *>(smraw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int L1 = pl.L1, L2 = pl.L2, t20 = blockIdx.y * G;
+  const int ng = min(G, L2 - t20), rows = ng * L1;           // t2 values here
+  const int i0 = 2 * kStepW * blockIdx.x;
+  const SmallDiv by_l1(L1);
+  const unsigned long long pol_stream = l2_evict_first(), pol_keep = l2_evict_last();
+  pdl_wait(x, y);
+  for (int q0 = 0; q0 < rows; q0 += kStepB * kStepWarps) {
+    if constexpr (NEUMANN) {
+#pragma unroll
+      for (int u = 0; u < kStepB; u++) {
+        const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
+        if (q < rows) {
+#pragma unroll
+          for (int h = 0; h < 2; h++)
+            Sf[q * 2 * kStepW + h * 32 + lane] = load_real<R, 0, true, YT>(
+                x, y, sigk, n, L2 * t1 + t20 + gi, i0 + h * 32 + lane, pol_stream);
+        }
+      }
+    } else {
+      XT d[kStepB][2];
+#pragma unroll
+      for (int u = 0; u < kStepB; u++) {
+        const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
+        const XT *row = x + (size_t)(L2 * t1 + t20 + gi) * n + i0 + lane;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const bool in = q < rows && i0 + h * 32 + lane < n;
+          if constexpr (sizeof(XT) == 8) d[u][h] = in ? ld_hint(row + h * 32, pol_stream) : 0.0;
+          else d[u][h] = in ? __ldg(row + h * 32) : (XT)0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kStepB; u++) {
+        const int q = q0 + warp + u * kStepWarps;
+        if (q < rows) {
+#pragma unroll
+          for (int h = 0; h < 2; h++) Sf[q * 2 * kStepW + h * 32 + lane] = from_any<R>(d[u][h]);
+        }
+      }
+    }
+  }
+  pdl_trigger();
+  __syncthreads();
+  S = dft_steps<R, -1>(S, S + rows * kStepW, ng, L1, pl.np1, pl.rad1, pl.L, tw);
+#pragma unroll 4
+  for (int q = warp; q < rows; q += kStepWarps) {
+    const int gi = by_l1(q), k1 = q - gi * L1, t2 = t20 + gi;
+    cx<R> v = S[q * kStepW + lane];
+    if (t2 * k1) v = twiddle<R, -1>(v, tw[t2 * k1]);
+    st_hint(inter + ((size_t)k1 * L2 + t2) * ncx + kStepW * blockIdx.x + lane, v, pol_keep);
+  }
+}
+
+// The buffers of G consecutive k1 groups {g, L1 - g}, g <= L1/2: buffer b =
+// 2 (g - g0) + member, L2 rows each; a group without a partner (k1 = 0, L1/2)
+// leaves its second buffer unused.  MULTI: G > 1.
+template <bool MULTI> struct StepGroups {
+  int L1, L2, g0, ng;
+  SmallDiv by_l2;
+  __device__ __forceinline__ StepGroups(const StepPlan &pl, int G)
+      : L1(pl.L1), L2(pl.L2), g0(MULTI ? blockIdx.y * G : blockIdx.y),
+        ng(MULTI ? min(G, pl.L1 / 2 + 1 - (int)blockIdx.y * G) : 1), by_l2(MULTI ? pl.L2 : 1) {}
+  __device__ __forceinline__ int rows() const { return 2 * ng * L2; }
+  // row q: its k1 (-1: unused), k2 and the row of the mirror frequency
+  // ell - k: L2 - 1 - k2 of the other member's buffer (k1 != 0; the same
+  // buffer where k1 = L1/2), or (L2 - k2) mod L2 of the same (k1 = 0)
+  __device__ __forceinline__ void row(int q, int &k1, int &k2, int &qm) const {
+    const int b = MULTI ? by_l2(q) : (q >= L2 ? 1 : 0);
+    const int g = MULTI ? g0 + (b >> 1) : g0, gb = g ? L1 - g : 0;
+    k2 = q - b * L2;
+    k1 = (b & 1) ? (gb != g ? gb : -1) : g;
+    qm = g == 0 ? (k2 ? b * L2 + L2 - k2 : q) : (gb != g ? (b ^ 1) : b) * L2 + L2 - 1 - k2;
+  }
+};
+
+// Forward 2.  grid (ncx / 32, ceil((L1/2 + 1) / G)); 4 G L2 x 32 complex of
+// dynamic shared memory.
+template <typename R, bool MULTI>
+__global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
+k_steps_forward2(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, int n, int ncx,
+                 int64_t n_pad, const cx<R> *__restrict__ tw, StepPlan pl, int G) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const StepGroups<MULTI> gr(pl, G);
+  const int rows = gr.rows(), cb = kStepW * blockIdx.x;
+  const unsigned long long pol_done = l2_evict_first(), pol_keep = l2_evict_last();
+  pdl_wait(inter);
+  for (int q0 = 0; q0 < rows; q0 += kStepB * kStepWarps) {
+    cx<R> d[kStepB];
+#pragma unroll
+    for (int u = 0; u < kStepB; u++) {
+      const int q = q0 + warp + u * kStepWarps;
+      int k1, k2, qm;
+      gr.row(q, k1, k2, qm);
+      d[u] = mk((R)0, (R)0);
+      if (q < rows && k1 >= 0)
+        d[u] = ld_hintc(inter + ((size_t)k1 * pl.L2 + k2) * ncx + cb + lane, pol_done);
+    }
+#pragma unroll
+    for (int u = 0; u < kStepB; u++) {
+      const int q = q0 + warp + u * kStepWarps;
+      if (q < rows) S[q * kStepW + lane] = d[u];
+    }
+  }
+  pdl_trigger();
+  __syncthreads();
+  S = dft_steps<R, -1>(S, S + rows * kStepW, 2 * gr.ng, pl.L2, pl.np2, pl.rad2, pl.L, tw);
+  // the two packed real columns X = (Z_k + conj Z_{ell-k})/2, Y = (Z_k - conj
+  // Z_{ell-k})/(2i) of k = k1 + L1 k2 <= ell/2; stored without the factor 1/2,
+  // which inverse B's scale carries (exactly: a power of two)
+  const int i = 2 * (cb + lane);
+#pragma unroll 4
+  for (int q = warp; q < rows; q += kStepWarps) {
+    int k1, k2, qm;
+    gr.row(q, k1, k2, qm);
+    const int k = k1 + pl.L1 * k2;
+    if (k1 < 0 || 2 * k > pl.L) continue;
+    const cx<R> zk = S[q * kStepW + lane], zm = S[qm * kStepW + lane];
+    const cx<R> X = mk(zk.re + zm.re, zk.im - zm.im);
+    const cx<R> Y = mk(zk.im + zm.im, zm.re - zk.re);
+    cx<R> *dst = spec + (size_t)k * n_pad + i;
+    if (i + 1 < n) st_hint2(dst, X, Y, pol_keep);
+    else if (i < n) st_hint(dst, X, pol_keep);
+  }
+}
+
+// Inverse A.  grid and shared memory as forward 2.
+template <typename R, bool MULTI>
+__global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
+k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int n, int ncx,
+                 int64_t n_pad, const cx<R> *__restrict__ tw, StepPlan pl, int G) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const StepGroups<MULTI> gr(pl, G);
+  const int rows = gr.rows(), cb = kStepW * blockIdx.x, i = 2 * (cb + lane);
+  const unsigned long long pol_done = l2_evict_first(), pol_keep = l2_evict_last();
+  pdl_wait(spec);
+  // X_k, Y_k of the stored half spectrum become Z_k = X + iY and, mirrored,
+  // Z_{ell-k} = conj X + i conj Y
+  constexpr int B = sizeof(R) == 8 ? kStepB / 2 : kStepB;
+  for (int q0 = 0; q0 < rows; q0 += B * kStepWarps) {
+    cx<R> X[B], Y[B];
+#pragma unroll
+    for (int u = 0; u < B; u++) {
+      const int q = q0 + warp + u * kStepWarps;
+      int k1, k2, qm;
+      gr.row(q, k1, k2, qm);
+      const int k = k1 + pl.L1 * k2;
+      X[u] = Y[u] = mk((R)0, (R)0);
+      if (q < rows && k1 >= 0 && 2 * k <= pl.L) {
+        const cx<R> *src = spec + (size_t)k * n_pad + i;
+        if (i + 1 < n) ld_hint2(src, X[u], Y[u], pol_done);
+        else if (i < n) X[u] = ld_hintc(src, pol_done);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < B; u++) {
+      const int q = q0 + warp + u * kStepWarps;
+      int k1, k2, qm;
+      gr.row(q, k1, k2, qm);
+      const int k = k1 + pl.L1 * k2;
+      if (q < rows && k1 >= 0 && 2 * k <= pl.L) {
+        cx<R> a = X[u], b = Y[u];
+        if (k == 0 || 2 * k == pl.L) { a.im = (R)0; b.im = (R)0; }
+        S[q * kStepW + lane] = mk(a.re - b.im, a.im + b.re);
+        if (k > 0 && 2 * k < pl.L) S[qm * kStepW + lane] = mk(a.re + b.im, b.re - a.im);
+      }
+    }
+  }
+  pdl_trigger();
+  __syncthreads();
+  S = dft_steps<R, +1>(S, S + rows * kStepW, 2 * gr.ng, pl.L2, pl.np2, pl.rad2, pl.L, tw);
+#pragma unroll 4
+  for (int q = warp; q < rows; q += kStepWarps) {
+    int k1, t2, qm;
+    gr.row(q, k1, t2, qm);
+    if (k1 < 0) continue;
+    cx<R> v = S[q * kStepW + lane];
+    if (t2 * k1) v = twiddle<R, +1>(v, tw[t2 * k1]);
+    st_hint(inter + ((size_t)k1 * pl.L2 + t2) * ncx + cb + lane, v, pol_keep);
+  }
+}
+
+// Inverse B.  grid and shared memory as forward 1.  With base (FP64 output
+// only) y = base - result.
+template <typename R, typename OT>
+__global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
+k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int ncx,
+                 const cx<R> *__restrict__ tw, const float *__restrict__ base, StepPlan pl, int G) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int L1 = pl.L1, L2 = pl.L2, t20 = blockIdx.y * G;
+  const int ng = min(G, L2 - t20), rows = ng * L1;
+  const int i0 = 2 * kStepW * blockIdx.x;
+  const SmallDiv by_l1(L1);
+  const unsigned long long pol_done = l2_evict_first();
+  pdl_wait(inter, base);
+  for (int q0 = 0; q0 < rows; q0 += kStepB * kStepWarps) {
+    cx<R> d[kStepB];
+#pragma unroll
+    for (int u = 0; u < kStepB; u++) {
+      const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), k1 = q - gi * L1;
+      if (q < rows)
+        d[u] = ld_hintc(inter + ((size_t)k1 * L2 + t20 + gi) * ncx + kStepW * blockIdx.x + lane, pol_done);
+    }
+#pragma unroll
+    for (int u = 0; u < kStepB; u++) {
+      const int q = q0 + warp + u * kStepWarps;
+      if (q < rows) S[q * kStepW + lane] = d[u];
+    }
+  }
+  pdl_trigger();
+  __syncthreads();
+  S = dft_steps<R, +1>(S, S + rows * kStepW, ng, L1, pl.np1, pl.rad1, pl.L, tw);
+  const R *Sf = reinterpret_cast<const R *>(S);
+  const R scale = (R)0.5 / (R)pl.L;   // with forward 2's 1/2
+  constexpr int B = 4;
+  for (int q0 = 0; q0 < rows; q0 += B * kStepWarps) {
+    float bv[B][2];
+    if constexpr (sizeof(OT) == 8) {
+      if (base) {
+#pragma unroll
+        for (int u = 0; u < B; u++) {
+          const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
+          const size_t row = (size_t)(L2 * t1 + t20 + gi) * n;
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            const int i = i0 + h * 32 + lane;
+            bv[u][h] = (q < rows && i < n) ? __ldg(&base[row + i]) : 0.f;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < B; u++) {
+      const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
+      const size_t row = (size_t)(L2 * t1 + t20 + gi) * n;
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        const int i = i0 + h * 32 + lane;
+        if (q < rows && i < n) {
+          const OT val = to_out<R, OT>(scale * Sf[q * 2 * kStepW + h * 32 + lane]);
+          if constexpr (sizeof(OT) == 8) y[row + i] = base ? to_f64(bv[u][h]) - val : val;
+          else y[row + i] = val;
+        }
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------- host side
+// Radices of an N-point transform (N = 2^a 3^b 5^c): the fewest passes, and
+// among those the smallest largest radix (more butterflies to share out).
+inline bool step_radices(int N, int *rad, int &np) {
+  static const int kRad[] = {2, 3, 4, 5, 6, 8, 9, 10};
+  if (N == 1) { np = 0; return true; }
+  int best = 1 << 30;
+  for (int a : kRad) {
+    if (N == a && a < best) { best = a; np = 1; rad[0] = a; }
+  }
+  if (best < (1 << 30)) return true;
+  for (int a : kRad) {
+    for (int b : kRad)
+      if (a * b == N && a >= b && a < best) { best = a; np = 2; rad[0] = a; rad[1] = b; }
+  }
+  if (best < (1 << 30)) return true;
+  for (int a : kRad) {
+    for (int b : kRad)
+      for (int c : kRad)
+        if (a * b * c == N && a >= b && b >= c && a < best) {
+          best = a; np = 3; rad[0] = a; rad[1] = b; rad[2] = c;
+        }
+  }
+  return best < (1 << 30);
+}
+
+// FP64: L1 >= L2, L1 as small as possible (a tile of 64 rows is 32 KB).
+// FP32: the smallest L1 >= 8 that leaves L2 <= 64.  The inverse's last DFT
+// has length L1, and the rounding of the twiddles before it reaches the
+// output shared by L1 time steps, so at the low frequencies that P^{-1}
+// amplifies it is about sqrt(L1) times that of a transform whose twiddles
+// come last; the refined apply squares that error.
+inline bool step_plan(int64_t ell, bool fp64, StepPlan &pl) {
+  pl = StepPlan{};
+  if (ell < AAO_STEPS_MIN) return false;
+  const bool wide = !fp64 && ell >= 64;
+  for (int64_t l1 = wide ? 8 : 1; l1 <= 128; l1++) {
+    if (ell % l1 || (wide ? ell / l1 > 64 : l1 * l1 < ell)) continue;
+    pl.L1 = (int)l1;
+    pl.L2 = (int)(ell / l1);
+    if (step_radices(pl.L1, pl.rad1, pl.np1) && step_radices(pl.L2, pl.rad2, pl.np2)) {
+      pl.L = (int)ell;
+      return true;
+    }
+  }
+  return false;
+}
+inline int64_t steps_ncx(int64_t n) { return ((n + 1) / 2 + kStepW - 1) / kStepW * kStepW; }
+template <typename R> size_t steps_inter_bytes(int64_t ell, int64_t n) {
+  return (size_t)ell * (size_t)steps_ncx(n) * sizeof(cx<R>);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t steps_launch(void (*kern)(KArgs...), dim3 grid, size_t smem, cudaStream_t s, Args &&...args) {
+  cudaError_t e = kernel_setup((const void *)kern, kStepT, smem, nullptr, true);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(kern, grid, dim3(kStepT), smem, s, std::forward<Args>(args)...);
+  note_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Units (t2 values, k1 groups) of `unit` rows per CTA: as many as fit in 64
+// rows, as long as two CTAs per SM remain.
+inline int steps_group(int cols, int units, int unit) {
+  int G = 64 / unit;
+  G = G < 1 ? 1 : (G > units ? units : G);
+  while (G > 1 && (int64_t)cols * ((units + G - 1) / G) < 2 * 152) G--;
+  return G;
+}
+
+template <typename R, typename XT, typename YT>
+cudaError_t steps_forward(const StepPlan &pl, int64_t n, int64_t n_pad, const XT *x, const YT *y, const R *sigk,
+                          cx<R> *spec, const cx<R> *tw, cudaStream_t s, void *inter) {
+  const int ncx = (int)steps_ncx(n), cols = ncx / kStepW;
+  cx<R> *ip = static_cast<cx<R> *>(inter);
+  const size_t row = kStepW * sizeof(cx<R>);
+  const int G1 = steps_group(cols, pl.L2, pl.L1), G2 = steps_group(cols, pl.L1 / 2 + 1, 2 * pl.L2);
+  const dim3 g1((unsigned)cols, (unsigned)((pl.L2 + G1 - 1) / G1)), g2((unsigned)cols, (unsigned)((pl.L1 / 2 + G2) / G2));
+  const size_t sm1 = 2 * (size_t)G1 * pl.L1 * row;
+  cudaError_t e;
+  if constexpr (sizeof(XT) == 8) {
+    e = y ? steps_launch(k_steps_forward1<R, XT, true, YT>, g1, sm1, s, x, y, sigk, ip, (int)n, ncx, tw, pl, G1)
+          : steps_launch(k_steps_forward1<R, XT, false, double>, g1, sm1, s, x, (const double *)nullptr, sigk, ip, (int)n, ncx, tw, pl, G1);
+  } else {
+    e = steps_launch(k_steps_forward1<R, XT, false, double>, g1, sm1, s, x, (const double *)nullptr, sigk, ip, (int)n, ncx, tw, pl, G1);
+  }
+  if (e != cudaSuccess) return e;
+  return steps_launch(G2 > 1 ? k_steps_forward2<R, true> : k_steps_forward2<R, false>, g2, 4 * (size_t)G2 * pl.L2 * row, s, ip, spec, (int)n, ncx, n_pad, tw, pl, G2);
+}
+
+template <typename R, typename OT>
+cudaError_t steps_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, const cx<R> *spec, OT *y, const cx<R> *tw,
+                          cudaStream_t s, void *inter, const float *base) {
+  const int ncx = (int)steps_ncx(n), cols = ncx / kStepW;
+  cx<R> *ip = static_cast<cx<R> *>(inter);
+  const size_t row = kStepW * sizeof(cx<R>);
+  const int G1 = steps_group(cols, pl.L2, pl.L1), G2 = steps_group(cols, pl.L1 / 2 + 1, 2 * pl.L2);
+  const dim3 g1((unsigned)cols, (unsigned)((pl.L2 + G1 - 1) / G1)), g2((unsigned)cols, (unsigned)((pl.L1 / 2 + G2) / G2));
+  const cudaError_t e = steps_launch(G2 > 1 ? k_steps_inverseA<R, true> : k_steps_inverseA<R, false>, g2, 4 * (size_t)G2 * pl.L2 * row, s, spec, ip, (int)n, ncx, n_pad, tw, pl, G2);
+  if (e != cudaSuccess) return e;
+  return steps_launch(k_steps_inverseB<R, OT>, g1, 2 * (size_t)G1 * pl.L1 * row, s, ip, y, (int)n, ncx, tw, base, pl, G1);
+}
+
+}  // namespace
+}  // namespace fft
+}  // namespace aao

@@ -38,7 +38,33 @@ __device__ __forceinline__ int swz(int chunk) { return chunk ^ ((chunk >> 3) & 7
 // Level buffers of the recursive form: one padding slot per CH values so
 // that the chunk-strided accesses of the threads fall in distinct banks.
 template <int CH>
-__device__ __forceinline__ int rpos(int e) { return e + e / CH; }
+__host__ __device__ __forceinline__ int rpos(int e) { return e + e / CH; }
+// Values of the buffer of level l: whole chunks, the tail past lsz[l] zeroed
+// by the caller, so that no chunk loop has to know the last chunk's length.
+template <int CH>
+__host__ __device__ __forceinline__ int level_size(const int *lsz, int levels, int l) {
+  return ((l + 1 < levels ? lsz[l + 1] : 0) + 1) * CH;
+}
+// Lay the buffers of levels 1 .. levels-1 out from `base` (B[l], NULL for a
+// size alone) and return the values they take.
+template <typename R, int CH>
+__host__ __device__ __forceinline__ size_t level_buffers(const int *lsz, int levels, cx<R> *base,
+                                                         cx<R> **B) {
+  size_t off = 0;
+  for (int l = 1; l < levels; l++) {
+    if (B) B[l] = base + off;
+    off += (size_t)rpos<CH>(level_size<CH>(lsz, levels, l)) + 1;
+  }
+  return off;
+}
+// Zero the tails of the level buffers (nthr threads, thread p).
+template <typename R, int CH>
+__device__ __forceinline__ void zero_tails(cx<R> *const *B, const int *lsz, int levels, int p,
+                                           int nthr) {
+  for (int l = 1; l < levels; l++)
+    for (int e = lsz[l] + p; e < level_size<CH>(lsz, levels, l); e += nthr)
+      B[l][rpos<CH>(e)] = mk((R)0, (R)0);
+}
 
 // Copy the levels in use of a frequency's table into shared memory,
 // conjugated for the transposed symbols; nthr threads, thread p.
@@ -68,20 +94,13 @@ __device__ __forceinline__ void chunk_solve(cx<R> *v, const cx<R> *inv, const cx
 
 // Levels 1 .. levels-1 of the recursive form on shared-memory buffers:
 // B[1] holds the level-1 right-hand sides on entry and the level-1 solution
-// (the level-0 separator values) on exit.  Called by all threads of one CTA
-// (WARP = false) or by the 32 lanes of one warp (WARP = true, p = lane).
-template <bool WARP>
-__device__ __forceinline__ void rec_sync() {
-  if constexpr (WARP) __syncwarp();
-  else __syncthreads();
-}
-template <typename R, int CH, bool WARP = false>
+// (the level-0 separator values) on exit.  Called by all threads of one CTA.
+template <typename R, int CH>
 __device__ __forceinline__ void rec_upper(cx<R> *const *B, const int *lsz, int levels,
                                           const RecLev<R, CH> *T, int p) {
-  const int nthr = WARP ? 32 : (int)blockDim.x;
+  const int nthr = (int)blockDim.x;
   const cx<R> zero = mk((R)0, (R)0);
   for (int l = 1; l < levels; l++) {
-    const int nl = lsz[l];
     const int Ml = l + 1 < levels ? lsz[l + 1] : 0, Pl = Ml + 1;
     cx<R> *Bl = B[l];
     const cx<R> el = T[l].e;
@@ -89,24 +108,22 @@ __device__ __forceinline__ void rec_upper(cx<R> *const *B, const int *lsz, int l
       const bool last = q == Ml;
       cx<R> w[CH];
 #pragma unroll
-      for (int i = 0; i < CH; i++) w[i] = (q * CH + i < nl) ? Bl[rpos<CH>(q * CH + i)] : zero;
+      for (int i = 0; i < CH; i++) w[i] = Bl[rpos<CH>(q * CH + i)];
       chunk_solve<R, CH>(w, last ? T[l].invt : T[l].invp, T[l].bp, el);
 #pragma unroll
-      for (int i = 0; i < CH - 1; i++)
-        if (q * CH + i < nl) Bl[rpos<CH>(q * CH + i)] = w[i];
-      if (last && q * CH + CH - 1 < nl) Bl[rpos<CH>(q * CH + CH - 1)] = w[CH - 1];
+      for (int i = 0; i < CH - 1; i++) Bl[rpos<CH>(q * CH + i)] = w[i];
+      if (last) Bl[rpos<CH>(q * CH + CH - 1)] = w[CH - 1];
     }
-    rec_sync<WARP>();
+    __syncthreads();
     for (int q = p; q < Ml; q += nthr) {
       const cx<R> sep = Bl[rpos<CH>(q * CH + CH - 1)];
       const cx<R> lastl = Bl[rpos<CH>(q * CH + CH - 2)];
       const cx<R> firstr = Bl[rpos<CH>((q + 1) * CH)];
       B[l + 1][rpos<CH>(q)] = cfnms(sep, el, lastl + firstr);
     }
-    if (Ml > 0) rec_sync<WARP>();
+    if (Ml > 0) __syncthreads();
   }
   for (int l = levels - 2; l >= 1; l--) {
-    const int nl = lsz[l];
     const int Ml = lsz[l + 1], Pl = Ml + 1;
     cx<R> *Bl = B[l];
     const cx<R> *Bu = B[l + 1];
@@ -118,13 +135,12 @@ __device__ __forceinline__ void rec_upper(cx<R> *const *B, const int *lsz, int l
 #pragma unroll
       for (int i = 0; i < CH - 1; i++) {
         const int pos = rpos<CH>(q * CH + i);
-        if (q * CH + i < nl) Bl[pos] = cfma(cfma(Bl[pos], sl, fl[i]), sr, T[l].fc[CH - 2 - i]);
+        Bl[pos] = cfma(cfma(Bl[pos], sl, fl[i]), sr, T[l].fc[CH - 2 - i]);
       }
       const int pe = rpos<CH>(q * CH + CH - 1);
-      if (!last) Bl[pe] = sr;
-      else if (q * CH + CH - 1 < nl) Bl[pe] = cfma(Bl[pe], sl, fl[CH - 1]);
+      Bl[pe] = last ? cfma(Bl[pe], sl, fl[CH - 1]) : sr;
     }
-    rec_sync<WARP>();
+    __syncthreads();
   }
 }
 
@@ -150,16 +166,13 @@ k_tridiag_rec(cx<R> *__restrict__ spec, int n, int64_t n_pad,
   extern __shared__ __align__(16) unsigned char smraw[];
   // level buffers B_1..B_{levels-1}, then the staged row
   cx<R> *B[kRecLevels];
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) {
-    B[l] = reinterpret_cast<cx<R> *>(smraw) + off;
-    off += (size_t)rpos<CH>(lsz[l]) + 1;
-  }
+  size_t off = level_buffers<R, CH>(lsz, levels, reinterpret_cast<cx<R> *>(smraw), B);
   cx<R> *s_first = reinterpret_cast<cx<R> *>(smraw) + off;   // [P]
   off += (size_t)P;
   float4 *s_row = reinterpret_cast<float4 *>(smraw + ((off * sizeof(cx<R>) + 15) & ~(size_t)15));
   constexpr int EPC = 16 / sizeof(cx<R>);
   load_levels<R, CH>(T, tabs + (size_t)k * levels, levels, conj_sym, p, P);
+  zero_tails<R, CH>(B, lsz, levels, p, P);
 
   cx<R> *row = spec + (size_t)k * n_pad;
   const int base = p * CH;
@@ -259,11 +272,7 @@ k_tridiag_cluster(cx<R> *__restrict__ spec, int n, int64_t n_pad,
   __shared__ RecLev<R, CH> T0[kRecLevels];
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<R> *B[kRecLevels];
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) {
-    B[l] = reinterpret_cast<cx<R> *>(smraw) + off;
-    off += (size_t)rpos<CH>(lsz[l]) + 1;
-  }
+  size_t off = level_buffers<R, CH>(lsz, levels, reinterpret_cast<cx<R> *>(smraw), B);
   cx<R> *s_first = reinterpret_cast<cx<R> *>(smraw) + off;   // [T]
   off += (size_t)T;
   float4 *s_row = reinterpret_cast<float4 *>(smraw + ((off * sizeof(cx<R>) + 15) & ~(size_t)15));
@@ -271,6 +280,7 @@ k_tridiag_cluster(cx<R> *__restrict__ spec, int n, int64_t n_pad,
   const int nchunks = (T * CH) / EPC;
 
   load_levels<R, CH>(T0, tabs + (size_t)k * levels, levels, conj_sym, p, T);
+  zero_tails<R, CH>(B, lsz, levels, p, T);
 
   cx<R> *row = spec + (size_t)k * n_pad + (size_t)rank * T * CH;   // this CTA's segment
   const int nseg = n - rank * T * CH;                                 // unknowns left from here
@@ -333,44 +343,38 @@ k_tridiag_cluster(cx<R> *__restrict__ spec, int n, int64_t n_pad,
 }
 
 // The separator system of the fused four-step apply (fft_four_fused.cuh):
-// one warp per frequency k.  The forward kernel left, for each chunk p of
-// row k, its first local value v_0 and its separator's partial right-hand
-// side x_sep - e v_14 in sepbuf[k P + p]; the level-1 right-hand side of
-// separator p is that partial value minus e times the first local value of
-// chunk p + 1.  Levels 1 .. levels-1 of the recursive form are solved as in
-// k_tridiag_rec (by one warp) and the separator values go to
-// sep[k sstride + p].  Per warp, wbytes of shared memory: the frequency's
-// levels in use (conjugated for the transpose), then the level buffers.
+// one CTA per frequency k, a thread per level-1 chunk up to 256 (a warp per
+// frequency left one warp on an SM at n = 65535, ell = 512: 8 chunks a lane
+// in turn, 30 us).  The forward kernel left, for each chunk p of row k, its
+// first local value v_0 and its separator's partial right-hand side
+// x_sep - e v_14 in sepbuf[k P + p]; the level-1 right-hand side of separator
+// p is that partial value minus e times the first local value of chunk p + 1.
+// Levels 1 .. levels-1 of the recursive form are solved as in k_tridiag_rec
+// and the separator values go to sep[k sstride + p].
 template <int CH>
 __global__ void __launch_bounds__(256)
 k_tridiag_reduced(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ sep,
                   int64_t sstride, const RecLev<float, CH> *__restrict__ tabs, int conj_sym,
-                  int levels, int4 lsz_lo, int2 lsz_hi, int nk, int wbytes) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = blockIdx.x * (blockDim.x >> 5) + w;
-  if (k >= nk) return;   // whole warps only; nothing below synchronises the CTA
+                  int levels, int4 lsz_lo, int2 lsz_hi) {
+  const int k = blockIdx.x, p = threadIdx.x, T = blockDim.x;
   const int lsz[kRecLevels] = {lsz_lo.x, lsz_lo.y, lsz_lo.z, lsz_lo.w, lsz_hi.x, lsz_hi.y};
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned char *mine = smraw + (size_t)w * wbytes;
-  RecLev<float, CH> *st = reinterpret_cast<RecLev<float, CH> *>(mine);
-  load_levels<float, CH>(st, tabs + (size_t)k * levels, levels, conj_sym, lane, 32);
+  RecLev<float, CH> *st = reinterpret_cast<RecLev<float, CH> *>(smraw);
+  load_levels<float, CH>(st, tabs + (size_t)k * levels, levels, conj_sym, p, T);
   cx<float> *B[kRecLevels];
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) {
-    B[l] = reinterpret_cast<cx<float> *>(mine + levels * sizeof(RecLev<float, CH>)) + off;
-    off += (size_t)rpos<CH>(lsz[l]) + 1;
-  }
-  __syncwarp();
+  level_buffers<float, CH>(lsz, levels, reinterpret_cast<cx<float> *>(st + levels), B);
+  zero_tails<float, CH>(B, lsz, levels, p, T);
+  __syncthreads();
   pdl_wait(sepbuf);   // the previous kernel's output
   const float4 *row = sepbuf + (size_t)k * sstride;
   const cx<float> e0 = st[0].e;
   const int M = lsz[1];
-  for (int q0 = 0; q0 < M; q0 += 8 * 32) {
+  for (int q0 = 0; q0 < M; q0 += 8 * T) {
     float4 a[8];
     float2 b[8];
 #pragma unroll
     for (int u = 0; u < 8; u++) {
-      const int q = q0 + lane + 32 * u;
+      const int q = q0 + p + T * u;
       if (q < M) {
         a[u] = row[q];                                         // (v0_q, partial_q)
         b[u] = *reinterpret_cast<const float2 *>(row + q + 1);  // v0_{q+1}
@@ -378,14 +382,15 @@ k_tridiag_reduced(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ sep
     }
 #pragma unroll
     for (int u = 0; u < 8; u++) {
-      const int q = q0 + lane + 32 * u;
+      const int q = q0 + p + T * u;
       if (q < M) B[1][rpos<CH>(q)] = cfnms(mk(a[u].z, a[u].w), e0, mk(b[u].x, b[u].y));
     }
   }
-  __syncwarp();
-  rec_upper<float, CH, true>(B, lsz, levels, st, lane);
+  pdl_trigger();
+  __syncthreads();
+  rec_upper<float, CH>(B, lsz, levels, st, p);
   cx<float> *out = sep + (size_t)k * sstride;
-  for (int q = lane; q < M; q += 32) out[q] = B[1][rpos<CH>(q)];
+  for (int q = p; q < M; q += T) out[q] = B[1][rpos<CH>(q)];
 }
 
 // The same separator system when the recursive form has at most three
@@ -501,34 +506,27 @@ cudaError_t launch_tridiag_reduced(const Ctx &c, const void *sepbuf, void *sep, 
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) off += (size_t)(lsz[l] + lsz[l] / CH) + 1;
-  const size_t wbytes =
-      (levels * sizeof(RecLev<float, CH>) + off * sizeof(cx<float>) + 15) & ~(size_t)15;
-  int wpb = (int)((200 * 1024) / wbytes);
-  wpb = wpb < 1 ? 1 : (wpb > 8 ? 8 : wpb);
-  if (wbytes > 200 * 1024) return cudaErrorNotSupported;
-  const size_t smem = (size_t)wpb * wbytes;
-  auto kern = k_tridiag_reduced<CH>;
-  cudaError_t e = kernel_setup((const void *)kern, 32 * wpb, smem);
+  const size_t off = level_buffers<float, CH>(lsz, levels, nullptr, nullptr);
+  const size_t smem = levels * sizeof(RecLev<float, CH>) + off * sizeof(cx<float>);
+  if (smem > 200 * 1024) return cudaErrorNotSupported;
+  const int chunks = lsz[2] + 1;                        // of level 1 (levels >= 4 here)
+  const int T = chunks >= 256 ? 256 : (chunks + 31) / 32 * 32;
+  cudaError_t e = kernel_setup((const void *)k_tridiag_reduced<CH>, T, smem);
   if (e != cudaSuccess) { cudaGetLastError(); return e; }
   const int4 lo = make_int4(lsz[0], lsz[1], lsz[2], lsz[3]);
   const int2 hi = make_int2(lsz[4], lsz[5]);
-  const unsigned grid = (unsigned)((c.nk + wpb - 1) / wpb);
-  kern<<<grid, 32 * wpb, smem, s>>>(static_cast<const float4 *>(sepbuf),
-                                     static_cast<cx<float> *>(sep), (int64_t)c.P32,
-                                     static_cast<const RecLev<float, CH> *>(c.rec32), transpose,
-                                     levels, lo, hi, (int)c.nk, (int)wbytes);
+  e = launch_pdl(k_tridiag_reduced<CH>, dim3((unsigned)c.nk), dim3(T), smem, s,
+                 static_cast<const float4 *>(sepbuf), static_cast<cx<float> *>(sep),
+                 (int64_t)c.P32, static_cast<const RecLev<float, CH> *>(c.rec32), transpose,
+                 levels, lo, hi);
   note_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename R, int CH>
 static cudaError_t run_tridiag_cluster(const Ctx &c, void *spec, const void *tab, int T, int S,
                                        int conj, int levels, const int *lsz, cudaStream_t s) {
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) off += (size_t)(lsz[l] + lsz[l] / CH) + 1;
-  off += (size_t)T;
+  const size_t off = level_buffers<R, CH>(lsz, levels, nullptr, nullptr) + (size_t)T;
   const size_t smem = ((off * sizeof(cx<R>) + 15) & ~(size_t)15) + (size_t)T * CH * sizeof(cx<R>);
   auto kern = k_tridiag_cluster<R, CH>;
   cudaError_t e = kernel_setup((const void *)kern, T, smem);
@@ -557,9 +555,7 @@ static cudaError_t run_tridiag_cluster(const Ctx &c, void *spec, const void *tab
 template <typename R, int CH>
 static cudaError_t run_tridiag_rec(const Ctx &c, void *spec, const void *tab, int P, int conj,
                                    int levels, const int *lsz, cudaStream_t s) {
-  size_t off = 0;
-  for (int l = 1; l < levels; l++) off += (size_t)(lsz[l] + lsz[l] / CH) + 1;
-  off += (size_t)P;
+  const size_t off = level_buffers<R, CH>(lsz, levels, nullptr, nullptr) + (size_t)P;
   const size_t upper = (off * sizeof(cx<R>) + 15) & ~(size_t)15;
   const size_t staged = upper + (size_t)P * CH * sizeof(cx<R>);
   const bool stage = staged <= 200 * 1024;
