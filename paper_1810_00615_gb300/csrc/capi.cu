@@ -923,6 +923,7 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       beta = std::sqrt(hs[320]);
       v0_sign = -1.0;
     }
+    if (!precond) Z[0] = V[0];   // V_0 may be b itself, not the basis slot
     relres_true = defer_b ? 1.0 : beta / bnorm;
     if (!std::isfinite(beta)) { status = AAO_ENUMERIC; break; }
     if (relres_true <= rtol) { status = AAO_OK; break; }

@@ -308,3 +308,22 @@ def test_zero_initial_guess_never_reads_x():
     # the Python wrapper's default (x0=None) takes the same path
     x_none, info_none = a.solve(b, rtol=1e-10)
     assert torch.equal(x_none, got[300]) and info_none["iters"] == info_given["iters"]
+
+
+def test_unpreconditioned_zero_guess_reads_the_right_hand_side():
+    """precond = 0 from x0 = 0: z_0 is b, not the first basis slot of the
+    workspace (filled with NaN here, so that any use of it shows)."""
+    torch = need_gpu()
+    from paper_1810_00615_gb300 import AllAtOnce
+    n, ell = 15, 16
+    a = AllAtOnce(n, ell, 1.0 / ell, restart=30)
+    b = a.build_rhs(to_dev(torch, syn.heat_initial(n)))
+    off = (-a._ws.data_ptr()) % 256
+    a._ws[off:].view(torch.uint8)[: (a._ws.numel() - off) // 8 * 8].view(torch.float64).fill_(float("nan"))
+    x, info = a.solve(b, restart=30, rtol=1e-14, maxit=1, precond=0)
+    assert torch.isfinite(x).all() and info["iters"] == 1
+    # one step minimises over span{b}: x = b (A b . b) / (A b . A b)
+    Ab = a.matvec(b)
+    want = b * ((Ab * b).sum() / (Ab * Ab).sum())
+    assert (x - want).abs().max() <= 1e-12 * want.abs().max()
+    a.ensure_workspace(31)   # a fresh workspace: the fill above went over its guard words
