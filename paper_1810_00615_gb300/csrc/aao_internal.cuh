@@ -541,16 +541,20 @@ bool dst_supported(int64_t n);
 cudaError_t launch_dst_solve(const Ctx &c, void *spec, int prec, int transpose, cudaStream_t s);
 // w = A x - sub (or A^T x - sub) with the Arnoldi dots of w in the same pass:
 // out = [v0 . w (when v0 is given),] sub . w, w . w (the layout launch_multidot
-// gives for the vectors (v0,) sub), then sub . sub with self_dot (no v0).
+// gives for the vectors (v0,) sub); SELF adds sub . sub (no v0), NORM gives
+// w . w alone (no v0).
 // dpart: matvec_dot_partials(c) doubles.  cudaErrorNotSupported for the
 // literal heat form (FP64 stencil kernel).
+enum class MvDots { ARNOLDI, SELF, NORM };
 size_t matvec_dot_partials(const Ctx &c);
 cudaError_t launch_matvec_dots(const Ctx &c, const double *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, bool self_dot = false);
+                               double *dpart, double *out,
+                               MvDots what = MvDots::ARNOLDI);
 cudaError_t launch_matvec_dots(const Ctx &c, const float *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, bool self_dot = false);
+                               double *dpart, double *out,
+                               MvDots what = MvDots::ARNOLDI);
 // y = A x (or A^T x); with `sub`, y = A x - sub (fused, for the shifted Arnoldi).
 cudaError_t launch_matvec(const Ctx &c, const double *x, double *y, int transpose,
                           cudaStream_t s, const double *sub = nullptr);

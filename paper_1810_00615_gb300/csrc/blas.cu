@@ -158,15 +158,23 @@ k_matvec(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
 // the tile maximum.  BD4's weights (sum of magnitudes 12) need two guard
 // bits more: 56 bits, truncation at 2^-55.  x is FP64 (the solution, the public matvec) or FP32
 // (the preconditioned basis of the mixed solver).
-constexpr int kFxRows = 32;   // output time steps per warp tile
-#ifndef AAO_MVFX_U1
-#define AAO_MVFX_U1 16     // unroll of the exponent pass (loads in flight)
-#endif
-#ifndef AAO_MVFX_PRE
-#define AAO_MVFX_PRE 2     // steps of prefetch in the walk
-#endif
-constexpr int kFxU1 = AAO_MVFX_U1;
-
+//
+// GB300: the kernel is bound by the FP64 pipe where it forms dots (an FP64
+// operation per element is ~30 us of that pipe at n 4095 x ell 4096) and by
+// instruction issue elsewhere, so each element is converted to fixed point
+// once, into a shared-memory tile with its two halo columns, and the walk
+// reads a value and its neighbours from there: no shuffles, no second pass
+// over x (whose tiles did not survive in L1: 29 M L2 sectors for 13 M's worth
+// of data at BD2 n 8191 x ell 2048).
+// (hi:lo) >> sh (0 <= sh; all bits out from 64 on), negated where neg is -1.
+__device__ __forceinline__ long long fx_shift(unsigned hi, unsigned lo, int sh, int neg) {
+  const unsigned s2 = (unsigned)max(sh - 32, 0);
+  const unsigned l = __funnelshift_rc(__funnelshift_rc(lo, hi, (unsigned)sh), 0u, s2);
+  const unsigned h = __funnelshift_rc(hi, 0u, (unsigned)sh);
+  const unsigned long long m = (unsigned long long)(long long)neg;
+  return (long long)(((((unsigned long long)h << 32) | l) ^ m) - m);
+}
+constexpr int kFastExp = 64;   // smallest tile exponent of the fast conversions
 
 template <typename XT> struct Fx;
 template <> struct Fx<float> {
@@ -188,6 +196,14 @@ template <> struct Fx<float> {
   }
   template <int G>
   __device__ static int unit(int emax) { return emax - 184 + G; }   // log2 of one unit
+  // the same for emax >= kFastExp: zeros and subnormals, whose missing
+  // implicit bit is not looked at, are shifted out with it
+  template <int G>
+  __device__ static long long fixed_fast(float v, int emax) {
+    const unsigned b = __float_as_uint(v);
+    const unsigned m = (b & 0x7fffffu) | 0x800000u;             // 24 bits, to 58 - G
+    return fx_shift(m << (2 - G), 0u, emax - (int)((b << 1) >> 24), (int)b >> 31);
+  }
 };
 template <> struct Fx<double> {
   static constexpr int kNonFinite = 2047;
@@ -207,6 +223,13 @@ template <> struct Fx<double> {
   }
   template <int G>
   __device__ static int unit(int emax) { return emax - 1080 + G; }
+  template <int G>
+  __device__ static long long fixed_fast(double v, int emax) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned m = (hi & 0xfffffu) | 0x100000u;
+    return fx_shift(__funnelshift_l(lo, m, 5 - G), lo << (5 - G), emax - (int)((hi << 1) >> 21),
+                    (int)hi >> 31);
+  }
 };
 
 // S * 2^unit rounded to nearest even (|S| < 2^63).  With RANGE, results
@@ -231,66 +254,84 @@ __device__ __forceinline__ double fx_to_f64(long long S, int unit) {
   return __longlong_as_double((long long)bits);
 }
 
-#ifndef AAO_MVFX_MINB
-#define AAO_MVFX_MINB 1
-#endif
-
-// The fused Arnoldi dots of the matvec: each warp sums its ND accumulators,
-// parks them in shared memory, and the last warp of the block to arrive adds
-// the warps' values in warp order and stores the block partial (the result
-// does not depend on the arrival order).  Every warp calls it exactly once,
-// with all 32 lanes.
+// The fused dots of the matvec: every lane parks its ND accumulators in shared
+// memory, and the last warp of the block to arrive adds the warps' values lane
+// by lane in warp order, sums the lanes and stores the block partial (the
+// result does not depend on the arrival order).  Every warp calls it exactly
+// once, with all 32 lanes.  The lane sums run ND values at once, each half of
+// the warp passing on half of them: 6 FP64 additions for three values instead
+// of 15 per warp, which at 16 steps a tile were one FP64 operation per element.
 template <int ND, int NW>
-__device__ __forceinline__ void dots_commit(double (&acc)[ND], double (*s_dot)[ND], int *s_cnt,
-                                            double *__restrict__ dpart) {
+__device__ __forceinline__ void dots_commit(const double (&acc)[ND], double (*s_dot)[ND][32],
+                                            int *s_cnt, double *__restrict__ dpart) {
+  static_assert(ND >= 1 && ND <= 3, "one to three values");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int q = 0; q < ND; q++) acc[q] = warp_sum(acc[q]);
-  if (lane == 0) {
+  for (int q = 0; q < ND; q++) s_dot[warp][q][lane] = acc[q];
+  __threadfence_block();
+  __syncwarp();
+  int last = 0;
+  if (lane == 0) last = atomicAdd(s_cnt, 1) == NW - 1;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __threadfence_block();
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int q = 0; q < ND; q++) s_dot[warp][q] = acc[q];
-    __threadfence_block();
-    if (atomicAdd(s_cnt, 1) == NW - 1) {
-      __threadfence_block();
-      const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
+  for (int q = 0; q < ND; q++)
 #pragma unroll
-      for (int q = 0; q < ND; q++) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < NW; w++) t += reinterpret_cast<volatile double *>(s_dot[w])[q];
-        dpart[b * ND + q] = t;
-      }
-    }
+    for (int w = 0; w < NW; w++) t[q] += reinterpret_cast<volatile double *>(s_dot[w][q])[lane];
+  auto cross = [](double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); };
+  double v;
+  if constexpr (ND == 1) {
+    v = t[0] + cross(t[0], 16);
+    v += cross(v, 8);
+  } else if constexpr (ND == 2) {
+    const bool up = lane & 16;                        // lanes 16..: value 1
+    v = (up ? t[1] : t[0]) + cross(up ? t[0] : t[1], 16);
+    v += cross(v, 8);
+  } else {
+    const bool up = lane & 16, odd = lane & 8;        // lanes 0, 8, 16..: values 0, 1, 2
+    const double a = (up ? t[2] : t[0]) + cross(up ? t[0] : t[2], 16);
+    const double b = (up ? t[3] : t[1]) + cross(up ? t[1] : t[3], 16);
+    v = (odd ? b : a) + cross(odd ? a : b, 8);
   }
+  v += cross(v, 4);
+  v += cross(v, 2);
+  v += cross(v, 1);
+  const size_t b = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * ND;
+  constexpr int per = ND == 3 ? 8 : 16;
+  if (lane % per == 0 && lane / per < ND) dpart[b + lane / per] = v;
 }
 
-// DK >= 0 (with SUB): the kernel also forms the Arnoldi dots of its output
-// w = A x - v, as block partials in dpart, ND values per block in order:
+// DK >= 0 (with SUB): the kernel also forms dots of its output w = A x - v,
+// as block partials in dpart, in order:
 //   DK = 0: v . w, w . w
 //   DK = 1: v0 . w, v . w, w . w
 //   DK = 2: v . w, w . w, v . v   (the first step from x0 = 0, v = b: ||b||^2)
-#ifndef AAO_MVFX_DOTS_MINB
-// fused-dots variants: ten CTAs of 128 threads per SM (51 registers, a few
-// words spilled to L1).  Measured at n 4095, ell 4096: 199 us per fused-dots
-// matvec against 211 us with eight CTAs (64 registers, no spills), 207 us
-// with twelve and 237 us with fourteen; the headline solve 1.458 against
-// 1.497 ms.  The walk is latency-bound, so resident warps pay more than
-// the registers they cost.
-#define AAO_MVFX_DOTS_MINB 10
+//   DK = 3: w . w                 (the true residual)
+__host__ __device__ constexpr int fx_dots(int DK) { return DK < 0 ? 0 : (DK == 3 ? 1 : (DK == 0 ? 2 : 3)); }
+
+// Resident CTAs per SM: the walk hides its latencies by warps.
+#ifndef AAO_MVFX_MINB
+#define AAO_MVFX_MINB 8
 #endif
-template <int NB, bool TR, bool SUB, typename XT, bool CIRC, int DK = -1>
-__global__ void __launch_bounds__(kMvCols, DK >= 0 ? AAO_MVFX_DOTS_MINB : AAO_MVFX_MINB)
+#ifndef AAO_MVFX_PRE
+#define AAO_MVFX_PRE 2     // steps of prefetch of the subtrahend
+#endif
+template <int NB, bool TR, bool SUB, typename XT, bool CIRC, int DK, int R>
+__global__ void __launch_bounds__(kMvCols, AAO_MVFX_MINB)
 k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
             const MvRow *__restrict__ rows, const double *__restrict__ sub,
-            const double *__restrict__ dv0 = nullptr, double *__restrict__ dpart = nullptr) {
-  constexpr int R = kFxRows, IN = R + NB - 1;   // input time steps per tile
+            const double *__restrict__ dv0, double *__restrict__ dpart) {
+  constexpr int IN = R + NB - 1;                // input time steps per tile
+  static_assert(IN <= 32, "a lane per halo row");
   constexpr int kWarps = kMvCols / 32;
   constexpr int G = NB == 4 ? 2 : 0;            // guard bits (sums below 2^63)
-  constexpr int ND = DK < 0 ? 1 : (DK == 0 ? 2 : 3);
+  constexpr int ND = fx_dots(DK) ? fx_dots(DK) : 1;
   static_assert(DK < 0 || SUB, "the dots need the subtrahend");
   using F = Fx<XT>;
-  __shared__ long long s_halo[kWarps][2][IN];   // converted halo columns, walk order
-  __shared__ double s_dot[kWarps][ND];
+  // columns iw - 1 .. iw + 32 of the walked steps, in fixed point
+  __shared__ long long s_x[kWarps][IN][34];
+  __shared__ double s_dot[DK >= 0 ? kWarps : 1][ND][32];
   __shared__ int s_cnt;
   if constexpr (DK >= 0) {
     if (threadIdx.x == 0) s_cnt = 0;
@@ -314,37 +355,39 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
   const int t0 = TR ? c0 + IN - 1 : c0 - (NB - 1);
   const int64_t step = (int64_t)dir * n;
   const int ic = col_ok ? i : iw;               // a valid column for every lane
-  const XT *px0 = x + (int64_t)t0 * n + ic;     // dereferenced only on valid steps
   auto t_ok = [&](int t) { return (unsigned)t < (unsigned)ell; };
-  // CIRC (the block circulant P): steps outside [0, ell) wrap around; the
-  // walk pointer is replaced by the wrapped row's address there
+  // CIRC (the block circulant P): steps outside [0, ell) wrap around
   auto wrap = [&](int t) { return ((t % ell) + ell) % ell; };
   // only the first (last) tile of a column walks past the ends in time
   const int t_min = TR ? t0 - (IN - 1) : t0, t_max = TR ? t0 : t0 + IN - 1;
-  const bool wrap_tile = CIRC && (t_min < 0 || t_max >= ell);
-  auto z_ok = [&](int t) { return col_ok && (wrap_tile || t_ok(t)); };
-  auto zaddr = [&](int t, const XT *pw) -> const XT * {
-    if (wrap_tile && !t_ok(t)) return x + (int64_t)wrap(t) * n + ic;
-    return pw;
-  };
+  const bool full = iw + 31 < n && t_min >= 0 && t_max < ell;   // the same for the warp
 
-  // pass 1: the tile's largest exponent (the values land in L1 for pass 2)
-  auto halo = [&](int col, int k) -> XT {
-    int t = t0 + k * dir;
-    if (CIRC) t = wrap(t);
-    return (k < IN && col >= 0 && col < n && t_ok(t)) ? __ldg(&x[(int64_t)t * n + col]) : (XT)0;
-  };
-  const XT hl0 = halo(iw - 1, lane), hr0 = halo(iw + 32, lane);
-  const XT hl1 = (IN > 32) ? halo(iw - 1, lane + 32) : (XT)0;
-  const XT hr1 = (IN > 32) ? halo(iw + 32, lane + 32) : (XT)0;
-  int em = max(max(F::exp(hl0), F::exp(hr0)), max(F::exp(hl1), F::exp(hr1)));
-  {
-    const XT *p = px0;
-    int t = t0;
-#pragma unroll kFxU1
-    for (int k = 0; k < IN; k++, p += step, t += dir)
-      if (z_ok(t)) em = max(em, F::exp(__ldg(zaddr(t, p))));
+  // the tile's values, all loads in flight together, and its largest exponent
+  XT z[IN];
+  const XT *px = x + (int64_t)t0 * n + ic;      // dereferenced only on valid steps
+  if (full) {
+#pragma unroll
+    for (int k = 0; k < IN; k++) z[k] = __ldg(px + k * step);
+  } else {
+#pragma unroll
+    for (int k = 0; k < IN; k++) {
+      const int t = t0 + k * dir;
+      const bool ok = col_ok && (CIRC || t_ok(t));
+      z[k] = ok ? __ldg(CIRC && !t_ok(t) ? x + (int64_t)wrap(t) * n + ic : px + k * step) : (XT)0;
+    }
   }
+  XT hl = (XT)0, hr = (XT)0;                    // lane k: the halo columns of walk step k
+  {
+    int t = t0 + lane * dir;
+    if (CIRC) t = wrap(t);
+    if (lane < IN && t_ok(t)) {
+      if (iw > 0) hl = __ldg(&x[(int64_t)t * n + iw - 1]);
+      if (iw + 32 < n) hr = __ldg(&x[(int64_t)t * n + iw + 32]);
+    }
+  }
+  int em = max(F::exp(hl), F::exp(hr));
+#pragma unroll
+  for (int k = 0; k < IN; k++) em = max(em, F::exp(z[k]));
   em = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
   if (em == F::kNonFinite) {                    // an inf or NaN in the tile
     if (col_ok)
@@ -358,67 +401,68 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
     return;
   }
   const int unit = F::template unit<G>(em);
-  if (lane < IN) {
-    s_halo[warp][0][lane] = F::template fixed<G>(hl0, em);
-    s_halo[warp][1][lane] = F::template fixed<G>(hr0, em);
+  long long(*sx)[34] = s_x[warp];
+  if (em >= kFastExp) {
+#pragma unroll
+    for (int k = 0; k < IN; k++) sx[k][lane + 1] = F::template fixed_fast<G>(z[k], em);
+  } else {
+#pragma unroll
+    for (int k = 0; k < IN; k++) sx[k][lane + 1] = F::template fixed<G>(z[k], em);
   }
-  if (IN > 32 && lane + 32 < IN) {
-    s_halo[warp][0][lane + 32] = F::template fixed<G>(hl1, em);
-    s_halo[warp][1][lane + 32] = F::template fixed<G>(hr1, em);
+  if (lane < IN) {
+    sx[lane][0] = F::template fixed<G>(hl, em);
+    sx[lane][33] = F::template fixed<G>(hr, em);
   }
   __syncwarp();
 
-  // pass 2: walk the steps; x and the subtrahend come kPre steps ahead so
-  // their latency hides behind the integer work of the steps in between
+  // walk the output steps; the subtrahend comes kPre steps ahead so that its
+  // latency hides behind the integer work of the steps in between.  FULL:
+  // every column of the warp and every walked step lie inside the system;
+  // RNG: results below or above the FP64 normal range are possible (FP64
+  // input with an extreme tile exponent); ZERO: v0 (DK = 1) or v (DK = 2) is
+  // zero on the whole tile.
   constexpr int kPre = AAO_MVFX_PRE;
-  const double *pv0 = SUB ? sub + (int64_t)t0 * n + ic : nullptr;
-  const double *pd0 = (DK == 1) ? dv0 + (int64_t)t0 * n + ic : nullptr;
-  XT zpre[kPre];
-  double vpre[kPre], dpre[kPre];
+  static_assert(R % kPre == 0, "whole prefetch rounds");
+  const int64_t first = (int64_t)(t0 + (NB - 1) * dir) * n + ic;   // output step 0
+  auto walk = [&](auto full_c, auto rng_c, auto zero_c) {
+    constexpr bool FULL = decltype(full_c)::value, RNG = decltype(rng_c)::value;
+    constexpr bool ZERO = decltype(zero_c)::value;
+    constexpr bool V = SUB && !(ZERO && DK == 2), D = DK == 1 && !ZERO;   // streams read
+    long long q1 = 0, q2 = 0, q3 = 0;           // q of the steps before
+    auto stencil = [&](int k, long long &X, long long &P) {
+      X = sx[k][lane + 1];
+      P = sx[k][lane] + sx[k][lane + 2];
+      return 4 * X + P;
+    };
 #pragma unroll
-  for (int k = 0; k < kPre; k++) {
-    const int t = t0 + k * dir;
-    zpre[k] = z_ok(t) ? __ldg(zaddr(t, px0 + k * step)) : (XT)0;
-    vpre[k] = (SUB && col_ok && t_ok(t) && k >= NB - 1) ? __ldg(pv0 + k * step) : 0.0;
-    dpre[k] = (DK == 1 && col_ok && t_ok(t) && k >= NB - 1) ? __ldg(pd0 + k * step) : 0.0;
-  }
-  const XT *pz = px0 + kPre * step;
-  const double *pv = SUB ? pv0 + kPre * step : nullptr;
-  const double *pd = (DK == 1) ? pd0 + kPre * step : nullptr;
-  double *py = y + (int64_t)t0 * n + ic;
-  // FULL: every column of the warp and every walked step lie inside the
-  // system (no per-step range checks); RNG: results below or above the FP64
-  // normal range are possible (FP64 input with an extreme tile exponent)
-  auto walk = [&](auto full_c, auto rng_c) {
-  constexpr bool FULL = decltype(full_c)::value, RNG = decltype(rng_c)::value;
-  long long q1 = 0, q2 = 0, q3 = 0;             // q of the previous steps walked
+    for (int k = 0; k < NB - 1; k++) {
+      long long X, P;
+      q3 = q2;
+      q2 = q1;
+      q1 = stencil(k, X, P);
+    }
+    double vpre[kPre], dpre[kPre];
+    const double *pv = V ? sub + first : nullptr, *pd = D ? dv0 + first : nullptr;
+    auto fetch = [&](int r, int u) {
+      const bool in = r < R && (FULL || (col_ok && t_ok(t0 + (NB - 1 + r) * dir)));
+      if (V) vpre[u] = in ? __ldg(pv) : 0.0;
+      if (D) dpre[u] = in ? __ldg(pd) : 0.0;
+      if (V) pv += step;
+      if (D) pd += step;
+    };
+#pragma unroll
+    for (int u = 0; u < kPre; u++) fetch(u, u);
+    double *py = y + first;
 #pragma unroll 1
-  for (int kb = 0; kb < IN; kb += kPre) {
+    for (int rb = 0; rb < R; rb += kPre) {
 #pragma unroll
-    for (int u = 0; u < kPre; u++) {
-      const int k = kb + u;
-      const int t = t0 + k * dir;
-      const XT zk = zpre[u];
-      const double vk = vpre[u], dk = dpre[u];
-      {
-        const int tn = t + kPre * dir;
-        const bool inb = k + kPre < IN;
-        const bool vin = inb && (FULL || (col_ok && t_ok(tn)));
-        zpre[u] = (inb && (FULL || z_ok(tn))) ? __ldg(FULL ? pz : zaddr(tn, pz)) : (XT)0;
-        if (SUB) vpre[u] = vin ? __ldg(pv) : 0.0;
-        if (DK == 1) dpre[u] = vin ? __ldg(pd) : 0.0;
-        pz += step;
-        if (SUB) pv += step;
-        if (DK == 1) pd += step;
-      }
-      const long long X = F::template fixed<G>(zk, em);
-      long long Xl = __shfl_up_sync(0xffffffffu, X, 1);
-      long long Xr = __shfl_down_sync(0xffffffffu, X, 1);
-      if (lane == 0) Xl = s_halo[warp][0][k < IN ? k : 0];
-      if (lane == 31) Xr = s_halo[warp][1][k < IN ? k : 0];
-      const long long P = Xl + Xr;
-      const long long q = 4 * X + P;
-      if (k >= NB - 1 && k < IN && (FULL || (col_ok && t_ok(t)))) {
+      for (int u = 0; u < kPre; u++) {
+        const int r = rb + u, t = t0 + (NB - 1 + r) * dir;
+        const double vk = V ? vpre[u] : 0.0;
+        [[maybe_unused]] const double dk = D ? dpre[u] : 0.0;
+        fetch(r + kPre, u);
+        long long X, P;
+        const long long q = stencil(NB - 1 + r, X, P);
         long long sm;
         if (NB == 2) {
           sm = q - q1;
@@ -431,42 +475,81 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
             else sm = t == 0 ? q - 2 * q1 + 4 * q2 - q3 : q - 5 * q1 + 4 * q2 - q3;
           }
         }
-        const long long sk = 2 * X - P;
-        // T = S_main + frac S_other, exact up to the truncated product; one
-        // rounding to FP64 and one FMA
-        const MvRow rw = rows[t];
-        const long long s_main = rw.main_k ? sk : sm, s_oth = rw.main_k ? sm : sk;
-        const unsigned long long so_neg = (unsigned long long)(s_oth >> 63);
-        const unsigned long long so_abs = ((unsigned long long)s_oth ^ so_neg) - so_neg;
-        const long long prod = (long long)__umul64hi(so_abs, rw.frac);
-        const long long T = s_main + (so_neg ? -prod : prod);
-        const double td = fx_to_f64<RNG>(T, unit);
-        const double yv = SUB ? fma(rw.coef, td, -vk) : rw.coef * td;
-        py[(int64_t)k * step] = yv;
-        if constexpr (DK == 1) {
-          dacc[0] = fma(dk, yv, dacc[0]);
-          dacc[1] = fma(vk, yv, dacc[1]);
-          dacc[2] = fma(yv, yv, dacc[2]);
-        } else if constexpr (DK >= 0) {
-          dacc[0] = fma(vk, yv, dacc[0]);
-          dacc[1] = fma(yv, yv, dacc[1]);
-          if constexpr (DK == 2) dacc[2] = fma(vk, vk, dacc[2]);
+        q3 = q2;
+        q2 = q1;
+        q1 = q;
+        if (FULL || (col_ok && t_ok(t))) {
+          const long long sk = 2 * X - P;
+          // T = S_main + frac S_other, exact up to the truncated product; one
+          // rounding to FP64 and one FMA
+          const MvRow rw = rows[t];
+          const long long s_main = rw.main_k ? sk : sm, s_oth = rw.main_k ? sm : sk;
+          // truncated towards zero: the one-sided rounding of a floor, though
+          // below a unit, adds up over a smooth field (it put a bias of 1e-10
+          // into the kappa gradient at n = 16383)
+          const unsigned long long so_neg = (unsigned long long)(s_oth >> 63);
+          const unsigned long long so_abs = ((unsigned long long)s_oth ^ so_neg) - so_neg;
+          const unsigned long long pa = __umul64hi(so_abs, rw.frac);
+          const long long prod = (long long)((pa ^ so_neg) - so_neg);
+          const double td = fx_to_f64<RNG>(s_main + prod, unit);
+          const double yv = V ? fma(rw.coef, td, -vk) : rw.coef * td;
+          *py = yv;
+          if constexpr (DK == 1) {
+            if constexpr (!ZERO) dacc[0] = fma(dk, yv, dacc[0]);
+            dacc[1] = fma(vk, yv, dacc[1]);
+            dacc[2] = fma(yv, yv, dacc[2]);
+          } else if constexpr (DK == 3) {
+            dacc[0] = fma(yv, yv, dacc[0]);
+          } else if constexpr (DK >= 0) {
+            if constexpr (!ZERO) dacc[0] = fma(vk, yv, dacc[0]);
+            dacc[1] = fma(yv, yv, dacc[1]);
+            if constexpr (DK == 2 && !ZERO) dacc[2] = fma(vk, vk, dacc[2]);
+          }
         }
+        py += step;
       }
-      q3 = q2;
-      q2 = q1;
-      q1 = q;
     }
-  }
   };
   // |S| < 2^63, so S 2^unit stays a normal FP64 number or zero for
   // -1022 <= unit <= 960; FP32 input always does
   constexpr bool RANGE = sizeof(XT) == 8;
   const bool in_range = !RANGE || (unit >= -1022 && unit <= 960);
-  const bool full = iw + 31 < n && t_min >= 0 && t_max < ell;   // the same for the warp
-  if (full && in_range) walk(std::true_type{}, std::false_type{});
-  else walk(std::false_type{}, std::integral_constant<bool, RANGE>{});
+  if constexpr (DK == 1 || DK == 2) {
+    // The right-hand side of an all-at-once system is zero past its first
+    // block rows, and in a solve from x = 0 it is v0 (DK = 1) and v (DK = 2):
+    // tiles where it is zero skip the products with it, one or two FP64
+    // operations of the bound pipe per element.  A dense vector costs a vote
+    // on the tile's first step.  (unit <= 0 keeps the outputs finite, so that
+    // no 0 x inf is dropped.)
+    if (full && in_range && unit <= 0) {
+      const double *pz = (DK == 1 ? dv0 : sub) + first;
+      auto nonzero = [](double a) { return (unsigned long long)__double_as_longlong(a) << 1; };
+      unsigned long long any = nonzero(__ldg(pz));
+      if (!__any_sync(0xffffffffu, any != 0)) {
+#pragma unroll
+        for (int r = 1; r < R; r++) any |= nonzero(__ldg(pz + r * step));
+        if (!__any_sync(0xffffffffu, any != 0)) {
+          walk(std::true_type{}, std::false_type{}, std::true_type{});
+          dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
+          return;
+        }
+      }
+    }
+  }
+  if (full && in_range) walk(std::true_type{}, std::false_type{}, std::false_type{});
+  else walk(std::false_type{}, std::integral_constant<bool, RANGE>{}, std::false_type{});
   if constexpr (DK >= 0) dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
+}
+
+// Output time steps per warp tile: 16, or 8 where the 16-step tiles leave
+// fewer than four CTAs per SM (short walks, more of them in flight).
+constexpr int kFxRows = 16, kFxRowsSmall = 8;
+static bool fx_small(const Ctx &c) {
+  return (c.n + kMvCols - 1) / kMvCols * ((c.ell + kFxRows - 1) / kFxRows) < 4 * 152;
+}
+static dim3 mv_fx_grid(const Ctx &c) {
+  const int R = fx_small(c) ? kFxRowsSmall : kFxRows;
+  return dim3((unsigned)((c.n + kMvCols - 1) / kMvCols), (unsigned)((c.ell + R - 1) / R));
 }
 
 template <int NB, bool TR, typename XT, bool CIRC>
@@ -498,15 +581,23 @@ static cudaError_t matvec_any(const Ctx &c, const XT *x, double *y, int transpos
   return cudaGetLastError();
 }
 
-template <int NB, bool TR, typename XT, bool CIRC>
-static void mv_fx(const Ctx &c, dim3 grid, const XT *x, double *y, const double *sub,
-                  cudaStream_t s) {
+template <int NB, bool TR, bool SUB, typename XT, bool CIRC, int DK>
+static void run_fx(const Ctx &c, const XT *x, double *y, const double *sub, const double *v0,
+                   double *dpart, cudaStream_t s) {
   const int n = (int)c.n, ell = (int)c.ell;
   const MvRow *rows = CIRC ? c.mv_rows_p : c.mv_rows;
-  if (sub)
-    k_matvec_fx<NB, TR, true, XT, CIRC><<<grid, kMvCols, 0, s>>>(x, y, n, ell, rows, sub);
+  const dim3 grid = mv_fx_grid(c);
+  if (fx_small(c))
+    k_matvec_fx<NB, TR, SUB, XT, CIRC, DK, kFxRowsSmall><<<grid, kMvCols, 0, s>>>(x, y, n, ell, rows, sub, v0, dpart);
   else
-    k_matvec_fx<NB, TR, false, XT, CIRC><<<grid, kMvCols, 0, s>>>(x, y, n, ell, rows, nullptr);
+    k_matvec_fx<NB, TR, SUB, XT, CIRC, DK, kFxRows><<<grid, kMvCols, 0, s>>>(x, y, n, ell, rows, sub, v0, dpart);
+  note_launch();
+}
+
+template <int NB, bool TR, typename XT, bool CIRC>
+static void mv_fx(const Ctx &c, const XT *x, double *y, const double *sub, cudaStream_t s) {
+  if (sub) run_fx<NB, TR, true, XT, CIRC, -1>(c, x, y, sub, nullptr, nullptr, s);
+  else run_fx<NB, TR, false, XT, CIRC, -1>(c, x, y, nullptr, nullptr, nullptr, s);
 }
 
 // Heat, BD2 and BD4 take the fixed-point kernel; the literal heat form (whose M
@@ -516,17 +607,13 @@ template <typename XT, bool CIRC = false>
 static cudaError_t matvec_dispatch(const Ctx &c, const XT *x, double *y, int transpose,
                                    cudaStream_t s, const double *sub) {
   if (c.equation == AAO_HEAT_LITERAL) return matvec_any<XT, CIRC>(c, x, y, transpose, s, sub);
-  const int n = (int)c.n, ell = (int)c.ell;
-  const dim3 grid((unsigned)((n + kMvCols - 1) / kMvCols),
-                  (unsigned)((ell + kFxRows - 1) / kFxRows));
   const bool bd2 = c.equation == AAO_WAVE_BD2, bd4 = c.equation == AAO_WAVE_BD4;
-  if (bd4 && transpose) mv_fx<4, true, XT, CIRC>(c, grid, x, y, sub, s);
-  else if (bd4) mv_fx<4, false, XT, CIRC>(c, grid, x, y, sub, s);
-  else if (bd2 && transpose) mv_fx<3, true, XT, CIRC>(c, grid, x, y, sub, s);
-  else if (bd2) mv_fx<3, false, XT, CIRC>(c, grid, x, y, sub, s);
-  else if (transpose) mv_fx<2, true, XT, CIRC>(c, grid, x, y, sub, s);
-  else mv_fx<2, false, XT, CIRC>(c, grid, x, y, sub, s);
-  note_launch();
+  if (bd4 && transpose) mv_fx<4, true, XT, CIRC>(c, x, y, sub, s);
+  else if (bd4) mv_fx<4, false, XT, CIRC>(c, x, y, sub, s);
+  else if (bd2 && transpose) mv_fx<3, true, XT, CIRC>(c, x, y, sub, s);
+  else if (bd2) mv_fx<3, false, XT, CIRC>(c, x, y, sub, s);
+  else if (transpose) mv_fx<2, true, XT, CIRC>(c, x, y, sub, s);
+  else mv_fx<2, false, XT, CIRC>(c, x, y, sub, s);
   return cudaGetLastError();
 }
 
@@ -549,43 +636,38 @@ k_finish_wide(const double *__restrict__ p, int nb, int nd, double *__restrict__
   }
 }
 
-static dim3 mv_fx_grid(const Ctx &c) {
-  return dim3((unsigned)((c.n + kMvCols - 1) / kMvCols),
-              (unsigned)((c.ell + kFxRows - 1) / kFxRows));
-}
-
 size_t matvec_dot_partials(const Ctx &c) {
   const dim3 g = mv_fx_grid(c);
   return (size_t)g.x * g.y * 3;
 }
 
-// w = A x - sub with the Arnoldi dots of w fused in: out = [v0 . w,] sub . w,
-// w . w (DK = 0, 1), or sub . w, w . w, sub . sub with self_dot (DK = 2).
+// w = A x - sub with dots of w fused in: out = [v0 . w,] sub . w, w . w
+// (DK = 0, 1), sub . w, w . w, sub . sub (MvDots::SELF) or w . w alone
+// (MvDots::NORM).
 template <typename XT>
 static cudaError_t matvec_dots_dispatch(const Ctx &c, const XT *x, double *y, int transpose,
                                         cudaStream_t s, const double *sub, const double *v0,
-                                        double *dpart, double *out, bool self_dot) {
-  if (c.equation == AAO_HEAT_LITERAL || !sub || (v0 && self_dot)) return cudaErrorNotSupported;
-  const dim3 grid = mv_fx_grid(c);
-  const int n = (int)c.n, ell = (int)c.ell;
+                                        double *dpart, double *out, MvDots what) {
+  if (c.equation == AAO_HEAT_LITERAL || !sub || (v0 && what != MvDots::ARNOLDI))
+    return cudaErrorNotSupported;
   const int nb = c.equation == AAO_WAVE_BD4 ? 4 : (c.equation == AAO_WAVE_BD2 ? 3 : 2);
-  const int dk = v0 ? 1 : (self_dot ? 2 : 0);
+  const int dk = v0 ? 1 : (what == MvDots::SELF ? 2 : (what == MvDots::NORM ? 3 : 0));
   const int key = nb * 8 + (transpose ? 4 : 0) + dk;
 #define AAO_MVD(NBV, TRV, DKV)                                                           \
   case NBV * 8 + (TRV ? 4 : 0) + DKV:                                                    \
-    k_matvec_fx<NBV, TRV, true, XT, false, DKV><<<grid, kMvCols, 0, s>>>(               \
-        x, y, n, ell, c.mv_rows, sub, v0, dpart);                                        \
+    run_fx<NBV, TRV, true, XT, false, DKV>(c, x, y, sub, v0, dpart, s);                  \
     break;
-#define AAO_MVD3(NBV, TRV) AAO_MVD(NBV, TRV, 0) AAO_MVD(NBV, TRV, 1) AAO_MVD(NBV, TRV, 2)
+#define AAO_MVD4(NBV, TRV) \
+  AAO_MVD(NBV, TRV, 0) AAO_MVD(NBV, TRV, 1) AAO_MVD(NBV, TRV, 2) AAO_MVD(NBV, TRV, 3)
   switch (key) {
-    AAO_MVD3(2, false) AAO_MVD3(2, true) AAO_MVD3(3, false) AAO_MVD3(3, true)
-    AAO_MVD3(4, false) AAO_MVD3(4, true)
+    AAO_MVD4(2, false) AAO_MVD4(2, true) AAO_MVD4(3, false) AAO_MVD4(3, true)
+    AAO_MVD4(4, false) AAO_MVD4(4, true)
     default: return cudaErrorNotSupported;
   }
-#undef AAO_MVD3
+#undef AAO_MVD4
 #undef AAO_MVD
-  note_launch();
-  const int nd = dk == 0 ? 2 : 3;
+  const dim3 grid = mv_fx_grid(c);
+  const int nd = fx_dots(dk);
   k_finish_wide<<<nd, kThreads, 0, s>>>(dpart, (int)(grid.x * grid.y), nd, out);
   note_launch();
   return cudaGetLastError();
@@ -593,14 +675,14 @@ static cudaError_t matvec_dots_dispatch(const Ctx &c, const XT *x, double *y, in
 
 cudaError_t launch_matvec_dots(const Ctx &c, const double *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, bool self_dot) {
-  return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, self_dot);
+                               double *dpart, double *out, MvDots what) {
+  return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, what);
 }
 
 cudaError_t launch_matvec_dots(const Ctx &c, const float *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, bool self_dot) {
-  return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, self_dot);
+                               double *dpart, double *out, MvDots what) {
+  return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, what);
 }
 
 // ------------------------------------------ compensated circulant residual

@@ -909,13 +909,12 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       // same kernel where the fixed-point matvec serves); v_0 = -V_0 / beta
       V[0] = v0_slot;
       if (c.equation != AAO_HEAT_LITERAL) {
-        // out = [b . V_0, V_0 . V_0] at d_nr
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-          return aao::launch_matvec_dots(c, x, V[0], tr, s, b, nullptr, dpart, d_nr);
+          return aao::launch_matvec_dots(c, x, V[0], tr, s, b, nullptr, dpart, d_nr,
+                                         aao::MvDots::NORM);
         }));
-        AAO_CK(c, fetch(d_nr, 2));
+        AAO_CK(c, fetch(d_nr, 1));
         AAO_CK(c, cudaStreamSynchronize(s));
-        hs[320] = hs[321];
       } else {
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] { return aao::launch_matvec(c, x, V[0], tr, s, b); }));
         AAO_CK(c, norm2(V[0]));
@@ -962,7 +961,8 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       const bool fused = nv <= 2 && c.equation != AAO_HEAT_LITERAL;
       if (fused) {
         const double *v0 = nv == 2 ? V[0] : nullptr;
-        const bool self = defer_b;   // also b . b (step 0 of the first cycle)
+        // also b . b at step 0 of the first cycle
+        const auto self = defer_b ? aao::MvDots::SELF : aao::MvDots::ARNOLDI;
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
           return zf ? aao::launch_matvec_dots(c, Zf[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, d_h1, self)
                     : aao::launch_matvec_dots(c, Z[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, d_h1, self);
@@ -1455,15 +1455,14 @@ int aao_residual(aao_ctx *ctx, const double *x, const double *b, double *r, int 
   const aao::WsLayout L = aao::ws_layout(c, 0);
   double *red = reinterpret_cast<double *>(c.ws + L.red);
   double *dpart = reinterpret_cast<double *>(c.ws + L.dots);
-  double *out = red + kPartials + 970;   // 2 doubles of the small-result area
+  double *out = red + kPartials + 970;   // in the small-result area
   cudaStream_t s = as_stream(stream);
   const int tr = transpose ? 1 : 0;
   if (c.equation != AAO_HEAT_LITERAL) {
     AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-      return aao::launch_matvec_dots(c, x, r, tr, s, b, nullptr, dpart, out);
+      return aao::launch_matvec_dots(c, x, r, tr, s, b, nullptr, dpart, out, aao::MvDots::NORM);
     }));
-    AAO_CK(c, cudaMemcpyAsync(c.host_small + 970, out + 1, sizeof(double),
-                              cudaMemcpyDeviceToHost, s));
+    AAO_CK(c, cudaMemcpyAsync(c.host_small + 970, out, sizeof(double), cudaMemcpyDeviceToHost, s));
   } else {
     AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] { return aao::launch_matvec(c, x, r, tr, s, b); }));
     AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
