@@ -539,6 +539,13 @@ cudaError_t fft_inverse_f32_correct(const Ctx &c, const void *spec, void *sep, d
 constexpr int64_t kDstMaxL = 4096;   // n + 1 <= kDstMaxL, a power of two
 bool dst_supported(int64_t n);
 cudaError_t launch_dst_solve(const Ctx &c, void *spec, int prec, int transpose, cudaStream_t s);
+// Where a reduction puts its sums: device memory and pinned host memory
+// (NULL: none).
+struct RedOut {
+  double *dev, *host;
+  RedOut at(int j) const { return RedOut{dev + j, host ? host + j : nullptr}; }
+};
+
 // w = A x - sub (or A^T x - sub) with the Arnoldi dots of w in the same pass:
 // out = [v0 . w (when v0 is given),] sub . w, w . w (the layout launch_multidot
 // gives for the vectors (v0,) sub); SELF adds sub . sub (no v0), NORM gives
@@ -549,11 +556,11 @@ enum class MvDots { ARNOLDI, SELF, NORM };
 size_t matvec_dot_partials(const Ctx &c);
 cudaError_t launch_matvec_dots(const Ctx &c, const double *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out,
+                               double *dpart, const RedOut &out,
                                MvDots what = MvDots::ARNOLDI);
 cudaError_t launch_matvec_dots(const Ctx &c, const float *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out,
+                               double *dpart, const RedOut &out,
                                MvDots what = MvDots::ARNOLDI);
 // y = A x (or A^T x); with `sub`, y = A x - sub (fused, for the shifted Arnoldi).
 cudaError_t launch_matvec(const Ctx &c, const double *x, double *y, int transpose,
@@ -583,19 +590,20 @@ cudaError_t launch_rhs(const Ctx &c, const double *u0, const double *v0, double 
 // writes the final sums to out (device).
 int  red_blocks(int64_t N);
 cudaError_t launch_norms2(const double *a, const double *b, int64_t N, double *partials,
-                          double *out, cudaStream_t s);
+                          const RedOut &out, cudaStream_t s);
 cudaError_t launch_multidot(const double *const *V, int nv, const double *w, int64_t N,
-                            bool with_norm, double *partials, double *out, cudaStream_t s);
+                            bool with_norm, double *partials, const RedOut &out, cudaStream_t s);
 // w -= sum_j hf[j] h[j] V_j (h on device, hf host factors, NULL = 1; with
-// div0 the j = 0 term is also divided by the device value *div0);
-// optionally fused: dots of the updated w with V_j (out2[j]); always its
-// squared norm (out2[nv]).
-cudaError_t launch_update_dots(const double *const *V, int nv, const double *h,
-                               double *w, int64_t N, bool want_dots, double *partials,
-                               double *out2, cudaStream_t s, const double *hf = nullptr,
-                               const double *div0 = nullptr);
-// x += sum_j y[j] Z_j (y on device)
-// x += Z y, or x = Z y (x not read) with assign
+// div0 the j = 0 term is also divided by the device value *div0) and the
+// updated w's squared norm.  With before (the device value ||w||^2 before the
+// update; nv <= 8): out = V_j . w (j < nv; formed where the norm is predicted to
+// fall below 0.55 of it), the norm, and 1 or 0 for dots formed or not;
+// otherwise out = the norm.
+cudaError_t launch_update(const double *const *V, int nv, const double *h, double *w, int64_t N,
+                          double *partials, const RedOut &out, cudaStream_t s,
+                          const double *hf = nullptr, const double *div0 = nullptr,
+                          const double *before = nullptr);
+// x += Z y (y on the host), or x = Z y (x not read) with assign
 cudaError_t launch_combine(const double *const *Z, int nv, const double *y, double *x,
                            int64_t N, cudaStream_t s, bool assign = false);
 cudaError_t launch_combine(const float *const *Z, int nv, const double *y, double *x,
@@ -603,10 +611,8 @@ cudaError_t launch_combine(const float *const *Z, int nv, const double *y, doubl
 // y = a*x (a on device, *a_scale of index)
 cudaError_t launch_scale(const double *x, double *y, const double *a, int64_t N,
                          bool invert, cudaStream_t s, bool negate = false);
-// r = b - r (in place on r)
-cudaError_t launch_sub_from(const double *b, double *r, int64_t N, cudaStream_t s);
 cudaError_t launch_adjoint_grads(const Ctx &c, const double *lam, const double *U,
-                                 double *g_u0, double *partials, double *out,
+                                 double *g_u0, double *partials, const RedOut &out,
                                  cudaStream_t s);
 // Conversion self-test: to_f32 / to_f64 beside __double2float_rn and the
 // widening cast, element by element (device arrays).

@@ -23,7 +23,7 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block-reduce NV values per thread into partials[blockIdx.x * NV + j].
+// Block-reduce NV values per thread into partials[block * NV + j].
 template <int NV>
 __device__ __forceinline__ void block_store(double (&acc)[NV], double *partials) {
   __shared__ double sm[kThreads / 32][NV > 0 ? NV : 1];
@@ -38,18 +38,48 @@ __device__ __forceinline__ void block_store(double (&acc)[NV], double *partials)
     double s = 0.0;
 #pragma unroll
     for (int w = 0; w < kThreads / 32; w++) s += sm[w][threadIdx.x];
-    partials[(size_t)blockIdx.x * NV + threadIdx.x] = s;
+    partials[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * NV + threadIdx.x] = s;
   }
 }
 
-// out[j] = sum_b partials[b * nv + j] in a fixed order (one warp per output).
-__global__ void k_finish(const double *__restrict__ partials, int nb, int nv,
-                         double *__restrict__ out) {
+// out[j] = sum_b partials[b * nv + j] in a fixed order, one block of NT threads
+// per output, into device memory and, straight over the host link, into
+// pinned host memory: a small result costs the stream no copy (6 of them,
+// 8 us of a 125 us solve at n 63 x ell 64).  Launched as a dependent of the
+// kernel that writes the partials.  (Letting that kernel's last block add them
+// saved this launch but cost every block a fence and an atomic: 145 -> 166 us
+// for the fused-dots matvec at n 4095 x ell 4096.)
+template <int NT>
+__global__ void __launch_bounds__(NT)
+k_finish(const double *__restrict__ partials, int nb, int nv, RedOut out) {
+  __shared__ double sm[NT / 32];
   const int j = blockIdx.x;
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nb; b += 32) s += partials[(size_t)b * nv + j];
-  s = warp_sum(s);
-  if (threadIdx.x == 0) out[j] = s;
+  pdl_wait(partials);
+  double v = 0.0;
+#pragma unroll 8
+  for (int b = threadIdx.x; b < nb; b += NT) v += partials[(size_t)b * nv + j];
+  v = warp_sum(v);
+  if constexpr (NT > 32) {
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int w = 0; w < NT / 32; w++) v += sm[w];
+    }
+  }
+  if (threadIdx.x == 0) {
+    out.dev[j] = v;
+    if (out.host) out.host[j] = v;
+  }
+}
+cudaError_t finish(const double *partials, int nb, int nv, const RedOut &out, cudaStream_t s) {
+  const cudaError_t e =
+      nb <= 64 ? launch_pdl(k_finish<32>, dim3(nv), dim3(32), 0, s, partials, nb, nv, out)
+      : nb <= 2048 ? launch_pdl(k_finish<256>, dim3(nv), dim3(256), 0, s, partials, nb, nv, out)
+                   : launch_pdl(k_finish<1024>, dim3(nv), dim3(1024), 0, s, partials, nb, nv, out);
+  note_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 struct Ptrs8 {
@@ -617,25 +647,6 @@ static cudaError_t matvec_dispatch(const Ctx &c, const XT *x, double *y, int tra
   return cudaGetLastError();
 }
 
-// out[j] = sum_b p[b * nd + j] in a fixed order, one 256-thread CTA per value
-// (the fused matvec leaves one partial per block: thousands of them).
-__global__ void __launch_bounds__(kThreads)
-k_finish_wide(const double *__restrict__ p, int nb, int nd, double *__restrict__ out) {
-  __shared__ double sm[kThreads / 32];
-  const int j = blockIdx.x;
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kThreads) v += p[(size_t)b * nd + j];
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; w++) t += sm[w];
-    out[j] = t;
-  }
-}
-
 size_t matvec_dot_partials(const Ctx &c) {
   const dim3 g = mv_fx_grid(c);
   return (size_t)g.x * g.y * 3;
@@ -647,7 +658,7 @@ size_t matvec_dot_partials(const Ctx &c) {
 template <typename XT>
 static cudaError_t matvec_dots_dispatch(const Ctx &c, const XT *x, double *y, int transpose,
                                         cudaStream_t s, const double *sub, const double *v0,
-                                        double *dpart, double *out, MvDots what) {
+                                        double *dpart, const RedOut &out, MvDots what) {
   if (c.equation == AAO_HEAT_LITERAL || !sub || (v0 && what != MvDots::ARNOLDI))
     return cudaErrorNotSupported;
   const int nb = c.equation == AAO_WAVE_BD4 ? 4 : (c.equation == AAO_WAVE_BD2 ? 3 : 2);
@@ -667,21 +678,18 @@ static cudaError_t matvec_dots_dispatch(const Ctx &c, const XT *x, double *y, in
 #undef AAO_MVD4
 #undef AAO_MVD
   const dim3 grid = mv_fx_grid(c);
-  const int nd = fx_dots(dk);
-  k_finish_wide<<<nd, kThreads, 0, s>>>(dpart, (int)(grid.x * grid.y), nd, out);
-  note_launch();
-  return cudaGetLastError();
+  return finish(dpart, (int)(grid.x * grid.y), fx_dots(dk), out, s);
 }
 
 cudaError_t launch_matvec_dots(const Ctx &c, const double *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, MvDots what) {
+                               double *dpart, const RedOut &out, MvDots what) {
   return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, what);
 }
 
 cudaError_t launch_matvec_dots(const Ctx &c, const float *x, double *y, int transpose,
                                cudaStream_t s, const double *sub, const double *v0,
-                               double *dpart, double *out, MvDots what) {
+                               double *dpart, const RedOut &out, MvDots what) {
   return matvec_dots_dispatch(c, x, y, transpose, s, sub, v0, dpart, out, what);
 }
 
@@ -985,24 +993,33 @@ cudaError_t launch_circ_residual(const Ctx &c, const float *z, double *y, int tr
 // u = x - E y with (E y)_t = sigk_t (2 y_i - y_{i-1} - y_{i+1}), sigk_t =
 // (tau_t - tau) kappa / h (Section 2): the right-hand side of a Neumann term,
 // formed in FP64 for the refined FP32 preconditioner.
-__global__ void k_neumann_rhs(const double *__restrict__ x, const double *__restrict__ y,
-                              const double *__restrict__ sigk, double *__restrict__ u, int n,
-                              int64_t N) {
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(g / n);
-    const int i = (int)(g - (int64_t)t * n);
+__global__ void __launch_bounds__(kThreads)
+k_neumann_rhs(const double *__restrict__ x, const double *__restrict__ y,
+              const double *__restrict__ sigk, double *__restrict__ u, int n, int ell) {
+  const int i = blockIdx.x * kThreads + threadIdx.x;
+  if (i >= n) return;
+  for (int t = blockIdx.y; t < ell; t += gridDim.y) {
+    const int64_t g = (int64_t)t * n + i;
     const double yc = y[g];
     const double s = ((i > 0) ? y[g - 1] : 0.0) + ((i + 1 < n) ? y[g + 1] : 0.0);
     u[g] = fma(-__ldg(&sigk[t]), fma(2.0, yc, -s), x[g]);
   }
 }
 
+// Grid of the kernels that walk a block vector with a thread per column and
+// the time steps dealt out over blockIdx.y: one element per thread at least,
+// about `want` blocks at most (no 64-bit division per element).
+static dim3 column_grid(int64_t n, int64_t ell, int64_t want) {
+  const int64_t gx = (n + kThreads - 1) / kThreads;
+  int64_t gy = want / gx;
+  gy = gy < 1 ? 1 : (gy > ell ? ell : gy);
+  return dim3((unsigned)gx, (unsigned)gy);
+}
+
 cudaError_t launch_neumann_rhs(const Ctx &c, const double *x, const double *y, double *u,
                                cudaStream_t s) {
-  int64_t blocks = (c.N + kThreads - 1) / kThreads;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  k_neumann_rhs<<<(unsigned)blocks, kThreads, 0, s>>>(x, y, c.sigk, u, (int)c.n, c.N);
+  k_neumann_rhs<<<column_grid(c.n, c.ell, 152 * 16), kThreads, 0, s>>>(x, y, c.sigk, u, (int)c.n,
+                                                                       (int)c.ell);
   note_launch();
   return cudaGetLastError();
 }
@@ -1025,11 +1042,9 @@ cudaError_t launch_matvec(const Ctx &c, const float *x, double *y, int transpose
 __global__ void k_rhs(const double *__restrict__ u0, const double *__restrict__ v0,
                       double *__restrict__ b, int n, int ell, int wave, double tau,
                       double mh, double kh) {
-  const int64_t N = (int64_t)n * ell;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(g / n);
-    const int i = (int)(g - (int64_t)t * n);
+  const int i = blockIdx.x * kThreads + threadIdx.x;
+  if (i >= n) return;
+  for (int t = blockIdx.y; t < ell; t += gridDim.y) {
     double out = 0.0;
     if (t <= 2) {
       auto at = [&](const double *v, int j) { return (j >= 0 && j < n) ? v[j] : 0.0; };
@@ -1048,15 +1063,13 @@ __global__ void k_rhs(const double *__restrict__ u0, const double *__restrict__ 
         out = t == 1 ? -m : m;
       }
     }
-    b[g] = out;
+    b[(int64_t)t * n + i] = out;
   }
 }
 
 cudaError_t launch_rhs(const Ctx &c, const double *u0, const double *v0, double *b,
                        cudaStream_t s) {
-  int64_t blocks = (c.N + kThreads - 1) / kThreads;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  k_rhs<<<(unsigned)blocks, kThreads, 0, s>>>(u0, v0, b, (int)c.n, (int)c.ell,
+  k_rhs<<<column_grid(c.n, c.ell, 152 * 16), kThreads, 0, s>>>(u0, v0, b, (int)c.n, (int)c.ell,
                                               c.equation == AAO_WAVE_BD2   ? 2
                                               : c.equation == AAO_WAVE_BD4 ? 3
                                                                            : 0,
@@ -1104,22 +1117,21 @@ k_norms2(const double *__restrict__ a, const double *__restrict__ b, int64_t N,
 }
 
 cudaError_t launch_norms2(const double *a, const double *b, int64_t N, double *partials,
-                          double *out, cudaStream_t s) {
+                          const RedOut &out, cudaStream_t s) {
   const int nb = red_blocks(N);
   k_norms2<<<nb, kThreads, 0, s>>>(a, b, N, partials); note_launch();
-  k_finish<<<2, 32, 0, s>>>(partials, nb, 2, out); note_launch();
-  return cudaGetLastError();
+  return finish(partials, nb, 2, out, s);
 }
 
 cudaError_t launch_multidot(const double *const *V, int nv, const double *w, int64_t N,
-                            bool with_norm, double *partials, double *out, cudaStream_t s) {
+                            bool with_norm, double *partials, const RedOut &out,
+                            cudaStream_t s) {
   const int nb = red_blocks(N);
   int done = 0;
   if (nv == 0 && with_norm) {
     Ptrs8 P{};
     run_multidot<0, true>(P, w, N, nb, partials, s);
-    k_finish<<<1, 32, 0, s>>>(partials, nb, 1, out); note_launch();
-    return cudaGetLastError();
+    return finish(partials, nb, 1, out, s);
   }
   while (done < nv) {
     const int g = (nv - done) > 8 ? 8 : (nv - done);
@@ -1136,106 +1148,135 @@ cudaError_t launch_multidot(const double *const *V, int nv, const double *w, int
     }
 #undef AAO_MD
     const int no = g + (norm ? 1 : 0);
-    k_finish<<<no, 32, 0, s>>>(partials, nb, no, out + done); note_launch();
+    const cudaError_t e = finish(partials, nb, no, out.at(done), s);
+    if (e != cudaSuccess) return e;
     done += g;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // --------------------------------------------- update (+ dots + norm) pass
-// w -= sum_j h_j V_j; then, if DOTS, acc_j += V_j . w_new, and always
-// acc_nv += w_new . w_new.
-template <int NV, bool DOTS>
+// w -= sum_j h_j V_j, its squared norm and, where they will be needed, the
+// dots V_j . w of the result: a second Gram-Schmidt pass follows where the
+// norm falls below half its value (the DGKS criterion), and for a nearly
+// orthonormal basis that fall is known from the first pass's dots, ||w||^2 -
+// sum_j h_j d_j.  AHEAD: the kernel forms that prediction from the device's own
+// numbers (before = ||w||^2 at *before; 0.55 leaves room for rounding) and adds
+// the dots only then, one FP64 operation per vector instead of another pass
+// over w and V (52 us at n 4095 x ell 4096).  out: the NV dots (zero if not
+// formed), the norm, 1 or 0 for formed or not; without AHEAD the norm alone.
+// A warp of a single vector whose 32 values are all zero (the right-hand side
+// of an all-at-once system past its first block rows) leaves w as it is.
+template <int NV, bool AHEAD>
 __global__ void __launch_bounds__(kThreads)
 k_update(Ptrs8 V, const double *__restrict__ h, Coef8 f, double *__restrict__ w, int64_t N,
-         double *__restrict__ partials, const double *__restrict__ div0) {
-  constexpr int NO = (DOTS ? NV : 0) + 1;
+         double *__restrict__ partials, const double *__restrict__ div0,
+         const double *__restrict__ before, RedOut flag) {
+  constexpr int NO = AHEAD ? NV + 1 : 1;
   double hv[NV];
 #pragma unroll
   for (int j = 0; j < NV; j++) hv[j] = h[j] * f.c[j];
   if (div0) hv[0] /= *div0;   // the first vector's squared norm, known only on the device
+  bool dots = false;
+  if (AHEAD) {
+    const double b = *before;
+    double left = b;
+#pragma unroll
+    for (int j = 0; j < NV; j++) left = fma(-hv[j], h[j], left);
+    dots = left < 0.55 * b;
+  }
   double acc[NO];
 #pragma unroll
   for (int j = 0; j < NO; j++) acc[j] = 0.0;
-  for (int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * kThreads) {
-    double v[NV];
-    double wv = w[g];
+  // U elements a thread at a time, all their loads first
+  constexpr int U = NV <= 2 ? 4 : (NV <= 4 ? 2 : 1);
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  auto pass = [&](auto dots_c) {
+    constexpr bool DOTS = decltype(dots_c)::value;
+    for (int64_t g0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; g0 < N; g0 += U * stride) {
+      double wv[U], v[U][NV];
 #pragma unroll
-    for (int j = 0; j < NV; j++) {
-      v[j] = __ldg(&V.p[j][g]);
-      wv = fma(-hv[j], v[j], wv);
-    }
-    w[g] = wv;
-    if (DOTS) {
+      for (int u = 0; u < U; u++) {
+        const int64_t g = g0 + u * stride;
+        wv[u] = g < N ? w[g] : 0.0;
 #pragma unroll
-      for (int j = 0; j < NV; j++) acc[j] = fma(v[j], wv, acc[j]);
+        for (int j = 0; j < NV; j++) v[u][j] = g < N ? __ldg(&V.p[j][g]) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const int64_t g = g0 + u * stride;
+        bool some = true;
+        if (NV == 1) {
+          const unsigned z = ((unsigned)__double2hiint(v[u][0]) << 1) | (unsigned)__double2loint(v[u][0]);
+          const unsigned e = (unsigned)__double2hiint(wv[u]) & 0x7ff00000u;   // inf, NaN: 0 x is a NaN
+          some = __any_sync(__activemask(), z != 0u || e == 0x7ff00000u);
+        }
+        if (some) {
+#pragma unroll
+          for (int j = 0; j < NV; j++) wv[u] = fma(-hv[j], v[u][j], wv[u]);
+          if (g < N) w[g] = wv[u];
+          if constexpr (DOTS) {
+#pragma unroll
+            for (int j = 0; j < NV; j++) acc[j] = fma(v[u][j], wv[u], acc[j]);
+          }
+        }
+        acc[NO - 1] = fma(wv[u], wv[u], acc[NO - 1]);
+      }
     }
-    acc[NO - 1] = fma(wv, wv, acc[NO - 1]);
+  };
+  if constexpr (AHEAD) {
+    if (dots) pass(std::true_type{});
+    else pass(std::false_type{});
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      flag.dev[0] = dots ? 1.0 : 0.0;
+      if (flag.host) flag.host[0] = dots ? 1.0 : 0.0;
+    }
+  } else {
+    pass(std::false_type{});
   }
   block_store<NO>(acc, partials);
 }
 
-cudaError_t launch_update_dots(const double *const *V, int nv, const double *h, double *w,
-                               int64_t N, bool want_dots, double *partials, double *out2,
-                               cudaStream_t s, const double *hf, const double *div0) {
-  // Groups of 8 vectors: every group but the last only updates; the dots of
-  // the final w with all vectors are then taken by a multi-dot pass when
-  // nv > 8 (the fused path covers nv <= 8, the common case).
+cudaError_t launch_update(const double *const *V, int nv, const double *h, double *w, int64_t N,
+                          double *partials, const RedOut &out, cudaStream_t s, const double *hf,
+                          const double *div0, const double *before) {
+  // groups of 8 vectors; the dots ahead are formed for at most 8
   const int nb = red_blocks(N);
-  auto coef = [&](int first, int g) {
-    Coef8 f{};
-    for (int j = 0; j < g; j++) f.c[j] = hf ? hf[first + j] : 1.0;
-    return f;
-  };
-  if (nv <= 8) {
-    Ptrs8 P{};
-    for (int j = 0; j < nv; j++) P.p[j] = V[j];
-    const Coef8 F = coef(0, nv);
-#define AAO_UP(G)                                                                          \
-  case G:                                                                                  \
-    if (want_dots) k_update<G, true><<<nb, kThreads, 0, s>>>(P, h, F, w, N, partials, div0); \
-    else k_update<G, false><<<nb, kThreads, 0, s>>>(P, h, F, w, N, partials, div0);        \
-    note_launch();                                                                         \
-    break;
-    switch (nv) {
-      AAO_UP(1) AAO_UP(2) AAO_UP(3) AAO_UP(4) AAO_UP(5) AAO_UP(6) AAO_UP(7) AAO_UP(8)
-      default: return cudaErrorInvalidValue;
-    }
-    const int no = (want_dots ? nv : 0) + 1;
-    if (want_dots) {
-      k_finish<<<no, 32, 0, s>>>(partials, nb, no, out2); note_launch();
-    } else {
-      k_finish<<<1, 32, 0, s>>>(partials, nb, 1, out2 + nv); note_launch();
-    }
-    return cudaGetLastError();
-  }
-  int done = 0;
-  while (done < nv) {
+  if (before && nv > 8) return cudaErrorInvalidValue;
+  for (int done = 0; done < nv;) {
     const int g = (nv - done) > 8 ? 8 : (nv - done);
     Ptrs8 P{};
-    for (int j = 0; j < g; j++) P.p[j] = V[done + j];
-    const Coef8 F = coef(done, g);
+    Coef8 F{};
+    for (int j = 0; j < g; j++) {
+      P.p[j] = V[done + j];
+      F.c[j] = hf ? hf[done + j] : 1.0;
+    }
+    const double *d0 = done == 0 ? div0 : nullptr;
     switch (g) {
-#define AAO_UP2(G) case G: k_update<G, false><<<nb, kThreads, 0, s>>>(P, h + done, F, w, N, partials, done == 0 ? div0 : nullptr); note_launch(); break;
-      AAO_UP2(1) AAO_UP2(2) AAO_UP2(3) AAO_UP2(4) AAO_UP2(5) AAO_UP2(6) AAO_UP2(7) AAO_UP2(8)
-#undef AAO_UP2
+#define AAO_UP(G)                                                                                \
+  case G:                                                                                        \
+    if (before) k_update<G, true><<<nb, kThreads, 0, s>>>(P, h + done, F, w, N, partials, d0, before, out.at(nv + 1)); \
+    else k_update<G, false><<<nb, kThreads, 0, s>>>(P, h + done, F, w, N, partials, d0, nullptr, out);               \
+    note_launch();                                                                               \
+    break;
+      AAO_UP(1) AAO_UP(2) AAO_UP(3) AAO_UP(4) AAO_UP(5) AAO_UP(6) AAO_UP(7) AAO_UP(8)
+#undef AAO_UP
     }
     done += g;
   }
-  if (want_dots) return launch_multidot(V, nv, w, N, true, partials, out2, s);
-  k_finish<<<1, 32, 0, s>>>(partials, nb, 1, out2 + nv); note_launch();
-  return cudaGetLastError();
+  return finish(partials, nb, before ? nv + 1 : 1, out, s);
 }
 
 // ------------------------------------------------------------ x += Z y
 template <int NV, typename ZT>
 __global__ void __launch_bounds__(kThreads)
-k_combine(PtrsT<ZT> Z, const double *__restrict__ yv, double *__restrict__ x, int64_t N,
-          int assign) {
+k_combine(PtrsT<ZT> Z, Coef8 yv, double *__restrict__ x, int64_t N, int assign) {
   double c[NV];
 #pragma unroll
-  for (int j = 0; j < NV; j++) c[j] = yv[j];
+  for (int j = 0; j < NV; j++) {
+    c[j] = yv.c[j];
+    asm volatile("" : "+d"(c[j]));   // in a register: 63 against 73 us from the constant bank
+  }
   for (int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x; g < N;
        g += (int64_t)gridDim.x * kThreads) {
     double a = assign ? 0.0 : x[g];   // assign: x = Z y (x not read)
@@ -1254,9 +1295,13 @@ static cudaError_t combine_any(const ZT *const *Z, int nv, const double *y, doub
   while (done < nv) {
     const int g = (nv - done) > 8 ? 8 : (nv - done);
     PtrsT<ZT> P{};
-    for (int j = 0; j < g; j++) P.p[j] = Z[done + j];
+    Coef8 Y{};
+    for (int j = 0; j < g; j++) {
+      P.p[j] = Z[done + j];
+      Y.c[j] = y[done + j];
+    }
     switch (g) {
-#define AAO_CB(G) case G: k_combine<G, ZT><<<(unsigned)blocks, kThreads, 0, s>>>(P, y + done, x, N, (assign && done == 0) ? 1 : 0); note_launch(); break;
+#define AAO_CB(G) case G: k_combine<G, ZT><<<(unsigned)blocks, kThreads, 0, s>>>(P, Y, x, N, (assign && done == 0) ? 1 : 0); note_launch(); break;
       AAO_CB(1) AAO_CB(2) AAO_CB(3) AAO_CB(4) AAO_CB(5) AAO_CB(6) AAO_CB(7) AAO_CB(8)
 #undef AAO_CB
     }
@@ -1297,19 +1342,6 @@ cudaError_t launch_scale(const double *x, double *y, const double *a, int64_t N,
   return cudaGetLastError();
 }
 
-__global__ void k_sub_from(const double *__restrict__ b, double *__restrict__ r, int64_t N) {
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * blockDim.x)
-    r[g] = b[g] - r[g];
-}
-
-cudaError_t launch_sub_from(const double *b, double *r, int64_t N, cudaStream_t s) {
-  int64_t blocks = (N + kThreads - 1) / kThreads;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  k_sub_from<<<(unsigned)blocks, kThreads, 0, s>>>(b, r, N); note_launch();
-  return cudaGetLastError();
-}
-
 // ------------------------------------------------------- adjoint gradients
 // g_u0 = M lam_1; sum_t tau_t lam_t^T K u_t (reduced; the caller negates).
 __global__ void k_grad_u0(const double *__restrict__ lam, double *__restrict__ g, int n,
@@ -1320,34 +1352,47 @@ __global__ void k_grad_u0(const double *__restrict__ lam, double *__restrict__ g
   }
 }
 
+// sum_t tau_t lam_t^T K u_t (times kappa, from tauk = tau_t kappa / h) by its
+// edges: lam^T (h K) u = sum_i (lam_{i+1} - lam_i)(u_{i+1} - u_i), i = 0 .. n
+// with zero ends, two subtractions and an FMA per element where the stencil
+// form took five FP64 operations (that pipe bounds the kernel: 167 us at n
+// 16383 x ell 1024), and no cancellation of second differences.  A row's sum
+// is scaled by tauk once per thread and row with variable steps, once per
+// thread with uniform ones.
+template <bool UNIFORM>
 __global__ void __launch_bounds__(kThreads)
 k_grad_kappa(const double *__restrict__ lam, const double *__restrict__ U, int n, int ell,
              const double *__restrict__ tauk, double *__restrict__ partials) {
-  const int64_t N = (int64_t)n * ell;
   double acc[1] = {0.0};
-  for (int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * kThreads) {
-    const int t = (int)(g / n);
-    const int i = (int)(g - (int64_t)t * n);
-    const double uc = U[g];
-    const double ul = (i > 0) ? U[g - 1] : 0.0;
-    const double ur = (i + 1 < n) ? U[g + 1] : 0.0;
-    const double ku = (uc - ul) - (ur - uc);
-    acc[0] = fma(__ldg(&tauk[t]) * lam[g], ku, acc[0]);
+  const int i = blockIdx.x * kThreads + threadIdx.x;   // edge between columns i - 1 and i
+  if (i <= n) {
+    const bool l = i > 0, r = i < n;
+#pragma unroll 4
+    for (int t = blockIdx.y; t < ell; t += gridDim.y) {
+      const int64_t g = (int64_t)t * n + i;
+      const double du = (r ? __ldg(&U[g]) : 0.0) - (l ? __ldg(&U[g - 1]) : 0.0);
+      const double dl = (r ? __ldg(&lam[g]) : 0.0) - (l ? __ldg(&lam[g - 1]) : 0.0);
+      acc[0] = fma(UNIFORM ? dl : __ldg(&tauk[t]) * dl, du, acc[0]);
+    }
+    if (UNIFORM) acc[0] *= __ldg(&tauk[0]);
   }
   block_store<1>(acc, partials);
 }
 
 cudaError_t launch_adjoint_grads(const Ctx &c, const double *lam, const double *U,
-                                 double *g_u0, double *partials, double *out, cudaStream_t s) {
+                                 double *g_u0, double *partials, const RedOut &out,
+                                 cudaStream_t s) {
   const int n = (int)c.n;
   k_grad_u0<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(lam, g_u0, n, c.h / 6.0); note_launch();
-  const int nb = red_blocks(c.N);
   // beta_t = tau_t kappa / h, so tau_t lam^T K u = (beta_t / kappa) lam^T (h K) u / h ... use
   // tau_t / h directly: the matvec's beta divided by kappa.
-  k_grad_kappa<<<nb, kThreads, 0, s>>>(lam, U, n, (int)c.ell, c.beta, partials); note_launch();
-  k_finish<<<1, 32, 0, s>>>(partials, nb, 1, out); note_launch();
-  return cudaGetLastError();
+  const dim3 grid = column_grid(c.n + 1, c.ell, kMaxRedBlocks);
+  if (c.variable_steps)
+    k_grad_kappa<false><<<grid, kThreads, 0, s>>>(lam, U, n, (int)c.ell, c.beta, partials);
+  else
+    k_grad_kappa<true><<<grid, kThreads, 0, s>>>(lam, U, n, (int)c.ell, c.beta, partials);
+  note_launch();
+  return finish(partials, (int)(grid.x * grid.y), 1, out, s);
 }
 
 // The library's integer-built conversions next to CUDA's own, element by

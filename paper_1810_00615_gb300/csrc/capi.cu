@@ -819,8 +819,9 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
   double *red = reinterpret_cast<double *>(c.ws + L.red);
   double *dpart = reinterpret_cast<double *>(c.ws + L.dots);
   double *small = red + kPartials;
-  double *d_h1 = small, *d_h2 = small + 160, *d_nr = small + 320, *d_y = small + 480;
+  double *d_h1 = small, *d_h2 = small + 160, *d_nr = small + 320;
   double *hs = c.host_small;   // pinned mirror of the same offsets
+  auto to = [&](double *dev) { return aao::RedOut{dev, hs + (dev - small)}; };
   std::vector<double *> V((size_t)m + 1), Z((size_t)m);
   for (int j = 0; j <= m; j++) V[(size_t)j] = vec_at(c, L, j);
   for (int j = 0; j < m; j++) Z[(size_t)j] = precond ? vec_at(c, L, m + 1 + j) : V[(size_t)j];
@@ -834,17 +835,11 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
     if (overlap(v, b, vb) || overlap(v, x, vb)) return AAO_EINVAL;
 
   if (info) { info->iters = 0; info->restarts = 0; info->history_len = 0; }
-  auto fetch = [&](double *dev, int count) -> cudaError_t {
-    return cudaMemcpyAsync(hs + (dev - small), dev, count * sizeof(double),
-                           cudaMemcpyDeviceToHost, s);
-  };
   auto norm2 = [&](const double *v) -> cudaError_t {
     cudaError_t e = run(c, AAO_K_DOTS, s, [&] {
-      return aao::launch_multidot(nullptr, 0, v, N, true, red, d_nr, s);
+      return aao::launch_multidot(nullptr, 0, v, N, true, red, to(d_nr), s);
     });
-    if (e != cudaSuccess) return e;
-    if ((e = fetch(d_nr, 1)) != cudaSuccess) return e;
-    return cudaStreamSynchronize(s);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(s);
   };
   // ||b||^2 and ||x0||^2 in one pass: a zero initial guess makes the first
   // residual -b, so the first cycle needs no matvec (V_0 aliases b, the sign
@@ -859,12 +854,10 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
   if (!defer_b) {
     if (guess_zero) {
       AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
-        return aao::launch_multidot(nullptr, 0, b, N, true, red, d_nr, s);
+        return aao::launch_multidot(nullptr, 0, b, N, true, red, to(d_nr), s);
       }));
-      AAO_CK(c, fetch(d_nr, 1));
     } else {
-      AAO_CK(c, run(c, AAO_K_DOTS, s, [&] { return aao::launch_norms2(b, x, N, red, d_nr, s); }));
-      AAO_CK(c, fetch(d_nr, 2));
+      AAO_CK(c, run(c, AAO_K_DOTS, s, [&] { return aao::launch_norms2(b, x, N, red, to(d_nr), s); }));
     }
     AAO_CK(c, cudaStreamSynchronize(s));
     bnorm = std::sqrt(hs[320]);
@@ -910,10 +903,9 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       V[0] = v0_slot;
       if (c.equation != AAO_HEAT_LITERAL) {
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-          return aao::launch_matvec_dots(c, x, V[0], tr, s, b, nullptr, dpart, d_nr,
+          return aao::launch_matvec_dots(c, x, V[0], tr, s, b, nullptr, dpart, to(d_nr),
                                          aao::MvDots::NORM);
         }));
-        AAO_CK(c, fetch(d_nr, 1));
         AAO_CK(c, cudaStreamSynchronize(s));
       } else {
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] { return aao::launch_matvec(c, x, V[0], tr, s, b); }));
@@ -964,8 +956,8 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
         // also b . b at step 0 of the first cycle
         const auto self = defer_b ? aao::MvDots::SELF : aao::MvDots::ARNOLDI;
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-          return zf ? aao::launch_matvec_dots(c, Zf[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, d_h1, self)
-                    : aao::launch_matvec_dots(c, Z[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, d_h1, self);
+          return zf ? aao::launch_matvec_dots(c, Zf[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, to(d_h1), self)
+                    : aao::launch_matvec_dots(c, Z[(size_t)j], w, tr, s, V[(size_t)j], v0, dpart, to(d_h1), self);
         }));
       } else {
         AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
@@ -973,7 +965,7 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
                     : aao::launch_matvec(c, Z[(size_t)j], w, tr, s, V[(size_t)j]);
         }));
         AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
-          return aao::launch_multidot(V.data(), nv, w, N, true, red, d_h1, s);
+          return aao::launch_multidot(V.data(), nv, w, N, true, red, to(d_h1), s);
         }));
       }
       for (int i = 0; i < nv; i++) sc2[(size_t)i] = sc[(size_t)i] * sc[(size_t)i];
@@ -1007,10 +999,9 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       // (h_{j+1,j} << h_{j,j}).
       const bool decide_first =
           j >= 1 && e_prev2 > 0.0 && e_prev * e_prev <= 1e4 * rtol * e_prev2;
-      bool skipped = false;
+      bool skipped = false, dots2 = false;   // dots2: d_nr holds V^T of the updated w~
       double before = 0.0, after = 0.0;   // ||w~||^2 before / after the projection (unscaled)
       if (decide_first) {
-        AAO_CK(c, fetch(d_h1, nv + 1));
         AAO_CK(c, cudaStreamSynchronize(s));
         before = hs[nv];
         double proj = 0.0;
@@ -1026,13 +1017,16 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       if (!skipped) {
         // deferred ||b||: the projection on V_0 = b divides by b . b on the
         // device (d_h1[2]), so the update needs no round trip to the host
+        // (up to 8 vectors: the dots of a second pass come with it where the
+        // device predicts one)
+        const bool ahead = nv <= 8;
         AAO_CK(c, run(c, AAO_K_UPDATE, s, [&] {
-          return aao::launch_update_dots(V.data(), nv, d_h1, w, N, false, red, d_nr, s,
-                                         sc2.data(), defer_b ? d_h1 + 2 : nullptr);
+          return aao::launch_update(V.data(), nv, d_h1, w, N, red, to(ahead ? d_nr : d_nr + nv),
+                                    s, sc2.data(), defer_b ? d_h1 + 2 : nullptr,
+                                    ahead ? d_h1 + nv : nullptr);
         }));
-        AAO_CK(c, fetch(d_h1, defer_b ? 3 : nv + 1));
-        AAO_CK(c, fetch(d_nr + nv, 1));
         AAO_CK(c, cudaStreamSynchronize(s));
+        dots2 = ahead && hs[320 + nv + 1] != 0.0;
         if (defer_b) {
           bnorm = std::sqrt(hs[2]);
           if (!std::isfinite(bnorm)) return AAO_ENUMERIC;
@@ -1054,16 +1048,17 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
           skipped || trial_est(after) <= rtol || iters + 1 >= maxit || j + 1 == m;
       if (after < 0.5 * before && !last_step) {
         // DGKS: lost more than half the norm, orthogonalise once more
-        AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
-          return aao::launch_multidot(V.data(), nv, w, N, false, red, d_h2, s);
-        }));
+        double *d2 = dots2 ? d_nr : d_h2;
+        if (!dots2)
+          AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
+            return aao::launch_multidot(V.data(), nv, w, N, false, red, to(d_h2), s);
+          }));
         AAO_CK(c, run(c, AAO_K_UPDATE, s, [&] {
-          return aao::launch_update_dots(V.data(), nv, d_h2, w, N, false, red, d_nr, s, sc2.data());
+          return aao::launch_update(V.data(), nv, d2, w, N, red, to(d_nr + nv), s, sc2.data());
         }));
-        AAO_CK(c, fetch(d_h2, nv));
-        AAO_CK(c, fetch(d_nr + nv, 1));
         AAO_CK(c, cudaStreamSynchronize(s));
-        for (int i = 0; i < nv; i++) Hij(i, j) += sc[(size_t)i] * sc[(size_t)j] * hs[160 + i];
+        for (int i = 0; i < nv; i++)
+          Hij(i, j) += sc[(size_t)i] * sc[(size_t)j] * hs[(d2 - small) + i];
         after = hs[320 + nv];
       }
       Hij(j, j) += 1.0;                      // undo the shift: A P^{-1} = (A P^{-1} - I) + I
@@ -1120,8 +1115,7 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       for (int l = i + 1; l < jd; l++) acc -= Hij(i, l) * y[(size_t)l];
       y[(size_t)i] = acc / Hij(i, i);
     }
-    for (int i = 0; i < jd; i++) hs[480 + i] = y[(size_t)i] * sc[(size_t)i];   // z_i = sc_i Z_i
-    AAO_CK(c, cudaMemcpyAsync(d_y, hs + 480, jd * sizeof(double), cudaMemcpyHostToDevice, s));
+    for (int i = 0; i < jd; i++) y[(size_t)i] *= sc[(size_t)i];   // z_i = sc_i Z_i
     if (copy_pending) AAO_CK(c, cudaStreamWaitEvent(s, c.ev_copy, 0));   // x is read by it
     if (x_host && jd > 0) {
       // x = Z y in kCopyPieces pieces, each sent to the host as soon as it
@@ -1137,8 +1131,8 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
           else Zp[(size_t)i] = Z[(size_t)i] + off;
         }
         AAO_CK(c, run(c, AAO_K_COMBINE, s, [&] {
-          return zf ? aao::launch_combine(Zfp.data(), jd, d_y, x + off, cnt, s, x_unset)
-                    : aao::launch_combine(Zp.data(), jd, d_y, x + off, cnt, s, x_unset);
+          return zf ? aao::launch_combine(Zfp.data(), jd, y.data(), x + off, cnt, s, x_unset)
+                    : aao::launch_combine(Zp.data(), jd, y.data(), x + off, cnt, s, x_unset);
         }));
         AAO_CK(c, cudaEventRecord(c.ev_x, s));
         AAO_CK(c, cudaStreamWaitEvent(c.copy_stream, c.ev_x, 0));
@@ -1149,8 +1143,8 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
       copy_pending = host_current = true;
     } else {
       AAO_CK(c, run(c, AAO_K_COMBINE, s, [&] {
-        return zf ? aao::launch_combine(Zf.data(), jd, d_y, x, N, s, x_unset)
-                  : aao::launch_combine(Z.data(), jd, d_y, x, N, s, x_unset);
+        return zf ? aao::launch_combine(Zf.data(), jd, y.data(), x, N, s, x_unset)
+                  : aao::launch_combine(Z.data(), jd, y.data(), x, N, s, x_unset);
       }));
     }
     if (jd > 0) x_unset = false;
@@ -1436,10 +1430,9 @@ int aao_matvec_dots(aao_ctx *ctx, const double *x, const double *v, const double
   cudaStream_t s = as_stream(stream);
   const int nd = v0 ? 3 : 2;
   AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-    return aao::launch_matvec_dots(c, x, w, transpose ? 1 : 0, s, v, v0, dpart, out);
+    return aao::launch_matvec_dots(c, x, w, transpose ? 1 : 0, s, v, v0, dpart,
+                                   aao::RedOut{out, c.host_small + 972});
   }));
-  AAO_CK(c, cudaMemcpyAsync(c.host_small + 972, out, nd * sizeof(double), cudaMemcpyDeviceToHost,
-                            s));
   AAO_CK(c, cudaStreamSynchronize(s));
   for (int q = 0; q < nd; q++) dots[q] = c.host_small[972 + q];
   return AAO_OK;
@@ -1458,18 +1451,16 @@ int aao_residual(aao_ctx *ctx, const double *x, const double *b, double *r, int 
   double *out = red + kPartials + 970;   // in the small-result area
   cudaStream_t s = as_stream(stream);
   const int tr = transpose ? 1 : 0;
+  const aao::RedOut to{out, c.host_small + 970};
   if (c.equation != AAO_HEAT_LITERAL) {
     AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] {
-      return aao::launch_matvec_dots(c, x, r, tr, s, b, nullptr, dpart, out, aao::MvDots::NORM);
+      return aao::launch_matvec_dots(c, x, r, tr, s, b, nullptr, dpart, to, aao::MvDots::NORM);
     }));
-    AAO_CK(c, cudaMemcpyAsync(c.host_small + 970, out, sizeof(double), cudaMemcpyDeviceToHost, s));
   } else {
     AAO_CK(c, run(c, AAO_K_MATVEC, s, [&] { return aao::launch_matvec(c, x, r, tr, s, b); }));
     AAO_CK(c, run(c, AAO_K_DOTS, s, [&] {
-      return aao::launch_multidot(nullptr, 0, r, c.N, true, red, out, s);
+      return aao::launch_multidot(nullptr, 0, r, c.N, true, red, to, s);
     }));
-    AAO_CK(c, cudaMemcpyAsync(c.host_small + 970, out, sizeof(double), cudaMemcpyDeviceToHost,
-                              s));
   }
   AAO_CK(c, cudaStreamSynchronize(s));
   *norm2 = c.host_small[970];
@@ -1521,8 +1512,10 @@ int aao_adjoint_grads(aao_ctx *ctx, const double *lambda, const double *U, doubl
   double *red = reinterpret_cast<double *>(c.ws + L.red);
   double *out = red + kPartials + 960;
   cudaStream_t s = as_stream(stream);
-  AAO_CK(c, run(c, AAO_K_OTHER, s, [&] { return aao::launch_adjoint_grads(c, lambda, U, g_u0, red, out, s); }));
-  AAO_CK(c, cudaMemcpyAsync(c.host_small + 960, out, sizeof(double), cudaMemcpyDeviceToHost, s));
+  AAO_CK(c, run(c, AAO_K_OTHER, s, [&] { 
+    return aao::launch_adjoint_grads(c, lambda, U, g_u0, red,
+                                     aao::RedOut{out, c.host_small + 960}, s);
+  }));
   AAO_CK(c, cudaStreamSynchronize(s));
   // the reduction used beta_t = tau_t kappa / h: it holds kappa sum_t tau_t lam_t^T K u_t
   *g_kappa = -c.host_small[960] / c.kappa;
