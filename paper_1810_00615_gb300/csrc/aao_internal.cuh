@@ -85,6 +85,27 @@ __device__ __forceinline__ double to_f64(float f) {
   return __hiloint2double((int)hi, (int)(u << 29));
 }
 
+// a - b of two FP32 numbers, rounded to FP64 as the FP64 subtraction rounds it,
+// on the FP32 and integer pipes (an FP64 operation per element is ~30 us of
+// its pipe at n 4095 x ell 4096).  TwoSum splits a - b = s + e exactly, |e| <=
+// half a unit of s; in units of s's last FP64 place e is below 2^28, so its
+// rounding to an integer, added to the bits of s, is the rounded sum as long
+// as it stays in s's binade.  Zeros, powers of two and s outside [2^-67,
+// 2^114) take the FP64 subtraction.
+__device__ __forceinline__ double diff_f64(float a, float b) {
+  const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
+  const float e = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+  const unsigned us = __float_as_uint(s), es = (us >> 23) & 0xffu;
+  if (es - 60u > 180u || (us & 0x7fffffu) == 0u) {
+    asm volatile("");   // a branch, not a predicated FP64 operation for every element
+    return (double)a - (double)b;
+  }
+  const int t = __float2int_rn(__fmul_rn(e, __uint_as_float((306u - es) << 23)));
+  const unsigned hi = (us & 0x80000000u) | (((us & 0x7fffffffu) >> 3) + (896u << 20));
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | (us << 29)) +
+                              ((int)us < 0 ? -t : t));
+}
+
 // ------------------------------------------------- programmatic dependent launch
 // The kernels of one preconditioner apply form a chain on one stream.  Each
 // is launched with programmatic stream serialisation: it may be scheduled

@@ -430,9 +430,9 @@ k_fft4_inverseB(const cx<float> *__restrict__ inter, OT *__restrict__ y, int n, 
     if (in) {
 #pragma unroll
       for (int u = 0; u < B; u++) {
-        const OT val = to_out<float, OT>(scale * Sf[(b0 + u) * kFourT + threadIdx.x]);
+        const float val = scale * Sf[(b0 + u) * kFourT + threadIdx.x];
         OT *dst = y + row0 + (b0 + u) * ustride;
-        if constexpr (sizeof(OT) == 8) *dst = base ? to_f64(bv[u]) - val : val;
+        if constexpr (sizeof(OT) == 8) *dst = base ? diff_f64(bv[u], val) : to_f64(val);
         else *dst = val;
       }
     }

@@ -349,8 +349,8 @@ k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int 
   }
 }
 
-// Inverse B.  grid and shared memory as forward 1.  With base (FP64 output
-// only) y = base - result.
+// Inverse B.  grid and shared memory as forward 1.  With base (FP64 output of
+// an FP32 transform only) y = base - result.
 template <typename R, typename OT>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int ncx,
@@ -386,7 +386,7 @@ k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int
   constexpr int B = 4;
   for (int q0 = 0; q0 < rows; q0 += B * kStepWarps) {
     float bv[B][2];
-    if constexpr (sizeof(OT) == 8) {
+    if constexpr (sizeof(OT) > sizeof(R)) {
       if (base) {
 #pragma unroll
         for (int u = 0; u < B; u++) {
@@ -408,9 +408,9 @@ k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int
       for (int h = 0; h < 2; h++) {
         const int i = i0 + h * 32 + lane;
         if (q < rows && i < n) {
-          const OT val = to_out<R, OT>(scale * Sf[q * 2 * kStepW + h * 32 + lane]);
-          if constexpr (sizeof(OT) == 8) y[row + i] = base ? to_f64(bv[u][h]) - val : val;
-          else y[row + i] = val;
+          const R val = scale * Sf[q * 2 * kStepW + h * 32 + lane];
+          if constexpr (sizeof(OT) == sizeof(R)) y[row + i] = val;
+          else y[row + i] = base ? diff_f64(bv[u][h], val) : to_f64(val);
         }
       }
     }
