@@ -39,9 +39,17 @@ def build(force: bool = False) -> str:
     return _build.build(force=force)
 
 
+# The current stream's handle without building a torch.cuda.Stream around it
+# (half the binding's own time in a small call).
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is None:
+        if _current_raw_stream is not None:
+            return _current_raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
+    return int(stream.cuda_stream)
 
 
 def _dev_f64(t: torch.Tensor, numel: int, name: str, dtype=torch.float64) -> torch.Tensor:

@@ -539,6 +539,19 @@ cudaError_t kernel_setup(const void *kern, int threads, size_t smem, int *reside
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
+  // this thread's last answer per slot: a launch path asks for the same few
+  // kernels over and over, and the shared maps cost it a lock and two searches
+  struct Slot {
+    const void *kern = nullptr;
+    int dev = -1, threads = 0, resident = 0;
+    size_t smem = 0;
+  };
+  static thread_local Slot slots[64];
+  Slot &slot = slots[(reinterpret_cast<uintptr_t>(kern) >> 4) % 64];
+  if (slot.kern == kern && slot.dev == dev && slot.threads == threads && slot.smem == smem) {
+    if (resident) *resident = slot.resident;
+    return cudaSuccess;
+  }
   static std::mutex mu;
   // the opt-in is one value per function and device: keep the largest set
   static std::map<std::pair<const void *, int>, size_t> optin;
@@ -573,6 +586,11 @@ cudaError_t kernel_setup(const void *kern, int threads, size_t smem, int *reside
     it = grid.emplace(key, sms * per).first;
   }
   if (resident) *resident = it->second;
+  slot.kern = kern;
+  slot.dev = dev;
+  slot.threads = threads;
+  slot.resident = it->second;
+  slot.smem = smem;
   return cudaSuccess;
 }
 
