@@ -823,122 +823,157 @@ k_circ_residual_df(const float *__restrict__ z, const double *__restrict__ x,
 // S = sum_j a_j q_{t-j} with the integer time weights (exact multiples by
 // 1, 2, 4; -5 q = -4 q - q), and r = mh S + bp k_t - x with two pair
 // products and two TwoSums.  Each row's stencil is formed once instead of
-// once per lag: 66 M against 77 M warp instructions per launch at n 4095 x
-// ell 4096 (the kernel is bound by instruction issue and load latency).
-// Rows of the residual's walk in flight: the next row is requested right
-// after the current one's stencil sums are formed.  Measured at n 4095 x
-// ell 4096: one row 373 us per refined apply, two or four 376 us.
-#ifndef AAO_RES_PRE
-#define AAO_RES_PRE 1
-#endif
-constexpr int kResPre = AAO_RES_PRE;
+// once per lag.  The kernel was bound by instruction issue (77%), so a thread
+// takes two columns kMvCols apart and forms both at once in packed FP32 pairs:
+// one f32x2 instruction for two additions or FMAs, with the roundings of one at
+// a time, so the same bits.  Per launch at n 4095 x ell 4096: 71 us with one
+// column a thread, 59 with two (268 MB: 4.6 TB/s, 40 us at the copy rate; the
+// load latency is what is left); n 16383 x ell 1024 transposed 74 -> 59, n 1568
+// x ell 1440 18 -> 11.  A walk has 8 steps: 16 or 32 leave the last wave emptier
+// than their fewer halo rows save (59.6 and 67.5 us, n 1568 x ell 1440 13), 12
+// differ by under 1%.
+constexpr int kResRows = 8;
 template <int NB> __device__ __forceinline__ constexpr int qweight(int j) {
   return NB == 2 ? (j == 0 ? 1 : -1)
                  : (NB == 3 ? (j == 1 ? -2 : 1) : (j == 0 ? 2 : (j == 1 ? -5 : (j == 2 ? 4 : -1))));
 }
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+
+// Two FP32 numbers in one 64-bit register pair.
+typedef unsigned long long f2x;
+__device__ __forceinline__ f2x pack2(float a, float b) {
+  f2x r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f2x v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2x dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ f2x add2(f2x a, f2x b) {
+  f2x r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2x sub2(f2x a, f2x b) {
+  f2x r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2x fma2(f2x a, f2x b, f2x c) {
+  f2x r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// The product as an FMA onto zero.  A packed multiplication followed by an
+// addition is contracted into one FMA in spite of its .rn, which leaves the
+// product unrounded where its rounding error is formed separately (a refined
+// apply was 6e-8 off).
+__device__ __forceinline__ f2x mul2(f2x a, f2x b) { return fma2(a, b, dup2(0.f)); }
+__device__ __forceinline__ void two_sum2(f2x a, f2x b, f2x &s, f2x &e) {
+  s = add2(a, b);
+  const f2x bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
 template <int NB, bool TR, typename RT>
 __global__ void __launch_bounds__(kMvCols)
 k_circ_residual_q(const float *__restrict__ z, const double *__restrict__ x,
                   RT *__restrict__ r, int n, int ell, CircDF cf) {
-  const int i = blockIdx.x * kMvCols + threadIdx.x;
+  const int i = blockIdx.x * (2 * kMvCols) + threadIdx.x, i2 = i + kMvCols;
   if (i >= n) return;                  // no barriers in this kernel
-  const int c0 = blockIdx.y * kMvRows;
-  const int c1 = min(ell, c0 + kMvRows);
-  auto load = [&](int t, float (&v)[3]) {
+  const bool two = i2 < n;
+  const int c0 = blockIdx.y * kResRows;
+  const int c1 = min(ell, c0 + kResRows);
+  auto load = [&](int t, f2x (&v)[3]) {
     const float *zr = z + (int64_t)t * n;
-    v[0] = __ldg(&zr[i]);
-    v[1] = (i > 0) ? __ldg(&zr[i - 1]) : 0.f;
-    v[2] = (i + 1 < n) ? __ldg(&zr[i + 1]) : 0.f;
+    v[0] = pack2(__ldg(&zr[i]), two ? __ldg(&zr[i2]) : 0.f);
+    v[1] = pack2((i > 0) ? __ldg(&zr[i - 1]) : 0.f, two ? __ldg(&zr[i2 - 1]) : 0.f);
+    v[2] = pack2((i + 1 < n) ? __ldg(&zr[i + 1]) : 0.f, (i2 + 1 < n) ? __ldg(&zr[i2 + 1]) : 0.f);
   };
+  auto loadx = [&](int t, double (&v)[2]) {
+    const double *xr = x + (int64_t)t * n;
+    v[0] = __ldg(&xr[i]);
+    v[1] = two ? __ldg(&xr[i2]) : 0.0;
+  };
+  const f2x zero = dup2(0.f), mhh = dup2(cf.mh_hi), mhl = dup2(cf.mh_lo), bph = dup2(cf.bp_hi),
+            bpl = dup2(cf.bp_lo);
   // q (and k) of a row as pairs: zl + zr first, then + 4 z (- for k, with 2 z)
-  auto qk = [](const float (&v)[3], float &qh, float &ql, float &kh, float &kl) {
-    float ah, ae, e;
-    two_sum(v[1], v[2], ah, ae);
-    two_sum(ah, 4.f * v[0], qh, e);
-    ql = __fadd_rn(e, ae);
-    two_sum(2.f * v[0], -ah, kh, e);
-    kl = __fsub_rn(e, ae);
+  auto qk = [&](const f2x (&v)[3], f2x &qh, f2x &ql, f2x &kh, f2x &kl) {
+    f2x ah, ae, e;
+    two_sum2(v[1], v[2], ah, ae);
+    two_sum2(ah, mul2(dup2(4.f), v[0]), qh, e);
+    ql = add2(e, ae);
+    two_sum2(mul2(dup2(2.f), v[0]), sub2(zero, ah), kh, e);
+    kl = sub2(e, ae);
   };
-  float qh[NB], ql[NB];                // [j]: the row j behind in walk order
+  f2x qh[NB], ql[NB];                  // [j]: the row j behind in walk order
   const int first = TR ? c1 - 1 : c0, stp = TR ? -1 : 1, cnt = c1 - c0;
 #pragma unroll
   for (int j = 1; j < NB; j++) {
     int tj = first - j * stp;
     tj = ((tj % ell) + ell) % ell;     // time wrapped around: P
-    float v[3], kh, kl;
+    f2x v[3], kh, kl;
     load(tj, v);
     qk(v, qh[j], ql[j], kh, kl);
   }
-  // the values of the next kResPre rows are in flight while a row is
-  // computed: slot u of the ring holds row kb + u
-  constexpr int D = kResPre;
-  float zq[D][3];
-  double xq[D];
-#pragma unroll
-  for (int u = 0; u < D; u++) {
-    zq[u][0] = zq[u][1] = zq[u][2] = 0.f;
-    xq[u] = 0.0;
-    if (u < cnt) {
-      load(first + u * stp, zq[u]);
-      xq[u] = __ldg(&x[(int64_t)(first + u * stp) * n + i]);
+  // the next row is requested right after the current one's stencil sums
+  f2x zq[3];
+  double xq[2];
+  load(first, zq);
+  loadx(first, xq);
+  for (int k = 0; k < cnt; k++) {
+    const int t = first + k * stp;
+    f2x kh, kl;
+    qk(zq, qh[0], ql[0], kh, kl);
+    const double xc[2] = {xq[0], xq[1]};
+    if (k + 1 < cnt) {
+      load(t + stp, zq);
+      loadx(t + stp, xq);
     }
-  }
-  for (int kb = 0; kb < cnt; kb += D) {
+    // S = sum_j a_j q_{t-j} as a pair
+    f2x sh = qh[0], sl = ql[0], e;
+    if (qweight<NB>(0) != 1) {
+      sh = mul2(dup2((float)qweight<NB>(0)), qh[0]);
+      sl = mul2(dup2((float)qweight<NB>(0)), ql[0]);
+    }
 #pragma unroll
-    for (int u = 0; u < D; u++) {
-      const int k = kb + u;
-      if (k < cnt) {
-        const int t = first + k * stp;
-        float kh, kl;
-        qk(zq[u], qh[0], ql[0], kh, kl);
-        const double xc = xq[u];
-        if (k + D < cnt) {             // refill the slot with row k + D
-          load(t + D * stp, zq[u]);
-          xq[u] = __ldg(&x[(int64_t)(t + D * stp) * n + i]);
-        }
-        // S = sum_j a_j q_{t-j} as a pair
-        float sh = (float)qweight<NB>(0) * qh[0], sl = (float)qweight<NB>(0) * ql[0], e;
-#pragma unroll
-        for (int j = 1; j < NB; j++) {
-          const int w = qweight<NB>(j);
-          if (w == -5) {               // -5 q = -4 q - q, each exact
-            two_sum(sh, -4.f * qh[j], sh, e);
-            sl = __fadd_rn(sl, e);
-            two_sum(sh, -qh[j], sh, e);
-            sl = __fadd_rn(sl, __fsub_rn(e, 5.f * ql[j]));
-          } else {
-            two_sum(sh, (float)w * qh[j], sh, e);
-            sl = __fadd_rn(sl, __fadd_rn(e, (float)w * ql[j]));
-          }
-        }
-        // mh S and bp k as pairs (exact high products by FMA)
-        const float p1 = __fmul_rn(cf.mh_hi, sh);
-        float e1 = __fmaf_rn(cf.mh_hi, sh, -p1);
-        e1 = __fmaf_rn(cf.mh_hi, sl, e1);
-        e1 = __fmaf_rn(cf.mh_lo, sh, e1);
-        const float p2 = __fmul_rn(cf.bp_hi, kh);
-        float e2 = __fmaf_rn(cf.bp_hi, kh, -p2);
-        e2 = __fmaf_rn(cf.bp_hi, kl, e2);
-        e2 = __fmaf_rn(cf.bp_lo, kh, e2);
-        float xh, xl;
-        split_f64(xc, xh, xl);
-        float s, er1, er2;
-        two_sum(-xh, p1, s, er1);
-        two_sum(s, p2, s, er2);
-        const float lo = __fadd_rn(__fadd_rn(__fsub_rn(e1, xl), e2), __fadd_rn(er1, er2));
-        store_r(r + (int64_t)t * n + i, __fadd_rn(s, lo));   // r to FP32: all the apply reads
-#pragma unroll
-        for (int j = NB - 1; j >= 1; j--) {
-          qh[j] = qh[j - 1];
-          ql[j] = ql[j - 1];
-        }
+    for (int j = 1; j < NB; j++) {
+      const int w = qweight<NB>(j);
+      if (w == -5) {                   // -5 q = -4 q - q, each exact
+        two_sum2(sh, mul2(dup2(-4.f), qh[j]), sh, e);
+        sl = add2(sl, e);
+        two_sum2(sh, sub2(zero, qh[j]), sh, e);
+        sl = add2(sl, sub2(e, mul2(dup2(5.f), ql[j])));
+      } else {
+        two_sum2(sh, w == 1 ? qh[j] : mul2(dup2((float)w), qh[j]), sh, e);
+        sl = add2(sl, fma2(dup2((float)w), ql[j], e));   // one rounding, as w q is exact
       }
+    }
+    // mh S and bp k as pairs (exact high products by FMA)
+    const f2x p1 = mul2(mhh, sh);
+    f2x e1 = fma2(mhh, sh, sub2(zero, p1));
+    e1 = fma2(mhh, sl, e1);
+    e1 = fma2(mhl, sh, e1);
+    const f2x p2 = mul2(bph, kh);
+    f2x e2 = fma2(bph, kh, sub2(zero, p2));
+    e2 = fma2(bph, kl, e2);
+    e2 = fma2(bpl, kh, e2);
+    float xh[2], xl[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) split_f64(xc[u], xh[u], xl[u]);
+    f2x sum, er1, er2;
+    two_sum2(pack2(-xh[0], -xh[1]), p1, sum, er1);
+    two_sum2(sum, p2, sum, er2);
+    const f2x lo = add2(add2(sub2(e1, pack2(xl[0], xl[1])), e2), add2(er1, er2));
+    float ra, rb;
+    unpack2(add2(sum, lo), ra, rb);    // r to FP32: all the apply reads
+    RT *rr = r + (int64_t)t * n;
+    store_r(rr + i, ra);
+    if (two) store_r(rr + i2, rb);
+#pragma unroll
+    for (int j = NB - 1; j >= 1; j--) {
+      qh[j] = qh[j - 1];
+      ql[j] = ql[j - 1];
     }
   }
 }
@@ -950,13 +985,15 @@ static cudaError_t circ_residual_df_any(const Ctx &c, const float *z, const doub
                   (unsigned)((c.ell + kMvRows - 1) / kMvRows));
   const int n = (int)c.n, ell = (int)c.ell;
   if (c.circ_df.int_weights) {
+    const dim3 qgrid((unsigned)((c.n + 2 * kMvCols - 1) / (2 * kMvCols)),
+                     (unsigned)((c.ell + kResRows - 1) / kResRows));
     switch (c.circ_df.taps * 2 + (transpose ? 1 : 0)) {
-      case 4: k_circ_residual_q<2, false, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 5: k_circ_residual_q<2, true, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 6: k_circ_residual_q<3, false, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 7: k_circ_residual_q<3, true, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 8: k_circ_residual_q<4, false, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 9: k_circ_residual_q<4, true, RT><<<grid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 4: k_circ_residual_q<2, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 5: k_circ_residual_q<2, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 6: k_circ_residual_q<3, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 7: k_circ_residual_q<3, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 8: k_circ_residual_q<4, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 9: k_circ_residual_q<4, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
       default: return cudaErrorInvalidValue;
     }
     note_launch();

@@ -1,11 +1,37 @@
-"""The refined apply's last subtraction z0 - d on the FP32 and integer pipes:
-the same bits as the FP64 subtraction that large results take."""
+"""The refined apply's residual with two columns a thread (csrc/blas.cu): column
+counts at the edges of a CTA's two halves of 128 columns, step counts at the
+edges of a walk of 8, for every form and both directions, within the bounds of
+test_gpu_refined.  And its last subtraction z0 - d on the FP32 and integer
+pipes: the same bits as the FP64 subtraction that large results take."""
 import numpy as np
 import pytest
 
-from tests._helpers import need_gpu, rand_block, to_dev, to_host
+from oracle import precond
+from tests._helpers import (backward_error, need_gpu, oracle_system, rand_block, refined_bw_tol,
+                            rel_max, to_dev, to_host)
+from tests.test_gpu_refined import ELEMENTWISE_MAX, refined_tol
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,ell", [(127, 8), (128, 9), (129, 16), (130, 6), (255, 8), (256, 15),
+                                   (257, 8), (385, 3), (512, 18)])
+@pytest.mark.parametrize("kind", ["heat", "wave_bd2", "wave_bd4"])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_refined_apply(n, ell, kind, transpose):
+    torch = need_gpu()
+    from paper_1810_00615_gb300 import AllAtOnce
+    S = oracle_system(kind, n, ell)
+    X = rand_block(n, ell, 4100 + n + ell)
+    a = AllAtOnce(n, ell, 1.0 / ell, equation=kind, precision="fp32_refined", restart=1)
+    got = to_host(a.precond_apply(to_dev(torch, X), transpose=transpose))
+    tol = refined_tol(S, kind, n, ell)
+    if tol < ELEMENTWISE_MAX:
+        assert rel_max(got, precond.circulant_inverse(S, X, transpose=transpose)) <= tol
+    a.set_precision("fp32")
+    z0 = to_host(a.precond_apply(to_dev(torch, X), transpose=transpose))
+    d = np.linalg.norm(z0 - got) / max(np.linalg.norm(got), 1e-300)
+    assert backward_error(S, X, got, transpose) <= refined_bw_tol(n, ell, d)
 
 
 @pytest.mark.parametrize("n,ell", [(40, 48), (33, 256), (255, 1024), (20, 8)])
