@@ -838,37 +838,6 @@ template <int NB> __device__ __forceinline__ constexpr int qweight(int j) {
                  : (NB == 3 ? (j == 1 ? -2 : 1) : (j == 0 ? 2 : (j == 1 ? -5 : (j == 2 ? 4 : -1))));
 }
 
-// Two FP32 numbers in one 64-bit register pair.
-typedef unsigned long long f2x;
-__device__ __forceinline__ f2x pack2(float a, float b) {
-  f2x r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f2x v, float &a, float &b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f2x dup2(float a) { return pack2(a, a); }
-__device__ __forceinline__ f2x add2(f2x a, f2x b) {
-  f2x r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2x sub2(f2x a, f2x b) {
-  f2x r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2x fma2(f2x a, f2x b, f2x c) {
-  f2x r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-// The product as an FMA onto zero.  A packed multiplication followed by an
-// addition is contracted into one FMA in spite of its .rn, which leaves the
-// product unrounded where its rounding error is formed separately (a refined
-// apply was 6e-8 off).
-__device__ __forceinline__ f2x mul2(f2x a, f2x b) { return fma2(a, b, dup2(0.f)); }
 __device__ __forceinline__ void two_sum2(f2x a, f2x b, f2x &s, f2x &e) {
   s = add2(a, b);
   const f2x bb = sub2(s, a);
