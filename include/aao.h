@@ -190,8 +190,8 @@ int aao_neumann_apply(aao_ctx *ctx, int terms, const double *x, double *y,
  * BD4: y_t = M(2x_t - 5x_{t-1} + 4x_{t-2} - x_{t-3}) + tau^2 K x_t, with the
  * BD2 rows B x_1 and C x_1 + B x_2 first;
  * the transpose shifts the other way.  For these forms the stencil sums
- * are formed exactly in 64-bit fixed point per 32-column, 32-step tile and
- * rounded once (elements more than 2^5 below their tile's largest enter with
+ * are formed exactly in 64-bit fixed point per tile of 32 columns and 8 or 16
+ * steps and rounded once (elements more than 2^5 below their tile's largest enter with
  * an absolute error under 2^-57 of it; BD4, whose larger weights need two
  * more guard bits: 2^3 and 2^-55); the literal heat form runs the FP64
  * stencil.  An inf or NaN in a tile makes that tile's outputs NaN.  No
@@ -214,8 +214,8 @@ int aao_matvec_sub(aao_ctx *ctx, const double *x, const double *sub, double *y, 
  * 2^34 below their tile's largest enter with an absolute error under 2^-57
  * of it); the literal heat form widens x and runs the FP64 stencil.  x:
  * device, N floats; sub, y: device, N doubles (sub must not overlap y); no
- * workspace needed.  An inf or NaN anywhere in a 32-column, 32-step tile
- * makes that tile's outputs NaN. */
+ * workspace needed.  An inf or NaN anywhere in a tile makes that tile's
+ * outputs NaN. */
 int aao_matvec_f32(aao_ctx *ctx, const float *x, const double *sub, double *y, int transpose,
                    void *stream);
 
@@ -244,7 +244,7 @@ int aao_residual(aao_ctx *ctx, const double *x, const double *b, double *r, int 
  * circulant of Section 3 with the constant step): the residual of the refined
  * FP32 preconditioner apply (AAO_PREC_FP32_REFINED), which corrects
  * z = P32^{-1} x by P32^{-1} r.  Evaluated like aao_matvec_f32 (exact
- * fixed-point stencil sums per 32-column, 32-step tile, time wrapped around,
+ * fixed-point stencil sums per tile, time wrapped around,
  * one rounding) so that r keeps its relative accuracy however much P z and x
  * cancel; the literal heat form widens z and runs the FP64 stencil.
  * z: device, N floats; x, r: device, N doubles; r overlaps neither. */
@@ -302,7 +302,7 @@ int aao_solve_host(aao_ctx *ctx, const double *u0_host, const double *v0_host,
  * the matvec, the Arnoldi kernels, and the residual P z0 - x (or the Neumann
  * right-hand side) of the refined FP32 apply.  Where the FP32 apply folds the
  * tridiagonal solves into its transform (ell = 256 ... 4096 a power of two,
- * n + 1 = 16 P), FFT_FORWARD is its first forward kernel, FFT_FORWARD_SOLVE
+ * n > 16), FFT_FORWARD is its first forward kernel, FFT_FORWARD_SOLVE
  * the second forward kernel with the chunk solves, TRIDIAG the separator
  * systems, FFT_INVERSE_SOLVE the first inverse kernel with the chunk
  * corrections and FFT_INVERSE the last inverse kernel; elsewhere the two
