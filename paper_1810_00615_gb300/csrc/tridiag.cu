@@ -82,14 +82,24 @@ __device__ __forceinline__ void load_levels(RecLev<R, CH> *dst, const RecLev<R, 
 }
 
 // Dirichlet solve of one chunk in registers with the pivots inv (invp, or
-// invt for the last chunk): entries whose 1/pivot is zero come out zero.
+// invt for the last chunk): entries whose 1/pivot is zero come out zero.  Only
+// a last chunk of CH unknowns (all) has one in the separator's place; the others
+// leave v[CH - 1] alone, a ninth of an FP64 chunk's arithmetic and two links
+// of its chain (whole FP64 apply n 4095 x ell 4096: 1871 -> 1857 us, n 16383 x
+// ell 16: 107.4 -> 105.2 with the upper levels).
 template <typename R, int CH>
-__device__ __forceinline__ void chunk_solve(cx<R> *v, const cx<R> *inv, const cx<R> *bp, cx<R> e) {
+__device__ __forceinline__ void chunk_solve(cx<R> *v, const cx<R> *inv, const cx<R> *bp, cx<R> e,
+                                            bool all) {
   v[0] = v[0] * inv[0];
 #pragma unroll
-  for (int i = 1; i < CH; i++) v[i] = cfnms(v[i], e, v[i - 1]) * inv[i];
+  for (int i = 1; i < CH - 1; i++) v[i] = cfnms(v[i], e, v[i - 1]) * inv[i];
+  if (all) {
+    if constexpr (sizeof(R) == 8) asm volatile("");   // a branch: one warp of the row takes it
+    v[CH - 1] = cfnms(v[CH - 1], e, v[CH - 2]) * inv[CH - 1];
+    v[CH - 2] = cfnms(v[CH - 2], bp[CH - 2], v[CH - 1]);
+  }
 #pragma unroll
-  for (int i = CH - 2; i >= 0; i--) v[i] = cfnms(v[i], bp[i], v[i + 1]);
+  for (int i = CH - 3; i >= 0; i--) v[i] = cfnms(v[i], bp[i], v[i + 1]);
 }
 
 // Levels 1 .. levels-1 of the recursive form on shared-memory buffers:
@@ -109,7 +119,10 @@ __device__ __forceinline__ void rec_upper(cx<R> *const *B, const int *lsz, int l
       cx<R> w[CH];
 #pragma unroll
       for (int i = 0; i < CH; i++) w[i] = Bl[rpos<CH>(q * CH + i)];
-      chunk_solve<R, CH>(w, last ? T[l].invt : T[l].invp, T[l].bp, el);
+      // FP32 takes every chunk for a full one (w[CH - 1] comes out zero): the
+      // branch costs more than it saves, n 65535 x ell 512 397 -> 402 us
+      chunk_solve<R, CH>(w, last ? T[l].invt : T[l].invp, T[l].bp, el,
+                         sizeof(R) == 4 || (last && lsz[l] == Pl * CH));
 #pragma unroll
       for (int i = 0; i < CH - 1; i++) Bl[rpos<CH>(q * CH + i)] = w[i];
       if (last) Bl[rpos<CH>(q * CH + CH - 1)] = w[CH - 1];
@@ -204,7 +217,7 @@ k_tridiag_rec(cx<R> *__restrict__ spec, int n, int64_t n_pad,
   // level 0: local Dirichlet solve of the chunk, its separator value aside
   const bool last = p == M;
   const cx<R> e0 = T[0].e, sep = v[CH - 1];
-  chunk_solve<R, CH>(v, last ? T[0].invt : T[0].invp, T[0].bp, e0);
+  chunk_solve<R, CH>(v, last ? T[0].invt : T[0].invp, T[0].bp, e0, last && n == P * CH);
   if (levels > 1) {
     // separator right-hand sides of level 1: needs the first local value of
     // the next chunk
@@ -300,7 +313,7 @@ k_tridiag_cluster(cx<R> *__restrict__ spec, int n, int64_t n_pad,
     }
   }
   const cx<R> e0 = T0[0].e, sep = v[CH - 1];
-  chunk_solve<R, CH>(v, T0[0].invp, T0[0].bp, e0);
+  chunk_solve<R, CH>(v, T0[0].invp, T0[0].bp, e0, false);   // n + 1 = P CH
   s_first[p] = v[0];
   cluster.sync();
   cx<R> *B1root = cluster.map_shared_rank(B[1], 0);
@@ -460,7 +473,7 @@ k_tridiag_reduced3(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ se
   }
   // level 1: the chunk's unknowns, its separator value aside
   const cx<float> sep1 = wv[CH - 1];
-  chunk_solve<float, CH>(wv, lane == M2 ? T1.invt : T1.invp, T1.bp, e1);
+  chunk_solve<float, CH>(wv, lane == M2 ? T1.invt : T1.invp, T1.bp, e1, lane == M2);
   // level-2 right-hand side of separator L: sep - e1 (last of chunk L + first of chunk L+1)
   const cx<float> firstr = mk(__shfl_down_sync(0xffffffffu, wv[0].re, 1),
                               __shfl_down_sync(0xffffffffu, wv[0].im, 1));
@@ -470,7 +483,7 @@ k_tridiag_reduced3(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ se
     cx<float> z[CH];
 #pragma unroll
     for (int i = 0; i < CH; i++) z[i] = (i < M2) ? s2[w][i] : mk(0.f, 0.f);
-    chunk_solve<float, CH>(z, T2.invt, T2.bp, T2.e);
+    chunk_solve<float, CH>(z, T2.invt, T2.bp, T2.e, true);
 #pragma unroll
     for (int i = 0; i < CH; i++)
       if (i < M2) s2[w][i] = z[i];
