@@ -428,7 +428,8 @@ struct CircDF {
 // (fft_steps.cuh) and the radices of its two short transforms; L = 0 where it
 // does not serve ell.
 struct StepPlan {
-  int L, L1, L2;
+  int L, L1, L2;        // L = 0: not these kernels
+  int split;            // the row and panel kernels instead (powers of two)
   int np1, np2;
   int rad1[4], rad2[4];
 };

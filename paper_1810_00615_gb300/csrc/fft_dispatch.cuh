@@ -25,20 +25,48 @@ static int persistent_grid(K kern, int threads, size_t smem, int npanels) {
 #endif
 // With scratch for the intermediate: FP32, ell = 256 ... 4096 a power of two
 // takes the four-step kernels compiled for it, every other length from
-// AAO_STEPS_MIN on (and every FP64 one) the run-time four-step kernels;
-// shorter transforms, and calls without scratch, one kernel per direction.
+// AAO_STEPS_MIN on (and FP64) what step_plan says: mostly the run-time
+// four-step kernels.  Shorter transforms, and calls without scratch, one
+// kernel per direction.
 template <typename R>
 inline bool use_four(int64_t ell) {
   return AAO_FFT_FOUR && std::is_same<R, float>::value && ell >= 256 && ell <= 4096 &&
          (ell & (ell - 1)) == 0;
 }
 
+// The row and panel kernels serve the powers of two that step_plan leaves
+// to them (large n): bytes of their panel-major intermediate.
+template <typename R, int L>
+static size_t split_bytes(int64_t n) {
+  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+    const int W = 2 * Shape<R, L>::C;
+    return (size_t)((n + W - 1) / W) * Split<R, L>::PANEL;
+  }
+  return 0;
+}
+
 template <typename R, int L, typename YT>
-static cudaError_t run_forward(int64_t n, int64_t n_pad, const double *x, const YT *y,
-                               const R *sigk, cx<R> *spec, const cx<R> *tw, cudaStream_t s) {
+static cudaError_t run_forward(const StepPlan &pl, int64_t n, int64_t n_pad, const double *x, const YT *y,
+                               const R *sigk, cx<R> *spec, const cx<R> *tw, cudaStream_t s, void *inter) {
   using S = Shape<R, L>;
   const int W = 2 * S::C;
   const int np = (int)((n + W - 1) / W);
+  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+    if (inter && pl.split) {
+      const int ncx = np * S::C;
+      const dim3 g1((unsigned)((ncx + kRowThreads - 1) / kRowThreads), (unsigned)Split<R, L>::LR);
+      cx<R> *ip = static_cast<cx<R> *>(inter);
+      if (y) k_fft_forward_rows<R, L, true, YT><<<g1, kRowThreads, 0, s>>>(x, y, sigk, ip, (int)n, ncx);
+      else k_fft_forward_rows<R, L, false, double><<<g1, kRowThreads, 0, s>>>(x, nullptr, sigk, ip, (int)n, ncx);
+      note_launch();
+      auto kern = k_fft_forward_panels<R, L>;
+      const int g = persistent_grid(kern, S::T, S::SMEM, np);
+      if (g <= 0) return cudaErrorInvalidConfiguration;
+      kern<<<g, S::T, S::SMEM, s>>>(ip, spec, (int)n, n_pad, tw, np);
+      note_launch();
+      return cudaGetLastError();
+    }
+  }
   if (y) {
     auto kern = k_fft_forward<R, L, true, YT>;
     const int g = persistent_grid(kern, S::T, S::SMEM, np);
@@ -55,11 +83,26 @@ static cudaError_t run_forward(int64_t n, int64_t n_pad, const double *x, const 
 }
 
 template <typename R, int L, typename OT>
-static cudaError_t run_inverse(int64_t n, int64_t n_pad, const cx<R> *spec, OT *y,
-                               const cx<R> *tw, cudaStream_t s, const float *base) {
+static cudaError_t run_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, const cx<R> *spec, OT *y,
+                               const cx<R> *tw, cudaStream_t s, void *inter, const float *base) {
   using S = Shape<R, L>;
   const int W = 2 * S::C;
   const int np = (int)((n + W - 1) / W);
+  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+    if (inter && pl.split) {
+      cx<R> *ip = static_cast<cx<R> *>(inter);
+      auto kern = k_fft_inverse_panels<R, L>;
+      const int g = persistent_grid(kern, S::T, S::SMEM, np);
+      if (g <= 0) return cudaErrorInvalidConfiguration;
+      kern<<<g, S::T, S::SMEM, s>>>(spec, ip, (int)n, n_pad, tw, np);
+      note_launch();
+      const int ncx = np * S::C;
+      const dim3 g2((unsigned)((ncx + kRowThreads - 1) / kRowThreads), (unsigned)(L / 16));
+      k_fft_inverse_rows<R, L, OT><<<g2, kRowThreads, 0, s>>>(ip, y, (int)n, ncx, tw, base);
+      note_launch();
+      return cudaGetLastError();
+    }
+  }
   auto kern = k_fft_inverse<R, L, OT>;
   const int g = persistent_grid(kern, S::T, S::SMEM, np);
   if (g <= 0) return cudaErrorInvalidConfiguration;
@@ -88,7 +131,7 @@ cudaError_t forward_any(int64_t ell, const StepPlan &pl, int64_t n, int64_t n_pa
   }
   if (inter && pl.L) return steps_forward<R>(pl, n, n_pad, x, y, sigk, spec, tw, s, inter);
   switch (ell) {
-#define AAO_F(L) case L: return run_forward<R, L, YT>(n, n_pad, x, y, sigk, spec, tw, s);
+#define AAO_F(L) case L: return run_forward<R, L, YT>(pl, n, n_pad, x, y, sigk, spec, tw, s, inter);
     AAO_FFT_CASES(AAO_F)
 #undef AAO_F
     default: return run_forward_mixed<R, YT>(ell, n, n_pad, x, y, sigk, spec, tw, s);
@@ -117,7 +160,13 @@ inline cudaError_t forward_four_f32_input(int64_t ell, const StepPlan &pl, int64
 template <typename R>
 size_t inter_bytes_any(int64_t ell, const StepPlan &pl, int64_t n) {
   if (use_four<R>(ell)) return four_inter_bytes(ell, n);
-  return pl.L ? steps_inter_bytes<R>(ell, n) : 0;
+  if (!pl.split) return pl.L ? steps_inter_bytes<R>(ell, n) : 0;
+  switch (ell) {
+#define AAO_B(L) case L: return split_bytes<R, L>(n);
+    AAO_FFT_CASES(AAO_B)
+#undef AAO_B
+    default: return 0;
+  }
 }
 
 template <typename R, typename OT>
@@ -135,7 +184,7 @@ cudaError_t inverse_any(int64_t ell, const StepPlan &pl, int64_t n, int64_t n_pa
   }
   if (inter && pl.L) return steps_inverse<R, OT>(pl, n, n_pad, spec, y, tw, s, inter, base);
   switch (ell) {
-#define AAO_I(L) case L: return run_inverse<R, L, OT>(n, n_pad, spec, y, tw, s, base);
+#define AAO_I(L) case L: return run_inverse<R, L, OT>(pl, n, n_pad, spec, y, tw, s, inter, base);
     AAO_FFT_CASES(AAO_I)
 #undef AAO_I
     default: return run_inverse_mixed<R, OT>(ell, n, n_pad, spec, y, tw, s, base);

@@ -3,8 +3,8 @@
 
 namespace aao {
 void fft_plan(Ctx &c) {
-  fft::step_plan(c.ell, false, c.step32);
-  fft::step_plan(c.ell, true, c.step64);
+  fft::step_plan(c.ell, c.n, false, c.step32);
+  fft::step_plan(c.ell, c.n, true, c.step64);
 }
 cudaError_t fft_forward_f32(const Ctx &c, const double *x, const double *y, void *spec,
                             cudaStream_t s, void *inter) {

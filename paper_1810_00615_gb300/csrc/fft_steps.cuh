@@ -449,9 +449,28 @@ inline bool step_radices(int N, int *rad, int &np) {
 // output shared by L1 time steps, so at the low frequencies that P^{-1}
 // amplifies it is about sqrt(L1) times that of a transform whose twiddles
 // come last; the refined apply squares that error.
-inline bool step_plan(int64_t ell, bool fp64, StepPlan &pl) {
+//
+// Large calls keep the compiled forms of fft_time.cuh and fft_mixed.cuh, which
+// spend fewer instructions per element once they fill the chip.  Powers of two
+// (row and panel kernels; whole apply, steps against them): FP32 n 65535 x ell
+// 64 83 / 61 us, 16383 x 128 59 / 50, but 8191 x 32 30 / 32 and 4095 x 128 28 /
+// 29; FP64 8191 x 128 162 / 146, 4095 x 256 159 / 126, 32767 x 256 937 / 800,
+// but 2047 x 256 93 / 114, 8191 x 512 449 / 478, 16383 x 1024 1704 / 1780; only
+// ell = 4096 turns again (8191: 3865 / 3791).  Other short lengths (one mixed-radix
+// kernel a direction): FP32 n 16383 x ell 20 38 / 33, 8191 x 40 31 / 26, but
+// refined 4095 x 30 49 / 56 and 32767 x 100 67 / 75; FP64 4095 x 40 67 / 62,
+// 16383 x 40 136 / 130, but 16383 x 100 200 / 208 and 65535 x 20 171 / 183.
+inline bool step_plan(int64_t ell, int64_t n, bool fp64, StepPlan &pl) {
   pl = StepPlan{};
   if (ell < AAO_STEPS_MIN) return false;
+  if ((ell & (ell - 1)) == 0) {
+    const bool big = n * ell > 1000000;
+    pl.split = fp64 ? (ell <= 256 && big) || (ell <= 512 && n >= 16383) || (ell == 4096 && n >= 4095)
+                    : ell <= 128 && (big || n >= 32767);
+    if (pl.split) return false;
+  } else if (n < 32767 && (fp64 ? ell <= 50 && n >= 3072 : ell <= 100 && n >= 6144)) {
+    return false;
+  }
   const bool wide = !fp64 && ell >= 64;
   for (int64_t l1 = wide ? 8 : 1; l1 <= 128; l1++) {
     if (ell % l1 || (wide ? ell / l1 > 64 : l1 * l1 < ell)) continue;

@@ -354,6 +354,269 @@ k_fft_forward(const double *__restrict__ x, const YT *__restrict__ y,
   }
 }
 
+// ------------------------------------------------ forward in two kernels
+// The single kernel above reads its panel as 2C doubles per time step, a
+// 32-64 byte piece of each of L rows far apart in memory, and that pattern
+// holds DRAM well below its streaming rate; its passes then run while the
+// DRAM idles.  For L >= 256 the forward transform is split instead:
+//
+//  rows   the first Stockham pass (radix R1, Ns = 1: no twiddles) needs time
+//         steps j + r L/R1 of a column, r < R1.  A CTA takes one j and 256
+//         complex columns, so it reads R1 row segments of 512 doubles each;
+//         it writes its R1 outputs per column into a panel-major intermediate
+//         laid out exactly like the panel kernel's shared-memory buffer.
+//  panels a persistent CTA copies one panel of that intermediate (one
+//         contiguous block, resident in L2) into shared memory with 16-byte
+//         asynchronous copies, runs passes 2..NP and writes the half spectrum.
+constexpr int kRowThreads = 256;
+
+template <typename R, int L> struct Split {
+  static constexpr bool OK = Passes<L>::NP >= 2;
+  static constexpr int R1 = Passes<L>::R1;
+  static constexpr int LR = L / (R1 < 1 ? 1 : R1);                    // butterflies per column
+  static constexpr size_t PANEL = Shape<R, L>::WORK;                   // bytes per panel
+};
+
+template <typename R, int L, bool NEUMANN, typename YT>
+__global__ void __launch_bounds__(kRowThreads)
+k_fft_forward_rows(const double *__restrict__ x, const YT *__restrict__ y,
+                   const R *__restrict__ sigk, cx<R> *__restrict__ inter, int n, int ncx) {
+  using S = Shape<R, L>;
+  using P = Split<R, L>;
+  constexpr int C = S::C, R1 = P::R1;
+  const int j = blockIdx.y;                                   // butterfly (time offset)
+  const int cg = blockIdx.x * kRowThreads + threadIdx.x;      // complex column
+  const bool act = cg < ncx;        // every thread stays for the barriers below
+  const int i = 2 * cg;
+  const unsigned long long pol_stream = l2_evict_first(), pol_keep = l2_evict_last();
+  cx<R> v[R1];
+  if constexpr (!NEUMANN) {
+    // The CTA's rows (512 real columns each) come in through shared memory,
+    // up to 8 at a time, so that every warp load is one contiguous segment
+    // instead of two interleaved 8-byte streams.
+    constexpr int H = R1 < 8 ? R1 : 8;
+    __shared__ __align__(16) double s_in[H][2 * kRowThreads];
+    const int i0 = 2 * blockIdx.x * kRowThreads;
+#pragma unroll
+    for (int h = 0; h < R1; h += H) {
+#pragma unroll
+      for (int rr = 0; rr < H; rr++) {
+        const size_t row = (size_t)(j + (h + rr) * P::LR) * n;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const int col = u * kRowThreads + threadIdx.x, ic = i0 + col;
+          s_in[rr][col] = (ic < n) ? ld_hint(&x[row + ic], pol_stream) : 0.0;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int rr = 0; rr < H; rr++) {
+        const double2 d = reinterpret_cast<const double2 *>(s_in[rr])[threadIdx.x];
+        v[h + rr] = mk(from_f64<R>(d.x), from_f64<R>(d.y));
+      }
+      __syncthreads();
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < R1; r++) {
+      const int t = j + r * P::LR;
+      v[r] = mk(load_real<R, L, NEUMANN, YT>(x, y, sigk, n, t, i, pol_stream),
+                load_real<R, L, NEUMANN, YT>(x, y, sigk, n, t, i + 1, pol_stream));
+    }
+  }
+  if (!act) return;
+  dft<R, -1, R1>(v);
+  cx<R> *dst = reinterpret_cast<cx<R> *>(reinterpret_cast<unsigned char *>(inter) +
+                                         (size_t)(cg / C) * P::PANEL) + (cg % C);
+#pragma unroll
+  for (int r = 0; r < R1; r++) st_hint(dst + phys<C>(j * R1 + r, 0), v[r], pol_keep);
+}
+
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+}
+
+template <typename R, int L>
+__global__ void __launch_bounds__(Shape<R, L>::T)
+k_fft_forward_panels(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, int n,
+                     int64_t n_pad, const cx<R> *__restrict__ tw, int npanels) {
+  using S = Shape<R, L>;
+  using PL = Passes<L>;
+  using P = Split<R, L>;
+  constexpr int C = S::C, T = S::T, W = 2 * C;
+  constexpr int CHUNKS = (int)(P::PANEL / 16);
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *sm = reinterpret_cast<cx<R> *>(smraw);
+  const unsigned long long pol_keep = l2_evict_last();
+  for (int panel = blockIdx.x; panel < npanels; panel += gridDim.x) {
+    const unsigned char *src = reinterpret_cast<const unsigned char *>(inter) + (size_t)panel * P::PANEL;
+    for (int q = threadIdx.x; q < CHUNKS; q += T) cp_async16(smraw + 16 * q, src + 16 * q);
+    cp_async_wait_all();
+    __syncthreads();
+    int Ns = P::R1;
+#pragma unroll
+    for (int p = 1; p < PL::NP; p++) {
+      pass<R, L, C, 16, -1, T>(sm, Ns, tw);
+      Ns *= 16;
+    }
+    const int i0 = panel * W;
+    constexpr int NK = L / 2 + 1;
+    for (int idx = threadIdx.x; idx < NK * C; idx += T) {
+      const int k = idx / C, c = idx - k * C;
+      const cx<R> zk = sm[phys<C>(k, c)];
+      const cx<R> zm = sm[phys<C>((L - k) & (L - 1), c)];
+      const R hf = (R)0.5;
+      const cx<R> X = mk(hf * (zk.re + zm.re), hf * (zk.im - zm.im));
+      const cx<R> Y = mk(hf * (zk.im + zm.im), hf * (zm.re - zk.re));
+      const int i = i0 + 2 * c;
+      cx<R> *dst = spec + (size_t)k * n_pad + i;
+      if (i + 1 < n) {
+        st_hint2(dst, X, Y, pol_keep);        // i even: the pair is 16/32-byte aligned
+      } else if (i < n) {
+        st_hint(dst, X, pol_keep);
+      }
+    }
+    __syncthreads();   // the work buffer is reused by the next panel
+  }
+}
+
+// ------------------------------------------------ inverse in two kernels
+// Mirror of the forward split (L >= 256): a persistent panel kernel loads the
+// half spectrum of its panel, extends it to the Hermitian full spectrum, runs
+// all Stockham passes but the last and stores its shared-memory image to the
+// panel-major intermediate; a row kernel runs the last radix-16 pass (whose
+// butterfly j yields time steps j + r L/16) and writes those rows of y as
+// contiguous segments of 512 columns.
+template <typename R, int L>
+__global__ void __launch_bounds__(Shape<R, L>::T)
+k_fft_inverse_panels(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int n,
+                     int64_t n_pad, const cx<R> *__restrict__ tw, int npanels) {
+  using S = Shape<R, L>;
+  using PL = Passes<L>;
+  using P = Split<R, L>;
+  constexpr int C = S::C, T = S::T, W = 2 * C;
+  constexpr int CHUNKS = (int)(P::PANEL / 16);
+  constexpr int NK = L / 2 + 1;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<R> *sm = reinterpret_cast<cx<R> *>(smraw);
+  const unsigned long long pol_done = l2_evict_first(), pol_keep = l2_evict_last();
+  for (int panel = blockIdx.x; panel < npanels; panel += gridDim.x) {
+    const int i0 = panel * W;
+    // all of a thread's spectrum loads are issued before any is used
+    constexpr int IT = (NK * C + T - 1) / T;
+    cx<R> A[IT], B[IT];
+#pragma unroll
+    for (int q = 0; q < IT; q++) {
+      const int idx = threadIdx.x + q * T;
+      const int k = idx / C, c = idx - k * C;
+      const int i = i0 + 2 * c;
+      const cx<R> *src = spec + (size_t)k * n_pad + i;
+      A[q] = mk((R)0, (R)0);
+      B[q] = mk((R)0, (R)0);
+      if (idx < NK * C) {
+        if (i + 1 < n) ld_hint2(src, A[q], B[q], pol_done);   // i even: aligned pair
+        else if (i < n) A[q] = ld_hintc(src, pol_done);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < IT; q++) {
+      const int idx = threadIdx.x + q * T;
+      if (idx >= NK * C) break;
+      const int k = idx / C, c = idx - k * C;
+      cx<R> a = A[q], b = B[q];
+      if (k == 0 || 2 * k == L) { a.im = (R)0; b.im = (R)0; }
+      sm[phys<C>(k, c)] = mk(a.re - b.im, a.im + b.re);
+      if (k > 0 && 2 * k < L) sm[phys<C>(L - k, c)] = mk(a.re + b.im, b.re - a.im);
+    }
+    __syncthreads();
+    pass<R, L, C, P::R1, +1, T>(sm, 1, tw);
+    int Ns = P::R1;
+#pragma unroll
+    for (int p = 1; p < PL::NP - 1; p++) {
+      pass<R, L, C, 16, +1, T>(sm, Ns, tw);
+      Ns *= 16;
+    }
+    float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(inter) +
+                                             (size_t)panel * P::PANEL);
+    const float4 *srcs = reinterpret_cast<const float4 *>(smraw);
+    for (int q = threadIdx.x; q < CHUNKS; q += T) st_hint4(dst + q, srcs[q], pol_keep);
+    __syncthreads();   // the work buffer is reused by the next panel
+  }
+}
+
+// With base (FP64 output only): y = base - (the transform), the correction
+// step of the refined FP32 preconditioner.
+template <typename R, int L, typename OT>
+__global__ void __launch_bounds__(kRowThreads)
+k_fft_inverse_rows(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int ncx,
+                   const cx<R> *__restrict__ tw, const float *__restrict__ base) {
+  using S = Shape<R, L>;
+  using P = Split<R, L>;
+  constexpr int C = S::C, NS = L / 16;                        // last pass: radix 16, Ns = L/16
+  const int j = blockIdx.y;                                   // butterfly = first time step
+  const int cg = blockIdx.x * kRowThreads + threadIdx.x;
+  const bool act = cg < ncx;        // every thread stays for the barriers below
+  const unsigned long long pol_done = l2_evict_first();
+  const cx<R> *src = reinterpret_cast<const cx<R> *>(reinterpret_cast<const unsigned char *>(inter) +
+                                                     (size_t)(act ? cg / C : 0) * P::PANEL) + (cg % C);
+  cx<R> v[16];
+#pragma unroll
+  for (int r = 0; r < 16; r++)
+    v[r] = act ? ld_hintc(src + phys<C>(j + r * NS, 0), pol_done) : mk((R)0, (R)0);
+#pragma unroll
+  for (int r = 1; r < 16; r++) v[r] = twiddle<R, +1>(v[r], tw[j * r]);
+  dft<R, +1, 16>(v);
+  const R scale = (R)1 / (R)L;
+  // The CTA's rows (16 time steps x 512 real columns) go out through shared
+  // memory in two halves, so that every warp store (and base load) is one
+  // contiguous segment instead of two interleaved 8-byte streams.
+  __shared__ __align__(16) OT s_out[8][2 * kRowThreads];
+  const int i0 = 2 * blockIdx.x * kRowThreads;                // first real column of the CTA
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    // the base values of this half are requested before the barrier
+    float bv[8][2];
+    if constexpr (sizeof(OT) == 8) {
+      if (base) {
+#pragma unroll
+        for (int rr = 0; rr < 8; rr++) {
+          const size_t row = (size_t)(j + (h * 8 + rr) * NS) * n;
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const int i = i0 + u * kRowThreads + threadIdx.x;
+            bv[rr][u] = (i < n) ? __ldg(&base[row + i]) : 0.0f;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int rr = 0; rr < 8; rr++)   // one 8/16-byte store of the pair: no bank conflicts
+      reinterpret_cast<cx<OT> *>(s_out[rr])[threadIdx.x] =
+          mk(to_out<R, OT>(scale * v[h * 8 + rr].re), to_out<R, OT>(scale * v[h * 8 + rr].im));
+    __syncthreads();
+#pragma unroll
+    for (int rr = 0; rr < 8; rr++) {
+      const size_t row = (size_t)(j + (h * 8 + rr) * NS) * n;
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        const int col = u * kRowThreads + threadIdx.x, i = i0 + col;
+        if (i >= n) continue;
+        const OT val = s_out[rr][col];
+        if constexpr (sizeof(OT) == 8) {
+          y[row + i] = base ? to_f64(bv[rr][u]) - val : val;
+        } else {
+          y[row + i] = val;
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // Inverse: half spectrum -> y, scaled by 1/L.  The result goes through shared
 // memory and is written row by row (2C contiguous values per time step).  OT
 // is the stored type: double for the public entry points, float for the
