@@ -52,8 +52,8 @@ L2_BYTES = 135528448
 ROOFLINE_KEY = "fft4_inverseA_correct"
 MATVEC_KEY = "matvec_dots1_double"
 RESIDUAL_KEY = "circ_residual_df"
-DOMINANT_NAMES = {"k_fft4_inverseA_correct<4096, 32>": "correction",
-                  "k_matvec_fx<2, 0, 1, double, 0, 1>": "matvec",
+DOMINANT_NAMES = {"k_fft4_inverseA_correct<4096, 32, 0>": "correction",
+                  "k_matvec_fx<2, 0, 1, double, 0, 1, 16>": "matvec",
                   "k_circ_residual_q<2, 0, float>": "residual"}
 
 

@@ -16,7 +16,7 @@ on the machine that ran ncu); bench.py uses a summary's figures only while
 that digest is still the current one.
 
     python -m paper_1810_00615_gb300.ncu_summary capture raw.csv out.md \\
-        --title "..." --command "..." --digest HEX --key 'k_matvec_fx<2, 0, 1, double, 0, 1>=matvec_dots1_double'
+        --title "..." --command "..." --digest HEX --key 'k_matvec_fx<2, 0, 1, double, 0, 1, 16>=matvec_dots1_double'
     python -m paper_1810_00615_gb300.ncu_summary launches launches.csv out.md \\
         --title "..." --command "..." --digest HEX
 """
