@@ -831,8 +831,10 @@ k_circ_residual_df(const float *__restrict__ z, const double *__restrict__ x,
 // load latency is what is left); n 16383 x ell 1024 transposed 74 -> 59, n 1568
 // x ell 1440 18 -> 11.  A walk has 8 steps: 16 or 32 leave the last wave emptier
 // than their fewer halo rows save (59.6 and 67.5 us, n 1568 x ell 1440 13), 12
-// differ by under 1%.
-constexpr int kResRows = 8;
+// differ by under 1%.  Where 8 leave fewer than two CTAs per SM a walk has 2:
+// it is a chain of loads then, and 8 steps of two columns were slower than 8 of
+// one (refined apply n 5000 x ell 8 58.8 us against 56.2).
+constexpr int kResRows = 8, kResRowsSmall = 2;
 template <int NB> __device__ __forceinline__ constexpr int qweight(int j) {
   return NB == 2 ? (j == 0 ? 1 : -1)
                  : (NB == 3 ? (j == 1 ? -2 : 1) : (j == 0 ? 2 : (j == 1 ? -5 : (j == 2 ? 4 : -1))));
@@ -844,15 +846,15 @@ __device__ __forceinline__ void two_sum2(f2x a, f2x b, f2x &s, f2x &e) {
   e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
-template <int NB, bool TR, typename RT>
+template <int NB, bool TR, typename RT, int ROWS>
 __global__ void __launch_bounds__(kMvCols)
 k_circ_residual_q(const float *__restrict__ z, const double *__restrict__ x,
                   RT *__restrict__ r, int n, int ell, CircDF cf) {
   const int i = blockIdx.x * (2 * kMvCols) + threadIdx.x, i2 = i + kMvCols;
   if (i >= n) return;                  // no barriers in this kernel
   const bool two = i2 < n;
-  const int c0 = blockIdx.y * kResRows;
-  const int c1 = min(ell, c0 + kResRows);
+  const int c0 = blockIdx.y * ROWS;
+  const int c1 = min(ell, c0 + ROWS);
   auto load = [&](int t, f2x (&v)[3]) {
     const float *zr = z + (int64_t)t * n;
     v[0] = pack2(__ldg(&zr[i]), two ? __ldg(&zr[i2]) : 0.f);
@@ -947,6 +949,17 @@ k_circ_residual_q(const float *__restrict__ z, const double *__restrict__ x,
   }
 }
 
+template <int NB, bool TR, typename RT>
+static void run_circ_q(const Ctx &c, const float *z, const double *x, RT *r, cudaStream_t s) {
+  const unsigned gx = (unsigned)((c.n + 2 * kMvCols - 1) / (2 * kMvCols));
+  const int n = (int)c.n, ell = (int)c.ell;
+  auto gy = [&](int rows) { return (unsigned)((ell + rows - 1) / rows); };
+  if ((int64_t)gx * gy(kResRows) >= 2 * 152)
+    k_circ_residual_q<NB, TR, RT, kResRows><<<dim3(gx, gy(kResRows)), kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df);
+  else
+    k_circ_residual_q<NB, TR, RT, kResRowsSmall><<<dim3(gx, gy(kResRowsSmall)), kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df);
+}
+
 template <typename RT>
 static cudaError_t circ_residual_df_any(const Ctx &c, const float *z, const double *x, RT *r,
                                         int transpose, cudaStream_t s) {
@@ -954,15 +967,13 @@ static cudaError_t circ_residual_df_any(const Ctx &c, const float *z, const doub
                   (unsigned)((c.ell + kMvRows - 1) / kMvRows));
   const int n = (int)c.n, ell = (int)c.ell;
   if (c.circ_df.int_weights) {
-    const dim3 qgrid((unsigned)((c.n + 2 * kMvCols - 1) / (2 * kMvCols)),
-                     (unsigned)((c.ell + kResRows - 1) / kResRows));
     switch (c.circ_df.taps * 2 + (transpose ? 1 : 0)) {
-      case 4: k_circ_residual_q<2, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 5: k_circ_residual_q<2, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 6: k_circ_residual_q<3, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 7: k_circ_residual_q<3, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 8: k_circ_residual_q<4, false, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
-      case 9: k_circ_residual_q<4, true, RT><<<qgrid, kMvCols, 0, s>>>(z, x, r, n, ell, c.circ_df); break;
+      case 4: run_circ_q<2, false, RT>(c, z, x, r, s); break;
+      case 5: run_circ_q<2, true, RT>(c, z, x, r, s); break;
+      case 6: run_circ_q<3, false, RT>(c, z, x, r, s); break;
+      case 7: run_circ_q<3, true, RT>(c, z, x, r, s); break;
+      case 8: run_circ_q<4, false, RT>(c, z, x, r, s); break;
+      case 9: run_circ_q<4, true, RT>(c, z, x, r, s); break;
       default: return cudaErrorInvalidValue;
     }
     note_launch();
