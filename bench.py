@@ -54,7 +54,7 @@ MATVEC_KEY = "matvec_dots1_double"
 RESIDUAL_KEY = "circ_residual_df"
 DOMINANT_NAMES = {"k_fft4_inverseA_correct<4096, 32, 0>": "correction",
                   "k_matvec_fx<2, 0, 1, double, 0, 1, 16>": "matvec",
-                  "k_circ_residual_q<2, 0, float>": "residual"}
+                  "k_circ_residual_q<2, 0, float, 8>": "residual"}
 
 
 def _peaks():
