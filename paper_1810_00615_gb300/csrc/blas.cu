@@ -549,8 +549,9 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
     // block rows, and in a solve from x = 0 it is v0 (DK = 1) and v (DK = 2):
     // tiles where it is zero skip the products with it, one or two FP64
     // operations of the bound pipe per element.  A dense vector costs a vote
-    // on the tile's first step.  (unit <= 0 keeps the outputs finite, so that
-    // no 0 x inf is dropped.)
+    // on the tile's first step.  An output that is not finite (v may hold an inf
+    // or NaN, and the scale may overflow) makes w . w so too: the tile is then
+    // walked again with the products, since 0 x inf and 0 x NaN are NaN.
     if (full && in_range && unit <= 0) {
       const double *pz = (DK == 1 ? dv0 : sub) + first;
       auto nonzero = [](double a) { return (unsigned long long)__double_as_longlong(a) << 1; };
@@ -560,8 +561,13 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
         for (int r = 1; r < R; r++) any |= nonzero(__ldg(pz + r * step));
         if (!__any_sync(0xffffffffu, any != 0)) {
           walk(std::true_type{}, std::false_type{}, std::true_type{});
-          dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
-          return;
+          const int ww = __double2hiint(dacc[DK == 1 ? 2 : 1]) & 0x7ff00000;
+          if (!__any_sync(0xffffffffu, ww == 0x7ff00000)) {
+            dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
+            return;
+          }
+#pragma unroll
+          for (int q = 0; q < ND; q++) dacc[q] = 0.0;
         }
       }
     }
