@@ -188,8 +188,10 @@ k_fft4_forward1(const XT *__restrict__ x, const YT *__restrict__ y,
       if (lane == 31) g = h;
       const float k = __ldg(sg + (kFourT / 32) * L2 * u);
       float2 v = X2[r * W + lane];
-      v.x -= k * ((c.x + c.x) - l - c.y);
-      v.y -= k * ((c.y + c.y) - c.x - g);
+      // columns past n stay zero: the first has a live left neighbour, and for
+      // odd n it is the last column's partner in the packed transform
+      if (i0 + 2 * lane < n) v.x -= k * ((c.x + c.x) - l - c.y);
+      if (i0 + 2 * lane + 1 < n) v.y -= k * ((c.y + c.y) - c.x - g);
       X2[r * W + lane] = v;
     }
   }
