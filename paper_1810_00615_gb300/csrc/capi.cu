@@ -151,13 +151,20 @@ void build_rec_tables(const Ctx &c, int levels, const int *lsz,
   for (int64_t k0 = 0; k0 < c.nk; k0 += 4) {
     const int cnt = (int)std::min<int64_t>(4, c.nk - k0);
     zq sig = one, e = one;
+    // the block is scaled by a power of two to elements of order 1, so that the
+    // squares below neither overflow nor vanish (tau may be 1e-180); pivots
+    // scale with it, everything else is free of it
+    double scale[4];
     for (int u = 0; u < 4; u++) {
       cd cM, s0, e0;
       double cK;
       block_symbol(c, k0 + (u < cnt ? u : 0), cM, cK);
       excess_form(c, cM, cK, s0, e0);
-      sig.re[u] = s0.real(); sig.im[u] = s0.imag();
-      e.re[u] = e0.real(); e.im[u] = e0.imag();
+      const double big = std::max(std::max(std::fabs(s0.real()), std::fabs(s0.imag())),
+                                  std::max(std::fabs(e0.real()), std::fabs(e0.imag())));
+      scale[u] = big > 0.0 ? std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(big)))) : 1.0;
+      sig.re[u] = s0.real() * scale[u]; sig.im[u] = s0.imag() * scale[u];
+      e.re[u] = e0.real() * scale[u]; e.im[u] = e0.imag() * scale[u];
     }
     zq sig_l = sig, off_l = e;
     for (int l = 0; l < levels; l++) {
@@ -194,15 +201,17 @@ void build_rec_tables(const Ctx &c, int levels, const int *lsz,
       }
       for (int u = 0; u < cnt; u++) {
         auto &V = tabs[(size_t)(k0 + u) * (size_t)levels + (size_t)l];
-        auto at = [u](const zq &z) { return aao::mk((R)z.re[u], (R)z.im[u]); };
+        auto at = [u](const zq &z, double f) {
+          return aao::mk((R)(z.re[u] * f), (R)(z.im[u] * f));
+        };
         for (int i = 0; i < CH; i++) {
-          V.invp[i] = at(invp[i]);
-          V.invt[i] = at(invt[i]);
-          V.bp[i] = at(bp[i]);
-          V.fc[i] = at(fc[i]);
-          V.fl[i] = at(fl[i]);
+          V.invp[i] = at(invp[i], scale[u]);
+          V.invt[i] = at(invt[i], scale[u]);
+          V.bp[i] = at(bp[i], 1.0);
+          V.fc[i] = at(fc[i], 1.0);
+          V.fl[i] = at(fl[i], 1.0);
         }
-        V.e = at(e);
+        V.e = at(e, 1.0 / scale[u]);
       }
       const zq sw = e * sig * w[0];
       sig_l = fnms(sig - sw, e, wl[0]);
