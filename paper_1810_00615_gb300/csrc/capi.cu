@@ -1262,14 +1262,19 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
   if (st == AAO_OK) {
     std::vector<cx<float>> t32((size_t)ell);
     std::vector<cx<double>> t64((size_t)ell);
+    std::vector<float4> ts((size_t)ell);
     for (int64_t m = 0; m < ell; m++) {
       const double co = sinpi_q(4 * m + ell, 2 * ell);   // cos(2 pi m / ell)
       const double si = sinpi_q(2 * m, ell);             // sin(2 pi m / ell)
       t64[(size_t)m] = aao::mk(co, -si);
       t32[(size_t)m] = aao::mk((float)co, (float)-si);
+      ts[(size_t)m] = make_float4((float)co, (float)-si, (float)(co - (double)(float)co),
+                                  (float)((double)(float)si - si));
     }
     cudaError_t e = upload((void **)&c.tw32, t32);
     if (e == cudaSuccess) e = upload((void **)&c.tw64, t64);
+    if (e == cudaSuccess && c.step32.L) e = upload((void **)&c.tws32, ts);
+    c.step32.tw32 = c.tws32;
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c.host_small, kSmall * sizeof(double));
     if (e != cudaSuccess) st = fail_cuda(c, e, "create");
   }
@@ -1284,7 +1289,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
 void aao_destroy(aao_ctx *ctx) {
   if (!ctx) return;
   Ctx &c = ctx->c;
-  void *ptrs[] = {c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.beta, c.beta_p,
+  void *ptrs[] = {c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.tws32, c.beta, c.beta_p,
                   c.mv_rows, c.mv_rows_p, c.mv_d0, c.mv_o0,
                   c.sigk, c.sigk32, c.dtw32, c.dtw64, c.dst_cm32, c.dst_cm64,
                   c.dst_mk32, c.dst_mk64};

@@ -129,7 +129,7 @@ cudaError_t forward_any(int64_t ell, const StepPlan &pl, int64_t n, int64_t n_pa
       }
     }
   }
-  if (inter && pl.L) return steps_forward<R>(pl, n, n_pad, x, y, sigk, spec, tw, s, inter);
+  if (inter && pl.L) return steps_forward<R>(pl, n, n_pad, x, y, sigk, spec, step_table<R, -1>(pl, tw), s, inter);
   switch (ell) {
 #define AAO_F(L) case L: return run_forward<R, L, YT>(pl, n, n_pad, x, y, sigk, spec, tw, s, inter);
     AAO_FFT_CASES(AAO_F)
@@ -153,7 +153,7 @@ inline cudaError_t forward_four_f32_input(int64_t ell, const StepPlan &pl, int64
     }
   }
   if (!pl.L) return cudaErrorNotSupported;
-  return steps_forward<float>(pl, n, n_pad, x, none, none, spec, tw, s, inter);
+  return steps_forward<float>(pl, n, n_pad, x, none, none, spec, step_table<float, -1>(pl, tw), s, inter);
 }
 
 // Bytes of the four-step intermediate (0 where a single kernel serves).
@@ -182,7 +182,7 @@ cudaError_t inverse_any(int64_t ell, const StepPlan &pl, int64_t n, int64_t n_pa
       }
     }
   }
-  if (inter && pl.L) return steps_inverse<R, OT>(pl, n, n_pad, spec, y, tw, s, inter, base);
+  if (inter && pl.L) return steps_inverse<R, OT>(pl, n, n_pad, spec, y, step_table<R, +1>(pl, tw), s, inter, base);
   switch (ell) {
 #define AAO_I(L) case L: return run_inverse<R, L, OT>(pl, n, n_pad, spec, y, tw, s, inter, base);
     AAO_FFT_CASES(AAO_I)

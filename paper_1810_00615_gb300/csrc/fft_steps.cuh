@@ -39,7 +39,121 @@ constexpr int kStepT = 256, kStepW = 32, kStepWarps = kStepT / 32;
 // Resident CTAs per SM the kernels are compiled for.
 template <typename R> struct StepOcc { static constexpr int V = sizeof(R) == 8 ? 3 : 4; };
 
+// Twiddles.  The rounding errors of a table are the same in the forward and in
+// the inverse transform, and a four-step transform applies its middle twiddles
+// to whole classes of frequencies: with rounded tables on both sides their
+// product acts on the low frequencies that P^{-1} amplifies with one sign for
+// every input.  The refined apply lives on the product of two such errors and
+// was up to three times as far off as with one kernel per direction (1.27 times
+// over 287 sizes).  So the FP32 forward transform takes its twiddles and
+// constants with what their rounding left out (re, im, re lo, im lo of
+// e^{-2 pi i m/ell}): 0.59 times over the same sizes, no length above 1.02, for
+// 1.3% of the time (5% at n 2047 x ell 1440).  The inverse with full tables in
+// its place: 0.61, ell = 16 at 1.07; both: 0.54, for 2% (7%).
+template <typename R, int DIR> struct StepTw {
+  static constexpr bool FULL = sizeof(R) == 4 && DIR < 0;
+  using T = typename std::conditional<FULL, float4, cx<R>>::type;
+};
+template <typename R, int DIR> using step_tw = typename StepTw<R, DIR>::T;
+template <typename R, int DIR>
+inline const step_tw<R, DIR> *step_table(const StepPlan &pl, const cx<R> *tw) {
+  if constexpr (StepTw<R, DIR>::FULL) return pl.tw32;
+  else return tw;
+}
+
+template <typename R, int DIR>
+__device__ __forceinline__ cx<R> twiddle_step(cx<R> v, cx<R> w) {
+  return twiddle<R, DIR>(v, w);
+}
+template <typename R, int DIR>
+__device__ __forceinline__ cx<float> twiddle_step(cx<float> v, float4 w) {
+  constexpr float sg = DIR > 0 ? -1.f : 1.f;
+  const float c = w.x, d = sg * w.y, cl = w.z, dl = sg * w.w;
+  return mk(__fmaf_rn(v.re, c, __fmaf_rn(-v.im, d, __fmaf_rn(v.re, cl, -v.im * dl))),
+            __fmaf_rn(v.re, d, __fmaf_rn(v.im, c, __fmaf_rn(v.re, dl, v.im * cl))));
+}
+
 // ---- butterflies beyond fft_time.cuh's 2, 4, 8, 16 and fft_mixed.cuh's 3, 5
+// (refined apply at ell = 200 = 8 x 25, error against one kernel per direction:
+// 2.3 with rounded tables, 1.35 with full twiddles and rounded constants, 0.85)
+template <typename R, int DIR> __device__ __forceinline__ R const_fma(R x, double c, R y) {
+  if constexpr (StepTw<R, DIR>::FULL) {
+    const float h = (float)c, l = (float)(c - (double)h);
+    return __fmaf_rn(x, h, __fmaf_rn(x, l, y));
+  } else {
+    return fma(x, (R)c, y);
+  }
+}
+template <typename R, int DIR> __device__ __forceinline__ R const_mul(R x, double c) {
+  if constexpr (StepTw<R, DIR>::FULL) {
+    const float h = (float)c, l = (float)(c - (double)h);
+    return __fmaf_rn(x, h, x * l);
+  } else {
+    return x * (R)c;
+  }
+}
+// times e^{DIR i th}, c = cos th, s = sin th
+template <typename R, int DIR>
+__device__ __forceinline__ cx<R> const_rot(cx<R> z, double c, double s) {
+  if constexpr (StepTw<R, DIR>::FULL) {
+    const float ch = (float)c, sh = (float)s;
+    return twiddle_step<R, DIR>(z, make_float4(ch, -sh, (float)(c - (double)ch), (float)((double)sh - s)));
+  } else {
+    return twiddle_step<R, DIR>(z, mk((R)c, (R)-s));
+  }
+}
+
+template <typename R, int DIR>
+__device__ __forceinline__ void step_dft3(cx<R> *v) {
+  const double h = 0.86602540378443864676;   // sin(2 pi / 3)
+  const cx<R> s = v[1] + v[2], d = v[1] - v[2];
+  const cx<R> m = mk(v[0].re - (R)0.5 * s.re, v[0].im - (R)0.5 * s.im);
+  const cx<R> jd = rot90<R, DIR>(mk(const_mul<R, DIR>(d.re, h), const_mul<R, DIR>(d.im, h)));
+  v[0] = v[0] + s;
+  v[1] = m + jd;
+  v[2] = m - jd;
+}
+
+template <typename R, int DIR>
+__device__ __forceinline__ void step_dft5(cx<R> *v) {
+  const double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;   // cos(2pi/5), cos(4pi/5)
+  const double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;    // sin(2pi/5), sin(4pi/5)
+  const cx<R> t1 = v[1] + v[4], t2 = v[2] + v[3], t3 = v[1] - v[4], t4 = v[2] - v[3], x0 = v[0];
+  auto lin = [](cx<R> x, cx<R> p, double a, cx<R> q, double b) {   // x + a p + b q
+    return mk(const_fma<R, DIR>(q.re, b, const_fma<R, DIR>(p.re, a, x.re)), const_fma<R, DIR>(q.im, b, const_fma<R, DIR>(p.im, a, x.im)));
+  };
+  auto lin0 = [](cx<R> p, double a, cx<R> q, double b) {           // a p + b q
+    return mk(const_fma<R, DIR>(q.re, b, const_mul<R, DIR>(p.re, a)), const_fma<R, DIR>(q.im, b, const_mul<R, DIR>(p.im, a)));
+  };
+  const cx<R> a1 = lin(x0, t1, c1, t2, c2), a2 = lin(x0, t1, c2, t2, c1);
+  const cx<R> b1 = rot90<R, DIR>(lin0(t3, s1, t4, s2)), b2 = rot90<R, DIR>(lin0(t3, s2, t4, -s1));
+  v[0] = x0 + t1 + t2;
+  v[1] = a1 + b1;
+  v[4] = a1 - b1;
+  v[2] = a2 + b2;
+  v[3] = a2 - b2;
+}
+
+// 8 = 2 x 4: n = q + 2m, k = k1 + 4 k2
+template <typename R, int DIR>
+__device__ __forceinline__ void step_dft8(cx<R> *v) {
+  const double c8 = 0.70710678118654752440;   // cos(pi / 4)
+  cx<R> b[2][4];
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    b[q][0] = v[q]; b[q][1] = v[q + 2]; b[q][2] = v[q + 4]; b[q][3] = v[q + 6];
+    dft4<R, DIR>(b[q][0], b[q][1], b[q][2], b[q][3]);
+  }
+  b[1][1] = const_rot<R, DIR>(b[1][1], c8, c8);
+  b[1][2] = rot90<R, DIR>(b[1][2]);
+  b[1][3] = const_rot<R, DIR>(b[1][3], -c8, c8);
+#pragma unroll
+  for (int k1 = 0; k1 < 4; k1++) {
+    v[k1] = b[0][k1] + b[1][k1];
+    v[k1 + 4] = b[0][k1] - b[1][k1];
+  }
+}
+
 // 6 = 2 x 3 and 10 = 2 x 5 by the Good-Thomas index maps (no twiddles):
 // n = n1 M + 2 n2, k = M k1 + (M + 1) k2 mod 2M for M = 3, 5 (2^-1 mod M =
 // (M + 1)/2).
@@ -52,8 +166,11 @@ __device__ __forceinline__ void dft_2m(cx<R> *v) {
     a[0][q] = x0 + x1;
     a[1][q] = x0 - x1;
   }
-  dft_mixed<R, DIR, M>(a[0]);
-  dft_mixed<R, DIR, M>(a[1]);
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    if constexpr (M == 3) step_dft3<R, DIR>(a[q]);
+    else step_dft5<R, DIR>(a[q]);
+  }
 #pragma unroll
   for (int q = 0; q < M; q++) {
     v[((M + 1) * q) % (2 * M)] = a[0][q];
@@ -68,20 +185,19 @@ __device__ __forceinline__ void dft9(cx<R> *v) {
 #pragma unroll
   for (int q = 0; q < 3; q++) {
     a[q][0] = v[q]; a[q][1] = v[q + 3]; a[q][2] = v[q + 6];
-    dft3<R, DIR>(a[q]);
+    step_dft3<R, DIR>(a[q]);
   }
-  const R c1 = (R)0.76604444311897803520, s1 = (R)0.64278760968653932632;    // 2 pi / 9
-  const R c2 = (R)0.17364817766693034885, s2 = (R)0.98480775301220805937;    // 4 pi / 9
-  const R c4 = (R)-0.93969262078590838405, s4 = (R)0.34202014332566873304;   // 8 pi / 9
-  auto rot = [](cx<R> z, R c, R s) { const R d = DIR < 0 ? -s : s; return mk(z.re * c - z.im * d, z.re * d + z.im * c); };
-  a[1][1] = rot(a[1][1], c1, s1);
-  a[1][2] = rot(a[1][2], c2, s2);
-  a[2][1] = rot(a[2][1], c2, s2);
-  a[2][2] = rot(a[2][2], c4, s4);
+  const double c1 = 0.76604444311897803520, s1 = 0.64278760968653932632;    // 2 pi / 9
+  const double c2 = 0.17364817766693034885, s2 = 0.98480775301220805937;    // 4 pi / 9
+  const double c4 = -0.93969262078590838405, s4 = 0.34202014332566873304;   // 8 pi / 9
+  a[1][1] = const_rot<R, DIR>(a[1][1], c1, s1);
+  a[1][2] = const_rot<R, DIR>(a[1][2], c2, s2);
+  a[2][1] = const_rot<R, DIR>(a[2][1], c2, s2);
+  a[2][2] = const_rot<R, DIR>(a[2][2], c4, s4);
 #pragma unroll
   for (int k1 = 0; k1 < 3; k1++) {
     cx<R> b[3] = {a[0][k1], a[1][k1], a[2][k1]};
-    dft3<R, DIR>(b);
+    step_dft3<R, DIR>(b);
     v[k1] = b[0]; v[k1 + 3] = b[1]; v[k1 + 6] = b[2];
   }
 }
@@ -91,7 +207,10 @@ __device__ __forceinline__ void dft_step(cx<R> *v) {
   if constexpr (RAD == 6) dft_2m<R, DIR, 3>(v);
   else if constexpr (RAD == 10) dft_2m<R, DIR, 5>(v);
   else if constexpr (RAD == 9) dft9<R, DIR>(v);
-  else dft_mixed<R, DIR, RAD>(v);
+  else if constexpr (RAD == 3) step_dft3<R, DIR>(v);
+  else if constexpr (RAD == 5) step_dft5<R, DIR>(v);
+  else if constexpr (RAD == 8 && StepTw<R, DIR>::FULL) step_dft8<R, DIR>(v);
+  else dft<R, DIR, RAD>(v);
 }
 
 // q / d for 0 <= q < 512, 1 <= d <= 128 by a multiplication (exact: the error
@@ -106,7 +225,7 @@ struct SmallDiv {
 // at src + m N 32), out of place.  nmem N <= 256 rows in all.
 template <typename R, int DIR, int RAD>
 __device__ __forceinline__ void pass_step(const cx<R> *src, cx<R> *dst, int nmem, int N, int Ns,
-                                          int L, const cx<R> *__restrict__ tw) {
+                                          int L, const step_tw<R, DIR> *__restrict__ tw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nb = N / RAD, tot = nmem * nb, tstep = L / (Ns * RAD);
   const SmallDiv by_nb(nb), by_ns(Ns);
@@ -119,7 +238,7 @@ __device__ __forceinline__ void pass_step(const cx<R> *src, cx<R> *dst, int nmem
     for (int r = 0; r < RAD; r++) v[r] = s[r * nb * kStepW];
     if (jm) {
 #pragma unroll
-      for (int r = 1; r < RAD; r++) v[r] = twiddle<R, DIR>(v[r], tw[jm * tstep * r]);
+      for (int r = 1; r < RAD; r++) v[r] = twiddle_step<R, DIR>(v[r], tw[jm * tstep * r]);
     }
     dft_step<R, DIR, RAD>(v);
     cx<R> *d = dst + (m * N + jd * Ns * RAD + jm) * kStepW + lane;
@@ -133,7 +252,7 @@ __device__ __forceinline__ void pass_step(const cx<R> *src, cx<R> *dst, int nmem
 // result.  All threads call it; a barrier before it is the caller's.
 template <typename R, int DIR>
 __device__ __forceinline__ cx<R> *dft_steps(cx<R> *a, cx<R> *b, int nmem, int N, int np,
-                                            const int *rad, int L, const cx<R> *__restrict__ tw) {
+                                            const int *rad, int L, const step_tw<R, DIR> *__restrict__ tw) {
   int Ns = 1;
   for (int p = 0; p < np; p++) {
     const int r = rad[p];
@@ -158,7 +277,7 @@ constexpr int kStepB = 8;   // rows a warp keeps in flight
 template <typename R, typename XT, bool NEUMANN, typename YT>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_forward1(const XT *__restrict__ x, const YT *__restrict__ y, const R *__restrict__ sigk,
-                 cx<R> *__restrict__ inter, int n, int ncx, const cx<R> *__restrict__ tw,
+                 cx<R> *__restrict__ inter, int n, int ncx, const step_tw<R, -1> *__restrict__ tw,
                  StepPlan pl, int G) {
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
@@ -212,7 +331,7 @@ k_steps_forward1(const XT *__restrict__ x, const YT *__restrict__ y, const R *__
   for (int q = warp; q < rows; q += kStepWarps) {
     const int gi = by_l1(q), k1 = q - gi * L1, t2 = t20 + gi;
     cx<R> v = S[q * kStepW + lane];
-    if (t2 * k1) v = twiddle<R, -1>(v, tw[t2 * k1]);
+    if (t2 * k1) v = twiddle_step<R, -1>(v, tw[t2 * k1]);
     st_hint(inter + ((size_t)k1 * L2 + t2) * ncx + kStepW * blockIdx.x + lane, v, pol_keep);
   }
 }
@@ -244,7 +363,7 @@ template <bool MULTI> struct StepGroups {
 template <typename R, bool MULTI>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_forward2(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, int n, int ncx,
-                 int64_t n_pad, const cx<R> *__restrict__ tw, StepPlan pl, int G) {
+                 int64_t n_pad, const step_tw<R, -1> *__restrict__ tw, StepPlan pl, int G) {
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -295,7 +414,7 @@ k_steps_forward2(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, int 
 template <typename R, bool MULTI>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int n, int ncx,
-                 int64_t n_pad, const cx<R> *__restrict__ tw, StepPlan pl, int G) {
+                 int64_t n_pad, const step_tw<R, +1> *__restrict__ tw, StepPlan pl, int G) {
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -344,7 +463,7 @@ k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int 
     gr.row(q, k1, t2, qm);
     if (k1 < 0) continue;
     cx<R> v = S[q * kStepW + lane];
-    if (t2 * k1) v = twiddle<R, +1>(v, tw[t2 * k1]);
+    if (t2 * k1) v = twiddle_step<R, +1>(v, tw[t2 * k1]);
     st_hint(inter + ((size_t)k1 * pl.L2 + t2) * ncx + cb + lane, v, pol_keep);
   }
 }
@@ -354,7 +473,7 @@ k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int 
 template <typename R, typename OT>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int ncx,
-                 const cx<R> *__restrict__ tw, const float *__restrict__ base, StepPlan pl, int G) {
+                 const step_tw<R, +1> *__restrict__ tw, const float *__restrict__ base, StepPlan pl, int G) {
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<R> *S = reinterpret_cast<cx<R> *>(smraw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -508,7 +627,7 @@ inline int steps_group(int cols, int units, int unit) {
 
 template <typename R, typename XT, typename YT>
 cudaError_t steps_forward(const StepPlan &pl, int64_t n, int64_t n_pad, const XT *x, const YT *y, const R *sigk,
-                          cx<R> *spec, const cx<R> *tw, cudaStream_t s, void *inter) {
+                          cx<R> *spec, const step_tw<R, -1> *tw, cudaStream_t s, void *inter) {
   const int ncx = (int)steps_ncx(n), cols = ncx / kStepW;
   cx<R> *ip = static_cast<cx<R> *>(inter);
   const size_t row = kStepW * sizeof(cx<R>);
@@ -527,7 +646,7 @@ cudaError_t steps_forward(const StepPlan &pl, int64_t n, int64_t n_pad, const XT
 }
 
 template <typename R, typename OT>
-cudaError_t steps_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, const cx<R> *spec, OT *y, const cx<R> *tw,
+cudaError_t steps_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, const cx<R> *spec, OT *y, const step_tw<R, +1> *tw,
                           cudaStream_t s, void *inter, const float *base) {
   const int ncx = (int)steps_ncx(n), cols = ncx / kStepW;
   cx<R> *ip = static_cast<cx<R> *>(inter);
