@@ -432,7 +432,7 @@ struct StepPlan {
   int split;            // the row and panel kernels instead (powers of two)
   int np1, np2;
   int rad1[4], rad2[4];
-  const float4 *tw32;   // FP32: e^{-2 pi i m/ell} as (re, im, re lo, im lo)
+  const float4 *tw32;   // FP32: the full twiddles (Ctx::tws32)
 };
 
 // ------------------------------------------------------------ context
@@ -462,7 +462,7 @@ struct Ctx {
   StepPlan step32{}, step64{};    // run-time four-step transforms (set by fft_plan)
   cx<float> *tw32 = nullptr;      // exp(-2 pi i m/ell), m < ell
   cx<double> *tw64 = nullptr;
-  float4 *tws32 = nullptr;        // the same for step32: each entry and what its rounding left out
+  float4 *tws32 = nullptr;        // the same with what the rounding left out: (re, im, re lo, im lo)
   int space = AAO_SPACE_TRIDIAG;  // per-frequency solver
   cx<float> *dtw32 = nullptr;     // DST form: exp(-2 pi i m/(2(n+1))), m < 2(n+1)
   cx<double> *dtw64 = nullptr;

@@ -123,7 +123,7 @@ cudaError_t forward_any(int64_t ell, const StepPlan &pl, int64_t n, int64_t n_pa
   if (inter && use_four<R>(ell)) {
     if constexpr (std::is_same<R, float>::value) {
       switch (ell) {
-#define AAO_F(L) case L: return four_forward<L>(n, n_pad, x, y, sigk, spec, tw, s, inter);
+#define AAO_F(L) case L: return four_forward<L>(n, n_pad, x, y, sigk, spec, tw, pl.tw32, s, inter);
         AAO_FOUR_CASES(AAO_F)
 #undef AAO_F
       }
@@ -147,7 +147,7 @@ inline cudaError_t forward_four_f32_input(int64_t ell, const StepPlan &pl, int64
   const float *none = nullptr;
   if (use_four<float>(ell)) {
     switch (ell) {
-#define AAO_F(L) case L: return four_forward<L>(n, n_pad, x, none, none, spec, tw, s, inter);
+#define AAO_F(L) case L: return four_forward<L>(n, n_pad, x, none, none, spec, tw, pl.tw32, s, inter);
       AAO_FOUR_CASES(AAO_F)
 #undef AAO_F
     }

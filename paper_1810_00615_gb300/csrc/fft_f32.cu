@@ -73,12 +73,12 @@ cudaError_t fft_forward_f32_solve(const Ctx &c, const double *x, const float *x3
 #define AAO_FS(L)                                                                                 \
   case L:                                                                                         \
     if (x32)                                                                                      \
-      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x32, y32, c.sigk32, sp, sb, c.tw32, s,  \
+      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x32, y32, c.sigk32, sp, sb, c.tw32, c.tws32, s,  \
                                         inter, tb, tr, ragged, part, c.rec32, rb);                \
     if (y32)                                                                                      \
-      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y32, c.sigk32, sp, sb, c.tw32, s,    \
+      return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y32, c.sigk32, sp, sb, c.tw32, c.tws32, s,    \
                                         inter, tb, tr, ragged, part, c.rec32, rb);                \
-    return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y, c.sigk32, sp, sb, c.tw32, s, inter, \
+    return fft::four_forward_solve<L>(c.n, c.n_pad, P, x, y, c.sigk32, sp, sb, c.tw32, c.tws32, s, inter, \
                                       tb, tr, ragged, part, c.rec32, rb);
   switch (c.ell) {
     AAO_FOUR_CASES(AAO_FS)

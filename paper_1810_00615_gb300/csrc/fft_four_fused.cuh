@@ -470,7 +470,7 @@ k_fft4_inverseA_correct(const cx<float> *__restrict__ spec, const cx<float> *__r
 // in sepbuf: forward 1 (part 1), forward 2 + solves (part 2), or both (0).
 template <int L, typename XT, typename YT>
 cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *x, const YT *y,
-                               const float *sigk, cx<float> *spec, float4 *sepbuf, const cx<float> *tw, cudaStream_t s, void *inter,
+                               const float *sigk, cx<float> *spec, float4 *sepbuf, const cx<float> *tw, const float4 *twf, cudaStream_t s, void *inter,
                                const float4 *tabs, int conj, int ragged, int part = 0,
                                const void *rtab = nullptr, int rtab_bytes = 0) {
   constexpr int L1 = Four<L>::L1, W = kFourW;
@@ -479,7 +479,7 @@ cudaError_t four_forward_solve(int64_t n, int64_t n_pad, int nchunks, const XT *
   cx<float> *ip = static_cast<cx<float> *>(inter);
   cudaError_t e = cudaSuccess;
   if (part != 2) {
-    e = four_forward1<L>(n, x, y, sigk, tw, s, ip);
+    e = four_forward1<L>(n, x, y, sigk, tw, twf, s, ip);
     if (e != cudaSuccess) return e;
   }
   if (part != 1) {

@@ -67,10 +67,7 @@ __device__ __forceinline__ cx<R> twiddle_step(cx<R> v, cx<R> w) {
 }
 template <typename R, int DIR>
 __device__ __forceinline__ cx<float> twiddle_step(cx<float> v, float4 w) {
-  constexpr float sg = DIR > 0 ? -1.f : 1.f;
-  const float c = w.x, d = sg * w.y, cl = w.z, dl = sg * w.w;
-  return mk(__fmaf_rn(v.re, c, __fmaf_rn(-v.im, d, __fmaf_rn(v.re, cl, -v.im * dl))),
-            __fmaf_rn(v.re, d, __fmaf_rn(v.im, c, __fmaf_rn(v.re, dl, v.im * cl))));
+  return twiddle_full<DIR>(v, w);
 }
 
 // ---- butterflies beyond fft_time.cuh's 2, 4, 8, 16 and fft_mixed.cuh's 3, 5

@@ -36,6 +36,16 @@ __device__ __forceinline__ cx<R> twiddle(cx<R> v, cx<R> w) {
   return v * w;
 }
 
+// The same with a table entry that carries what its rounding left out
+// (re, im, re lo, im lo).
+template <int DIR>
+__device__ __forceinline__ cx<float> twiddle_full(cx<float> v, float4 w) {
+  constexpr float sg = DIR > 0 ? -1.f : 1.f;
+  const float c = w.x, d = sg * w.y, cl = w.z, dl = sg * w.w;
+  return mk(__fmaf_rn(v.re, c, __fmaf_rn(-v.im, d, __fmaf_rn(v.re, cl, -v.im * dl))),
+            __fmaf_rn(v.re, d, __fmaf_rn(v.im, c, __fmaf_rn(v.re, dl, v.im * cl))));
+}
+
 // multiply by DIR*i : forward (DIR = -1) -i, inverse +i
 template <typename R, int DIR>
 __device__ __forceinline__ cx<R> rot90(cx<R> a) {

@@ -1,10 +1,10 @@
 """The right-hand side x - E y of a Neumann term past the last column
 (csrc/fft_four.cuh): columns that a tile has beyond n stay zero, so that for
 an odd n they add nothing to the last column, whose partner they are in the
-packed transform.  The second term of Q_2^{-1} x is then, bit for bit, the
-plain FP32 apply of x - E y formed on the host: y is large at column n - 1
-alone, and the steps make sigma_t a power of two, so that sigma_t K y is exact
-and x - E y has one rounding."""
+packed transform.  The second term of Q_2^{-1} x is then, bit for bit, that of x
+- E y formed on the host with sigma = 0: y is large at column n - 1 alone, and
+the steps make sigma_t a power of two, so that sigma_t K y is exact and x - E y
+has one rounding."""
 import numpy as np
 import pytest
 
@@ -42,6 +42,8 @@ def test_second_term_is_the_apply_of_its_right_hand_side(n, ell, transpose):
     left, right = np.hstack([z, y32[:, :-1]]), np.hstack([y32[:, 1:], z])
     k = ((y32 + y32) - left) - right
     u = (X.astype(np.float32) - sig.astype(np.float32)[:, None] * k).astype(np.float32)
-    want = to_host(a.precond_apply(to_dev(torch, u.astype(np.float64)), transpose=transpose))
+    b = AllAtOnce(n, ell, tau, precision="fp32", restart=1)
+    b.set_steps(np.full(ell, tau))                             # sigma = 0, term by term
+    want = to_host(b.neumann_apply(to_dev(torch, u.astype(np.float64)), 2, transpose=transpose))
     got = to_host(a.neumann_apply(xd, 2, transpose=transpose))
     assert np.array_equal(got, want)
