@@ -98,8 +98,8 @@ typedef struct {
  * or 4096 chunks (n = 32767, 49151, 65535; other n give AAO_EUNSUPPORTED).
  * Computes the per-frequency
  * tridiagonal symbols A0 + w_k A1 (+ w_k^2 A2), w_k = exp(-2 pi i k/ell),
- * k = 0..ell/2 (Section 3, Fourier diagonalisation of P), in FP64 on the
- * host and uploads them; the context owns that device memory.
+ * k = 0..ell/2 (Section 3, Fourier diagonalisation of P), in FP64 and from
+ * them the tables of their solves on the device; the context owns that memory.
  * Defaults: kappa = 1, uniform steps, AAO_PREC_FP32.
  * Errors: AAO_EINVAL (n < 1, tau <= 0, bad equation, out == NULL),
  * AAO_EUNSUPPORTED (ell), AAO_ENOMEM, AAO_ECUDA. */

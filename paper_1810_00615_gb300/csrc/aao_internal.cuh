@@ -375,8 +375,8 @@ template <typename R, typename OT> __device__ __forceinline__ OT to_out(R v) {
 // sigma_L - e - o_L (excess sigma_L, virtual right coupling o_L; level 0 has
 // sigma_L = sigma, o_L = e): so any n >= 1 is served, and n + 1 a multiple of
 // CH at every level is the case in which the last chunk is like the others.
-// Everything here is per frequency k and RHS-independent, so the host
-// computes it once in FP64.  Zeros in the tables keep the device code free of
+// Everything here is per frequency k and RHS-independent, so it is computed
+// once, in FP64 (tables.cu).  Zeros in the tables keep the device code free of
 // lengths: invp[CH-1] = 0 clears a chunk's separator slot, invt and fl are
 // zero past the last chunk's end.
 constexpr int kRecLevels = 6;
@@ -391,6 +391,12 @@ struct RecLev {
   cx<R> pad;
 };
 // The table of frequency k is tab[k levels .. k levels + levels).
+
+// One frequency block as the tables are built from it: row excess and
+// off-diagonal, times the power of two `scale`.
+struct BlockSymbol {
+  double sig_re, sig_im, e_re, e_im, scale;
+};
 
 // Factor L1 of the four-step FP32 time transform, ell = L1 L2 (ell = 256 ...
 // 4096, L1 >= L2, both in {16, 32, 64}).
@@ -452,6 +458,7 @@ struct Ctx {
   int P32 = 1, P64 = 1;      // chunks per row
 
   // device-side constants (owned)
+  void *symbols = nullptr; // BlockSymbol[nk]
   void *rec32 = nullptr;   // RecLev<float, ch32>[nk][lev32]; the transposed symbols are their conjugates
   void *rec64 = nullptr;   // RecLev<double, ch64>[nk][lev64]
   void *fuse32 = nullptr;  // float4[kFusePairs(Ragged)][ell]: level-0 tables of the fused apply
@@ -593,6 +600,9 @@ cudaError_t fft_forward_f32_from_f32(const Ctx &c, const float *x, void *spec, c
                                      void *inter);
 cudaError_t fft_inverse_f32_to_f32(const Ctx &c, const void *spec, float *y, cudaStream_t s,
                                    void *inter = nullptr);
+// Build rec32, rec64 and fuse32 (sizes and level sizes set) from symbols.
+size_t rec_table_bytes(const Ctx &c, bool fp64);
+cudaError_t launch_build_tables(const Ctx &c, cudaStream_t s);
 cudaError_t launch_tridiag(const Ctx &c, void *spec, int prec, int transpose,
                            cudaStream_t s);
 // The FP32 apply with the tridiagonal solves folded into the four-step

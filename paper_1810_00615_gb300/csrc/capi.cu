@@ -85,142 +85,9 @@ void excess_form(const Ctx &c, const cd &cM, double cK, cd &sig, cd &e) {
   e = cM * (c.h / 6.0) - cd(cK / c.h, 0.0);
 }
 
-template <typename R>
-cx<R> to_cx(const cd &z) { return aao::mk((R)z.real(), (R)z.imag()); }
-
 // Chunks of a system of m unknowns with chunk length CH (CH-1 unknowns + one
 // separator, the last chunk 1 .. CH unknowns): the number of separators.
 int64_t separators(int64_t m, int CH) { return m >= CH + 1 ? (m - 1 - CH) / CH + 1 : 0; }
-
-// Four complex numbers, one per frequency.  The table construction is a chain
-// of about 2 CH dependent operations per level, so it runs four frequencies
-// side by side, in plain arithmetic: std::complex products and quotients
-// carry NaN and overflow recoveries that cost more than the arithmetic.
-struct zq {
-  double re[4], im[4];
-};
-template <class F>
-inline zq zmap(F &&f) {
-  zq z;
-  for (int u = 0; u < 4; u++) f(u, z.re[u], z.im[u]);
-  return z;
-}
-inline zq operator-(const zq &a, const zq &b) {
-  return zmap([&](int u, double &r, double &i) { r = a.re[u] - b.re[u]; i = a.im[u] - b.im[u]; });
-}
-inline zq operator*(const zq &a, const zq &b) {
-  return zmap([&](int u, double &r, double &i) {
-    r = a.re[u] * b.re[u] - a.im[u] * b.im[u];
-    i = a.re[u] * b.im[u] + a.im[u] * b.re[u];
-  });
-}
-inline zq fnms(const zq &a, const zq &b, const zq &c) {   // a - b c
-  return zmap([&](int u, double &r, double &i) {
-    r = a.re[u] - b.re[u] * c.re[u] + b.im[u] * c.im[u];
-    i = a.im[u] - b.re[u] * c.im[u] - b.im[u] * c.re[u];
-  });
-}
-inline zq recip(const zq &a) {
-  return zmap([&](int u, double &r, double &i) {
-    const double d = 1.0 / (a.re[u] * a.re[u] + a.im[u] * a.im[u]);
-    r = a.re[u] * d;
-    i = -a.im[u] * d;
-  });
-}
-
-// Tables of the recursive form (aao_internal.cuh, RecLev), all in FP64.
-// Level l is the system (sigma, e) with last-row excess sigma_L and virtual
-// right coupling o_L, so its last diagonal is sigma_L - e - o_L.
-//   pivots in excess form: q_0 = sigma - e, q_i = sigma - e q_{i-1}/p_{i-1},
-//     p_i = q_i - e; the last row: q = sigma_L - e q/p (sigma_L - e alone),
-//     p = q - o_L;
-//   Green's functions g = T_c^{-1} e_1 (regular chunk), gl (last chunk), and
-//     w = T_c^{-1} (sigma 1), wl = Tlast^{-1} (sigma, ..., sigma, sigma_L):
-//     1 + e (g_0 + g_{c-1}) = w_0 and 1 + e gl_0 + o_L gl_{cl-1} = wl_0, so
-//     the separators' excesses sigma - 2 e w_0 and sigma - e w_0 - e wl_0
-//     come without cancellation;
-//   level l+1: off-diagonal -e^2 g_{c-1}, virtual coupling -e o_L gl_{cl-1}.
-template <typename R, int CH>
-void build_rec_tables(const Ctx &c, int levels, const int *lsz,
-                      std::vector<aao::RecLev<R, CH>> &tabs) {
-  tabs.assign((size_t)c.nk * (size_t)levels, aao::RecLev<R, CH>{});
-  constexpr int cr = CH - 1;
-  const zq zero = zmap([](int, double &r, double &i) { r = i = 0.0; });
-  const zq one = zmap([](int, double &r, double &i) { r = 1.0; i = 0.0; });
-  zq invp[CH], bp[CH], invt[CH], g[CH], w[CH], gl[CH], wl[CH], fc[CH], fl[CH];
-  for (int64_t k0 = 0; k0 < c.nk; k0 += 4) {
-    const int cnt = (int)std::min<int64_t>(4, c.nk - k0);
-    zq sig = one, e = one;
-    // the block is scaled by a power of two to elements of order 1, so that the
-    // squares below neither overflow nor vanish (tau may be 1e-180); pivots
-    // scale with it, everything else is free of it
-    double scale[4];
-    for (int u = 0; u < 4; u++) {
-      cd cM, s0, e0;
-      double cK;
-      block_symbol(c, k0 + (u < cnt ? u : 0), cM, cK);
-      excess_form(c, cM, cK, s0, e0);
-      const double big = std::max(std::max(std::fabs(s0.real()), std::fabs(s0.imag())),
-                                  std::max(std::fabs(e0.real()), std::fabs(e0.imag())));
-      scale[u] = big > 0.0 ? std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(big)))) : 1.0;
-      sig.re[u] = s0.real() * scale[u]; sig.im[u] = s0.imag() * scale[u];
-      e.re[u] = e0.real() * scale[u]; e.im[u] = e0.imag() * scale[u];
-    }
-    zq sig_l = sig, off_l = e;
-    for (int l = 0; l < levels; l++) {
-      const int M = l + 1 < levels ? lsz[l + 1] : 0;   // separators
-      const int cl = lsz[l] - M * CH;                  // unknowns of the last chunk
-      zq q = sig - e, qp = zero;
-      for (int i = 0; i < CH; i++) {
-        if (i > 0) q = fnms(sig, e, q * invp[i - 1]);
-        invp[i] = recip(q - e);
-        bp[i] = e * invp[i];
-        if (i == cl - 2) qp = q * invp[i];
-      }
-      for (int i = 0; i < CH; i++) invt[i] = i < cl - 1 ? invp[i] : zero;
-      invt[cl - 1] = recip((cl == 1 ? sig_l - e : fnms(sig_l, e, qp)) - off_l);
-      invp[cr] = zero;   // a chunk has CH-1 unknowns: its separator slot stays zero
-      g[0] = w[0] = invp[0];
-      gl[0] = invt[0];
-      wl[0] = (cl == 1 ? sig_l : sig) * invt[0];
-      for (int i = 1; i < CH; i++) {
-        g[i] = fnms(zero, e, g[i - 1]) * invp[i];
-        w[i] = fnms(one, e, w[i - 1]) * invp[i];
-        gl[i] = fnms(zero, e, gl[i - 1]) * invt[i];
-        wl[i] = fnms(i < cl - 1 ? sig : sig_l, e, wl[i - 1]) * invt[i];
-      }
-      for (int i = CH - 2; i >= 0; i--) {
-        g[i] = fnms(g[i], bp[i], g[i + 1]);
-        w[i] = fnms(w[i], bp[i], w[i + 1]);
-        gl[i] = fnms(gl[i], bp[i], gl[i + 1]);
-        wl[i] = fnms(wl[i], bp[i], wl[i + 1]);
-      }
-      for (int i = 0; i < CH; i++) {
-        fc[i] = fnms(zero, e, g[i]);
-        fl[i] = fnms(zero, e, gl[i]);
-      }
-      for (int u = 0; u < cnt; u++) {
-        auto &V = tabs[(size_t)(k0 + u) * (size_t)levels + (size_t)l];
-        auto at = [u](const zq &z, double f) {
-          return aao::mk((R)(z.re[u] * f), (R)(z.im[u] * f));
-        };
-        for (int i = 0; i < CH; i++) {
-          V.invp[i] = at(invp[i], scale[u]);
-          V.invt[i] = at(invt[i], scale[u]);
-          V.bp[i] = at(bp[i], 1.0);
-          V.fc[i] = at(fc[i], 1.0);
-          V.fl[i] = at(fl[i], 1.0);
-        }
-        V.e = at(e, 1.0 / scale[u]);
-      }
-      const zq sw = e * sig * w[0];
-      sig_l = fnms(sig - sw, e, wl[0]);
-      sig = sig - sw - sw;
-      off_l = fnms(zero, e * off_l, gl[cl - 1]);
-      e = fnms(zero, e * e, g[cr - 1]);
-    }
-  }
-}
 
 // Level sizes of the recursive form.
 int rec_levels(int64_t n, int CH, int *lsz) {
@@ -248,10 +115,16 @@ void choose_form(int64_t n, int CH, size_t elem, int tpb, int &lev, int *lsz, in
   }
 }
 
+// Device memory for a constant, in place of what it had (cudaFree waits for
+// every kernel that may still read it).
+cudaError_t reserve(void **dst, size_t bytes) {
+  if (*dst) { cudaFree(*dst); *dst = nullptr; }
+  return cudaMalloc(dst, bytes);
+}
+
 template <typename T>
 cudaError_t upload(void **dst, const std::vector<T> &v) {
-  if (*dst) { cudaFree(*dst); *dst = nullptr; }
-  cudaError_t e = cudaMalloc(dst, v.size() * sizeof(T));
+  cudaError_t e = reserve(dst, v.size() * sizeof(T));
   if (e != cudaSuccess) return e;
   return cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
@@ -374,50 +247,35 @@ cudaError_t upload_dst_tables(Ctx &c) {
 
 // (Re)compute everything that depends on kappa, the steps or tau.
 int refresh_constants(Ctx &c) {
-  // per-frequency tridiagonal tables
+  // per-frequency tridiagonal tables (tables.cu): the symbols here, scaled to
+  // elements of order 1, the recursion on the device
   c.P32 = (int)separators(c.n, c.ch32) + 1;
   c.P64 = (int)separators(c.n, c.ch64) + 1;
   choose_form(c.n, c.ch32, sizeof(cx<float>), 1024, c.lev32, c.lsz32, c.clu32, c.cta32);
-  {
-    std::vector<aao::RecLev<float, 16>> r32;
-    build_rec_tables<float, 16>(c, c.lev32, c.lsz32, r32);
-    AAO_CK(c, upload(&c.rec32, r32));
-    // level 0 again, in the layout of the fused four-step apply
-    if (c.lev32 >= 2 && c.ell >= 256 && c.ell <= 4096 && (c.ell & (c.ell - 1)) == 0) {
-      const int64_t L1 = aao::four_l1(c.ell), L2 = c.ell / L1;
-      const bool ragged = (c.n + 1) % 16 != 0;
-      const int pairs = ragged ? aao::kFusePairsRagged : aao::kFusePairs;
-      std::vector<float4> ft((size_t)pairs * (size_t)c.ell, make_float4(0, 0, 0, 0));
-      auto pack = [](const cx<float> &a, const cx<float> &b) {
-        return make_float4(a.re, a.im, b.re, b.im);
-      };
-      for (int64_t k = 0; k < c.nk; k++) {
-        const auto &T = r32[(size_t)k * (size_t)c.lev32];
-        const size_t pos = (size_t)((k % L1) * L2 + k / L1);
-        auto at = [&](int j) -> float4 & { return ft[(size_t)j * (size_t)c.ell + pos]; };
-        for (int j = 0; j < 7; j++) at(j) = pack(T.invp[2 * j], T.invp[2 * j + 1]);
-        at(7) = pack(T.invp[14], T.e);
-        for (int j = 0; j < 7; j++) at(8 + j) = pack(T.bp[2 * j], T.bp[2 * j + 1]);
-        for (int j = 0; j < 7; j++) at(15 + j) = pack(T.fc[2 * j], T.fc[2 * j + 1]);
-        at(22) = pack(T.fc[14], T.bp[14]);
-        for (int j = 0; ragged && j < 8; j++) {
-          at(aao::kFuseTailInv + j) = pack(T.invt[2 * j], T.invt[2 * j + 1]);
-          at(aao::kFuseTailGreen + j) = pack(T.fl[2 * j], T.fl[2 * j + 1]);
-        }
-      }
-      AAO_CK(c, upload(&c.fuse32, ft));
-    }
-  }
   choose_form(c.n, c.ch64, sizeof(cx<double>), 512, c.lev64, c.lsz64, c.clu64, c.cta64);
-  if (c.ch64 == 8) {
-    std::vector<aao::RecLev<double, 8>> r64;
-    build_rec_tables<double, 8>(c, c.lev64, c.lsz64, r64);
-    AAO_CK(c, upload(&c.rec64, r64));
-  } else {
-    std::vector<aao::RecLev<double, 16>> r64;
-    build_rec_tables<double, 16>(c, c.lev64, c.lsz64, r64);
-    AAO_CK(c, upload(&c.rec64, r64));
+  std::vector<aao::BlockSymbol> sym((size_t)c.nk);
+  for (int64_t k = 0; k < c.nk; k++) {
+    cd cM, s0, e0;
+    double cK;
+    block_symbol(c, k, cM, cK);
+    excess_form(c, cM, cK, s0, e0);
+    const double big = std::max(std::max(std::fabs(s0.real()), std::fabs(s0.imag())),
+                                std::max(std::fabs(e0.real()), std::fabs(e0.imag())));
+    const double f =
+        big > 0.0 ? std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(big)))) : 1.0;
+    sym[(size_t)k] = {s0.real() * f, s0.imag() * f, e0.real() * f, e0.imag() * f, f};
   }
+  AAO_CK(c, upload(&c.symbols, sym));
+  AAO_CK(c, reserve(&c.rec32, aao::rec_table_bytes(c, false)));
+  AAO_CK(c, reserve(&c.rec64, aao::rec_table_bytes(c, true)));
+  // level 0 again, in the layout of the fused four-step apply
+  if (c.lev32 >= 2 && c.ell >= 256 && c.ell <= 4096 && (c.ell & (c.ell - 1)) == 0) {
+    const int pairs = (c.n + 1) % 16 != 0 ? aao::kFusePairsRagged : aao::kFusePairs;
+    const size_t bytes = (size_t)pairs * (size_t)c.ell * sizeof(float4);
+    AAO_CK(c, reserve(&c.fuse32, bytes));
+    AAO_CK(c, cudaMemsetAsync(c.fuse32, 0, bytes, nullptr));
+  }
+  AAO_CK(c, aao::launch_build_tables(c, nullptr));
   // DST-in-space form: cM_k per frequency, (m_j, cK k_j) per mode
   if (c.space == AAO_SPACE_DST) AAO_CK(c, upload_dst_tables(c));
   // matvec K coefficients beta_t and Neumann coefficients (tau_t - tau) kappa / h
@@ -463,14 +321,12 @@ int refresh_constants(Ctx &c) {
       sk32[(size_t)t] = (float)sk[(size_t)t];
     }
   }
-  AAO_CK(c, upload((void **)&c.beta, beta));
   // K coefficient of the circulant P (Section 3): the constant-step blocks
   std::vector<double> beta_p((size_t)c.ell,
                              c.equation == AAO_WAVE_BD2 || c.equation == AAO_WAVE_BD4
                                                               ? c.tau * c.tau / c.h
                              : c.equation == AAO_HEAT_LITERAL ? 1.0 / c.h
                                                               : c.tau * c.kappa / c.h);
-  AAO_CK(c, upload((void **)&c.beta_p, beta_p));
   // the same circulant's stencil per time lag, FP32 hi + lo pairs
   {
     const double bp = beta_p.empty() ? 0.0 : beta_p[0];
@@ -519,14 +375,17 @@ int refresh_constants(Ctx &c) {
   AAO_CK(c, upload((void **)&c.mv_rows_p, rows_p));
   AAO_CK(c, upload((void **)&c.mv_d0, d0));
   AAO_CK(c, upload((void **)&c.mv_o0, o0));
+  AAO_CK(c, upload((void **)&c.beta, beta));
+  AAO_CK(c, upload((void **)&c.beta_p, beta_p));
+  AAO_CK(c, upload((void **)&c.sigk, sk));
+  AAO_CK(c, upload((void **)&c.sigk32, sk32));
   // A1 = -M (heat) or -2M (BD2), A2 = M (BD2)
   const double a1 = (c.equation == AAO_WAVE_BD2) ? -2.0 : -1.0;
   c.mv_d1 = a1 * 4 * mh;
   c.mv_o1 = a1 * mh;
   c.mv_d2 = (c.equation == AAO_WAVE_BD2) ? 4 * mh : 0.0;
   c.mv_o2 = (c.equation == AAO_WAVE_BD2) ? mh : 0.0;
-  AAO_CK(c, upload((void **)&c.sigk, sk));
-  AAO_CK(c, upload((void **)&c.sigk32, sk32));
+  AAO_CK(c, cudaStreamSynchronize(nullptr));   // the tables stand for every stream
   return AAO_OK;
 }
 
@@ -1289,7 +1148,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
 void aao_destroy(aao_ctx *ctx) {
   if (!ctx) return;
   Ctx &c = ctx->c;
-  void *ptrs[] = {c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.tws32, c.beta, c.beta_p,
+  void *ptrs[] = {c.symbols, c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.tws32, c.beta, c.beta_p,
                   c.mv_rows, c.mv_rows_p, c.mv_d0, c.mv_o0,
                   c.sigk, c.sigk32, c.dtw32, c.dtw64, c.dst_cm32, c.dst_cm64,
                   c.dst_mk32, c.dst_mk64};
