@@ -477,6 +477,7 @@ struct Ctx {
   void *dst_cm64 = nullptr;
   void *dst_mk32 = nullptr;       // (m_j, cK k_j) per mode j = 1..n (same forms)
   void *dst_mk64 = nullptr;
+  void *per_step = nullptr;       // one buffer for the arrays below, beta ... sigk32
   double *beta = nullptr;         // per-step K coefficient tau_t kappa / h (ell)
   double *beta_p = nullptr;       // K coefficient of the circulant P (constant step) (ell)
   struct MvRow *mv_rows = nullptr;     // fixed-point matvec: per-step combination of A

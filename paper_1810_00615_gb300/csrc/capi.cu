@@ -115,11 +115,18 @@ void choose_form(int64_t n, int CH, size_t elem, int tpb, int &lev, int *lsz, in
   }
 }
 
-// Device memory for a constant, in place of what it had (cudaFree waits for
-// every kernel that may still read it).
+// Device memory for a constant.  Its size follows from n and ell, so a context
+// allocates it once.
 cudaError_t reserve(void **dst, size_t bytes) {
-  if (*dst) { cudaFree(*dst); *dst = nullptr; }
-  return cudaMalloc(dst, bytes);
+  return *dst ? cudaSuccess : cudaMalloc(dst, bytes);
+}
+
+// Frees a buffer.  cudaFree returns when every kernel that may still read it, or
+// any other constant, is done (a device synchronisation would do as well, but
+// is refused while another thread captures a stream).
+void drop(void **p) {
+  if (*p) cudaFree(*p);
+  *p = nullptr;
 }
 
 template <typename T>
@@ -236,6 +243,7 @@ cudaError_t upload_dst_tables(Ctx &c) {
     split(mj, q.x, q.y);
     split(cK * kj, q.z, q.w);
   }
+  drop(&c.dst_cm32);   // written in place from here on
   cudaError_t e = upload((void **)&c.dtw32, tw32);
   if (e == cudaSuccess) e = upload((void **)&c.dtw64, tw64);
   if (e == cudaSuccess) e = upload(&c.dst_cm32, cm32);
@@ -265,6 +273,7 @@ int refresh_constants(Ctx &c) {
         big > 0.0 ? std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(big)))) : 1.0;
     sym[(size_t)k] = {s0.real() * f, s0.imag() * f, e0.real() * f, e0.imag() * f, f};
   }
+  drop(&c.symbols);   // the constants are written in place from here on
   AAO_CK(c, upload(&c.symbols, sym));
   AAO_CK(c, reserve(&c.rec32, aao::rec_table_bytes(c, false)));
   AAO_CK(c, reserve(&c.rec64, aao::rec_table_bytes(c, true)));
@@ -371,14 +380,25 @@ int refresh_constants(Ctx &c) {
     rows_a[(size_t)t] = mvrow(beta[(size_t)t]);
     rows_p[(size_t)t] = mvrow(beta_p[(size_t)t]);
   }
-  AAO_CK(c, upload((void **)&c.mv_rows, rows_a));
-  AAO_CK(c, upload((void **)&c.mv_rows_p, rows_p));
-  AAO_CK(c, upload((void **)&c.mv_d0, d0));
-  AAO_CK(c, upload((void **)&c.mv_o0, o0));
-  AAO_CK(c, upload((void **)&c.beta, beta));
-  AAO_CK(c, upload((void **)&c.beta_p, beta_p));
-  AAO_CK(c, upload((void **)&c.sigk, sk));
-  AAO_CK(c, upload((void **)&c.sigk32, sk32));
+  // everything per step in one buffer and one copy
+  std::vector<char> host;
+  std::vector<std::pair<void **, size_t>> places;
+  auto put = [&](auto **dst, const auto &v) {
+    places.emplace_back((void **)dst, host.size());
+    const size_t bytes = v.size() * sizeof(v[0]);
+    host.resize(host.size() + round_up(bytes, kAlign));
+    std::memcpy(host.data() + places.back().second, v.data(), bytes);
+  };
+  put(&c.beta, beta);
+  put(&c.beta_p, beta_p);
+  put(&c.mv_rows, rows_a);
+  put(&c.mv_rows_p, rows_p);
+  put(&c.mv_d0, d0);
+  put(&c.mv_o0, o0);
+  put(&c.sigk, sk);
+  put(&c.sigk32, sk32);
+  AAO_CK(c, upload(&c.per_step, host));
+  for (auto &p : places) *p.first = static_cast<char *>(c.per_step) + p.second;
   // A1 = -M (heat) or -2M (BD2), A2 = M (BD2)
   const double a1 = (c.equation == AAO_WAVE_BD2) ? -2.0 : -1.0;
   c.mv_d1 = a1 * 4 * mh;
@@ -1148,9 +1168,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
 void aao_destroy(aao_ctx *ctx) {
   if (!ctx) return;
   Ctx &c = ctx->c;
-  void *ptrs[] = {c.symbols, c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.tws32, c.beta, c.beta_p,
-                  c.mv_rows, c.mv_rows_p, c.mv_d0, c.mv_o0,
-                  c.sigk, c.sigk32, c.dtw32, c.dtw64, c.dst_cm32, c.dst_cm64,
+  void *ptrs[] = {c.symbols, c.rec32, c.rec64, c.fuse32, c.tw32, c.tw64, c.tws32, c.per_step, c.dtw32, c.dtw64, c.dst_cm32, c.dst_cm64,
                   c.dst_mk32, c.dst_mk64};
   for (void *p : ptrs)
     if (p) cudaFree(p);

@@ -32,6 +32,11 @@
 // an instruction.  So a block takes one level, and walks the levels below it
 // for itself, and one of two roles: what belongs to the regular chunks, or to
 // the last one.
+// aao_set_kappa, the one allocation and the copies around it included: n 63 x
+// ell 64 175 us (with all levels of a role in one thread 268; tables built and
+// copied by the host 121, by the host before the recursion served every row
+// 229), n 5000 x ell 300 371 (542, 406, 307), n 1000 x ell 900 310 (463, 944,
+// 698), n 12345 x ell 4096 678 (890, 7089, 3599).
 #include "aao_internal.cuh"
 
 namespace aao {
