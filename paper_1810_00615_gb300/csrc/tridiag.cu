@@ -415,6 +415,11 @@ k_tridiag_reduced(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ sep
 // sweep, and every lane corrects its chunk with the two level-2 values
 // around it.  No level buffer round trips: the chain of dependent steps is
 // two Thomas sweeps.
+// It does not let its successor be scheduled early: the correction kernel's CTAs
+// then wait beside it, and what a wait costs at the end is more than the prologue
+// they save (FP32 apply, with / without: n 255 x ell 4096 31.2 / 24.2 us, 127 x
+// 4096 29.7 / 20.6, 511 x 4096 39.4 / 34.2, 1023 x 1024 22.1 / 19.6; before this
+// kernel served two levels 28.7, 24.6, 40.2, 21.6).
 template <int CH>
 __global__ void __launch_bounds__(256)
 k_tridiag_reduced3(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ sep,
@@ -452,7 +457,6 @@ k_tridiag_reduced3(const float4 *__restrict__ sepbuf, cx<float> *__restrict__ se
     if (own && q0 + j <= M1) a[j] = row[q0 + j];
   }
   if (own && q0 + CH <= M1) nxt = *reinterpret_cast<const float2 *>(row + q0 + CH);
-  pdl_trigger();
   {
     const float sg = conj_sym ? -1.f : 1.f;   // every entry is complex: (re, im) pairs
     float4 *dst = reinterpret_cast<float4 *>(&s_tab[w][0]);
