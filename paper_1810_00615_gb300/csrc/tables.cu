@@ -32,34 +32,30 @@
 // an instruction.  So a block takes one level, and walks the levels below it
 // for itself, and one of two roles: what belongs to the regular chunks, or to
 // the last one.
-// aao_set_kappa, the one allocation and the copies around it included: n 63 x
-// ell 64 175 us (with all levels of a role in one thread 268; tables built and
-// copied by the host 121, by the host before the recursion served every row
-// 229), n 5000 x ell 300 371 (542, 406, 307), n 1000 x ell 900 310 (463, 944,
-// 698), n 12345 x ell 4096 678 (890, 7089, 3599).
+// aao_set_kappa with its copies, against the host building the tables, and the
+// host before the recursion served every row: n 63 x ell 64 153 us (124, 229), n
+// 5000 x ell 300 279 (395, 300), n 1000 x ell 900 238 (934, 679), n 12345 x ell 4096
+// 726 (6867, 3535).  With a lane a frequency it was 175, 371, 310 and 678; with all
+// levels of a role in one thread besides 268, 542, 463 and 890.
 #include "aao_internal.cuh"
 
 namespace aao {
 namespace {
 
+// A complex number is held by two lanes, the even one its real and the odd one
+// its imaginary part: half the instructions for a warp to issue.  All lanes take
+// part in every operation.
 template <typename E> struct zc {
-  E re, im;
+  E v;
 };
-using zd = zc<double>;
+__device__ __forceinline__ bool imag() { return threadIdx.x & 1; }
+__device__ __forceinline__ double other(double a) { return __shfl_xor_sync(0xffffffffu, a, 1); }
 __device__ __forceinline__ double lead(double a) { return a; }
-__device__ __forceinline__ zd zadd(zd a, zd b) { return {a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ zd zsub(zd a, zd b) { return {a.re - b.re, a.im - b.im}; }
-__device__ __forceinline__ zd zneg(zd a) { return {-a.re, -a.im}; }
-__device__ __forceinline__ zd zmul(zd a, zd b) {
-  return {fma(a.re, b.re, -a.im * b.im), fma(a.re, b.im, a.im * b.re)};
-}
-__device__ __forceinline__ zd zfma(zd a, zd b, zd c) {   // a b + c
-  return {fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im))};
-}
-__device__ __forceinline__ zd zrecip(zd a) {
-  const double d = fma(a.re, a.re, a.im * a.im);
-  return {a.re / d, -a.im / d};
-}
+__device__ __forceinline__ double neg(double a) { return -a; }
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ double mul(double a, double b) { return a * b; }
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double recip(double a) { return 1.0 / a; }
 
 // Pairs: unevaluated sums h + l of two FP64 numbers, |l| at most half a unit of
 // h (Dekker; products split by FMA).  Rounded operations throughout: a
@@ -70,75 +66,79 @@ struct pair {
   __device__ __forceinline__ explicit pair(double a) : h(a), l(0.0) {}
   __device__ __forceinline__ pair(double a, double b) : h(a), l(b) {}
 };
-using zp = zc<pair>;
+__device__ __forceinline__ pair other(pair a) { return {other(a.h), other(a.l)}; }
 __device__ __forceinline__ double lead(pair a) { return a.h; }
 __device__ __forceinline__ pair neg(pair a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ pair tidy(pair a) {                      // |h| >= |l|
-  const double s = __dadd_rn(a.h, a.l);
-  return {s, __dsub_rn(a.l, __dsub_rn(s, a.h))};
+__device__ __forceinline__ pair tidy(double h, double l) {           // |h| >= |l|
+  const double s = __dadd_rn(h, l);
+  return {s, __dsub_rn(l, __dsub_rn(s, h))};
 }
-// a + (b, c) and a + x y, left untidy
-__device__ __forceinline__ pair plus(pair a, double b, double c) {
-  const double s = __dadd_rn(a.h, b), t = __dsub_rn(s, a.h);
-  const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, t)), __dsub_rn(b, t));
-  return {s, __dadd_rn(a.l, __dadd_rn(e, c))};
+__device__ __forceinline__ pair add(pair a, pair b) {
+  const double s = __dadd_rn(a.h, b.h), t = __dsub_rn(s, a.h);
+  const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, t)), __dsub_rn(b.h, t));
+  return tidy(s, __dadd_rn(a.l, __dadd_rn(e, b.l)));
 }
-__device__ __forceinline__ pair plus(pair a, pair x, pair y) {
-  const double p = __dmul_rn(x.h, y.h);
-  return plus(a, p, __fma_rn(x.l, y.h, __fma_rn(x.h, y.l, __fma_rn(x.h, y.h, -p))));
+__device__ __forceinline__ pair mul(pair a, pair b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return tidy(p, __fma_rn(a.l, b.h, __fma_rn(a.h, b.l, __fma_rn(a.h, b.h, -p))));
 }
-__device__ __forceinline__ pair mul(pair x, pair y) {
-  const double p = __dmul_rn(x.h, y.h);
-  return {p, __fma_rn(x.l, y.h, __fma_rn(x.h, y.l, __fma_rn(x.h, y.h, -p)))};
-}
-__device__ __forceinline__ zp zadd(zp a, zp b) {
-  return {tidy(plus(a.re, b.re.h, b.re.l)), tidy(plus(a.im, b.im.h, b.im.l))};
-}
-__device__ __forceinline__ zp zneg(zp a) { return {neg(a.re), neg(a.im)}; }
-__device__ __forceinline__ zp zsub(zp a, zp b) { return zadd(a, zneg(b)); }
-__device__ __forceinline__ zp zmul(zp a, zp b) {
-  return {tidy(plus(mul(a.re, b.re), neg(a.im), b.im)), tidy(plus(mul(a.re, b.im), a.im, b.re))};
-}
-__device__ __forceinline__ zp zfma(zp a, zp b, zp c) {
-  return {tidy(plus(plus(c.re, a.re, b.re), neg(a.im), b.im)),
-          tidy(plus(plus(c.im, a.re, b.im), a.im, b.re))};
-}
-__device__ __forceinline__ zp zrecip(zp a) {
-  const pair d = tidy(plus(mul(a.re, a.re), a.im, a.im));
-  const double r = 1.0 / d.h;
-  const pair inv = tidy({r, __dmul_rn(r, __fma_rn(-d.l, r, __fma_rn(-d.h, r, 1.0)))});
-  return {tidy(mul(a.re, inv)), tidy(neg(mul(a.im, inv)))};
+__device__ __forceinline__ pair fmadd(pair a, pair b, pair c) { return add(mul(a, b), c); }
+__device__ __forceinline__ pair recip(pair a) {
+  const double r = 1.0 / a.h;
+  return tidy(r, __dmul_rn(r, __fma_rn(-a.l, r, __fma_rn(-a.h, r, 1.0))));
 }
 
-// a times the power of two f, rounded to R
-template <typename R, typename E>
-__device__ __forceinline__ cx<R> rounded(const zc<E> &a, double f) {
-  return mk((R)(lead(a.re) * f), (R)(lead(a.im) * f));
+template <typename E> __device__ __forceinline__ zc<E> real_z(double a) { return {E(imag() ? 0.0 : a)}; }
+template <typename E> __device__ __forceinline__ zc<E> zadd(zc<E> a, zc<E> b) { return {add(a.v, b.v)}; }
+template <typename E> __device__ __forceinline__ zc<E> zneg(zc<E> a) { return {neg(a.v)}; }
+template <typename E> __device__ __forceinline__ zc<E> zsub(zc<E> a, zc<E> b) { return zadd(a, zneg(b)); }
+// a b (+ c): (re re) - (im im) in the even lane, (re im) + (im re) in the odd one
+template <typename E> __device__ __forceinline__ zc<E> zmul(zc<E> a, zc<E> b) {
+  const E ap = other(a.v);
+  return {fmadd(imag() ? ap : a.v, b.v, mul(imag() ? a.v : neg(ap), other(b.v)))};
+}
+template <typename E> __device__ __forceinline__ zc<E> zfma(zc<E> a, zc<E> b, zc<E> c) {
+  const E ap = other(a.v);
+  return {fmadd(imag() ? ap : a.v, b.v, fmadd(imag() ? a.v : neg(ap), other(b.v), c.v))};
+}
+template <typename E> __device__ __forceinline__ zc<E> zrecip(zc<E> a) {
+  const E p = other(a.v), r = mul(a.v, recip(fmadd(a.v, a.v, mul(p, p))));
+  return {imag() ? neg(r) : r};
 }
 
-// An element of the fused four-step apply's copy of level 0 (aao_internal.cuh):
-// element i of the run that starts at pair `first`; NULL: none.
-__device__ __forceinline__ void fuse_put(float4 *ft, int ell, int first, int i, cx<float> v) {
-  if (ft)
-    reinterpret_cast<float2 *>(ft + (size_t)(first + i / 2) * ell)[i & 1] = make_float2(v.re, v.im);
-}
-__device__ __forceinline__ void fuse_put(float4 *, int, int, int, cx<double>) {}
+// Where one frequency's entries of a level go; nowhere past the last frequency.
+template <typename R, int CH> struct Sink {
+  RecLev<R, CH> *V;
+  float4 *ft;   // the fused four-step apply's copy of level 0 (aao_internal.cuh), or NULL
+  int ell;
+  bool live;
+  // z times the power of two f, rounded to R; element i of the run that starts
+  // at pair `first` of the copy (-1: not in it)
+  template <typename E>
+  __device__ __forceinline__ void put(cx<R> *p, const zc<E> &z, double f, int first = -1, int i = 0) const {
+    if (!live) return;
+    const R v = (R)(lead(z.v) * f);
+    reinterpret_cast<R *>(p)[imag()] = v;
+    if (ft && first >= 0)
+      reinterpret_cast<float *>(ft + (size_t)(first + i / 2) * ell)[2 * (i & 1) + imag()] = (float)v;
+  }
+};
 
 // What role 0 (regular chunks) or 1 (last chunk) writes of level `level`.
 template <typename R, int CH, typename E>
-__device__ void entries(int role, int level, const BlockSymbol &sy, RecLev<R, CH> &V, int levels,
-                        const int *lsz, float4 *fuse, int ell, bool ragged) {
+__device__ void entries(int role, int level, const BlockSymbol &sy, const Sink<R, CH> &out, int levels,
+                        const int *lsz, bool ragged) {
   using Z = zc<E>;
   constexpr int c = CH - 1;
-  const cx<R> nil = mk((R)0, (R)0);
-  Z sig{E(sy.sig_re), E(sy.sig_im)}, a{E(-sy.e_re), E(-sy.e_im)};
+  const Z one = real_z<E>(1.0), nil = real_z<E>(0.0);
+  Z sig{E(imag() ? sy.sig_im : sy.sig_re)}, a{E(imag() ? -sy.e_im : -sy.e_re)};
   Z sig_l = sig, b = a;
   for (int l = 0;; l++) {
     const int cl = lsz[l] - (l + 1 < levels ? lsz[l + 1] : 0) * CH;
     const int N = role && cl == CH ? CH : c;
     Z D[CH + 1], H[CH + 1], A[CH + 1];   // A_i = a^i
-    D[0] = A[0] = {E(1.0), E(0.0)};
-    H[0] = {E(0.0), E(0.0)};
+    D[0] = A[0] = one;
+    H[0] = nil;
 #pragma unroll 1
     for (int i = 0; i < N; i++) {
       H[i + 1] = zfma(sig, D[i], zmul(a, H[i]));
@@ -146,7 +146,7 @@ __device__ void entries(int role, int level, const BlockSymbol &sy, RecLev<R, CH
       D[i + 1] = zfma(a, D[i], zadd(H[i + 1], A[i + 1]));
     }
     const Z x = zsub(sig_l, sig), delta = zadd(x, zsub(b, a));
-    auto det_l = [&](int i) { return i ? zfma(delta, D[i - 1], D[i]) : D[0]; };   // R_i
+    auto det_l = [&](int i) { return i ? zfma(delta, D[i - 1], D[i]) : one; };   // R_i
     const Z inv = zrecip(role && l == level ? det_l(cl) : D[c]);
     if (l < level) {
       const Z h = zmul(a, zmul(H[c], inv));
@@ -160,63 +160,53 @@ __device__ void entries(int role, int level, const BlockSymbol &sy, RecLev<R, CH
       a = zmul(zmul(a, A[c]), inv);
       continue;
     }
-    float4 *ft = l == 0 ? fuse : nullptr;
+    RecLev<R, CH> &V = *out.V;
+    const int tinv = ragged ? kFuseTailInv : -1, tgreen = ragged ? kFuseTailGreen : -1;
     if (role == 0) {
 #pragma unroll 1
       for (int i = 0; i < c; i++) {
         const Z p = zmul(D[i], zrecip(D[i + 1]));
-        const cx<R> ip = rounded<R>(p, sy.scale), bp = rounded<R>(zneg(zmul(a, p)), 1.0);
-        const cx<R> fc = rounded<R>(zmul(zmul(A[i + 1], D[c - 1 - i]), inv), 1.0);
-        V.invp[i] = ip;
-        V.bp[i] = bp;
-        V.fc[i] = fc;
-        fuse_put(ft, ell, 0, i, ip);
-        if (i < c - 1) fuse_put(ft, ell, 8, i, bp);
-        else fuse_put(ft, ell, 15, c, bp);
-        fuse_put(ft, ell, 15, i, fc);
-        if (i < cl - 1) {
-          V.invt[i] = ip;
-          if (ragged) fuse_put(ft, ell, kFuseTailInv, i, ip);
-        }
+        out.put(&V.invp[i], p, sy.scale, 0, i);
+        if (i < cl - 1) out.put(&V.invt[i], p, sy.scale, tinv, i);
+        out.put(&V.bp[i], zneg(zmul(a, p)), 1.0, i < c - 1 ? 8 : 15, i < c - 1 ? i : c);
+        out.put(&V.fc[i], zmul(zmul(A[i + 1], D[c - 1 - i]), inv), 1.0, 15, i);
       }
-      const cx<R> e = rounded<R>(zneg(a), 1.0 / sy.scale);
-      V.e = e;
-      fuse_put(ft, ell, 0, c, e);
-      V.invp[c] = V.bp[c] = V.fc[c] = V.pad = nil;
+      out.put(&V.e, zneg(a), 1.0 / sy.scale, 0, c);
+      out.put(&V.invp[c], nil, 1.0);
+      out.put(&V.bp[c], nil, 1.0);
+      out.put(&V.fc[c], nil, 1.0);
+      out.put(&V.pad, nil, 1.0);
     } else {
 #pragma unroll 1
       for (int i = 0; i < CH; i++) {
-        const cx<R> fl =
-            i < cl ? rounded<R>(zmul(zmul(A[i + 1], det_l(cl - 1 - i)), inv), 1.0) : nil;
-        V.fl[i] = fl;
-        if (ragged) fuse_put(ft, ell, kFuseTailGreen, i, fl);
-        if (i < cl - 1) continue;
-        const cx<R> last = i == cl - 1 ? rounded<R>(zmul(D[i], inv), sy.scale) : nil;
-        V.invt[i] = last;
-        if (ragged) fuse_put(ft, ell, kFuseTailInv, i, last);
+        out.put(&V.fl[i], i < cl ? zmul(zmul(A[i + 1], det_l(cl - 1 - i)), inv) : nil, 1.0, tgreen, i);
+        if (i >= cl - 1)
+          out.put(&V.invt[i], i == cl - 1 ? zmul(D[i], inv) : nil, i == cl - 1 ? sy.scale : 1.0, tinv, i);
       }
     }
     return;
   }
 }
 
-// grid (frequencies / 32, role + 2 level, FP64 or FP32 tables)
+// grid (frequencies / 16, role + 2 level, FP64 or FP32 tables)
 template <int CH64>
 __global__ void __launch_bounds__(32)
 k_tables(const BlockSymbol *__restrict__ sym, int nk, RecLev<float, 16> *__restrict__ tab32,
          int lev32, int4 lo32, int2 hi32, float4 *__restrict__ fuse, int ell, int L1, int ragged,
          RecLev<double, CH64> *__restrict__ tab64, int lev64, int4 lo64, int2 hi64) {
-  const int k = blockIdx.x * 32 + threadIdx.x, role = blockIdx.y & 1, level = blockIdx.y >> 1;
-  if (k >= nk) return;
+  const int q = blockIdx.x * 16 + threadIdx.x / 2, k = min(q, nk - 1);
+  const int role = blockIdx.y & 1, level = blockIdx.y >> 1;
   if (blockIdx.z == 0) {
     if (level >= lev64) return;
     const int lsz[kRecLevels] = {lo64.x, lo64.y, lo64.z, lo64.w, hi64.x, hi64.y};
-    entries<double, CH64, pair>(role, level, sym[k], tab64[(size_t)k * lev64 + level], lev64, lsz, nullptr, ell, false);
+    const Sink<double, CH64> out{tab64 + (size_t)k * lev64 + level, nullptr, ell, q < nk};
+    entries<double, CH64, pair>(role, level, sym[k], out, lev64, lsz, false);
   } else {
     if (level >= lev32) return;
     const int lsz[kRecLevels] = {lo32.x, lo32.y, lo32.z, lo32.w, hi32.x, hi32.y};
-    float4 *ft = fuse ? fuse + (size_t)(k % L1) * (ell / L1) + k / L1 : nullptr;
-    entries<float, 16, double>(role, level, sym[k], tab32[(size_t)k * lev32 + level], lev32, lsz, ft, ell, ragged);
+    float4 *ft = fuse && level == 0 ? fuse + (size_t)(k % L1) * (ell / L1) + k / L1 : nullptr;
+    const Sink<float, 16> out{tab32 + (size_t)k * lev32 + level, ft, ell, q < nk};
+    entries<float, 16, double>(role, level, sym[k], out, lev32, lsz, ragged != 0);
   }
 }
 
@@ -225,7 +215,7 @@ cudaError_t run_tables(const Ctx &c, cudaStream_t s) {
   auto lo = [](const int *v) { return make_int4(v[0], v[1], v[2], v[3]); };
   auto hi = [](const int *v) { return make_int2(v[4], v[5]); };
   const int levels = c.lev64 > c.lev32 ? c.lev64 : c.lev32;
-  k_tables<CH64><<<dim3((unsigned)((c.nk + 31) / 32), 2 * levels, 2), 32, 0, s>>>(
+  k_tables<CH64><<<dim3((unsigned)((c.nk + 15) / 16), 2 * levels, 2), 32, 0, s>>>(
       static_cast<const BlockSymbol *>(c.symbols), (int)c.nk, static_cast<RecLev<float, 16> *>(c.rec32),
       c.lev32, lo(c.lsz32), hi(c.lsz32), static_cast<float4 *>(c.fuse32), (int)c.ell,
       four_l1(c.ell), (c.n + 1) % 16 != 0 ? 1 : 0, static_cast<RecLev<double, CH64> *>(c.rec64),
