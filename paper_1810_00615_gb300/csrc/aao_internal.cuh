@@ -466,7 +466,9 @@ struct Ctx {
   int clu32 = 1, clu64 = 1;             // CTAs per row (cluster size) for rows beyond one CTA
   int cta32 = 0, cta64 = 0;             // threads per CTA in the cluster form
   int lsz32[kRecLevels] = {0}, lsz64[kRecLevels] = {0};   // unknowns per level
-  StepPlan step32{}, step64{};    // run-time four-step transforms (set by fft_plan)
+  StepPlan step32{}, step32r{}, step64{};   // run-time four-step transforms of the plain and
+                                            // refined FP32 and the FP64 apply (set by fft_plan)
+  const StepPlan &plan32() const { return refine ? step32r : step32; }
   cx<float> *tw32 = nullptr;      // exp(-2 pi i m/ell), m < ell
   cx<double> *tw64 = nullptr;
   float4 *tws32 = nullptr;        // the same with what the rounding left out: (re, im, re lo, im lo)
@@ -575,7 +577,7 @@ cudaError_t kernel_setup(const void *kern, int threads, size_t smem, int *reside
 // half spectrum; half spectrum -> y.  One instantiation per precision.
 // `inter` (may be NULL: single-kernel transform) is the scratch of the
 // four-step transforms, fft_inter_bytes_* bytes.
-void fft_plan(Ctx &c);   // sets c.step32 and c.step64 from c.ell
+void fft_plan(Ctx &c);   // sets the plans from c.ell and c.n
 cudaError_t fft_forward_f32(const Ctx &c, const double *x, const double *yprev, void *spec,
                             cudaStream_t s, void *inter = nullptr);
 cudaError_t fft_inverse_f32(const Ctx &c, const void *spec, double *y, cudaStream_t s,

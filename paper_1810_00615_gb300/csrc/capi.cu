@@ -1153,7 +1153,7 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
     cudaError_t e = upload((void **)&c.tw32, t32);
     if (e == cudaSuccess) e = upload((void **)&c.tw64, t64);
     if (e == cudaSuccess) e = upload((void **)&c.tws32, ts);
-    c.step32.tw32 = c.tws32;
+    c.step32.tw32 = c.step32r.tw32 = c.tws32;
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c.host_small, kSmall * sizeof(double));
     if (e != cudaSuccess) st = fail_cuda(c, e, "create");
   }

@@ -3,38 +3,44 @@
 
 namespace aao {
 void fft_plan(Ctx &c) {
-  fft::step_plan(c.ell, c.n, false, c.step32);
-  fft::step_plan(c.ell, c.n, true, c.step64);
+  fft::step_plan(c.ell, c.n, false, false, c.step32);
+  fft::step_plan(c.ell, c.n, false, true, c.step32r);
+  fft::step_plan(c.ell, c.n, true, false, c.step64);
 }
 cudaError_t fft_forward_f32(const Ctx &c, const double *x, const double *y, void *spec,
                             cudaStream_t s, void *inter) {
-  return fft::forward_any<float, double>(c.ell, c.step32, c.n, c.n_pad, x, y, c.sigk32,
+  return fft::forward_any<float, double>(c.ell, c.plan32(), c.n, c.n_pad, x, y, c.sigk32,
                                          static_cast<cx<float> *>(spec), c.tw32, s, inter);
 }
 cudaError_t fft_inverse_f32(const Ctx &c, const void *spec, double *y, cudaStream_t s,
                             void *inter, const float *base) {
-  return fft::inverse_any<float, double>(c.ell, c.step32, c.n, c.n_pad,
+  return fft::inverse_any<float, double>(c.ell, c.plan32(), c.n, c.n_pad,
                                          static_cast<const cx<float> *>(spec), y, c.tw32, s, inter,
                                          base);
 }
 cudaError_t fft_forward_f32_yf(const Ctx &c, const double *x, const float *y, void *spec,
                                cudaStream_t s, void *inter) {
-  return fft::forward_any<float, float>(c.ell, c.step32, c.n, c.n_pad, x, y, c.sigk32,
+  return fft::forward_any<float, float>(c.ell, c.plan32(), c.n, c.n_pad, x, y, c.sigk32,
                                         static_cast<cx<float> *>(spec), c.tw32, s, inter);
 }
-size_t fft_inter_bytes_f32(const Ctx &c) { return fft::inter_bytes_any<float>(c.ell, c.step32, c.n); }
+// (for both plans: one workspace serves every mode)
+size_t fft_inter_bytes_f32(const Ctx &c) {
+  const size_t a = fft::inter_bytes_any<float>(c.ell, c.step32, c.n);
+  const size_t b = fft::inter_bytes_any<float>(c.ell, c.step32r, c.n);
+  return a > b ? a : b;
+}
 bool fft_four_supported(const Ctx &c) { return fft::use_four<float>(c.ell); }
 bool fft_f32_input_supported(const Ctx &c) {
-  return fft::use_four<float>(c.ell) || c.step32.L;
+  return fft::use_four<float>(c.ell) || c.plan32().L;
 }
 cudaError_t fft_forward_f32_from_f32(const Ctx &c, const float *x, void *spec, cudaStream_t s,
                                      void *inter) {
-  return fft::forward_four_f32_input(c.ell, c.step32, c.n, c.n_pad, x, static_cast<cx<float> *>(spec),
+  return fft::forward_four_f32_input(c.ell, c.plan32(), c.n, c.n_pad, x, static_cast<cx<float> *>(spec),
                                      c.tw32, s, inter);
 }
 cudaError_t fft_inverse_f32_to_f32(const Ctx &c, const void *spec, float *y, cudaStream_t s,
                                    void *inter) {
-  return fft::inverse_any<float, float>(c.ell, c.step32, c.n, c.n_pad,
+  return fft::inverse_any<float, float>(c.ell, c.plan32(), c.n, c.n_pad,
                                         static_cast<const cx<float> *>(spec), y, c.tw32, s, inter);
 }
 

@@ -566,38 +566,69 @@ inline bool step_radices(int N, int *rad, int &np) {
 // amplifies it is about sqrt(L1) times that of a transform whose twiddles
 // come last; the refined apply squares that error.
 //
-// Large calls keep the compiled forms of fft_time.cuh and fft_mixed.cuh, which
-// spend fewer instructions per element once they fill the chip.  Powers of two
-// (row and panel kernels; whole apply, steps against them): FP32 n 65535 x ell
-// 64 83 / 61 us, 16383 x 128 59 / 50, but 8191 x 32 30 / 32 and 4095 x 128 28 /
-// 29; FP64 8191 x 128 162 / 146, 4095 x 256 159 / 126, 32767 x 256 937 / 800,
-// but 2047 x 256 93 / 114, 8191 x 512 449 / 478, 16383 x 1024 1704 / 1780; only
-// ell = 4096 turns again (8191: 3865 / 3791).  Other short lengths (one mixed-radix
-// kernel a direction): FP32 n 16383 x ell 20 38 / 33, 8191 x 40 31 / 26, but
-// refined 4095 x 30 49 / 56 and 32767 x 100 67 / 75; FP64 4095 x 40 67 / 62,
-// 16383 x 40 136 / 130, but 16383 x 100 200 / 208 and 65535 x 20 171 / 183.
-inline bool step_plan(int64_t ell, int64_t n, bool fp64, StepPlan &pl) {
+// Where n fills the chip with panels of 32 columns, the forms of fft_time.cuh
+// (powers of two: row and panel kernels) and fft_mixed.cuh (one kernel a
+// direction) can be the faster ones, which spend fewer instructions per element.
+// Whole applies, steps / the other form, on both sides of each line:
+//   FP32, powers of two up to 128: n ell = 480000 up to ell 32 (32: n 14000 1.00,
+//     15000 1.06, 16383 1.09; 16: 16383 0.99, 32767 1.05), 10^6 above (64: 10000
+//     0.98, 16383 1.06; 128: 7500 1.01, 8191 1.10).
+//   FP64, powers of two: n ell = 240000 at 16 (12000 1.00, 16383 1.08), 620000 up to
+//     64 (64: 8191 0.93, 10000 1.07; 32: 16383 1.00, 32767 1.06), 850000 up to 256
+//     (128: 6200 0.91, 7000 1.12; 256: 3071 0.93, 4000 1.25), never at 512 ... 2048
+//     (0.94 ... 1.00 up to n 65535), n = 4000 at 4096 (2500 0.94, 4000 1.01, 8191 1.02).
+//   Other lengths:
+//     FP32, ell <= 64 in at most three passes, n < 32767 (there 0.9 ... 1.05): n = 4000
+//       up to 40 (30: 3071 1.02, 4095 1.03, 5000 1.17), 5000 above (60: 4095 1.00,
+//       5000 1.04); up to 200 in no more passes than the steps take: n = 64 ell (96:
+//       5000 0.94, 6200 1.00, 8191 1.05; 120: 6200 0.94, 8191 1.02; 192: 8191 1.01,
+//       16383 1.06; n >= 32767 1.02 ... 1.13).
+//     FP32 refined, which has no FP32 residual with these kernels: n = 5000 (40: 4095
+//       0.98, 5000 1.12), 8000 (50: 6200 0.95, 8191 1.03) and 128 ell (96: 8191 0.94,
+//       16383 1.04), all n < 32767 (there 0.74 ... 1.05).
+//     FP64, ell <= 64 in at most three passes, none of 16 (48: 0.83 ... 0.97), n < 32767
+//       (there 0.82 ... 1.0): n = 3072 up to 50 (40: 2047 0.96, 4095 1.03, 16383 1.05),
+//       6000 above (60: 5000 1.00, 6143 1.04).
+//     FP64, 90 <= ell <= 192: where the panels fill the second wave of 152 SMs to
+//       three quarters (n = 7300 ... 9728: 1.01 ... 1.11, but 162 0.92; beside it, n 5500
+//       0.78 ... 0.91, 12000 0.84 ... 1.04).
+// `steps`: the passes of the four-step plan.
+inline bool panels_faster(int64_t ell, int64_t n, bool fp64, bool refined, int steps) {
+  const int64_t work = n * ell;
+  if ((ell & (ell - 1)) == 0) {
+    if (!fp64) return ell <= 128 && work >= (ell <= 32 ? 480000 : 1000000);
+    if (ell > 256) return ell == 4096 && n >= 4000;
+    return work >= (ell <= 16 ? 240000 : ell <= 64 ? 620000 : 850000);
+  }
+  const int64_t second = (n + 31) / 32 - 152;   // panels of the second wave
+  if (fp64 && ell >= 90) return ell <= 192 && 4 * second > 3 * 152 && second <= 152;
+  MixedPlan mp;
+  if (ell > 200 || !mixed_plan((int)ell, mp)) return false;
+  if (ell > 64) return !fp64 && mp.np <= steps && (refined ? n >= 128 * ell && n < 32767 : n >= 64 * ell);
+  if (mp.np > 3 || n >= 32767) return false;
+  if (!fp64) return n >= (ell <= 40 ? (refined ? 5000 : 4000) : (refined ? 8000 : 5000));
+  for (int p = 0; p < mp.np; p++)
+    if (mp.rad[p] == 16) return false;
+  return n >= (ell <= 50 ? 3072 : 6000);
+}
+
+inline bool step_plan(int64_t ell, int64_t n, bool fp64, bool refined, StepPlan &pl) {
   pl = StepPlan{};
   if (ell < AAO_STEPS_MIN) return false;
-  if ((ell & (ell - 1)) == 0) {
-    const bool big = n * ell > 1000000;
-    pl.split = fp64 ? (ell <= 256 && big) || (ell <= 512 && n >= 16383) || (ell == 4096 && n >= 4095)
-                    : ell <= 128 && (big || n >= 32767);
-    if (pl.split) return false;
-  } else if (n < 32767 && (fp64 ? ell <= 50 && n >= 3072 : ell <= 100 && n >= 6144)) {
+  const bool wide = !fp64 && ell >= 64;
+  StepPlan st{};
+  for (int64_t l1 = wide ? 8 : 1; l1 <= 128 && !st.L; l1++) {
+    if (ell % l1 || (wide ? ell / l1 > 64 : l1 * l1 < ell)) continue;
+    st.L1 = (int)l1;
+    st.L2 = (int)(ell / l1);
+    if (step_radices(st.L1, st.rad1, st.np1) && step_radices(st.L2, st.rad2, st.np2)) st.L = (int)ell;
+  }
+  if (!st.L || panels_faster(ell, n, fp64, refined, st.np1 + st.np2)) {
+    pl.split = (ell & (ell - 1)) == 0;
     return false;
   }
-  const bool wide = !fp64 && ell >= 64;
-  for (int64_t l1 = wide ? 8 : 1; l1 <= 128; l1++) {
-    if (ell % l1 || (wide ? ell / l1 > 64 : l1 * l1 < ell)) continue;
-    pl.L1 = (int)l1;
-    pl.L2 = (int)(ell / l1);
-    if (step_radices(pl.L1, pl.rad1, pl.np1) && step_radices(pl.L2, pl.rad2, pl.np2)) {
-      pl.L = (int)ell;
-      return true;
-    }
-  }
-  return false;
+  pl = st;
+  return true;
 }
 inline int64_t steps_ncx(int64_t n) { return ((n + 1) / 2 + kStepW - 1) / kStepW * kStepW; }
 template <typename R> size_t steps_inter_bytes(int64_t ell, int64_t n) {
