@@ -22,6 +22,12 @@
 // (75 + 52 us, with row passes of 7 and 21 us).  Here the same shapes give
 // 49 x 36 and 16 x 32 CTAs.
 // FP64 is bound by the FP64 pipe, FP32 by latency and issue.
+//
+// The kernels are launched as dependents but do not let their successors be
+// scheduled early: CTAs that wait beside the last ones cost more than their
+// prologues save (whole applies with the trigger / without, n 63 ... 65535 x ell
+// 16 ... 4096: 1.02 on average, n 1023 x ell 512 in FP64 1.19, n 1023 x ell 500 in
+// FP32 1.14, n 5000 x ell 40 0.92).
 #pragma once
 #include "fft_time.cuh"
 #include "fft_mixed.cuh"
@@ -321,7 +327,6 @@ k_steps_forward1(const XT *__restrict__ x, const YT *__restrict__ y, const R *__
       }
     }
   }
-  pdl_trigger();
   __syncthreads();
   S = dft_steps<R, -1>(S, S + rows * kStepW, ng, L1, pl.np1, pl.rad1, pl.L, tw);
 #pragma unroll 4
@@ -385,7 +390,6 @@ k_steps_forward2(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, int 
       if (q < rows) S[q * kStepW + lane] = d[u];
     }
   }
-  pdl_trigger();
   __syncthreads();
   S = dft_steps<R, -1>(S, S + rows * kStepW, 2 * gr.ng, pl.L2, pl.np2, pl.rad2, pl.L, tw);
   // the two packed real columns X = (Z_k + conj Z_{ell-k})/2, Y = (Z_k - conj
@@ -451,7 +455,6 @@ k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int 
       }
     }
   }
-  pdl_trigger();
   __syncthreads();
   S = dft_steps<R, +1>(S, S + rows * kStepW, 2 * gr.ng, pl.L2, pl.np2, pl.rad2, pl.L, tw);
 #pragma unroll 4
@@ -494,7 +497,6 @@ k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int
       if (q < rows) S[q * kStepW + lane] = d[u];
     }
   }
-  pdl_trigger();
   __syncthreads();
   S = dft_steps<R, +1>(S, S + rows * kStepW, ng, L1, pl.np1, pl.rad1, pl.L, tw);
   const R *Sf = reinterpret_cast<const R *>(S);
