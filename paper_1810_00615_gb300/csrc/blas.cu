@@ -674,14 +674,23 @@ static cudaError_t matvec_dots_dispatch(const Ctx &c, const XT *x, double *y, in
   case NBV * 8 + (TRV ? 4 : 0) + DKV:                                                    \
     run_fx<NBV, TRV, true, XT, false, DKV>(c, x, y, sub, v0, dpart, s);                  \
     break;
-#define AAO_MVD4(NBV, TRV) \
-  AAO_MVD(NBV, TRV, 0) AAO_MVD(NBV, TRV, 1) AAO_MVD(NBV, TRV, 2) AAO_MVD(NBV, TRV, 3)
+#define AAO_MVD3(NBV, TRV) AAO_MVD(NBV, TRV, 0) AAO_MVD(NBV, TRV, 1) AAO_MVD(NBV, TRV, 2)
   switch (key) {
-    AAO_MVD4(2, false) AAO_MVD4(2, true) AAO_MVD4(3, false) AAO_MVD4(3, true)
-    AAO_MVD4(4, false) AAO_MVD4(4, true)
-    default: return cudaErrorNotSupported;
+    AAO_MVD3(2, false) AAO_MVD3(2, true) AAO_MVD3(3, false) AAO_MVD3(3, true)
+    AAO_MVD3(4, false) AAO_MVD3(4, true)
+    default:
+      // the true residual's norm: of an FP64 solution only
+      if constexpr (sizeof(XT) == 8) {
+        switch (key) {
+          AAO_MVD(2, false, 3) AAO_MVD(2, true, 3) AAO_MVD(3, false, 3) AAO_MVD(3, true, 3)
+          AAO_MVD(4, false, 3) AAO_MVD(4, true, 3)
+          default: return cudaErrorNotSupported;
+        }
+        break;
+      }
+      return cudaErrorNotSupported;
   }
-#undef AAO_MVD4
+#undef AAO_MVD3
 #undef AAO_MVD
   const dim3 grid = mv_fx_grid(c);
   return finish(dpart, (int)(grid.x * grid.y), fx_dots(dk), out, s);

@@ -34,11 +34,15 @@ inline bool use_four(int64_t ell) {
          (ell & (ell - 1)) == 0;
 }
 
-// The row and panel kernels serve the powers of two that step_plan leaves
-// to them (large n): bytes of their panel-major intermediate.
+// The row and panel kernels serve the powers of two that step_plan may leave
+// to them (large n).
+template <typename R, int L>
+constexpr bool kSplitUsed = Split<R, L>::OK && (sizeof(R) == 4 ? L <= 128 : L <= 256 || L == 4096);
+
+// Bytes of their panel-major intermediate.
 template <typename R, int L>
 static size_t split_bytes(int64_t n) {
-  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+  if constexpr (kSplitUsed<R, L>) {
     const int W = 2 * Shape<R, L>::C;
     return (size_t)((n + W - 1) / W) * Split<R, L>::PANEL;
   }
@@ -51,7 +55,7 @@ static cudaError_t run_forward(const StepPlan &pl, int64_t n, int64_t n_pad, con
   using S = Shape<R, L>;
   const int W = 2 * S::C;
   const int np = (int)((n + W - 1) / W);
-  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+  if constexpr (kSplitUsed<R, L>) {
     if (inter && pl.split) {
       const int ncx = np * S::C;
       const dim3 g1((unsigned)((ncx + kRowThreads - 1) / kRowThreads), (unsigned)Split<R, L>::LR);
@@ -88,7 +92,7 @@ static cudaError_t run_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, con
   using S = Shape<R, L>;
   const int W = 2 * S::C;
   const int np = (int)((n + W - 1) / W);
-  if constexpr (Split<R, L>::OK && !(std::is_same<R, float>::value && L >= 256)) {
+  if constexpr (kSplitUsed<R, L>) {
     if (inter && pl.split) {
       cx<R> *ip = static_cast<cx<R> *>(inter);
       auto kern = k_fft_inverse_panels<R, L>;

@@ -161,7 +161,7 @@ __device__ __forceinline__ void rec_upper(cx<R> *const *B, const int *lsz, int l
 // shared memory.  SMALL: at most 256 threads (rows up to 4096), compiled for
 // AAO_TRI_MINB resident CTAs per SM so that the ell/2 + 1 frequencies take
 // fewer waves.  STAGE: the row fits in shared memory and moves through it;
-// otherwise (FP64 rows beyond 8191) each thread reads its chunk directly.
+// otherwise (FP64 rows beyond 11264, 200 KB) each thread reads its chunk directly.
 #ifndef AAO_TRI_MINB
 #define AAO_TRI_MINB 3
 #endif
@@ -577,8 +577,12 @@ static cudaError_t run_tridiag_rec(const Ctx &c, void *spec, const void *tab, in
   const size_t staged = upper + (size_t)P * CH * sizeof(cx<R>);
   const bool stage = staged <= 200 * 1024;
   const size_t smem = stage ? staged : upper;
-  auto kern = P <= 256 ? k_tridiag_rec<R, CH, true, true>
-                       : (stage ? k_tridiag_rec<R, CH, false, true> : k_tridiag_rec<R, CH, false, false>);
+  auto kern = k_tridiag_rec<R, CH, false, true>;
+  if constexpr (sizeof(R) == 8 && CH == 16) {   // n > 8191: 512 chunks and more
+    if (!stage) kern = k_tridiag_rec<R, CH, false, false>;
+  } else {                                      // at most 169 KB a row
+    if (P <= 256) kern = k_tridiag_rec<R, CH, true, true>;
+  }
   cudaError_t e = kernel_setup((const void *)kern, P, smem);
   if (e != cudaSuccess) { cudaGetLastError(); return e; }
   const int4 lo = make_int4(lsz[0], lsz[1], lsz[2], lsz[3]);
