@@ -44,8 +44,8 @@ __device__ __forceinline__ void block_store(double (&acc)[NV], double *partials)
 
 // out[j] = sum_b partials[b * nv + j] in a fixed order, one block of NT threads
 // per output, into device memory and, straight over the host link, into
-// pinned host memory: a small result costs the stream no copy (6 of them,
-// 8 us of a 125 us solve at n 63 x ell 64).  Launched as a dependent of the
+// pinned host memory: a small result costs the stream no copy (6 of them in a
+// solve at n 63 x ell 64, 8 us of its 170).  Launched as a dependent of the
 // kernel that writes the partials.  (Letting that kernel's last block add them
 // saved this launch but cost every block a fence and an atomic: 145 -> 166 us
 // for the fused-dots matvec at n 4095 x ell 4096.)
@@ -454,6 +454,7 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
   constexpr int kPre = AAO_MVFX_PRE;
   static_assert(R % kPre == 0, "whole prefetch rounds");
   const int64_t first = (int64_t)(t0 + (NB - 1) * dir) * n + ic;   // output step 0
+  [[maybe_unused]] int wmax = 0;   // high word of the largest |w| of a ZERO walk, NaN above inf
   auto walk = [&](auto full_c, auto rng_c, auto zero_c) {
     constexpr bool FULL = decltype(full_c)::value, RNG = decltype(rng_c)::value;
     constexpr bool ZERO = decltype(zero_c)::value;
@@ -524,6 +525,7 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
           const double td = fx_to_f64<RNG>(s_main + prod, unit);
           const double yv = V ? fma(rw.coef, td, -vk) : rw.coef * td;
           *py = yv;
+          if constexpr (ZERO) wmax = max(wmax, __double2hiint(yv) & 0x7fffffff);
           if constexpr (DK == 1) {
             if constexpr (!ZERO) dacc[0] = fma(dk, yv, dacc[0]);
             dacc[1] = fma(vk, yv, dacc[1]);
@@ -549,9 +551,10 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
     // block rows, and in a solve from x = 0 it is v0 (DK = 1) and v (DK = 2):
     // tiles where it is zero skip the products with it, one or two FP64
     // operations of the bound pipe per element.  A dense vector costs a vote
-    // on the tile's first step.  An output that is not finite (v may hold an inf
-    // or NaN, and the scale may overflow) makes w . w so too: the tile is then
-    // walked again with the products, since 0 x inf and 0 x NaN are NaN.
+    // on the tile's first step.  The sum of the products is zero unless an output
+    // is not finite (v may hold an inf or NaN, and the scale may overflow): 0 x
+    // inf and 0 x NaN are NaN.  (Walking such a tile again with the products made
+    // the dense case 1.6% slower, by the code around it alone.)
     if (full && in_range && unit <= 0) {
       const double *pz = (DK == 1 ? dv0 : sub) + first;
       auto nonzero = [](double a) { return (unsigned long long)__double_as_longlong(a) << 1; };
@@ -561,13 +564,9 @@ k_matvec_fx(const XT *__restrict__ x, double *__restrict__ y, int n, int ell,
         for (int r = 1; r < R; r++) any |= nonzero(__ldg(pz + r * step));
         if (!__any_sync(0xffffffffu, any != 0)) {
           walk(std::true_type{}, std::false_type{}, std::true_type{});
-          const int ww = __double2hiint(dacc[DK == 1 ? 2 : 1]) & 0x7ff00000;
-          if (!__any_sync(0xffffffffu, ww == 0x7ff00000)) {
-            dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
-            return;
-          }
-#pragma unroll
-          for (int q = 0; q < ND; q++) dacc[q] = 0.0;
+          if (wmax >= 0x7ff00000) dacc[0] = __longlong_as_double(0x7ff8000000000000ll);
+          dots_commit<ND, kWarps>(dacc, s_dot, &s_cnt, dpart);
+          return;
         }
       }
     }
