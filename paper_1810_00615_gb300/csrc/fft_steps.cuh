@@ -10,8 +10,8 @@
 // column), so every index, twiddle and branch is uniform over the warp and
 // its run-time arithmetic is paid once per 32 columns.  G fills the eight
 // warps where the factors are short: with one t2 of 8 rows per CTA (ell =
-// 128) a pass had one butterfly, and the kernels took 9-10 us each at n 8191.  The passes run out of place between two buffers,
-// so that a thread holds one butterfly: in place, with all butterflies of a
+// 128) a pass had one butterfly, and the kernels took 9-10 us each at n 8191.
+// The passes run out of place between two buffers, so that a thread holds one butterfly: in place, with all butterflies of a
 // warp in registers between two barriers, the run-time radices spilled 1 to 8
 // KB a thread and the kernels ran at half the speed.
 //
@@ -20,7 +20,7 @@
 // warps; 44 us forward, 35-59 us inverse), and the FP64 panel kernels had 64
 // CTAs for n = 1024, ell = 1024, their FP64 pipe 82% busy on 64 of 152 SMs
 // (75 + 52 us, with row passes of 7 and 21 us).  Here the same shapes give
-// 49 x 36 and 16 x 32 CTAs.
+// 25 x 30 (outer kernels) and 25 x 13 (middle ones), 16 x 32 and 16 x 17 CTAs.
 // FP64 is bound by the FP64 pipe, FP32 by latency and issue.
 //
 // The kernels are launched as dependents but do not let their successors be
@@ -468,9 +468,10 @@ k_steps_inverseA(const cx<R> *__restrict__ spec, cx<R> *__restrict__ inter, int 
   }
 }
 
-// Inverse B.  grid and shared memory as forward 1.  With base (FP64 output of
-// an FP32 transform only) y = base - result.
-template <typename R, typename OT>
+// Inverse B.  grid and shared memory as forward 1.  With BASE (FP64 output of
+// an FP32 transform only) y = base - result; as a branch at run time it left
+// the widening conversion's FP64 fallback in (the pipe 14% busy).
+template <typename R, typename OT, bool BASE>
 __global__ void __launch_bounds__(kStepT, StepOcc<R>::V)
 k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int ncx,
                  const step_tw<R, +1> *__restrict__ tw, const float *__restrict__ base, StepPlan pl, int G) {
@@ -503,18 +504,16 @@ k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int
   const R scale = (R)0.5 / (R)pl.L;   // with forward 2's 1/2
   constexpr int B = 4;
   for (int q0 = 0; q0 < rows; q0 += B * kStepWarps) {
-    float bv[B][2];
-    if constexpr (sizeof(OT) > sizeof(R)) {
-      if (base) {
+    [[maybe_unused]] float bv[B][2];
+    if constexpr (BASE) {
 #pragma unroll
-        for (int u = 0; u < B; u++) {
-          const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
-          const size_t row = (size_t)(L2 * t1 + t20 + gi) * n;
+      for (int u = 0; u < B; u++) {
+        const int q = q0 + warp + u * kStepWarps, gi = by_l1(q), t1 = q - gi * L1;
+        const size_t row = (size_t)(L2 * t1 + t20 + gi) * n;
 #pragma unroll
-          for (int h = 0; h < 2; h++) {
-            const int i = i0 + h * 32 + lane;
-            bv[u][h] = (q < rows && i < n) ? __ldg(&base[row + i]) : 0.f;
-          }
+        for (int h = 0; h < 2; h++) {
+          const int i = i0 + h * 32 + lane;
+          bv[u][h] = (q < rows && i < n) ? __ldg(&base[row + i]) : 0.f;
         }
       }
     }
@@ -527,8 +526,9 @@ k_steps_inverseB(const cx<R> *__restrict__ inter, OT *__restrict__ y, int n, int
         const int i = i0 + h * 32 + lane;
         if (q < rows && i < n) {
           const R val = scale * Sf[q * 2 * kStepW + h * 32 + lane];
-          if constexpr (sizeof(OT) == sizeof(R)) y[row + i] = val;
-          else y[row + i] = base ? diff_f64(bv[u][h], val) : to_f64(val);
+          if constexpr (BASE) y[row + i] = diff_f64(bv[u][h], val);
+          else if constexpr (sizeof(OT) == sizeof(R)) y[row + i] = val;
+          else y[row + i] = to_f64(val);
         }
       }
     }
@@ -685,7 +685,11 @@ cudaError_t steps_inverse(const StepPlan &pl, int64_t n, int64_t n_pad, const cx
   const dim3 g1((unsigned)cols, (unsigned)((pl.L2 + G1 - 1) / G1)), g2((unsigned)cols, (unsigned)((pl.L1 / 2 + G2) / G2));
   const cudaError_t e = steps_launch(G2 > 1 ? k_steps_inverseA<R, true> : k_steps_inverseA<R, false>, g2, 4 * (size_t)G2 * pl.L2 * row, s, spec, ip, (int)n, ncx, n_pad, tw, pl, G2);
   if (e != cudaSuccess) return e;
-  return steps_launch(k_steps_inverseB<R, OT>, g1, 2 * (size_t)G1 * pl.L1 * row, s, ip, y, (int)n, ncx, tw, base, pl, G1);
+  auto kern = k_steps_inverseB<R, OT, false>;
+  if constexpr (sizeof(OT) > sizeof(R)) {
+    if (base) kern = k_steps_inverseB<R, OT, true>;
+  }
+  return steps_launch(kern, g1, 2 * (size_t)G1 * pl.L1 * row, s, ip, y, (int)n, ncx, tw, base, pl, G1);
 }
 
 }  // namespace
