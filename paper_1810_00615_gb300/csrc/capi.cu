@@ -1075,8 +1075,8 @@ int solve_core(Ctx &c, int tr, const double *b, double *x, int m, double rtol, i
   return status;
 }
 
-// ell = 2^a 3^b 5^c: powers of two run the radix-16 kernels, the rest the
-// mixed-radix kernels.
+// ell = 2^a 3^b 5^c (the radices of every transform form; fft_dispatch.cuh says
+// which serves what).
 bool fft_length_ok(int64_t ell) {
   for (int64_t r : {2, 3, 5})
     while (ell % r == 0) ell /= r;

@@ -368,7 +368,8 @@ k_fft_forward(const double *__restrict__ x, const YT *__restrict__ y,
 // The single kernel above reads its panel as 2C doubles per time step, a
 // 32-64 byte piece of each of L rows far apart in memory, and that pattern
 // holds DRAM well below its streaming rate; its passes then run while the
-// DRAM idles.  For L >= 256 the forward transform is split instead:
+// DRAM idles.  For large n the forward transform is split instead (from L = 32;
+// panels_faster in fft_steps.cuh has the lines):
 //
 //  rows   the first Stockham pass (radix R1, Ns = 1: no twiddles) needs time
 //         steps j + r L/R1 of a column, r < R1.  A CTA takes one j and 256
@@ -495,7 +496,7 @@ k_fft_forward_panels(const cx<R> *__restrict__ inter, cx<R> *__restrict__ spec, 
 }
 
 // ------------------------------------------------ inverse in two kernels
-// Mirror of the forward split (L >= 256): a persistent panel kernel loads the
+// Mirror of the forward split: a persistent panel kernel loads the
 // half spectrum of its panel, extends it to the Hermitian full spectrum, runs
 // all Stockham passes but the last and stores its shared-memory image to the
 // panel-major intermediate; a row kernel runs the last radix-16 pass (whose
