@@ -129,7 +129,10 @@ int aao_set_steps(aao_ctx *ctx, const double *tau_steps_host);
  * product of two FP32 errors (about 1e-9 relative where FP32 alone gives
  * 3e-7), so FGMRES needs the iterations of the FP64 preconditioner at about
  * twice the cost of an FP32 apply.  The paper has no counterpart: it is a
- * choice of how to evaluate the Section 3 preconditioner on this hardware. */
+ * choice of how to evaluate the Section 3 preconditioner on this hardware.
+ * Entering FP64 mode builds the FP64 tables of the tridiagonal solves from the
+ * context's symbols (once, and again after a change of kappa or the steps in
+ * another mode) and waits for that; AAO_ECUDA if it fails. */
 int aao_set_precision(aao_ctx *ctx, int prec);
 
 /* How the per-frequency blocks cM_k M + cK K of P are solved (Section 3).

@@ -461,6 +461,8 @@ struct Ctx {
   void *symbols = nullptr; // BlockSymbol[nk]
   void *rec32 = nullptr;   // RecLev<float, ch32>[nk][lev32]; the transposed symbols are their conjugates
   void *rec64 = nullptr;   // RecLev<double, ch64>[nk][lev64]
+  bool rec64_current = false;             // built from symbols (in FP64 mode, and on entering it)
+  cudaStream_t setup_stream = nullptr;    // builds rec64 on entering FP64 mode
   void *fuse32 = nullptr;  // float4[kFusePairs(Ragged)][ell]: level-0 tables of the fused apply
   int lev32 = 1, lev64 = 1;             // levels of the recursive form
   int clu32 = 1, clu64 = 1;             // CTAs per row (cluster size) for rows beyond one CTA
@@ -603,9 +605,9 @@ cudaError_t fft_forward_f32_from_f32(const Ctx &c, const float *x, void *spec, c
                                      void *inter);
 cudaError_t fft_inverse_f32_to_f32(const Ctx &c, const void *spec, float *y, cudaStream_t s,
                                    void *inter = nullptr);
-// Build rec32, rec64 and fuse32 (sizes and level sizes set) from symbols.
+// Build rec64, or rec32 and fuse32, from symbols (level sizes set).
 size_t rec_table_bytes(const Ctx &c, bool fp64);
-cudaError_t launch_build_tables(const Ctx &c, cudaStream_t s);
+cudaError_t launch_build_tables(const Ctx &c, bool fp64, cudaStream_t s);
 cudaError_t launch_tridiag(const Ctx &c, void *spec, int prec, int transpose,
                            cudaStream_t s);
 // The FP32 apply with the tridiagonal solves folded into the four-step

@@ -253,7 +253,8 @@ cudaError_t upload_dst_tables(Ctx &c) {
   return e;
 }
 
-// (Re)compute everything that depends on kappa, the steps or tau.
+// (Re)compute everything that depends on kappa, the steps or tau; the caller
+// waits for the table kernel (settle).
 int refresh_constants(Ctx &c) {
   // per-frequency tridiagonal tables (tables.cu): the symbols here, scaled to
   // elements of order 1, the recursion on the device
@@ -274,6 +275,7 @@ int refresh_constants(Ctx &c) {
     sym[(size_t)k] = {s0.real() * f, s0.imag() * f, e0.real() * f, e0.imag() * f, f};
   }
   drop(&c.symbols);   // the constants are written in place from here on
+  c.rec64_current = false;
   AAO_CK(c, upload(&c.symbols, sym));
   AAO_CK(c, reserve(&c.rec32, aao::rec_table_bytes(c, false)));
   AAO_CK(c, reserve(&c.rec64, aao::rec_table_bytes(c, true)));
@@ -284,7 +286,11 @@ int refresh_constants(Ctx &c) {
     AAO_CK(c, reserve(&c.fuse32, bytes));
     AAO_CK(c, cudaMemsetAsync(c.fuse32, 0, bytes, nullptr));
   }
-  AAO_CK(c, aao::launch_build_tables(c, nullptr));
+  AAO_CK(c, aao::launch_build_tables(c, false, nullptr));
+  if (c.prec == AAO_PREC_FP64) {
+    AAO_CK(c, aao::launch_build_tables(c, true, nullptr));
+    c.rec64_current = true;
+  }
   // DST-in-space form: cM_k per frequency, (m_j, cK k_j) per mode
   if (c.space == AAO_SPACE_DST) AAO_CK(c, upload_dst_tables(c));
   // matvec K coefficients beta_t and Neumann coefficients (tau_t - tau) kappa / h
@@ -405,8 +411,33 @@ int refresh_constants(Ctx &c) {
   c.mv_o1 = a1 * mh;
   c.mv_d2 = (c.equation == AAO_WAVE_BD2) ? 4 * mh : 0.0;
   c.mv_o2 = (c.equation == AAO_WAVE_BD2) ? mh : 0.0;
-  AAO_CK(c, cudaStreamSynchronize(nullptr));   // the tables stand for every stream
   return AAO_OK;
+}
+
+// The FP64 tables, on entering FP64 mode (their pair arithmetic is most of the
+// time of a small context's set-up, and FP32 contexts never read them).  On a
+// stream of its own, which waits for nothing and may run beside a capture, as
+// setting the precision may always have been part of one.  No apply reads the
+// old tables any more: they are only stale after a change of constants, which
+// waited for them.
+int enter_fp64(Ctx &c) {
+  if (c.rec64_current) return AAO_OK;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaError_t e = cudaSuccess;
+  if (!c.setup_stream) e = cudaStreamCreateWithFlags(&c.setup_stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = aao::launch_build_tables(c, true, c.setup_stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c.setup_stream);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return fail_cuda(c, e, "set_precision");
+  c.rec64_current = true;
+  return AAO_OK;
+}
+
+// The constants stand for every stream.
+int settle(Ctx &c, int status) {
+  if (status == AAO_OK) AAO_CK(c, cudaStreamSynchronize(nullptr));
+  return status;
 }
 
 // Do [a, a + na) and [b, b + nb) intersect?
@@ -1150,11 +1181,13 @@ int aao_create(int64_t n, int64_t ell, double tau, int equation, aao_ctx **out) 
       ts[(size_t)m] = make_float4((float)co, (float)-si, (float)(co - (double)(float)co),
                                   (float)((double)(float)si - si));
     }
-    cudaError_t e = upload((void **)&c.tw32, t32);
+    // the pinned allocation while the table kernel runs; the copies wait for it
+    cudaError_t e = cudaMallocHost((void **)&c.host_small, kSmall * sizeof(double));
+    if (e == cudaSuccess) e = upload((void **)&c.tw32, t32);
     if (e == cudaSuccess) e = upload((void **)&c.tw64, t64);
     if (e == cudaSuccess) e = upload((void **)&c.tws32, ts);
     c.step32.tw32 = c.step32r.tw32 = c.tws32;
-    if (e == cudaSuccess) e = cudaMallocHost((void **)&c.host_small, kSmall * sizeof(double));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) st = fail_cuda(c, e, "create");
   }
   if (st != AAO_OK) {
@@ -1176,6 +1209,7 @@ void aao_destroy(aao_ctx *ctx) {
   if (c.ev_x) cudaEventDestroy(c.ev_x);
   if (c.ev_copy) cudaEventDestroy(c.ev_copy);
   if (c.copy_stream) cudaStreamDestroy(c.copy_stream);
+  if (c.setup_stream) cudaStreamDestroy(c.setup_stream);
   for (auto &p : c.pending) {
     cudaEventDestroy(p.a);
     cudaEventDestroy(p.b);
@@ -1188,7 +1222,7 @@ int aao_set_kappa(aao_ctx *ctx, double kappa) {
   if (!ctx || !(kappa > 0.0) || !std::isfinite(kappa)) return AAO_EINVAL;
   if (ctx->c.equation != AAO_HEAT) return AAO_EINVAL;
   ctx->c.kappa = kappa;
-  return refresh_constants(ctx->c);
+  return settle(ctx->c, refresh_constants(ctx->c));
 }
 
 int aao_set_steps(aao_ctx *ctx, const double *tau_steps_host) {
@@ -1204,12 +1238,14 @@ int aao_set_steps(aao_ctx *ctx, const double *tau_steps_host) {
     c.taus.assign(tau_steps_host, tau_steps_host + c.ell);
     c.variable_steps = true;
   }
-  return refresh_constants(c);
+  return settle(c, refresh_constants(c));
 }
 
 int aao_set_precision(aao_ctx *ctx, int prec) {
   if (!ctx || (prec != AAO_PREC_FP32 && prec != AAO_PREC_FP64 && prec != AAO_PREC_FP32_REFINED))
     return AAO_EINVAL;
+  const int st = prec == AAO_PREC_FP64 ? enter_fp64(ctx->c) : AAO_OK;
+  if (st != AAO_OK) return st;
   ctx->c.refine = prec == AAO_PREC_FP32_REFINED;
   ctx->c.prec = ctx->c.refine ? AAO_PREC_FP32 : prec;
   return AAO_OK;

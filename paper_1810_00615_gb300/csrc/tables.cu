@@ -16,7 +16,10 @@
 //   sigma' = sigma + 2a H_c/D_c,  sigma_L' = sigma + a H_c/D_c + a S_cl/R_cl,
 //   a' = a^{c+1} / D_c,           b' = a^cl b / R_cl.
 // No excess comes from a difference of diagonals, however nearly singular the
-// block is, and the chain has two quotients a level.
+// block is, and the chain has two quotients a level.  Pairs can afford such
+// differences and take the shorter recurrence D_{i+1} = (sigma + 2a) D_i - a^2
+// D_{i-1}, H_i = D_i - a D_{i-1} - a^i, off by some 2^-100 of a, which no solution
+// in FP64 can tell.
 //
 // The FP64 tables are formed in pairs of FP64 numbers and rounded once.  Their
 // errors are the same for every chunk of a row, so they add up: with tables
@@ -32,11 +35,13 @@
 // an instruction.  So a block takes one level, and walks the levels below it
 // for itself, and one of two roles: what belongs to the regular chunks, or to
 // the last one.
-// aao_set_kappa with its copies, against the host building the tables, and the
-// host before the recursion served every row: n 63 x ell 64 153 us (124, 229), n
-// 5000 x ell 300 279 (395, 300), n 1000 x ell 900 238 (934, 679), n 12345 x ell 4096
-// 726 (6867, 3535).  With a lane a frequency it was 175, 371, 310 and 678; with all
-// levels of a role in one thread besides 268, 542, 463 and 890.
+// aao_set_kappa with its copies, FP32 mode / FP64 mode too (the host building all
+// tables; the host before the recursion served every row): n 63 x ell 64 60 / 103 us
+// (120; 225), n 5000 x ell 300 85 / 202 (391; 307), n 1000 x ell 900 86 / 173 (931;
+// 694), n 12345 x ell 4096 168 / 527 (7180; 3591).  Few frequencies of long rows are
+// all latency: n 5000 x ell 16 79 / 195 (118; 110).  Both with one lane a number:
+// 175, 371, 310 and 678; with all levels of a role in one thread besides 268, 542,
+// 463 and 890.
 #include "aao_internal.cuh"
 
 namespace aao {
@@ -54,12 +59,14 @@ __device__ __forceinline__ double lead(double a) { return a; }
 __device__ __forceinline__ double neg(double a) { return -a; }
 __device__ __forceinline__ double add(double a, double b) { return a + b; }
 __device__ __forceinline__ double mul(double a, double b) { return a * b; }
-__device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double dot(double a, double b, double x, double y) { return fma(a, b, x * y); }
+__device__ __forceinline__ double dot(double a, double b, double x, double y, double c) { return fma(a, b, fma(x, y, c)); }
 __device__ __forceinline__ double recip(double a) { return 1.0 / a; }
 
 // Pairs: unevaluated sums h + l of two FP64 numbers, |l| at most half a unit of
 // h (Dekker; products split by FMA).  Rounded operations throughout: a
-// contracted product would undo the splitting.
+// contracted product would undo the splitting.  A chain of them costs its
+// latency here, so products are added up before the sum is put in order once.
 struct pair {
   double h, l;
   __device__ __forceinline__ pair() {}
@@ -69,40 +76,47 @@ struct pair {
 __device__ __forceinline__ pair other(pair a) { return {other(a.h), other(a.l)}; }
 __device__ __forceinline__ double lead(pair a) { return a.h; }
 __device__ __forceinline__ pair neg(pair a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ pair tidy(double h, double l) {           // |h| >= |l|
-  const double s = __dadd_rn(h, l);
-  return {s, __dsub_rn(l, __dsub_rn(s, h))};
+__device__ __forceinline__ pair tidy(pair a) {                                  // |h| >= |l|
+  const double s = __dadd_rn(a.h, a.l);
+  return {s, __dsub_rn(a.l, __dsub_rn(s, a.h))};
 }
-__device__ __forceinline__ pair add(pair a, pair b) {
+__device__ __forceinline__ pair loose(pair a, pair b) {                         // a + b, not tidy
   const double s = __dadd_rn(a.h, b.h), t = __dsub_rn(s, a.h);
   const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, t)), __dsub_rn(b.h, t));
-  return tidy(s, __dadd_rn(a.l, __dadd_rn(e, b.l)));
+  return {s, __dadd_rn(__dadd_rn(a.l, b.l), e)};
 }
-__device__ __forceinline__ pair mul(pair a, pair b) {
+__device__ __forceinline__ pair prod(pair a, pair b) {                          // a b, not tidy
   const double p = __dmul_rn(a.h, b.h);
-  return tidy(p, __fma_rn(a.l, b.h, __fma_rn(a.h, b.l, __fma_rn(a.h, b.h, -p))));
+  return {p, __dadd_rn(__fma_rn(a.h, b.h, -p), __fma_rn(a.l, b.h, __dmul_rn(a.h, b.l)))};
 }
-__device__ __forceinline__ pair fmadd(pair a, pair b, pair c) { return add(mul(a, b), c); }
+__device__ __forceinline__ pair add(pair a, pair b) { return tidy(loose(a, b)); }
+__device__ __forceinline__ pair mul(pair a, pair b) { return tidy(prod(a, b)); }
+__device__ __forceinline__ pair dot(pair a, pair b, pair x, pair y) {           // a b + x y
+  return tidy(loose(prod(a, b), prod(x, y)));
+}
+__device__ __forceinline__ pair dot(pair a, pair b, pair x, pair y, pair c) {   // a b + x y + c
+  return tidy(loose(loose(prod(a, b), prod(x, y)), c));
+}
 __device__ __forceinline__ pair recip(pair a) {
   const double r = 1.0 / a.h;
-  return tidy(r, __dmul_rn(r, __fma_rn(-a.l, r, __fma_rn(-a.h, r, 1.0))));
+  return tidy({r, __dmul_rn(r, __fma_rn(-a.l, r, __fma_rn(-a.h, r, 1.0)))});
 }
 
 template <typename E> __device__ __forceinline__ zc<E> real_z(double a) { return {E(imag() ? 0.0 : a)}; }
 template <typename E> __device__ __forceinline__ zc<E> zadd(zc<E> a, zc<E> b) { return {add(a.v, b.v)}; }
 template <typename E> __device__ __forceinline__ zc<E> zneg(zc<E> a) { return {neg(a.v)}; }
 template <typename E> __device__ __forceinline__ zc<E> zsub(zc<E> a, zc<E> b) { return zadd(a, zneg(b)); }
-// a b (+ c): (re re) - (im im) in the even lane, (re im) + (im re) in the odd one
+// a b (+ c): (re re) - (im im) in the even lane, (im re) + (re im) in the odd one
 template <typename E> __device__ __forceinline__ zc<E> zmul(zc<E> a, zc<E> b) {
   const E ap = other(a.v);
-  return {fmadd(imag() ? ap : a.v, b.v, mul(imag() ? a.v : neg(ap), other(b.v)))};
+  return {dot(imag() ? ap : a.v, b.v, imag() ? a.v : neg(ap), other(b.v))};
 }
 template <typename E> __device__ __forceinline__ zc<E> zfma(zc<E> a, zc<E> b, zc<E> c) {
   const E ap = other(a.v);
-  return {fmadd(imag() ? ap : a.v, b.v, fmadd(imag() ? a.v : neg(ap), other(b.v), c.v))};
+  return {dot(imag() ? ap : a.v, b.v, imag() ? a.v : neg(ap), other(b.v), c.v)};
 }
 template <typename E> __device__ __forceinline__ zc<E> zrecip(zc<E> a) {
-  const E p = other(a.v), r = mul(a.v, recip(fmadd(a.v, a.v, mul(p, p))));
+  const E p = other(a.v), r = mul(a.v, recip(dot(a.v, a.v, p, p)));
   return {imag() ? neg(r) : r};
 }
 
@@ -130,30 +144,46 @@ __device__ void entries(int role, int level, const BlockSymbol &sy, const Sink<R
                         const int *lsz, bool ragged) {
   using Z = zc<E>;
   constexpr int c = CH - 1;
+  constexpr bool PAIRS = sizeof(E) == 16;
   const Z one = real_z<E>(1.0), nil = real_z<E>(0.0);
   Z sig{E(imag() ? sy.sig_im : sy.sig_re)}, a{E(imag() ? -sy.e_im : -sy.e_re)};
   Z sig_l = sig, b = a;
   for (int l = 0;; l++) {
     const int cl = lsz[l] - (l + 1 < levels ? lsz[l + 1] : 0) * CH;
     const int N = role && cl == CH ? CH : c;
-    Z D[CH + 1], H[CH + 1], A[CH + 1];   // A_i = a^i
+    Z D[CH + 1], A[CH + 1], Hs[PAIRS ? 1 : CH + 1];   // A_i = a^i
     D[0] = A[0] = one;
-    H[0] = nil;
+    if constexpr (PAIRS) {
+      const Z d = zadd(sig, zadd(a, a)), q = zneg(zmul(a, a));
+      D[1] = d;
+      A[1] = a;
 #pragma unroll 1
-    for (int i = 0; i < N; i++) {
-      H[i + 1] = zfma(sig, D[i], zmul(a, H[i]));
-      A[i + 1] = zmul(a, A[i]);
-      D[i + 1] = zfma(a, D[i], zadd(H[i + 1], A[i + 1]));
+      for (int i = 1; i < N; i++) {
+        A[i + 1] = zmul(a, A[i]);
+        D[i + 1] = zfma(d, D[i], zmul(q, D[i - 1]));
+      }
+    } else {
+      Hs[0] = nil;
+#pragma unroll 1
+      for (int i = 0; i < N; i++) {
+        Hs[i + 1] = zfma(sig, D[i], zmul(a, Hs[i]));
+        A[i + 1] = zmul(a, A[i]);
+        D[i + 1] = zfma(a, D[i], zadd(Hs[i + 1], A[i + 1]));
+      }
     }
+    auto excess = [&](int i) {   // H_i
+      if constexpr (PAIRS) return i ? zsub(zfma(zneg(a), D[i - 1], D[i]), A[i]) : nil;
+      else return Hs[i];
+    };
     const Z x = zsub(sig_l, sig), delta = zadd(x, zsub(b, a));
     auto det_l = [&](int i) { return i ? zfma(delta, D[i - 1], D[i]) : one; };   // R_i
     const Z inv = zrecip(role && l == level ? det_l(cl) : D[c]);
     if (l < level) {
-      const Z h = zmul(a, zmul(H[c], inv));
+      const Z h = zmul(zmul(a, excess(c)), inv);
       if (role) {
         const Z invl = zrecip(det_l(cl));
-        const Z S = zfma(x, A[cl - 1], zfma(delta, H[cl - 1], H[cl]));
-        sig_l = zadd(sig, zfma(a, zmul(S, invl), h));
+        const Z S = zfma(x, A[cl - 1], zfma(delta, excess(cl - 1), excess(cl)));
+        sig_l = zadd(sig, zfma(zmul(a, S), invl, h));
         b = zmul(zmul(A[cl], b), invl);
       }
       sig = zadd(sig, zadd(h, h));
@@ -188,38 +218,25 @@ __device__ void entries(int role, int level, const BlockSymbol &sy, const Sink<R
   }
 }
 
-// grid (frequencies / 16, role + 2 level, FP64 or FP32 tables)
-template <int CH64>
+// grid (frequencies / 16, role + 2 level)
+template <typename R, int CH, typename E>
 __global__ void __launch_bounds__(32)
-k_tables(const BlockSymbol *__restrict__ sym, int nk, RecLev<float, 16> *__restrict__ tab32,
-         int lev32, int4 lo32, int2 hi32, float4 *__restrict__ fuse, int ell, int L1, int ragged,
-         RecLev<double, CH64> *__restrict__ tab64, int lev64, int4 lo64, int2 hi64) {
+k_tables(const BlockSymbol *__restrict__ sym, int nk, RecLev<R, CH> *__restrict__ tabs, int levels,
+         int4 lsz_lo, int2 lsz_hi, float4 *__restrict__ fuse, int ell, int L1, int ragged) {
   const int q = blockIdx.x * 16 + threadIdx.x / 2, k = min(q, nk - 1);
   const int role = blockIdx.y & 1, level = blockIdx.y >> 1;
-  if (blockIdx.z == 0) {
-    if (level >= lev64) return;
-    const int lsz[kRecLevels] = {lo64.x, lo64.y, lo64.z, lo64.w, hi64.x, hi64.y};
-    const Sink<double, CH64> out{tab64 + (size_t)k * lev64 + level, nullptr, ell, q < nk};
-    entries<double, CH64, pair>(role, level, sym[k], out, lev64, lsz, false);
-  } else {
-    if (level >= lev32) return;
-    const int lsz[kRecLevels] = {lo32.x, lo32.y, lo32.z, lo32.w, hi32.x, hi32.y};
-    float4 *ft = fuse && level == 0 ? fuse + (size_t)(k % L1) * (ell / L1) + k / L1 : nullptr;
-    const Sink<float, 16> out{tab32 + (size_t)k * lev32 + level, ft, ell, q < nk};
-    entries<float, 16, double>(role, level, sym[k], out, lev32, lsz, ragged != 0);
-  }
+  const int lsz[kRecLevels] = {lsz_lo.x, lsz_lo.y, lsz_lo.z, lsz_lo.w, lsz_hi.x, lsz_hi.y};
+  float4 *ft = fuse && level == 0 ? fuse + (size_t)(k % L1) * (ell / L1) + k / L1 : nullptr;
+  const Sink<R, CH> out{tabs + (size_t)k * levels + level, ft, ell, q < nk};
+  entries<R, CH, E>(role, level, sym[k], out, levels, lsz, ragged != 0);
 }
 
-template <int CH64>
-cudaError_t run_tables(const Ctx &c, cudaStream_t s) {
-  auto lo = [](const int *v) { return make_int4(v[0], v[1], v[2], v[3]); };
-  auto hi = [](const int *v) { return make_int2(v[4], v[5]); };
-  const int levels = c.lev64 > c.lev32 ? c.lev64 : c.lev32;
-  k_tables<CH64><<<dim3((unsigned)((c.nk + 15) / 16), 2 * levels, 2), 32, 0, s>>>(
-      static_cast<const BlockSymbol *>(c.symbols), (int)c.nk, static_cast<RecLev<float, 16> *>(c.rec32),
-      c.lev32, lo(c.lsz32), hi(c.lsz32), static_cast<float4 *>(c.fuse32), (int)c.ell,
-      four_l1(c.ell), (c.n + 1) % 16 != 0 ? 1 : 0, static_cast<RecLev<double, CH64> *>(c.rec64),
-      c.lev64, lo(c.lsz64), hi(c.lsz64));
+template <typename R, int CH, typename E>
+cudaError_t run_tables(const Ctx &c, void *tab, int levels, const int *lsz, void *fuse, cudaStream_t s) {
+  k_tables<R, CH, E><<<dim3((unsigned)((c.nk + 15) / 16), 2 * levels), 32, 0, s>>>(
+      static_cast<const BlockSymbol *>(c.symbols), (int)c.nk, static_cast<RecLev<R, CH> *>(tab), levels,
+      make_int4(lsz[0], lsz[1], lsz[2], lsz[3]), make_int2(lsz[4], lsz[5]), static_cast<float4 *>(fuse),
+      (int)c.ell, four_l1(c.ell), (c.n + 1) % 16 != 0 ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -230,8 +247,10 @@ size_t rec_table_bytes(const Ctx &c, bool fp64) {
   return (size_t)c.nk * c.lev64 * (c.ch64 == 8 ? sizeof(RecLev<double, 8>) : sizeof(RecLev<double, 16>));
 }
 
-cudaError_t launch_build_tables(const Ctx &c, cudaStream_t s) {
-  return c.ch64 == 8 ? run_tables<8>(c, s) : run_tables<16>(c, s);
+cudaError_t launch_build_tables(const Ctx &c, bool fp64, cudaStream_t s) {
+  if (!fp64) return run_tables<float, 16, double>(c, c.rec32, c.lev32, c.lsz32, c.fuse32, s);
+  return c.ch64 == 8 ? run_tables<double, 8, pair>(c, c.rec64, c.lev64, c.lsz64, nullptr, s)
+                     : run_tables<double, 16, pair>(c, c.rec64, c.lev64, c.lsz64, nullptr, s);
 }
 
 }  // namespace aao

@@ -36,3 +36,37 @@ def test_updated_context_equals_a_new_one(n, ell, prec):
         want = c.precond_apply(x)
         s.synchronize()
         assert all(torch.equal(o, want) for o in old)
+
+
+@pytest.mark.parametrize("n,ell", [(63, 64), (1000, 60), (9001, 16)])
+def test_constants_changed_in_another_precision(n, ell):
+    torch = need_gpu()
+    from paper_1810_00615_gb300 import AllAtOnce
+    x = to_dev(torch, rand_block(n, ell, 23))
+    a = AllAtOnce(n, ell, 1.0 / ell, precision="fp64", restart=1)
+    for kappa in (0.5, 3.0):
+        a.set_precision("fp32")
+        a.set_kappa(kappa)
+        a.set_precision("fp64")
+        b = AllAtOnce(n, ell, 1.0 / ell, precision="fp64", restart=1, kappa=kappa)
+        assert torch.equal(a.precond_apply(x), b.precond_apply(x))
+
+
+@pytest.mark.parametrize("n,ell", [(63, 64), (1000, 60)])
+def test_entering_fp64_inside_a_capture(n, ell):
+    """Setting the precision may be part of a stream capture."""
+    torch = need_gpu()
+    from paper_1810_00615_gb300 import AllAtOnce
+    x = to_dev(torch, rand_block(n, ell, 24))
+    b = AllAtOnce(n, ell, 1.0 / ell, precision="fp64", restart=1)
+    want = b.precond_apply(x)                  # and every kernel of it loaded
+    a = AllAtOnce(n, ell, 1.0 / ell, precision="fp32", restart=1)
+    y = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        a.set_precision("fp64")
+        a.precond_apply(x, out=y)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
