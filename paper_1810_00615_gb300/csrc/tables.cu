@@ -35,13 +35,13 @@
 // an instruction.  So a block takes one level, and walks the levels below it
 // for itself, and one of two roles: what belongs to the regular chunks, or to
 // the last one.
-// aao_set_kappa with its copies, FP32 mode / FP64 mode too (the host building all
-// tables; the host before the recursion served every row): n 63 x ell 64 60 / 103 us
-// (120; 225), n 5000 x ell 300 85 / 202 (391; 307), n 1000 x ell 900 86 / 173 (931;
-// 694), n 12345 x ell 4096 168 / 527 (7180; 3591).  Few frequencies of long rows are
-// all latency: n 5000 x ell 16 79 / 195 (118; 110).  Both with one lane a number:
-// 175, 371, 310 and 678; with all levels of a role in one thread besides 268, 542,
-// 463 and 890.
+// aao_set_kappa and a synchronise, FP32 modes / FP64 mode (the host building all
+// tables; the host before the recursion served every row): n 63 x ell 64 70 / 152 us
+// (131; 243), n 74 x ell 64 71 / 176 (135; 145), n 1000 x ell 900 98 / 237 (959;
+// 701), n 4095 x ell 4096 168 / 386 (4222; 10467), n 16383 x ell 64 87 / 340 (186;
+// 352): few frequencies are all latency, which the pairs' chains lengthen.  With
+// one lane a number n 63 x ell 64 and n 1000 x ell 900 took 175 and 310 in FP64
+// mode, with all levels of a role in one thread besides 268 and 463.
 #include "aao_internal.cuh"
 
 namespace aao {
